@@ -148,6 +148,9 @@ void set_band(LevelParams &p, const Camera *cam) {
     p.band_tlo = cam->band_tlo;
     p.band_thi = cam->band_thi;
     p.az_half = cam->az_half;
+    p.W = cam->W;
+    p.H = cam->H;
+    set_visit_params(p, cam->s.hfov_deg, cam->s.vfov_deg);
 }
 
 void set_pano_params(LevelParams &p, const Camera *cam, int32_t *pcnt) {
@@ -194,9 +197,10 @@ void launch_level_count_timed(mig_ctx *ctx, const LevelParams &p, int Ld, int co
     }
 }
 
-int steps_cap_for(const mig_ctx *ctx, int Lmax, int K, int W, int H, int mode) {
-    if (ctx->ray_count || mode == MIG_MODE_INTERVAL || mode == MIG_MODE_PANORAMIC) return 0;
-    return (int)steps_pairs((long long)std::max(1, Lmax) * K, W, H, ctx->steps_budget);
+StepsLayout steps_for(const mig_ctx *ctx, int Lmax, const mig_sensor &s, float voxel, int mode) {
+    if (ctx->ray_count || mode == MIG_MODE_INTERVAL || mode == MIG_MODE_PANORAMIC) return StepsLayout{};
+    return steps_layout(SensorDims{s.width, s.height, s.yaw_bins, range_q16(s.range_m, voxel)}, Lmax, ctx->steps_budget,
+                        ctx->voxel_pass != MIG_COUNT_PAIRS);
 }
 
 void prof_begin(mig_ctx *ctx, int kind, cudaEvent_t *a) {
@@ -442,7 +446,7 @@ mig_status mig_map_create(mig_ctx *ctx, int nx, int ny, int nz, float voxel_size
     m->ny = ny;
     m->nz = nz;
     m->grid_bytes = map_layout_bytes(nx, ny, nz, &m->nbx, &m->nby, &m->nbz);
-    if (m->grid_bytes >= ((size_t)1 << 32)) return fail(MIG_EINVAL, "map_create: padded grid above 2^32 voxels");
+    if (map_codes_bytes(nx, ny, nz) >= ((size_t)1 << 32)) return fail(MIG_EINVAL, "map_create: padded grid above 2^32 voxels");
     m->voxel = voxel_size_m;
     for (int a = 0; a < 3; ++a) m->origin[a] = origin_m ? origin_m[a] : 0.f;
     const size_t nvox = (size_t)nx * ny * nz;
@@ -465,6 +469,9 @@ mig_status mig_map_create(mig_ctx *ctx, int nx, int ny, int nz, float voxel_size
         launch_map_scatter(m->d_grid, m->nx, m->ny, m->nz, m->nbx, m->nby, tmp, 0, 0, 0, nx, ny, nz, ctx->stream);
         MIG_CUDA_TRY(cudaGetLastError());
         ctx->alloc.free(tmp, nvox, ctx->stream);
+    } else {
+        launch_brick_update(m->d_grid, nx, ny, nz, 0, 0, 0, nx, ny, nz, ctx->stream);
+        MIG_CUDA_TRY(cudaGetLastError());
     }
     MIG_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
     *out = m.release();
@@ -585,15 +592,16 @@ static mig_status eval_host(mig_map *m, int n, const int32_t *parent, const floa
     const size_t o_cnt = cv.take<int32_t>((size_t)n * K * 2);
     const size_t o_work = cv.take<int32_t>(L);
     const size_t o_arena = cv.take<uint32_t>((size_t)std::max(1, plan.n_internal) * WH);
+    const size_t o_dpyr = cv.take<uint2>((size_t)std::max(1, plan.n_internal) * hz_entries(cam->W, cam->H));
     const size_t o_stats = cv.take<unsigned long long>(kStatsCounters);
     const size_t o_pcnt = cv.take<int32_t>(pano ? (size_t)n * cam->pano_A * 2 : 1);
     int Lmax = 1;
     for (int d = 0; d < L; ++d) Lmax = std::max(Lmax, plan.level_off[d + 1] - plan.level_off[d]);
-    const int steps_cap = steps_cap_for(ctx, Lmax, K, cam->W, cam->H, mode);
-    const size_t o_steps = cv.take<char>(steps_region_bytes(steps_cap, WH));
+    const StepsLayout steps = steps_for(ctx, Lmax, *sensor, m->voxel, mode);
+    const size_t o_steps = cv.take<char>(steps.bytes);
     // instrumented pass: the ray-by-ray count kernel is re-run into scratch counters afterwards,
     // for the method's own work counts (rays, DDA steps, owner tests) and as a cross-check
-    const bool rerun = stats && steps_cap > 0;
+    const bool rerun = stats && steps.cap > 0;
     const size_t o_cnt2 = cv.take<int32_t>(rerun ? (size_t)n * K * 2 + L : 1);
     char *dev = nullptr;
     st = ctx_workspace(ctx, cv.off, (void **)&dev);
@@ -636,14 +644,12 @@ static mig_status eval_host(mig_map *m, int n, const int32_t *parent, const floa
     p.bounds_err = ctx->d_err + 16;  // checked build: out-of-buffer indices are recorded here
     MIG_CUDA_TRY(cudaMemsetAsync(p.bounds_err, 0, 4, ctx->stream));
 #endif
-    p.steps = steps_cap ? (uint16_t *)(dev + o_steps) : nullptr;
-    p.vctr = steps_counter((uint16_t *)(dev + o_steps), steps_cap, WH);
-    p.steps_cap = steps_cap;
+    if (steps.cap) set_steps(p, dev + o_steps, steps);
+    p.dpyr = (uint2 *)(dev + o_dpyr);
     if (stats) {
         p.stats = (unsigned long long *)(dev + o_stats);
         MIG_CUDA_TRY(cudaMemsetAsync(p.stats, 0, kStatsCounters * sizeof(unsigned long long), ctx->stream));
     }
-    const int cap = ctx->num_sms * 16;
     const int count_cap = ctx->num_sms * std::min(ctx->count_ctas, std::max(1, (int)ctx->tiles.ctas_per_sm));
     uint64_t n_count = 0, n_render = 0;
     for (int d = 0; d < L; ++d) {
@@ -652,10 +658,10 @@ static mig_status eval_host(mig_map *m, int n, const int32_t *parent, const floa
         launch_level_count_timed(ctx, p, Ld, count_cap);
         timed_launch(ctx, kProfSelect,
                      [&] { launch_select(p, std::max(1, std::min((Ld + 127) / 128, 1024)), ctx->stream); });
-        const int ritems = plan.level_int[d] * render_tiles(p.W, p.H);
-        if (ritems > 0) timed_launch(ctx, kProfRender, [&] { launch_render(p, std::min(ritems, cap), ctx->stream); });
+        const int inner = plan.level_int[d];
+        if (inner > 0) timed_launch(ctx, kProfRender, [&] { launch_render(p, inner, ctx->num_sms, ctx->stream); });
         n_count++;
-        n_render += ritems > 0;
+        n_render += inner > 0;
     }
     std::vector<int32_t> cnt_rerun;
     if (rerun) {
@@ -773,10 +779,11 @@ mig_status mig_tree_eval_device(mig_map *m, int n, const int32_t *parent, const 
     const size_t o_anc = cv.take<int32_t>(std::max<size_t>(1, (size_t)n * max_depth)), o_node = cv.take<int4>(n);
     const size_t o_sel = cv.take<int32_t>(n);
     const size_t o_arena = cv.take<uint32_t>((size_t)n * WH);
+    const size_t o_dpyr = cv.take<uint2>((size_t)n * hz_entries(cam->W, cam->H));
     // level sizes are known on the device only: the step-count buffer is sized for n nodes (its
     // chunks beyond a level's pairs return at once)
-    const int steps_cap = steps_cap_for(ctx, n, K, cam->W, cam->H, MIG_MODE_MARGINAL);
-    const size_t o_steps = cv.take<char>(steps_region_bytes(steps_cap, WH));
+    const StepsLayout steps = steps_for(ctx, n, *sensor, m->voxel, MIG_MODE_MARGINAL);
+    const size_t o_steps = cv.take<char>(steps.bytes);
     char *dev = nullptr;
     st = ctx_workspace(ctx, cv.off, (void **)&dev);
     if (st != MIG_OK) return st;
@@ -828,17 +835,15 @@ mig_status mig_tree_eval_device(mig_map *m, int n, const int32_t *parent, const 
     p.arena = (uint32_t *)(dev + o_arena);
     p.mode = MIG_MODE_MARGINAL;
     p.max_anc = std::max(1, max_depth);
-    p.steps = steps_cap ? (uint16_t *)(dev + o_steps) : nullptr;
-    p.vctr = steps_counter((uint16_t *)(dev + o_steps), steps_cap, WH);
-    p.steps_cap = steps_cap;
-    const int cap = ctx->num_sms * 16;
+    if (steps.cap) set_steps(p, dev + o_steps, steps);
+    p.dpyr = (uint2 *)(dev + o_dpyr);
     const int count_cap = ctx->num_sms * std::min(ctx->count_ctas, std::max(1, (int)ctx->tiles.ctas_per_sm));
     const int sel_grid = std::max(1, std::min((n + 127) / 128, 1024));
     for (int d = 0; d < L; ++d) {
         p.lvl = d;
         launch_level_count_timed(ctx, p, n, count_cap);
         timed_launch(ctx, kProfSelect, [&] { launch_select(p, sel_grid, ctx->stream); });
-        timed_launch(ctx, kProfRender, [&] { launch_render(p, cap, ctx->stream); });
+        timed_launch(ctx, kProfRender, [&] { launch_render(p, n, ctx->num_sms, ctx->stream); });
     }
     MIG_CUDA_TRY(cudaGetLastError());
     return MIG_OK;

@@ -606,7 +606,7 @@ mig_status batch_run_streams(mig_ctx *ctx, std::vector<BatchItem> &items) {
     const mig_tile_config tc = ctx->tiles;
     Carve cv;
     struct TreeOff {
-        size_t node, ar, anc, loff, lint, lnodes, cnt, work, sel, out, arena, pcnt;
+        size_t node, ar, anc, loff, lint, lnodes, cnt, work, sel, out, arena, dpyr, pcnt;
     };
     std::vector<TreeOff> to(T);
     for (int t = 0; t < T; ++t) {
@@ -630,6 +630,7 @@ mig_status batch_run_streams(mig_ctx *ctx, std::vector<BatchItem> &items) {
     for (int t = 0; t < T; ++t) {
         to[t].sel = cv.take(4 * (size_t)items[t].plan.n);
         to[t].arena = cv.take(4 * (size_t)std::max(1, items[t].plan.n_internal) * items[t].cam->W * items[t].cam->H);
+        to[t].dpyr = cv.take(sizeof(uint2) * (size_t)std::max(1, items[t].plan.n_internal) * hz_entries(items[t].cam->W, items[t].cam->H));
         to[t].pcnt = items[t].mode == MIG_MODE_PANORAMIC ? cv.take(8 * (size_t)items[t].plan.n * items[t].cam->pano_A) : 0;
     }
     // longest trees first, round-robin over the stream pool; the trees of one stream run one after
@@ -638,16 +639,15 @@ mig_status batch_run_streams(mig_ctx *ctx, std::vector<BatchItem> &items) {
     std::vector<int> order(T);
     for (int t = 0; t < T; ++t) order[t] = t;
     std::sort(order.begin(), order.end(), [&](int a, int c) { return items[a].plan.n > items[c].plan.n; });
-    std::vector<int> steps_cap(T, 0);
+    std::vector<StepsLayout> steps(T);
     std::vector<size_t> stream_steps(S, 0);
     for (int oi = 0; oi < T; ++oi) {
         const int t = order[oi];
         const HostPlan &pl = items[t].plan;
         int Lmax = 1;
         for (int d = 0; d <= pl.max_depth; ++d) Lmax = std::max(Lmax, pl.level_off[d + 1] - pl.level_off[d]);
-        steps_cap[t] = steps_cap_for(ctx, Lmax, items[t].cam->K, items[t].cam->W, items[t].cam->H, items[t].mode);
-        stream_steps[oi % S] = std::max(stream_steps[oi % S],
-                                        steps_region_bytes(steps_cap[t], (size_t)items[t].cam->W * items[t].cam->H));
+        steps[t] = steps_for(ctx, Lmax, items[t].sensor, items[t].map->voxel, items[t].mode);
+        stream_steps[oi % S] = std::max(stream_steps[oi % S], steps[t].bytes);
     }
     std::vector<size_t> o_steps(S);
     for (int i = 0; i < S; ++i) o_steps[i] = cv.take(std::max<size_t>(stream_steps[i], 1));
@@ -699,6 +699,7 @@ mig_status batch_run_streams(mig_ctx *ctx, std::vector<BatchItem> &items) {
         p.out_abs = (int32_t *)(dev + to[t].out);
         p.out_marg = p.out_abs + n;
         p.out_yaw = p.out_abs + 2 * (size_t)n;
+        p.dpyr = (uint2 *)(dev + to[t].dpyr);
         p.mode = it.mode;
         p.max_anc = std::max(1, pl.max_depth);
         if (it.mode == MIG_MODE_PANORAMIC) set_pano_params(p, it.cam, (int32_t *)(dev + to[t].pcnt));
@@ -706,11 +707,8 @@ mig_status batch_run_streams(mig_ctx *ctx, std::vector<BatchItem> &items) {
     }
     for (int oi = 0; oi < T; ++oi) {
         const int t = order[oi];
-        lp[t].steps = steps_cap[t] ? (uint16_t *)(dev + o_steps[oi % S]) : nullptr;
+        if (steps[t].cap) set_steps(lp[t], dev + o_steps[oi % S], steps[t]);
         lp[t].voxel_pass = ctx->voxel_pass;
-        lp[t].vctr = steps_counter((uint16_t *)(dev + o_steps[oi % S]), steps_cap[t],
-                                   (size_t)items[t].cam->W * items[t].cam->H);
-        lp[t].steps_cap = steps_cap[t];
     }
     if (!ctx->batch) ctx->batch = new mig_ctx::Batch();
     mig_ctx::Batch *B = ctx->batch;
@@ -724,7 +722,6 @@ mig_status batch_run_streams(mig_ctx *ctx, std::vector<BatchItem> &items) {
     }
     if (!B->fork) MIG_CUDA_TRY(cudaEventCreateWithFlags(&B->fork, cudaEventDisableTiming));
     cudaStream_t s0 = ctx->stream;
-    const int cap = ctx->num_sms * 16;
     const int count_cap = ctx->num_sms * std::min(ctx->count_ctas, std::max(1, (int)ctx->tiles.ctas_per_sm));
     auto enqueue = [&]() -> cudaError_t {
         cudaError_t e = cudaMemcpyAsync(dev, host, up_bytes, cudaMemcpyHostToDevice, s0);
@@ -736,13 +733,12 @@ mig_status batch_run_streams(mig_ctx *ctx, std::vector<BatchItem> &items) {
             cudaStream_t s = B->pool[oi % S];
             LevelParams p = lp[t];
             const HostPlan &pl = items[t].plan;
-            const int rt = render_tiles(p.W, p.H);
             for (int d = 0; d <= pl.max_depth; ++d) {
                 p.lvl = d;
                 const int Ld = pl.level_off[d + 1] - pl.level_off[d];
                 launch_level_count(ctx, p, Ld, count_cap, s);
                 launch_select(p, std::max(1, std::min((Ld + 127) / 128, 1024)), s);
-                if (pl.level_int[d] > 0) launch_render(p, std::min(pl.level_int[d] * rt, cap), s);
+                if (pl.level_int[d] > 0) launch_render(p, pl.level_int[d], ctx->num_sms, s);
             }
             e = cudaGetLastError();
         }

@@ -1,5 +1,5 @@
 // Device kernels: fused per-level count (3D DDA + owner test + ancestor depth test + integer
-// reductions), yaw selection, depth-buffer render, map brick scatter/gather, device planning.
+// reductions), yaw selection, map scatter/gather, device planning.
 //
 // All result-deciding arithmetic is integer (the fixed-point reading of Sec. IV-A..C):
 // positions Q16 voxel units, ray directions Q30, projection rows Q16, depths Q16.16.
@@ -8,10 +8,10 @@
 #include <algorithm>
 #include <cstdint>
 
+#include "bricks.cuh"
 #include "dev_path.cuh"
 #include "kernels.h"
 #include "mig.h"
-#include "voxcount.cuh"
 #include "voxcount.h"
 
 namespace mig {
@@ -48,36 +48,6 @@ __global__ void select_kernel(const LevelParams p) {
     const int L = p.level_off[p.lvl + 1] - l0;
     for (int li = blockIdx.x * blockDim.x + threadIdx.x; li < L; li += gridDim.x * blockDim.x)
         select_node(p, p.level_nodes[l0 + li]);
-}
-
-// ------------------------------------------------------------------------------ render kernel
-// Depth buffer of the selected yaw (Sec. IV-A): per pixel ray, camera z of the entry point of
-// the first occupied voxel, else of the range endpoint. Only nodes with children (the level's
-// first level_int nodes) are rendered; descendants read them in the ancestor test.
-template <bool STATS>
-__global__ void __launch_bounds__(256) render_kernel(const LevelParams p) {
-    constexpr int RT = 16;  // render tile: 16 x 16 pixels, one ray per thread
-    const int l0 = p.level_off[p.lvl];
-    const int Li = p.level_int[p.lvl];
-    const int rtx = (p.W + RT - 1) / RT;
-    const int rtiles = rtx * ((p.H + RT - 1) / RT);
-    const int items = Li * rtiles;
-    const int tid = threadIdx.x;
-    for (int item = blockIdx.x; item < items; item += gridDim.x) {
-        const int tile = item % rtiles;
-        const int li = item / rtiles;
-        const int n = p.level_nodes[l0 + li];
-        const int4 nd = p.node[n];
-        if (nd.w < 0) continue;
-        const int ti = (tile % rtx) * RT + tid % RT;
-        const int tj = (tile / rtx) * RT + tid / RT;
-        if (ti >= p.W || tj >= p.H) continue;
-        const uint32_t st_steps = render_pixel(p, n, nd, ti, tj);
-        if constexpr (STATS) {
-            atomicAdd(p.stats + 6, 1ull);
-            atomicAdd(p.stats + 7, (unsigned long long)st_steps);
-        }
-    }
 }
 
 // ------------------------------------------------------------------------------- map kernels
@@ -203,14 +173,16 @@ void launch_count(const LevelParams &p, int grid, cudaStream_t s) {
     else count_kernel<false><<<grid, kWarps * 32, smem, s>>>(p);
 }
 
+size_t map_codes_bytes(int nx, int ny, int nz) { return occ_summary_end(nx, ny, nz); }
+
 size_t map_layout_bytes(int nx, int ny, int nz, int *nbx, int *nby, int *nbz) {
     *nbx = (nx + 7) / 8;
     *nby = (ny + 7) / 8;
     *nbz = (nz + 7) / 8;
 #if MIG_LAYOUT == 1
-    // voxel codes, then (256-byte aligned) one occupancy byte per 8x8x8 brick and (256-byte aligned)
-    // one per 32x32x32 super-brick
-    return occ_summary_end(nx, ny, nz);
+    // voxel codes, then (each 256-byte aligned) one occupancy byte per 8x8x8 brick and one per 32x32x32
+    // super-brick, and the masks and distances of the 4x4x4 bricks
+    return brick_data_end(nx, ny, nz);
 #else
     return (size_t)*nbx * *nby * *nbz * 512;
 #endif
@@ -227,19 +199,14 @@ int count_ctas_per_sm() {
     return std::max(1, std::min(a, b));
 }
 void launch_select(const LevelParams &p, int grid, cudaStream_t s) { select_kernel<<<grid, 128, 0, s>>>(p); }
-void launch_render(const LevelParams &p, int grid, cudaStream_t s) {
-    if (p.stats) render_kernel<true><<<grid, 256, 0, s>>>(p);
-    else render_kernel<false><<<grid, 256, 0, s>>>(p);
-}
-
-int render_tiles(int W, int H) { return ((W + 15) / 16) * ((H + 15) / 16); }
 void launch_map_scatter(uint8_t *bricks, int nx, int ny, int nz, int nbx, int nby, const uint8_t *box, int x0, int y0,
                         int z0, int dx, int dy, int dz, cudaStream_t s) {
     const size_t total = (size_t)dx * dy * dz;
     const int grid = (int)std::min<size_t>((total + 255) / 256, 4096);
     map_scatter_kernel<<<grid, 256, 0, s>>>(bricks, nx, ny, nbx, nby, box, x0, y0, z0, dx, dy, dz);
 #if MIG_LAYOUT == 1
-    launch_bocc(bricks, nx, ny, nz, x0, y0, z0, dx, dy, dz, s);  // the occupancy bytes of the bricks it touched
+    launch_bocc(bricks, nx, ny, nz, x0, y0, z0, dx, dy, dz, s);  // the summaries of the bricks it touched
+    launch_brick_update(bricks, nx, ny, nz, x0, y0, z0, dx, dy, dz, s);
 #else
     (void)nz;
 #endif

@@ -15,6 +15,17 @@ struct GridView {
     int nbx, nby;
 };
 
+// A brick that the per-node pass leaves to its voxel stage: unknown voxels, those an ancestor is known
+// to observe, the ancestors (bit = place in the node's list) still to test, and by yaw (bit = yaw -
+// first) those that count every unknown voxel, those undecided, and of these the ones whose voxels
+// need the test against the owner ray's first hit, and against the owner ray itself. brick: x | y << 10 |
+// z << 20 (4x4x4 bricks); node: its place in the chunk | first yaw / 64 << kRecNodeBits.
+struct BrickRec {
+    uint64_t U, O, anc, all, part, rch, vis;
+    uint32_t brick, node;
+};
+constexpr int kRecNodeBits = 27;
+
 // One tree level's work (Sec. IV-C): the nodes level_nodes[level_off[lvl] ..), the first
 // level_int[lvl] of which have children and need their depth buffer rendered.
 struct LevelParams {
@@ -53,23 +64,35 @@ struct LevelParams {
     // owned-voxel count (voxcount.cu): per-ray DDA step counts of a chunk of (node, yaw) pairs
     // [q0, q1) of the level, steps_cap pairs of W * H each; NULL = the ray-by-ray count kernel
     uint16_t *steps;
-    int32_t *vctr;  // work counter of the voxel pass (zeroed by the cast launch before it)
+    int32_t *vctr;  // [0] work counter of the voxel pass, [1] records queued, [2] records handed out
+                    // (zeroed by the cast launch before it)
     int steps_cap;
     int q0, q1;
     // per-node voxel pass: the frustum's elevation band (tangents) and azimuth half-width
     float band_tlo, band_thi, az_half;
     int voxel_pass;  // MIG_COUNT_AUTO, MIG_COUNT_PAIRS or MIG_COUNT_NODES
+    // bounds of the step counts (hz, pairs of the chunk) and of the depth buffers (dpyr, arena slots)
+    // over pixel tiles, hz_entries(W, H) each; dpyr NULL: not kept
+    uint32_t *hz;
+    uint2 *dpyr;
+    BrickRec *queue;  // per-node pass: undecided bricks of the chunk
+    int queue_cap;
+    // per-node pass: half a pixel at unit depth along the image axes, the depth below which the owner
+    // ray certainly visits its voxel, and the reciprocal focal lengths (set_visit_params)
+    float vis_hu, vis_hv, vis_zl2, ifx, ify;
 };
 
 void launch_count(const LevelParams &p, int grid, cudaStream_t s);
 int count_ctas_per_sm();  // resident CTAs per SM of the count kernel
 void launch_select(const LevelParams &p, int grid, cudaStream_t s);
-void launch_render(const LevelParams &p, int grid, cudaStream_t s);
-int render_tiles(int W, int H);  // 16x16 pixel tiles of the render pass
-// Writes a box of voxel codes into a grid of nx * ny * nz and refreshes the brick occupancy bytes
-// of the bricks it touches.
+void launch_render(const LevelParams &p, int nodes, int num_sms, cudaStream_t s);  // nodes: at least the level's internal ones
+void set_visit_params(LevelParams &p, float hfov_deg, float vfov_deg);  // the vis_* fields, from p.W and p.H
+// Writes a box of voxel codes into a grid of nx * ny * nz and refreshes the occupancy bytes, masks
+// and distances of the bricks it touches.
 void launch_map_scatter(uint8_t *bricks, int nx, int ny, int nz, int nbx, int nby, const uint8_t *box, int x0, int y0,
                         int z0, int dx, int dy, int dz, cudaStream_t s);
+// device bytes of an nx*ny*nz grid's voxel codes and occupancy bytes
+size_t map_codes_bytes(int nx, int ny, int nz);
 // device bytes of an nx*ny*nz grid in the traversal layout (and its brick counts)
 size_t map_layout_bytes(int nx, int ny, int nz, int *nbx, int *nby, int *nbz);
 void launch_map_gather(const uint8_t *bricks, int nbx, int nby, uint8_t *lin, int nx, int ny, int nz, cudaStream_t s);

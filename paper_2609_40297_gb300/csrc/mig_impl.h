@@ -167,9 +167,10 @@ void set_pano_params(LevelParams &p, const Camera *cam, int32_t *pcnt);
 void launch_level_count(const mig_ctx *ctx, const LevelParams &p, int Ld, int count_cap, cudaStream_t s);
 // The same on the context stream, each launch timed under its own kind (mig_ctx_profile).
 void launch_level_count_timed(mig_ctx *ctx, const LevelParams &p, int Ld, int count_cap);
-// (node, yaw) pairs per owned-voxel chunk for a tree whose widest level has Lmax nodes (0 when the
-// context counts ray by ray); the step-count buffer holds steps_cap * W * H uint16.
-int steps_cap_for(const mig_ctx *ctx, int Lmax, int K, int W, int H, int mode);
+// The owned-voxel count's region for a tree whose widest level has Lmax nodes (empty when the context
+// counts ray by ray or the mode does).
+struct StepsLayout;
+StepsLayout steps_for(const mig_ctx *ctx, int Lmax, const mig_sensor &s, float voxel, int mode);
 // records an event pair around launch() on the context stream when profiling is on
 void prof_begin(mig_ctx *ctx, int kind, cudaEvent_t *a);
 void prof_end(mig_ctx *ctx, int kind, cudaEvent_t a);

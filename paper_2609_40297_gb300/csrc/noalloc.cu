@@ -221,14 +221,13 @@ extern "C" mig_status mig_tree_eval_device_noalloc(mig_map *m, int n, const int3
     p.mode = MIG_MODE_MARGINAL;
     p.stats = nullptr;
     p.max_anc = std::max(1, max_depth);
-    const int cap = ctx->num_sms * 16;
     const int count_cap = ctx->num_sms * std::min(ctx->count_ctas, std::max(1, (int)ctx->tiles.ctas_per_sm));
     const int sel_grid = std::max(1, std::min((n + 127) / 128, 1024));
     for (int d = 0; d < L; ++d) {
         p.lvl = d;
         timed_launch(ctx, kProfCount, [&] { launch_count(p, count_cap, s); });
         timed_launch(ctx, kProfSelect, [&] { launch_select(p, sel_grid, s); });
-        timed_launch(ctx, kProfRender, [&] { launch_render(p, cap, s); });
+        timed_launch(ctx, kProfRender, [&] { launch_render(p, n, ctx->num_sms, s); });
     }
     MIG_CUDA_TRY(cudaGetLastError());
     return MIG_OK;

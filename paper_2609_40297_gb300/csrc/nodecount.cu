@@ -1,0 +1,1149 @@
+// The owned-voxel count of one tree level by 4x4x4 bricks, and the depth-buffer render.
+//
+//   cast_kernel   - every pixel ray of every (node, yaw) pair runs to its first occupied voxel
+//                   (cast_bricks, bricks.cuh) and stores that voxel's step index (uint16; kNoHit if
+//                   none), with the minimum and maximum of every 8x8, 16x16 and 32x32 pixel tile.
+//   node_kernel   - every node's range ball is enumerated once for all yaws, 32 bricks of 64 voxels
+//                   at a time. A brick's unknown voxels are one 64-bit mask. Against each yaw, and each
+//                   ancestor's depth buffer, a brick is decided as a whole where it can be (all in the
+//                   image, all before the first hit of their pixels' rays, all visited for certain; or
+//                   none of them), so a yaw's counts are mostly sums of population counts of masks.
+//   brick_kernel  - the bricks left undecided, voxel by voxel.
+//   render_kernel - the depth buffer of each internal node's selected yaw (Sec. IV-A) with the
+//                   same tile bounds.
+// Every whole-brick decision is conservative (boxes widened by proven rounding bounds) and every
+// undecided voxel takes the exact integer tests of Sec. IV-B, so the counts equal the ray-by-ray
+// walk's and the oracle's bit for bit.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cstdint>
+
+#include "bricks.cuh"
+#include "kernels.h"
+#include "mig.h"
+#include "voxcount.h"
+
+namespace mig {
+
+namespace {
+
+using namespace dev;
+
+constexpr int kWarpsN = 8;  // warps per CTA of the kernels below
+
+__device__ __forceinline__ const uint64_t *grid_umask(const GridView &g) {
+    return reinterpret_cast<const uint64_t *>(g.g + umask_offset(g.nx, g.ny, g.nz));
+}
+__device__ __forceinline__ const uint64_t *grid_omask(const GridView &g) {
+    return reinterpret_cast<const uint64_t *>(g.g + omask_offset(g.nx, g.ny, g.nz));
+}
+
+__device__ __forceinline__ float q16f(int v) { return (float)v * (1.0f / 65536.0f); }
+
+// ------------------------------------------------------------------------- cast and render kernels
+// The rays of an image are cast 8x4 pixels at a time, one ray per lane. Before that, lanes follow one
+// such part each as a beam (beam_free): the part's rays start where the beam stopped, and are not
+// cast at all if it met nothing within the range (60 % of the parts on the large workload, 16 % at
+// paper scale). Three layouts, by the number of tiles of the level:
+//   large - one warp per 32x32 pixel tile, its 32 parts' beams on its 32 lanes;
+//   mid   - one CTA per 32x32 tile, the beams on its first warp, for levels of fewer tiles than keep every
+//           warp busy with several;
+//   small - one CTA per 16x16 tile, one part per warp, no beams and no 32x32 bounds, for levels that do
+//           not fill the GPU: their time is one warp's chain of dependent steps.
+// The level's size is only known on the device (tree_eval_device), so the kernels choose.
+constexpr int kCastCtas = 3;  // resident CTAs per SM: 80 registers; at 64 (4 CTAs) 2 % slower
+enum CastLayout { kCastSmall, kCastMid, kCastLarge };
+__device__ __forceinline__ CastLayout cast_layout(long long images, int W, int H, int num_sms) {
+    const long long tiles = images * ((W + 31) >> 5) * ((H + 31) >> 5), warps = (long long)num_sms * kCastCtas * kWarpsN;
+    return tiles >= 6 * warps ? kCastLarge : (2 * tiles >= warps ? kCastMid : kCastSmall);
+}
+
+// The beam of the 8x4 part at pixel (i0, j0).
+__device__ __forceinline__ float tile_beam(const LevelParams &p, const uint8_t *dist, const int4 nd, int ck, int sk, int i0, int j0) {
+    if (i0 >= p.W || j0 >= p.H) return 0.0f;
+    const int i1 = min(i0 + 7, p.W - 1), j1 = min(j0 + 3, p.H - 1);
+    const float q30 = 9.31322574615478515625e-10f, c = (float)ck * q30, s = (float)sk * q30;
+    float lo[3] = {1e30f, 1e30f, 1e30f}, hi[3] = {-1e30f, -1e30f, -1e30f};
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+        const int4 b = p.body[(t & 2 ? j1 : j0) * p.W + (t & 1 ? i1 : i0)];
+        const float z = __fdividef(1.0f, (float)b.w), x = (float)b.x * z, y = (float)b.y * z;
+        const float w[3] = {fmaf(c, x, -(s * y)), fmaf(s, x, c * y), (float)b.z * z};
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            lo[a] = fminf(lo[a], w[a]);
+            hi[a] = fmaxf(hi[a], w[a]);
+        }
+    }
+    // the largest camera depth of a unit ray: the part's pixel nearest the image centre on each axis
+    const float a0 = ((float)i0 + 0.5f - 0.5f * (float)p.W) * p.ifx, a1 = ((float)i1 + 0.5f - 0.5f * (float)p.W) * p.ifx;
+    const float b0 = ((float)j0 + 0.5f - 0.5f * (float)p.H) * p.ify, b1 = ((float)j1 + 0.5f - 0.5f * (float)p.H) * p.ify;
+    const float am = a0 * a1 <= 0.0f ? 0.0f : fminf(fabsf(a0), fabsf(a1)), bm = b0 * b1 <= 0.0f ? 0.0f : fminf(fabsf(b0), fabsf(b1));
+    const float s_end = q16f((int)p.Tq) * rsqrtf(1.0f + am * am + bm * bm) * 1.00001f;
+    return beam_free(dist, p.grid.nx, p.grid.ny, p.grid.nz, nd.x, nd.y, nd.z, lo, hi, s_end);
+}
+// The time before which a ray of camera depth cz (Q30, per unit length) of a beam free to depth s
+// meets no occupied voxel.
+__device__ __forceinline__ float beam_time(float s, int cz) {
+    return s > 0.0f ? fmaxf(0.0f, __fdividef(s * 1073741824.0f, (float)cz) * (1.0f - 1e-6f) - kCastEps) : 0.0f;
+}
+
+struct CastCnt {  // statistics
+    uint32_t rays = 0, fine = 0, jump = 0;
+};
+
+// What a pass keeps per ray and per tile: the cast the step index (16 bits, bounds packed as min |
+// ~max << 16), the render the depth.
+struct CastOut {
+    uint16_t *out;
+    uint32_t *hz;
+    static constexpr bool kDepth = false;
+    static constexpr uint32_t kMin = 0xFFFFu;
+    __device__ __forceinline__ uint32_t put(const LevelParams &, size_t i, int, uint32_t m, uint32_t, uint32_t) const {
+        out[i] = (uint16_t)m;
+        return m;
+    }
+    __device__ __forceinline__ void tile(size_t i, uint32_t lo, uint32_t hi) const { hz[i] = lo | ((hi ^ 0xFFFFu) << 16); }
+};
+struct RenderOut {
+    uint2 *pyr;  // NULL: not kept
+    int slot;
+    static constexpr bool kDepth = true;
+    static constexpr uint32_t kMin = 0xFFFFFFFFu;
+    __device__ __forceinline__ uint32_t put(const LevelParams &p, size_t i, int dzc, uint32_t m, uint32_t ne, uint32_t ade) const {
+        const uint32_t D = hit_depth(m != kNoHit, ne, ade, dzc, p.Tq);
+        arena_store(p.arena, p.arena_slots, slot, i, (size_t)p.W * p.H, D, p.bounds_err);
+        return D;
+    }
+    __device__ __forceinline__ void tile(size_t i, uint32_t lo, uint32_t hi) const {
+        if (pyr) pyr[i] = make_uint2(lo, hi);
+    }
+};
+
+// One ray, out of line: the layouts' loops keep their state in other registers than the walk's.
+struct RayHit {
+    uint32_t m, ne, ade;
+};
+template <bool STATS, bool DEPTH>
+__device__ __noinline__ RayHit cast_ray(const uint64_t *om, const uint8_t *dist, int gnx, int gny, int gnz, int Px, int Py, int Pz,
+                                       int dx, int dy, int dz, int Tq, float t0, CastCnt *st) {
+    RayHit h{0, 0, 1};
+    uint32_t fine = 0, jump = 0;
+    h.m = cast_bricks<DEPTH, STATS>(om, dist, gnx, gny, gnz, Px, Py, Pz, dx, dy, dz, Tq, t0, h.ne, h.ade, fine, jump);
+    if constexpr (STATS) {
+        st->fine += fine;
+        st->jump += jump;
+    }
+    return h;
+}
+
+// Casts the 8x4 part at pixel (i0, j0), lane l the pixel (l & 7, l >> 3); lo, hi gather its bounds.
+template <bool STATS, class OUT>
+__device__ __forceinline__ void cast_part(const LevelParams &p, const uint64_t *om, const uint8_t *dist, const int4 nd, int ck, int sk,
+                                          int i0, int j0, float beam, const OUT &o, int lane, uint32_t &lo, uint32_t &hi,
+                                          CastCnt &st) {
+    const int i = i0 + (lane & 7), j = j0 + (lane >> 3);
+    if (i >= p.W || j >= p.H) return;
+    const size_t at = (size_t)j * p.W + i;
+    RayHit hit{kNoHit, 0, 1};
+    int dzc = 0;
+    if (OUT::kDepth || beam < 1e29f) {
+        const int4 b = p.body[at];
+        dzc = b.w;
+        if (beam < 1e29f) {
+            int dx, dy, dz;
+            ray_dir(b, ck, sk, dx, dy, dz);
+            hit = cast_ray<STATS, OUT::kDepth>(om, dist, p.grid.nx, p.grid.ny, p.grid.nz, nd.x, nd.y, nd.z, dx, dy, dz, (int)p.Tq,
+                                               beam_time(beam, b.w), &st);
+        }
+    }
+    const uint32_t v = o.put(p, at, dzc, hit.m, hit.ne, hit.ade);
+    lo = min(lo, v);
+    hi = max(hi, v);
+    if constexpr (STATS) ++st.rays;
+}
+
+// The pixel of part t (0..7) of the 16x16 quadrant at (x0, y0): half t & 1 of 8x8 tile t >> 1.
+__device__ __forceinline__ int2 part_at(int x0, int y0, int t) {
+    return make_int2(x0 + ((t >> 1) & 1) * 8, y0 + (t >> 2) * 8 + (t & 1) * 4);
+}
+
+// One 16x16 quadrant by one warp, part t's beam in lane base + t of s; returns its bounds.
+template <bool STATS, class OUT>
+__device__ __forceinline__ uint2 cast_quad(const LevelParams &p, const uint64_t *om, const uint8_t *dist, const Pyramid &y,
+                                           const int4 nd, int ck, int sk, int x0, int y0, float s, int base, const OUT &o, int lane,
+                                           CastCnt &st) {
+    uint32_t lo = OUT::kMin, hi = 0u, lo16 = OUT::kMin, hi16 = 0u;
+#pragma unroll 1
+    for (int t = 0; t < 8; ++t) {
+        const int2 at = part_at(x0, y0, t);
+        const float beam = __shfl_sync(0xffffffffu, s, base + t);
+        cast_part<STATS>(p, om, dist, nd, ck, sk, at.x, at.y, beam, o, lane, lo, hi, st);
+        __syncwarp();
+        if (t & 1) {
+            lo = __reduce_min_sync(0xffffffffu, lo);
+            hi = __reduce_max_sync(0xffffffffu, hi);
+            if (lane == 0 && at.x < p.W && at.y - 4 < p.H) o.tile((size_t)(at.y >> 3) * y.w0 + (at.x >> 3), lo, hi);
+            lo16 = min(lo16, lo);
+            hi16 = max(hi16, hi);
+            lo = OUT::kMin;
+            hi = 0u;
+        }
+    }
+    if (lane == 0 && x0 < p.W && y0 < p.H) o.tile(y.o1 + (size_t)(y0 >> 4) * y.w1 + (x0 >> 4), lo16, hi16);
+    return make_uint2(lo16, hi16);
+}
+
+// One 32x32 tile at pixel (x0, y0) by one warp.
+template <bool STATS, class OUT>
+__device__ __forceinline__ void cast_large(const LevelParams &p, const uint64_t *om, const uint8_t *dist, const Pyramid &y,
+                                           const int4 nd, int ck, int sk, int x0, int y0, const OUT &o, int lane, CastCnt &st) {
+    const int2 at = part_at(x0 + ((lane >> 3) & 1) * 16, y0 + (lane >> 4) * 16, lane & 7);
+    const float s = tile_beam(p, dist, nd, ck, sk, at.x, at.y);
+    uint2 b = make_uint2(OUT::kMin, 0u);
+#pragma unroll 1
+    for (int q = 0; q < 4; ++q) {
+        const uint2 v = cast_quad<STATS>(p, om, dist, y, nd, ck, sk, x0 + (q & 1) * 16, y0 + (q >> 1) * 16, s, 8 * q, o, lane, st);
+        b = make_uint2(min(b.x, v.x), max(b.y, v.y));
+    }
+    if (lane == 0) o.tile(y.o2 + (size_t)(y0 >> 5) * y.w2 + (x0 >> 5), b.x, b.y);
+}
+
+// One 32x32 tile at pixel (x0, y0) by a CTA of 8 warps: warp w casts half of quadrant w >> 1.
+template <bool STATS, class OUT>
+__device__ __forceinline__ void cast_mid(const LevelParams &p, const uint64_t *om, const uint8_t *dist, const Pyramid &y,
+                                         const int4 nd, int ck, int sk, int x0, int y0, const OUT &o, uint2 *s_t, float *s_beam, int warp,
+                                         int lane, CastCnt &st) {
+    if (warp == 0) {
+        const int2 at = part_at(x0 + ((lane >> 3) & 1) * 16, y0 + (lane >> 4) * 16, lane & 7);
+        s_beam[lane] = tile_beam(p, dist, nd, ck, sk, at.x, at.y);
+    }
+    __syncthreads();
+    const int qx = x0 + ((warp >> 1) & 1) * 16, qy = y0 + (warp >> 2) * 16;
+    uint32_t lo = OUT::kMin, hi = 0u, lo2 = OUT::kMin, hi2 = 0u;
+#pragma unroll 1
+    for (int t = 4 * (warp & 1); t < 4 * (warp & 1) + 4; ++t) {
+        const int2 at = part_at(qx, qy, t);
+        cast_part<STATS>(p, om, dist, nd, ck, sk, at.x, at.y, s_beam[8 * (warp >> 1) + t], o, lane, lo, hi, st);
+        __syncwarp();
+        if (t & 1) {
+            lo = __reduce_min_sync(0xffffffffu, lo);
+            hi = __reduce_max_sync(0xffffffffu, hi);
+            if (lane == 0 && at.x < p.W && at.y - 4 < p.H) o.tile((size_t)(at.y >> 3) * y.w0 + (at.x >> 3), lo, hi);
+            lo2 = min(lo2, lo);
+            hi2 = max(hi2, hi);
+            lo = OUT::kMin;
+            hi = 0u;
+        }
+    }
+    if (lane == 0) s_t[warp] = make_uint2(lo2, hi2);
+    __syncthreads();
+    if (threadIdx.x < 4) {
+        const uint2 a = s_t[2 * threadIdx.x], b = s_t[2 * threadIdx.x + 1];
+        lo = min(a.x, b.x);
+        hi = max(a.y, b.y);
+        const int i0 = x0 + (threadIdx.x & 1) * 16, j0 = y0 + (threadIdx.x >> 1) * 16;
+        if (i0 < p.W && j0 < p.H) o.tile(y.o1 + (size_t)(j0 >> 4) * y.w1 + (i0 >> 4), lo, hi);
+        lo = __reduce_min_sync(0xfu, lo);
+        hi = __reduce_max_sync(0xfu, hi);
+        if (threadIdx.x == 0) o.tile(y.o2 + (size_t)(y0 >> 5) * y.w2 + (x0 >> 5), lo, hi);
+    }
+    __syncthreads();
+}
+
+// One 16x16 tile at pixel (x0, y0) by a CTA of 8 warps.
+template <bool STATS, class OUT>
+__device__ __forceinline__ void cast_small(const LevelParams &p, const uint64_t *om, const uint8_t *dist, const Pyramid &y,
+                                            const int4 nd, int ck, int sk, int x0, int y0, const OUT &o, uint2 *s_t, int warp, int lane,
+                                            CastCnt &st) {
+    uint32_t lo = OUT::kMin, hi = 0u;
+    const int2 at = part_at(x0, y0, warp);
+    cast_part<STATS>(p, om, dist, nd, ck, sk, at.x, at.y, 0.0f, o, lane, lo, hi, st);
+    __syncwarp();
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if (lane == 0) s_t[warp] = make_uint2(lo, hi);
+    __syncthreads();
+    if (threadIdx.x < 4) {
+        const uint2 a = s_t[2 * threadIdx.x], b = s_t[2 * threadIdx.x + 1];
+        lo = min(a.x, b.x);
+        hi = max(a.y, b.y);
+        const int i0 = x0 + (threadIdx.x & 1) * 8, j0 = y0 + (threadIdx.x >> 1) * 8;
+        if (i0 < p.W && j0 < p.H) o.tile((size_t)(j0 >> 3) * y.w0 + (i0 >> 3), lo, hi);
+        lo = __reduce_min_sync(0xfu, lo);
+        hi = __reduce_max_sync(0xfu, hi);
+        if (threadIdx.x == 0) o.tile(y.o1 + (size_t)(y0 >> 4) * y.w1 + (x0 >> 4), lo, hi);
+    }
+    __syncthreads();
+}
+
+template <bool STATS>
+__global__ void __launch_bounds__(kWarpsN * 32, kCastCtas) cast_kernel(const LevelParams p, int num_sms) {
+    __shared__ uint2 s_t[kWarpsN];
+    __shared__ float s_beam[32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (blockIdx.x == 0 && threadIdx.x < 3) p.vctr[threadIdx.x] = 0;  // the counters of the passes that follow
+    const int l0 = p.level_off[p.lvl];
+    const int q1 = min(p.q1, (p.level_off[p.lvl + 1] - l0) * p.K);
+    if (p.q0 >= q1) return;
+    const CastLayout lay = cast_layout(q1 - p.q0, p.W, p.H, num_sms);
+    const int T = lay == kCastSmall ? 16 : 32;
+    const int tx = (p.W + T - 1) / T, ty = (p.H + T - 1) / T;
+    const size_t WH = (size_t)p.W * p.H;
+    const Pyramid y = pyramid(p.W, p.H);
+    const uint64_t *om = grid_omask(p.grid);
+    const uint8_t *dist = p.grid.g + dist_offset(p.grid.nx, p.grid.ny, p.grid.nz);
+    CastCnt st;
+    const long long items = (long long)(q1 - p.q0) * tx * ty;
+    const int per = lay == kCastLarge ? kWarpsN : 1, mine = lay == kCastLarge ? warp : 0;  // items at a time per CTA
+    for (long long it = (long long)blockIdx.x * per + mine; it < items; it += (long long)gridDim.x * per) {
+        const int tile = (int)(it % (tx * ty)), ql = (int)(it / (tx * ty));
+        const int q = p.q0 + ql;
+        const int4 nd = p.node[p.level_nodes[l0 + q / p.K]];
+        const int32_t *yk = p.yawtab + (q % p.K) * 12;
+        const CastOut o{p.steps + (size_t)ql * WH, p.hz + (size_t)ql * y.n};
+        const int x0 = tile % tx * T, y0 = tile / tx * T;
+        if (lay == kCastLarge) {
+            cast_large<STATS>(p, om, dist, y, nd, yk[0], yk[1], x0, y0, o, lane, st);
+        } else if (lay == kCastMid) {
+            cast_mid<STATS>(p, om, dist, y, nd, yk[0], yk[1], x0, y0, o, s_t, s_beam, warp, lane, st);
+        } else {
+            cast_small<STATS>(p, om, dist, y, nd, yk[0], yk[1], x0, y0, o, s_t, warp, lane, st);
+        }
+    }
+    if constexpr (STATS) {
+        atomicAdd(p.stats + 8, (unsigned long long)st.rays);
+        atomicAdd(p.stats + 9, (unsigned long long)st.fine);
+        atomicAdd(p.stats + 10, (unsigned long long)st.jump);
+    }
+}
+
+// Depth buffer of the selected yaw (Sec. IV-A): per pixel ray, camera z of the entry point of the
+// first occupied voxel, else of the range endpoint. Only nodes with children (the level's first
+// level_int nodes) are rendered; descendants read them in the ancestor test.
+template <bool STATS>
+__global__ void __launch_bounds__(kWarpsN * 32, kCastCtas) render_kernel(const LevelParams p, int num_sms) {
+    __shared__ uint2 s_t[kWarpsN];
+    __shared__ float s_beam[32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int l0 = p.level_off[p.lvl], Li = p.level_int[p.lvl];
+    const CastLayout lay = cast_layout(Li, p.W, p.H, num_sms);
+    const int T = lay == kCastSmall ? 16 : 32;
+    const int tx = (p.W + T - 1) / T, ty = (p.H + T - 1) / T;
+    const int items = Li * tx * ty;
+    const Pyramid y = pyramid(p.W, p.H);
+    const uint64_t *om = grid_omask(p.grid);
+    const uint8_t *dist = p.grid.g + dist_offset(p.grid.nx, p.grid.ny, p.grid.nz);
+    CastCnt st;
+    const int per = lay == kCastLarge ? kWarpsN : 1, mine = lay == kCastLarge ? warp : 0;  // items at a time per CTA
+    for (int it = blockIdx.x * per + mine; it < items; it += gridDim.x * per) {
+        const int tile = it % (tx * ty);
+        const int n = p.level_nodes[l0 + it / (tx * ty)];
+        const int4 nd = p.node[n];
+        if (nd.w < 0) continue;  // uniform over the warps of the item
+        const int32_t *yk = p.yawtab + p.sel_yaw[n] * 12;
+        const RenderOut o{p.dpyr ? p.dpyr + (size_t)nd.w * y.n : nullptr, nd.w};
+        const int x0 = tile % tx * T, y0 = tile / tx * T;
+        if (lay == kCastLarge) {
+            cast_large<STATS>(p, om, dist, y, nd, yk[0], yk[1], x0, y0, o, lane, st);
+        } else if (lay == kCastMid) {
+            cast_mid<STATS>(p, om, dist, y, nd, yk[0], yk[1], x0, y0, o, s_t, s_beam, warp, lane, st);
+        } else {
+            cast_small<STATS>(p, om, dist, y, nd, yk[0], yk[1], x0, y0, o, s_t, warp, lane, st);
+        }
+    }
+    if constexpr (STATS) {
+        atomicAdd(p.stats + 6, (unsigned long long)st.rays);
+        atomicAdd(p.stats + 7, (unsigned long long)(st.fine + st.jump));
+    }
+}
+
+// ---------------------------------------------------------------------------- the per-node count
+// Two kernels per chunk of nodes. node_kernel takes macro blocks of 16x16x8 voxels, 4x4x2 bricks, one
+// brick per lane, and decides whole bricks against every yaw and ancestor; what it cannot decide as a
+// whole it appends to a queue, one record per brick. brick_kernel takes the records, one warp each,
+// one voxel of the brick's lower and upper half per lane. (As one kernel the two stages' code, 4300
+// instructions, did not fit the instruction cache, and a warp's block took 10 to 100 times as long as
+// another's: 338 ms on the large workload.)
+constexpr int kMacX = 16, kMacZ = 8;
+__host__ __device__ inline int mac_xy(int64_t Tq) { return (2 * ((int)(Tq >> 16) + 2)) / kMacX + 2; }
+__host__ __device__ inline int mac_z(int64_t Tq) { return (2 * ((int)(Tq >> 16) + 2)) / kMacZ + 2; }
+
+struct NodeAnc {
+    int px, py, pz, yaw;
+    const uint32_t *D;
+    const uint2 *pyr;
+};
+
+struct NodeCnt {  // statistics
+    uint32_t cand = 0, unk = 0, visit = 0, anc = 0, reads = 0, smp = 0;
+};
+
+__device__ __forceinline__ uint64_t shfl64(uint64_t v, int src) {
+    return (uint64_t)__shfl_sync(0xffffffffu, (unsigned long long)v, src);
+}
+__device__ __forceinline__ uint64_t or64(uint64_t v) {  // over the warp
+    return (uint64_t)__reduce_or_sync(0xffffffffu, (unsigned)v) | ((uint64_t)__reduce_or_sync(0xffffffffu, (unsigned)(v >> 32)) << 32);
+}
+
+// Bounds of the step counts under a pixel box: min in the low half, ~max in the high half.
+__device__ __forceinline__ uint32_t hz_box(const uint32_t *hz, const Pyramid &y, int top, const BoxView &b) {
+    int sh, off, w;
+    pyramid_level(y, max(b.u1 - b.u0, b.v1 - b.v0), top, sh, off, w);
+    const uint32_t *t = hz + off;
+    uint32_t r = 0xFFFFFFFFu;
+#pragma unroll 1
+    for (int ty = b.v0 >> sh; ty <= (b.v1 >> sh); ++ty)
+#pragma unroll 1
+        for (int tx = b.u0 >> sh; tx <= (b.u1 >> sh); ++tx) r = __vminu2(r, __ldg(t + ty * w + tx));
+    return r;
+}
+// Bounds of the stored depths under a pixel box (the 32x32 level is not kept by every render).
+__device__ __forceinline__ uint2 depth_box(const uint2 *pyr, const Pyramid &y, const BoxView &b) {
+    int sh, off, w;
+    pyramid_level(y, max(b.u1 - b.u0, b.v1 - b.v0), 4, sh, off, w);
+    const uint2 *t = pyr + off;
+    uint2 r = make_uint2(0xFFFFFFFFu, 0u);
+#pragma unroll 1
+    for (int ty = b.v0 >> sh; ty <= (b.v1 >> sh); ++ty)
+#pragma unroll 1
+        for (int tx = b.u0 >> sh; tx <= (b.u1 >> sh); ++tx) {
+            const uint2 v = __ldg(t + ty * w + tx);
+            r.x = min(r.x, v.x);
+            r.y = max(r.y, v.y);
+        }
+    return r;
+}
+__device__ __forceinline__ bool box_lookup(const BoxView &b) {
+    return b.zlo >= 0.5f && b.u1 - b.u0 <= kPyramidSpan && b.v1 - b.v0 <= kPyramidSpan;
+}
+
+// Float pixel of a voxel centre at camera depth >= 1/2. c = 5e-7 (largest offset + 1) bounds a row
+// product's error per unit of the row's L1 norm, so eu = 2 c (norm_u + W norm_z) / Z + 1e-6 (W + 1)
+// bounds the error of u for every pixel inside the image, and of an outside one by less than its
+// distance to the image. su, sv: 2 c (norm + size norm_z).
+struct PixelErr {
+    float su, sv, bu, bv;
+};
+// 1: inside the image, pixel index pix; 0: outside; -1: undecided.
+__device__ __forceinline__ int pixel_float(const PixelErr &e, float Z, float U, float V, float fW, float fH, int &pix) {
+    const float kMagic = 12582912.0f;
+    const float zi = __fdividef(1.0f, Z);
+    const float u = fmaf(U, zi, -0.5f), v = fmaf(V, zi, -0.5f);
+    const float fu = (u + kMagic) - kMagic, fv = (v + kMagic) - kMagic;  // floors: nearest integers of u - 1/2
+    const bool sure = Z >= 0.5f && fmaf(zi, e.su, fabsf(u - fu)) <= e.bu && fmaf(zi, e.sv, fabsf(v - fv)) <= e.bv;
+    pix = __float_as_int(fmaf(fv, fW, fu) + 8388608.0f) & 0x7FFFFF;
+    if (!sure) return -1;
+    return fu >= 0.0f && fu < fW && fv >= 0.0f && fv < fH;
+}
+// The exact pixel index (Eq. 5) in integers, or -1 outside the image; Z (Q32).
+__device__ __forceinline__ int pixel_index(const int32_t *row, int rx, int ry, int rz, int W, int H, int64_t &Z) {
+    Z = (int64_t)row[8] * rx + (int64_t)row[9] * ry + (int64_t)row[10] * rz;
+    if (Z <= 0) return -1;
+    const int64_t U = (int64_t)row[2] * rx + (int64_t)row[3] * ry + (int64_t)row[4] * rz;
+    const int64_t V = (int64_t)row[5] * rx + (int64_t)row[6] * ry + (int64_t)row[7] * rz;
+    const float zi = __fdividef(1.0f, (float)Z);
+    int pu, pv;
+    if (!pixel_in(U, Z, (float)U * zi, W, pu) || !pixel_in(V, Z, (float)V * zi, H, pv)) return -1;
+    return pv * W + pu;
+}
+__device__ __noinline__ int pixel_exact(const int32_t *row, int rx, int ry, int rz, int W, int H) {
+    int64_t Z;
+    return pixel_index(row, rx, ry, rz, W, H, Z);
+}
+// The exact ancestor test (Sec. IV-B): inside the image and z <= D.
+__device__ __noinline__ bool observed_exact(const int32_t *row, int rx, int ry, int rz, int W, int H, const uint32_t *D) {
+    int64_t Z;
+    const int pix = pixel_index(row, rx, ry, rz, W, H, Z);
+    return pix >= 0 && Z < (((int64_t)__ldg(D + pix) + 1) << 16);
+}
+// The exact visit test of a voxel by its owner ray.
+__device__ __noinline__ bool visit_exact(int Px, int Py, int Pz, int bx, int by, int bz, int ck, int sk, int x, int y, int z,
+                                         int64_t Tq) {
+    int dx, dy, dz;
+    ray_dir(make_int4(bx, by, bz, 0), ck, sk, dx, dy, dz);
+    return visit_index(Px, Py, Pz, dx, dy, dz, x, y, z, Tq) >= 0;
+}
+
+// Per-launch constants of the voxel stage.
+struct VoxConst {
+    float fW, fH, bu, bv, Tv, out2, inf2, l22;
+};
+__device__ __forceinline__ VoxConst vox_const(const LevelParams &p) {
+    VoxConst c;
+    c.fW = (float)p.W;
+    c.fH = (float)p.H;
+    c.bu = 0.5f - 1.0e-6f * (c.fW + 1.0f);
+    c.bv = 0.5f - 1.0e-6f * (c.fH + 1.0f);
+    c.Tv = q16f((int)p.Tq);
+    // squared centre distances: no visit beyond out2; certain visits by the yaw's limit and by zl2
+    c.out2 = (c.Tv + 0.88f) * (c.Tv + 0.88f);
+    c.inf2 = fmaxf(c.Tv - 0.86f, 0.f) * fmaxf(c.Tv - 0.86f, 0.f);
+    c.l22 = fmaxf(c.Tv - 0.02f, 0.f) * fmaxf(c.Tv - 0.02f, 0.f);
+    return c;
+}
+
+// The ancestors of node n that the mode tests (Sec. IV-B), parent first; returns their number.
+__device__ __forceinline__ int node_ancestors(const LevelParams &p, int n, NodeAnc *anc, size_t WH, int pyr_n, int lane) {
+    const int2 ar = p.anc_range[n];
+    int na = p.mode == MIG_MODE_ABSOLUTE ? 0 : (p.mode == MIG_MODE_SINGLE_PARENT ? min(ar.y, 1) : ar.y);
+    na = min(na, p.max_anc);
+    __syncwarp();
+    for (int t = lane; t < na; t += 32) {
+        const int a = p.anc[ar.x + t];
+        const int4 an = p.node[a];
+        anc[t] = NodeAnc{an.x, an.y, an.z, p.sel_yaw[a], p.arena + (size_t)an.w * WH, p.dpyr + (size_t)an.w * pyr_n};
+    }
+    __syncwarp();
+    return na;
+}
+
+// One undecided brick (warp-uniform record r; lane = voxel of its lower and upper half): the
+// ancestor tests left, then each yaw's counts into c_abs / c_mrg of lane (yaw - first) % 32, slot
+// (yaw - first) / 32.
+template <bool STATS>
+__device__ __forceinline__ void count_brick(const LevelParams &p, const VoxConst &vc, const YawRows *s_y, const NodeAnc *anc,
+                                            const int4 nd, const uint16_t *steps, const BrickRec &r, int lane, int c_abs[2],
+                                            int c_mrg[2], NodeCnt &st) {
+    const int W = p.W, H = p.H, kb = (int)(r.node >> kRecNodeBits) * 64;
+    const size_t WH = (size_t)W * H;
+    const int x = 4 * (int)(r.brick & 1023) + (lane & 3), y = 4 * (int)((r.brick >> 10) & 1023) + ((lane >> 2) & 3),
+              z0 = 4 * (int)(r.brick >> 20) + (lane >> 4);
+    const uint64_t U = r.U;
+    uint64_t O = r.O;
+    const int rx = (x << 16) + 32768 - nd.x, ry = (y << 16) + 32768 - nd.y, rz0 = (z0 << 16) + 32768 - nd.z;
+    const float rinf = fmaxf(fmaxf(fabsf(q16f(rx)), fabsf(q16f(ry))), fabsf(q16f(rz0))) + 8.0f;
+    // error of a row product per unit of the row's norm, for every voxel of the brick
+    const float verr = 5e-7f * (__uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(rinf))) + 1.0f);
+    // ---- the ancestors that were not decided for the whole brick
+    for (uint64_t as = r.anc; as; as &= as - 1) {
+        const NodeAnc A = anc[__ffsll((long long)as) - 1];
+        const float4 ru = s_y[A.yaw].u, rv = s_y[A.yaw].v, rz = s_y[A.yaw].z;
+        const int32_t *row = p.yawtab + A.yaw * 12;
+        const int ax = (x << 16) + 32768 - A.px, ay = (y << 16) + 32768 - A.py, az0 = (z0 << 16) + 32768 - A.pz;
+        const float ex = q16f(ax), ey = q16f(ay);
+        const float Zxy = fmaf(rz.x, ex, rz.y * ey), Uxy = fmaf(ru.x, ex, ru.y * ey), Vxy = fmaf(rv.x, ex, rv.y * ey);
+        const float c = verr + 5e-7f * fmaxf(fmaxf(fabsf(q16f(A.px - nd.x)), fabsf(q16f(A.py - nd.y))), fabsf(q16f(A.pz - nd.z)));
+        const PixelErr pe{2.0f * c * fmaf(vc.fW, rz.w, ru.w), 2.0f * c * fmaf(vc.fH, rz.w, rv.w), vc.bu, vc.bv};
+        const float e_z = c * rz.w;
+        const uint64_t rem = U & ~O;
+        bool obs[2] = {false, false};
+        int pix[2], in[2];
+        float Zf[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float ez = q16f(az0 + (h << 17));
+            Zf[h] = fmaf(rz.z, ez, Zxy);
+            in[h] = pixel_float(pe, Zf[h], fmaf(ru.z, ez, Uxy), fmaf(rv.z, ez, Vxy), vc.fW, vc.fH, pix[h]);
+            if (!((uint32_t)(rem >> (32 * h)) >> lane & 1)) in[h] = 0;
+            if constexpr (STATS) st.anc += (uint32_t)(rem >> (32 * h)) >> lane & 1;
+        }
+        uint32_t D[2] = {0u, 0u};
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            if (in[h] > 0) D[h] = __ldg(A.D + pix[h]);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if constexpr (STATS) st.reads += in[h] > 0;
+            // z <= D  <=>  Z < (D + 1) / 2^16 (voxels); lim within 2^-23 of that
+            const float lim = ((float)D[h] + 1.0f) * (1.0f / 65536.0f);
+            obs[h] = in[h] > 0 && Zf[h] + e_z < lim * (1.0f - 2.4e-7f);
+            if (in[h] < 0 || (in[h] > 0 && !obs[h] && Zf[h] - e_z < lim * (1.0f + 2.4e-7f)))
+                obs[h] = observed_exact(row, ax, ay, az0 + (h << 17), W, H, A.D);
+        }
+        O |= (uint64_t)__ballot_sync(0xffffffffu, obs[0]) | ((uint64_t)__ballot_sync(0xffffffffu, obs[1]) << 32);
+    }
+    // ---- yaws that count every unknown voxel
+    {
+        const int cu = __popcll(U), cm = __popcll(U & ~O);
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+            if ((uint32_t)(r.all >> (32 * i)) >> lane & 1) {
+                c_abs[i] += cu;
+                c_mrg[i] += cm;
+                if constexpr (STATS) st.visit += cu;
+            }
+    }
+    // ---- yaws that left the brick undecided
+    const float ex = q16f(rx), ey = q16f(ry), ez[2] = {q16f(rz0), q16f(rz0 + 131072)};
+    const float exy2 = fmaf(ex, ex, ey * ey);
+    const int v0z = nd.z >> 16, mxy = abs(x - (nd.x >> 16)) + abs(y - (nd.y >> 16));
+    bool has[2], near_inf[2], near_l2[2];
+    int man[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const float r2 = fmaf(ez[h], ez[h], exy2);
+        has[h] = ((uint32_t)(U >> (32 * h)) >> lane & 1) && r2 < vc.out2;
+        near_inf[h] = r2 < vc.inf2;
+        near_l2[h] = r2 < vc.l22;
+        man[h] = mxy + abs(z0 + 2 * h - v0z);
+    }
+    const uint64_t rv64 = r.rch | r.vis;
+    for (uint64_t ks = r.part; ks; ks &= ks - 1) {
+        const int j = __ffsll((long long)ks) - 1, k = kb + j;
+        const float4 ru = s_y[k].u, rv = s_y[k].v, rz = s_y[k].z;
+        const float Zxy = fmaf(rz.x, ex, rz.y * ey), Uxy = fmaf(ru.x, ex, ru.y * ey), Vxy = fmaf(rv.x, ex, rv.y * ey);
+        const int32_t *row = p.yawtab + k * 12;
+        bool c[2] = {false, false};
+        if (!((rv64 >> j) & 1)) {
+            // every voxel is reached and visited: only the image test, without the pixel
+            const float cz = verr * rz.w, cu = verr * ru.w, cv = verr * rv.w, cr = fmaf(vc.fW, cz, cu), cb = fmaf(vc.fH, cz, cv);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float Zf = fmaf(rz.z, ez[h], Zxy), Uf = fmaf(ru.z, ez[h], Uxy), Vf = fmaf(rv.z, ez[h], Vxy);
+                const float Rf = fmaf(vc.fW, Zf, -Uf), Bf = fmaf(vc.fH, Zf, -Vf);
+                const bool in = fminf(fminf(Uf - cu, Vf - cv), fminf(Rf - cr, Bf - cb)) > 0.0f;
+                const bool out = fminf(fminf(Uf + cu, Vf + cv), fminf(Rf + cr, Bf + cb)) < 0.0f;
+                c[h] = has[h] && in;
+                if (has[h] && !in && !out) c[h] = pixel_exact(row, rx, ry, rz0 + (h << 17), W, H) >= 0;
+            }
+            if constexpr (STATS) st.visit += (int)c[0] + (int)c[1];
+        } else {
+            const PixelErr pe{2.0f * verr * fmaf(vc.fW, rz.w, ru.w), 2.0f * verr * fmaf(vc.fH, rz.w, rv.w), vc.bu, vc.bv};
+            const bool nr = (r.rch >> j) & 1, nv = (r.vis >> j) & 1;
+            const uint16_t *stp = steps + (size_t)k * WH;
+            int pix[2];
+            float Zf[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                Zf[h] = fmaf(rz.z, ez[h], Zxy);
+                const int in = pixel_float(pe, Zf[h], fmaf(ru.z, ez[h], Uxy), fmaf(rv.z, ez[h], Vxy), vc.fW, vc.fH, pix[h]);
+                c[h] = has[h] && in > 0;
+                if (has[h] && in < 0) {
+                    pix[h] = pixel_exact(row, rx, ry, rz0 + (h << 17), W, H);
+                    c[h] = pix[h] >= 0;
+                }
+            }
+            if (nr) {  // before the owner ray's hit
+                int m[2] = {0, 0};
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    if (c[h]) m[h] = __ldg(stp + pix[h]);
+                c[0] = man[0] < m[0];
+                c[1] = man[1] < m[1];
+            }
+            if constexpr (STATS) st.visit += (int)c[0] + (int)c[1];
+            if (nv) {  // the owner ray visits the voxel
+                const float4 rq = s_y[k].x;
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    if (c[h] && !(Zf[h] >= 0.5f && ((near_inf[h] && Zf[h] < rq.x) || (near_l2[h] && Zf[h] < p.vis_zl2)))) {
+                        const int4 b = p.body[pix[h]];
+                        const float q30 = 9.31322574615478515625e-10f;
+                        const float bxf = (float)b.x * q30, byf = (float)b.y * q30;
+                        const int d = visit_slab(ex, ey, ez[h], fmaf(rq.y, bxf, -(rq.z * byf)), fmaf(rq.z, bxf, rq.y * byf),
+                                                 (float)b.z * q30, vc.Tv);
+                        c[h] = d > 0;
+                        if (d < 0) c[h] = visit_exact(nd.x, nd.y, nd.z, b.x, b.y, b.z, row[0], row[1], x, y, z0 + 2 * h, p.Tq);
+                    }
+            }
+        }
+        const unsigned m0 = __ballot_sync(0xffffffffu, c[0]), m1 = __ballot_sync(0xffffffffu, c[1]);
+        if (lane == (j & 31)) {
+            const int a = __popc(m0) + __popc(m1), m = __popc(m0 & ~(unsigned)O) + __popc(m1 & ~(unsigned)(O >> 32));
+            c_abs[0] += j < 32 ? a : 0;
+            c_mrg[0] += j < 32 ? m : 0;
+            c_abs[1] += j < 32 ? 0 : a;
+            c_mrg[1] += j < 32 ? 0 : m;
+        }
+    }
+}
+
+// Adds a warp's counts of node n's yaws [kb, kb + 64) to the level's counters and clears them: one
+// 64-bit addition for the (abs, marginal) pair, whose halves stay below 2^31.
+template <bool STATS>
+__device__ __forceinline__ void flush_counts(const LevelParams &p, int n, int kb, int lane, int c_abs[2], int c_mrg[2], NodeCnt &st) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const int k = kb + 32 * i + lane;
+        if (k < p.K && (c_abs[i] | c_mrg[i]))
+            atomicAdd(reinterpret_cast<unsigned long long *>(p.cnt) + (size_t)n * p.K + k,
+                      (unsigned long long)(unsigned)c_abs[i] | ((unsigned long long)(unsigned)c_mrg[i] << 32));
+        if constexpr (STATS) st.smp += c_abs[i];
+        c_abs[i] = c_mrg[i] = 0;
+    }
+}
+
+template <bool STATS>
+__device__ __forceinline__ void add_stats(const LevelParams &p, const NodeCnt &st) {
+    if constexpr (STATS) {
+        const uint32_t v[6] = {st.cand, st.unk, st.visit, st.smp, st.anc, st.reads};
+        for (int i = 0; i < 6; ++i) atomicAdd(p.stats + 11 + i, (unsigned long long)v[i]);
+    }
+}
+
+template <bool STATS>
+__global__ void __launch_bounds__(kWarpsN * 32, 3) node_kernel(const LevelParams p, int num_sms) {
+    extern __shared__ __align__(16) unsigned char s_dyn[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int K = p.K;
+    YawRows *s_y = reinterpret_cast<YawRows *>(s_dyn);
+    NodeAnc *anc = reinterpret_cast<NodeAnc *>(s_y + K) + warp * p.max_anc;
+    const int l0 = p.level_off[p.lvl];
+    const int Ld = p.level_off[p.lvl + 1] - l0;
+    const int nb0 = p.q0 / K, nn = min(p.q1 / K, Ld) - nb0;
+    if (nn <= 0) return;
+    for (int k = threadIdx.x; k < K; k += blockDim.x)
+        s_y[k] = yaw_rows(p.yawtab + k * 12, p.W, p.H, p.vis_hu, p.vis_hv, p.ifx, p.ify);
+    __syncthreads();
+    const int W = p.W, H = p.H;
+    const size_t WH = (size_t)W * H;
+    const Pyramid pyr = pyramid(W, H);
+    const int top = cast_layout((long long)nn * K, W, H, num_sms) == kCastSmall ? 4 : 5;  // the bounds the cast kept
+    const BrickDims bd = brick_dims(p.grid.nx, p.grid.ny, p.grid.nz);
+    const uint64_t *umask = grid_umask(p.grid);
+    const VoxConst vc = vox_const(p);
+    const float R2 = (vc.Tv + 1.0f) * (vc.Tv + 1.0f);
+    const int Rv = (int)(p.Tq >> 16) + 2;
+    const int mxy = mac_xy(p.Tq), mn = mxy * mxy * mac_z(p.Tq);
+    // macro blocks per work item: enough items for every warp to get several, at most one per lane
+    const int group = (int)max(1ll, min(32ll, (long long)nn * mn / ((long long)gridDim.x * kWarpsN * 8)));
+    // too few blocks to fill the GPU: an item takes every split-th yaw of a block
+    const int split = (long long)nn * mn < 2ll * gridDim.x * kWarpsN ? min(K, 8) : 1;
+    const int gpn = (mn + group - 1) / group * split;
+    NodeCnt st;
+    int cur = -1, cur_kb = 0, na = 0;
+    int c_abs[2] = {0, 0}, c_mrg[2] = {0, 0};  // node cur, yaws cur_kb + lane and cur_kb + 32 + lane
+    for (;;) {
+        int it = 0;
+        if (lane == 0) it = atomicAdd(p.vctr, 1);
+        it = __shfl_sync(0xffffffffu, it, 0);
+        if (it >= nn * gpn) break;
+        const int ln = it / gpn, sub = (it - ln * gpn) % split, g0 = (it - ln * gpn) / split * group;
+        const int n = p.level_nodes[l0 + nb0 + ln];
+        const int4 nd = p.node[n];
+        const int v0x = nd.x >> 16, v0y = nd.y >> 16, v0z = nd.z >> 16;
+        // lane = macro block of the item: inside the grid, the ball and the elevation band?
+        int mX = 0, mY = 0, mZ = 0;
+        bool live = false;
+        {
+            const int mi = g0 + lane;
+            if (lane < group && mi < mn) {
+                const int a = mi / mxy;
+                mX = ((v0x - Rv) >> 4) + (mi - a * mxy);
+                mZ = ((v0z - Rv) >> 3) + a / mxy;
+                mY = ((v0y - Rv) >> 4) + (a - (a / mxy) * mxy);
+                if (mX >= 0 && mY >= 0 && mZ >= 0 && 16 * mX < p.grid.nx && 16 * mY < p.grid.ny && 8 * mZ < p.grid.nz) {
+                    const float cx = q16f(((16 * mX + 8) << 16) - nd.x), cy = q16f(((16 * mY + 8) << 16) - nd.y),
+                                cz = q16f(((8 * mZ + 4) << 16) - nd.z);
+                    const float dx = fmaxf(fabsf(cx) - 7.5f, 0.f), dy = fmaxf(fabsf(cy) - 7.5f, 0.f),
+                                dz = fmaxf(fabsf(cz) - 3.5f, 0.f);
+                    const float rho = sqrtf(cx * cx + cy * cy), r0 = fmaxf(rho - 10.7f, 0.f), r1 = rho + 10.7f;
+                    const float eps = 0.01f * (r1 + fabsf(cz) + 4.f) + 0.05f;
+                    live = dx * dx + dy * dy + dz * dz <= R2 &&
+                           (p.band_thi >= 1e29f || cz - 3.5f <= p.band_thi * (p.band_thi > 0.f ? r1 : r0) + eps) &&
+                           (p.band_tlo <= -1e29f || cz + 3.5f >= p.band_tlo * (p.band_tlo < 0.f ? r1 : r0) - eps);
+                }
+            }
+        }
+        unsigned todo = __ballot_sync(0xffffffffu, live);
+        if (todo && n != cur) {
+            if (cur >= 0) flush_counts<STATS>(p, cur, cur_kb, lane, c_abs, c_mrg, st);
+            cur = n;
+            na = node_ancestors(p, n, anc, WH, pyr.n, lane);
+        }
+        const uint32_t *hz = p.hz + (size_t)ln * K * pyr.n;
+#pragma unroll 1
+        for (; todo; todo &= todo - 1) {
+            const int src = __ffs(todo) - 1;
+            const int X = __shfl_sync(0xffffffffu, mX, src) * 4, Y = __shfl_sync(0xffffffffu, mY, src) * 4,
+                      Z = __shfl_sync(0xffffffffu, mZ, src) * 2;  // the block's first brick
+            // ---- lane = brick
+            const int bx = X + (lane & 3), by = Y + ((lane >> 2) & 3), bz = Z + (lane >> 4);
+            uint64_t U = 0;
+            if (bx < bd.nbx && by < bd.nby && bz < bd.nbz) U = ld_u64(umask + ((size_t)(bz * bd.nby + by) * bd.nbx + bx));
+            const float cx = q16f(((4 * bx + 2) << 16) - nd.x), cy = q16f(((4 * by + 2) << 16) - nd.y),
+                        cz = q16f(((4 * bz + 2) << 16) - nd.z);
+            float far;
+            {
+                const float dx = fmaxf(fabsf(cx) - 1.5f, 0.f), dy = fmaxf(fabsf(cy) - 1.5f, 0.f), dz = fmaxf(fabsf(cz) - 1.5f, 0.f);
+                if (dx * dx + dy * dy + dz * dz > R2) U = 0;
+                const float ex = fabsf(cx) + 1.5f, ey = fabsf(cy) + 1.5f, ez = fabsf(cz) + 1.5f;
+                far = sqrtf(ex * ex + ey * ey + ez * ez);
+            }
+            if (!__any_sync(0xffffffffu, U != 0)) continue;
+            // Manhattan distances (step indices) of the brick's voxels from the start voxel
+            int man0, man1;
+            {
+                const int ax = 4 * bx - v0x, ay = 4 * by - v0y, az = 4 * bz - v0z;
+                man0 = max(max(ax, -ax - 3), 0) + max(max(ay, -ay - 3), 0) + max(max(az, -az - 3), 0);
+                man1 = max(abs(ax), abs(ax + 3)) + max(abs(ay), abs(ay + 3)) + max(abs(az), abs(az + 3));
+            }
+            const float gx = q16f(((4 * X + 8) << 16) - nd.x), gy = q16f(((4 * Y + 8) << 16) - nd.y),
+                        gz = q16f(((4 * Z + 4) << 16) - nd.z);  // the block's centre
+            const int mac_man0 = __reduce_min_sync(0xffffffffu, U ? man0 : 0x7fffffff);
+#pragma unroll 1
+            for (int kb = 0; kb < K; kb += 64) {
+                // ---- lane = yaw: which yaws may count a voxel of the block?
+                uint64_t yaws = 0;
+#pragma unroll 1
+                for (int i = 0; i < 64 && kb + i < K; i += 32) {
+                    bool may = false;
+                    const int k = kb + i + lane;
+                    if (k < K && k % split == sub) {
+                        const BoxView b = box_view<false>(s_y[k], gx, gy, gz, 7.5f, 7.5f, 3.5f, W, H);
+                        may = b.in >= 0;
+                        if (may && box_lookup(b)) {
+                            const uint32_t hm = hz_box(hz + (size_t)k * pyr.n, pyr, top, b);
+                            may = mac_man0 < (int)((hm >> 16) ^ 0xFFFFu);  // else every ray stops before the block
+                        }
+                    }
+                    yaws |= (uint64_t)__ballot_sync(0xffffffffu, may) << i;
+                }
+                // ---- lane = brick against each of them
+                uint64_t all = 0, part = 0, rch = 0, vis = 0;  // bit k - kb
+#pragma unroll 1
+                for (uint64_t ks = yaws; ks; ks &= ks - 1) {
+                    const int j = __ffsll((long long)ks) - 1;
+                    if (U) {
+                        const BoxView b = box_view<true>(s_y[kb + j], cx, cy, cz, 1.5f, 1.5f, 1.5f, W, H);
+                        bool some = b.in >= 0, reach = false, sure = false;  // all reached; all visited for certain
+                        if constexpr (STATS) {
+                            st.cand += 64;
+                            st.unk += __popcll(U);
+                        }
+                        if (some && b.zlo >= 0.5f) {
+                            if (box_lookup(b)) {
+                                const uint32_t hm = hz_box(hz + (size_t)(kb + j) * pyr.n, pyr, top, b);
+                                some = man0 < (int)((hm >> 16) ^ 0xFFFFu);
+                                reach = man1 < (int)(hm & 0xFFFFu);
+                            }
+                            sure = (b.zhi < s_y[kb + j].x.x && far + 0.86f < vc.Tv) || (b.zhi < p.vis_zl2 && far + 0.02f < vc.Tv);
+                        }
+                        if (some) {
+                            const uint64_t bit = 1ull << j;
+                            const bool whole = b.in > 0 && reach && sure;
+                            all |= whole ? bit : 0ull;
+                            part |= whole ? 0ull : bit;
+                            rch |= reach ? 0ull : bit;
+                            vis |= sure ? 0ull : bit;
+                        }
+                    }
+                }
+                const bool want = (all | part) != 0;
+                if (!__any_sync(0xffffffffu, want)) continue;
+                // ---- the ancestors' test (Sec. IV-B) of the bricks some yaw may count
+                uint64_t O = 0, left = 0;  // observed voxels; ancestors undecided for the brick
+#pragma unroll 1
+                for (int ab = 0; ab < na; ab += 32) {
+                    bool rel = false;  // lane = ancestor: does it look at the block, not behind its depths?
+                    if (ab + lane < na) {
+                        const NodeAnc A = anc[ab + lane];
+                        const float ox = q16f(((4 * X + 8) << 16) - A.px), oy = q16f(((4 * Y + 8) << 16) - A.py),
+                                    oz = q16f(((4 * Z + 4) << 16) - A.pz);
+                        const BoxView b = box_view<false>(s_y[A.yaw], ox, oy, oz, 7.5f, 7.5f, 3.5f, W, H);
+                        rel = b.in >= 0;
+                        if (rel && box_lookup(b)) {
+                            const uint2 D = depth_box(A.pyr, pyr, b);
+                            rel = b.zlo * (65536.0f * (1.0f - 1e-6f)) <= (float)D.y + 1.5f;
+                        }
+                    }
+#pragma unroll 1
+                    for (unsigned as = __ballot_sync(0xffffffffu, rel); as; as &= as - 1) {
+                        const int a = ab + __ffs(as) - 1;
+                        if (want && O != U) {
+                            const NodeAnc A = anc[a];
+                            const float ox = q16f(((4 * bx + 2) << 16) - A.px), oy = q16f(((4 * by + 2) << 16) - A.py),
+                                        oz = q16f(((4 * bz + 2) << 16) - A.pz);
+                            const BoxView b = box_view<true>(s_y[A.yaw], ox, oy, oz, 1.5f, 1.5f, 1.5f, W, H);
+                            bool vox = b.in >= 0;
+                            if (vox && box_lookup(b)) {
+                                const uint2 D = depth_box(A.pyr, pyr, b);
+                                if (b.zlo * (65536.0f * (1.0f - 1e-6f)) > (float)D.y + 1.5f) {
+                                    vox = false;
+                                } else if (b.in > 0 && b.zhi * (65536.0f * (1.0f + 1e-6f)) < (float)D.x) {
+                                    O = U;
+                                    vox = false;
+                                }
+                            }
+                            if (vox) left |= 1ull << a;
+                        }
+                    }
+                }
+                if (O == U) left = 0;
+                if (kb != cur_kb) {
+                    flush_counts<STATS>(p, cur, cur_kb, lane, c_abs, c_mrg, st);
+                    cur_kb = kb;
+                }
+                // ---- decided bricks: population counts; lane j % 32 keeps the counts of yaw kb + j
+                const bool rec = part != 0 || (all != 0 && left != 0);
+                const unsigned pc = (unsigned)__popcll(U) | ((unsigned)__popcll(U & ~O) << 16);
+#pragma unroll 1
+                for (uint64_t ks = or64(rec ? 0ull : all); ks; ks &= ks - 1) {
+                    const int j = __ffsll((long long)ks) - 1;
+                    const unsigned v = __reduce_add_sync(0xffffffffu, !rec && ((all >> j) & 1) ? pc : 0u);
+                    if (lane == (j & 31)) {
+                        const int i = j >> 5;
+                        c_abs[0] += i ? 0 : (int)(v & 0xFFFF);
+                        c_mrg[0] += i ? 0 : (int)(v >> 16);
+                        c_abs[1] += i ? (int)(v & 0xFFFF) : 0;
+                        c_mrg[1] += i ? (int)(v >> 16) : 0;
+                        if constexpr (STATS) st.visit += v & 0xFFFF;
+                    }
+                }
+                // ---- undecided bricks: to the queue (counted here if it is full)
+                const unsigned recs = __ballot_sync(0xffffffffu, rec);
+                if (recs) {
+                    int at = 0;
+                    if (lane == 0) at = atomicAdd(p.vctr + 1, __popc(recs));
+                    at = __shfl_sync(0xffffffffu, at, 0) + __popc(recs & ((1u << lane) - 1u));
+                    BrickRec r{U, O, left, all, part, rch, vis, (uint32_t)bx | ((uint32_t)by << 10) | ((uint32_t)bz << 20),
+                               (uint32_t)ln | ((uint32_t)(kb >> 6) << kRecNodeBits)};
+                    if (rec && at < p.queue_cap) p.queue[at] = r;
+#pragma unroll 1
+                    for (unsigned full = __ballot_sync(0xffffffffu, rec && at >= p.queue_cap); full; full &= full - 1) {
+                        const int s = __ffs(full) - 1;
+                        BrickRec q{shfl64(r.U, s), shfl64(r.O, s), shfl64(r.anc, s), shfl64(r.all, s), shfl64(r.part, s),
+                                   shfl64(r.rch, s), shfl64(r.vis, s), __shfl_sync(0xffffffffu, r.brick, s), r.node};
+                        count_brick<STATS>(p, vc, s_y, anc, nd, p.steps + (size_t)ln * K * WH, q, lane, c_abs, c_mrg, st);
+                    }
+                }
+            }
+        }
+    }
+    if (cur >= 0) flush_counts<STATS>(p, cur, cur_kb, lane, c_abs, c_mrg, st);
+    add_stats<STATS>(p, st);
+}
+
+// The queue's records, one warp each, in slices of consecutive records (mostly of one node).
+template <bool STATS>
+__global__ void __launch_bounds__(kWarpsN * 32, 4) brick_kernel(const LevelParams p) {
+    extern __shared__ __align__(16) unsigned char s_dyn[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int K = p.K;
+    YawRows *s_y = reinterpret_cast<YawRows *>(s_dyn);
+    NodeAnc *anc = reinterpret_cast<NodeAnc *>(s_y + K) + warp * p.max_anc;
+    const int l0 = p.level_off[p.lvl];
+    const int nb0 = p.q0 / K;
+    if (min(p.q1 / K, p.level_off[p.lvl + 1] - l0) <= nb0) return;
+    const int total = min(p.vctr[1], p.queue_cap);
+    const int slice = max(1, min(64, total / (int)(gridDim.x * kWarpsN * 8)));
+    if (blockIdx.x * kWarpsN * slice >= total) return;
+    for (int k = threadIdx.x; k < K; k += blockDim.x)
+        s_y[k] = yaw_rows(p.yawtab + k * 12, p.W, p.H, p.vis_hu, p.vis_hv, p.ifx, p.ify);
+    __syncthreads();
+    const size_t WH = (size_t)p.W * p.H;
+    const int pyr_n = pyramid(p.W, p.H).n;
+    const VoxConst vc = vox_const(p);
+    NodeCnt st;
+    uint32_t cur = 0xFFFFFFFFu;
+    int n = 0, c_abs[2] = {0, 0}, c_mrg[2] = {0, 0};
+    int4 nd = make_int4(0, 0, 0, 0);
+    for (;;) {
+        int i = 0;
+        if (lane == 0) i = atomicAdd(p.vctr + 2, slice);
+        i = __shfl_sync(0xffffffffu, i, 0);
+        if (i >= total) break;
+        const int end = min(i + slice, total);
+#pragma unroll 1
+        for (; i < end; ++i) {
+            const BrickRec r = p.queue[i];
+            if (r.node != cur) {
+                if (cur != 0xFFFFFFFFu) flush_counts<STATS>(p, n, (int)(cur >> kRecNodeBits) * 64, lane, c_abs, c_mrg, st);
+                cur = r.node;
+                n = p.level_nodes[l0 + nb0 + (int)(cur & ((1u << kRecNodeBits) - 1))];
+                nd = p.node[n];
+                node_ancestors(p, n, anc, WH, pyr_n, lane);
+            }
+            count_brick<STATS>(p, vc, s_y, anc, nd, p.steps + (size_t)(cur & ((1u << kRecNodeBits) - 1)) * K * WH, r, lane, c_abs,
+                               c_mrg, st);
+        }
+    }
+    if (cur != 0xFFFFFFFFu) flush_counts<STATS>(p, n, (int)(cur >> kRecNodeBits) * 64, lane, c_abs, c_mrg, st);
+    add_stats<STATS>(p, st);
+}
+
+// ---------------------------------------------------------------------------- brick data update
+// Masks of the bricks [b0, b1) from the voxel codes: one thread per brick. A row of four codes is
+// one 32-bit load where rows are 4-byte aligned; the codes 0 / 1 / 2 differ in their two low bits.
+__device__ __forceinline__ uint32_t nibble(uint32_t v) { return ((v & 0x01010101u) * 0x01020408u) >> 24; }
+
+__global__ void brick_mask_kernel(uint8_t *grid, int nx, int ny, int nz, int bx0, int by0, int bz0, int bx1, int by1, int bz1) {
+    const int nbx = (nx + 3) >> 2, nby = (ny + 3) >> 2;
+    uint64_t *um = reinterpret_cast<uint64_t *>(grid + umask_offset(nx, ny, nz));
+    uint64_t *om = reinterpret_cast<uint64_t *>(grid + omask_offset(nx, ny, nz));
+    const int wx = bx1 - bx0, wy = by1 - by0;
+    const long long total = (long long)wx * wy * (bz1 - bz0);
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
+        const int bx = bx0 + (int)(i % wx), by = by0 + (int)((i / wx) % wy), bz = bz0 + (int)(i / ((long long)wx * wy));
+        const int w = min(4, nx - 4 * bx);
+        uint64_t u = 0, o = 0;
+        for (int z = 0; z < 4 && 4 * bz + z < nz; ++z)
+            for (int y = 0; y < 4 && 4 * by + y < ny; ++y) {
+                const uint8_t *r = grid + ((size_t)(4 * bz + z) * ny + (4 * by + y)) * nx + 4 * bx;
+                uint32_t c = 0x01010101u;  // beyond the grid: neither unknown nor occupied
+                if ((nx & 3) == 0) c = *reinterpret_cast<const uint32_t *>(r);
+                else
+                    for (int x = 0; x < w; ++x) c = (c & ~(0xFFu << (8 * x))) | ((uint32_t)r[x] << (8 * x));
+                u |= (uint64_t)nibble(~(c | (c >> 1))) << (16 * z + 4 * y);
+                o |= (uint64_t)nibble(c >> 1) << (16 * z + 4 * y);
+            }
+        const size_t b = ((size_t)bz * nby + by) * nbx + bx;
+        um[b] = u;
+        om[b] = o;
+    }
+}
+
+// One pass of the Chebyshev distance to the nearest brick with an occupied voxel, over the bricks of
+// a box: along x from the masks (pass 0, into scratch 0), along y (pass 1, scratch 0 to 1), along
+// z (pass 2, scratch 1 to dist). d = min over j of max(|j|, the previous pass at offset j).
+__global__ void brick_dist_kernel(uint8_t *grid, int nx, int ny, int nz, int pass, int bx0, int by0, int bz0, int bx1, int by1,
+                                  int bz1) {
+    const int nbx = (nx + 3) >> 2, nby = (ny + 3) >> 2, nbz = (nz + 3) >> 2;
+    const uint64_t *om = reinterpret_cast<const uint64_t *>(grid + omask_offset(nx, ny, nz));
+    const uint8_t *src = grid + dist_scratch_offset(nx, ny, nz, pass == 2);
+    uint8_t *dst = grid + (pass == 2 ? dist_offset(nx, ny, nz) : dist_scratch_offset(nx, ny, nz, pass));
+    const int wx = bx1 - bx0, wy = by1 - by0;
+    const long long total = (long long)wx * wy * (bz1 - bz0);
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
+        const int bx = bx0 + (int)(i % wx), by = by0 + (int)((i / wx) % wy), bz = bz0 + (int)(i / ((long long)wx * wy));
+        const size_t b = ((size_t)bz * nby + by) * nbx + bx;
+        int d = kDistCap;
+        if (pass == 0) {
+            for (int j = 0; j < d; ++j)
+                if ((bx - j >= 0 && om[b - j]) || (bx + j < nbx && om[b + j])) d = j;
+        } else {
+            const int c = pass == 1 ? by : bz, n = pass == 1 ? nby : nbz;
+            const ptrdiff_t step = pass == 1 ? nbx : (ptrdiff_t)nbx * nby;
+            for (int j = 0; j < d; ++j) {
+                int e = kDistCap;
+                if (c - j >= 0) e = min(e, (int)src[(ptrdiff_t)b - j * step]);
+                if (c + j < n) e = min(e, (int)src[(ptrdiff_t)b + j * step]);
+                d = min(d, max(e, j));
+            }
+        }
+        dst[b] = (uint8_t)d;
+    }
+}
+
+size_t node_dyn_smem(int K, int max_anc) {
+    return (size_t)K * sizeof(YawRows) + (size_t)kWarpsN * std::max(1, max_anc) * sizeof(NodeAnc);
+}
+
+}  // namespace
+
+size_t hz_entries(int W, int H) { return (size_t)pyramid(W, H).n; }
+
+void set_visit_params(LevelParams &p, float hfov_deg, float vfov_deg) {
+    const VisitLimits l = visit_limits(hfov_deg, vfov_deg, p.W, p.H);
+    p.vis_hu = l.hu;
+    p.vis_hv = l.hv;
+    p.vis_zl2 = l.zl2;
+    p.ifx = (float)(std::tan(hfov_deg * 0.5 * (3.14159265358979323846 / 180.0)) / (p.W * 0.5));
+    p.ify = (float)(std::tan(vfov_deg * 0.5 * (3.14159265358979323846 / 180.0)) / (p.H * 0.5));
+}
+
+// CTAs for a cast of `images` images (an upper bound of the level's): one per 16x16 tile, at most as
+// many as keep the kernel's loops short.
+static int cast_grid(long long images, int W, int H, int num_sms) {
+    const long long tiles = images * ((W + 15) / 16) * ((H + 15) / 16);
+    return (int)std::max<long long>(1, std::min<long long>(tiles, (long long)num_sms * 64));
+}
+
+void launch_cast_chunk(const LevelParams &c, int num_sms, cudaStream_t s) {
+    const int g = cast_grid(c.q1 - c.q0, c.W, c.H, num_sms);
+    if (c.stats) cast_kernel<true><<<g, kWarpsN * 32, 0, s>>>(c, num_sms);
+    else cast_kernel<false><<<g, kWarpsN * 32, 0, s>>>(c, num_sms);
+}
+
+void launch_render(const LevelParams &p, int nodes, int num_sms, cudaStream_t s) {
+    const int g = cast_grid(nodes, p.W, p.H, num_sms);
+    if (p.stats) render_kernel<true><<<g, kWarpsN * 32, 0, s>>>(p, num_sms);
+    else render_kernel<false><<<g, kWarpsN * 32, 0, s>>>(p, num_sms);
+}
+
+int node_ctas_per_sm() {
+    // the most yaws and the deepest tree: 112 KB
+    const int smem = (int)node_dyn_smem(MIG_MAX_YAW_BINS, MIG_MAX_DEPTH);
+    cudaFuncSetAttribute(node_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaFuncSetAttribute(node_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaFuncSetAttribute(brick_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaFuncSetAttribute(brick_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    int a = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, node_kernel<false>, kWarpsN * 32, node_dyn_smem(36, 16));
+    cudaGetLastError();
+    return std::max(1, a);
+}
+
+// Macro blocks of a node's range ball (its bounding box): the node pass's items per node.
+long long node_items(int64_t Tq) { return (long long)mac_xy(Tq) * mac_xy(Tq) * mac_z(Tq); }
+
+void launch_node_chunk(const LevelParams &c, int num_sms, int node_ctas, cudaStream_t s) {
+    const long long items = (long long)((c.q1 - c.q0) / c.K) * node_items(c.Tq);
+    const int g = (int)std::max<long long>(1, std::min<long long>((items + kWarpsN - 1) / kWarpsN, (long long)num_sms * node_ctas));
+    const size_t smem = node_dyn_smem(c.K, c.max_anc);
+    const int gb = num_sms * 4;
+    if (c.stats) {
+        node_kernel<true><<<g, kWarpsN * 32, smem, s>>>(c, num_sms);
+        brick_kernel<true><<<gb, kWarpsN * 32, smem, s>>>(c);
+    } else {
+        node_kernel<false><<<g, kWarpsN * 32, smem, s>>>(c, num_sms);
+        brick_kernel<false><<<gb, kWarpsN * 32, smem, s>>>(c);
+    }
+}
+
+// Bricks that a node's range ball can touch, and the records a chunk's queue has room for per node
+// (measured: up to 0.27 of them are left undecided as a whole; a fuller queue only sends its last
+// bricks through the slower path inside node_kernel).
+static long long node_bricks(int64_t Tq) {
+    const double r = ((double)Tq / 65536.0 + 1.0) / 4.0 + 1.74;
+    return (long long)(4.19 * r * r * r) + 1;
+}
+constexpr double kQueueShare = 0.3;
+constexpr long long kQueueMax = 8ll << 20;  // records (512 MB)
+
+StepsLayout steps_layout(const SensorDims &d, int max_nodes, size_t budget_bytes, bool node_pass) {
+    StepsLayout L{};
+    const size_t WH = (size_t)d.W * d.H;
+    const long long pairs = (long long)std::max(1, max_nodes) * d.K;
+    L.cap = (int)steps_pairs(pairs, d.W, d.H, budget_bytes);
+    const long long per_node = (long long)(kQueueShare * (double)node_bricks(d.Tq)) + 1;
+    if (node_pass && L.cap >= d.K) {  // whole nodes, as many as the queue has room for
+        const long long nodes = std::max<long long>(1, std::min<long long>(L.cap / d.K, kQueueMax / per_node));
+        L.cap = (int)nodes * d.K;
+        L.queue_cap = (int)std::min(kQueueMax, std::max<long long>(nodes * per_node, 1ll << 16));
+    }
+    auto align = [](size_t b) { return (b + 255) & ~(size_t)255; };
+    L.o_ctr = align((size_t)L.cap * WH * sizeof(uint16_t));
+    L.o_hz = L.o_ctr + 256;
+    L.o_queue = align(L.o_hz + (size_t)L.cap * hz_entries(d.W, d.H) * sizeof(uint32_t));
+    L.bytes = L.o_queue + (size_t)L.queue_cap * sizeof(BrickRec);
+    return L;
+}
+
+void set_steps(LevelParams &p, void *base, const StepsLayout &L) {
+    char *b = static_cast<char *>(base);
+    p.steps = reinterpret_cast<uint16_t *>(b);
+    p.vctr = reinterpret_cast<int32_t *>(b + L.o_ctr);
+    p.hz = reinterpret_cast<uint32_t *>(b + L.o_hz);
+    p.queue = reinterpret_cast<BrickRec *>(b + L.o_queue);
+    p.queue_cap = L.queue_cap;
+    p.steps_cap = L.cap;
+}
+
+void launch_brick_update(uint8_t *grid, int nx, int ny, int nz, int x0, int y0, int z0, int dx, int dy, int dz, cudaStream_t s) {
+    const BrickDims n = brick_dims(nx, ny, nz);
+    const int lo[3] = {x0 >> 2, y0 >> 2, z0 >> 2}, hi[3] = {(x0 + dx + 3) >> 2, (y0 + dy + 3) >> 2, (z0 + dz + 3) >> 2};
+    auto blocks = [](long long t) { return (int)std::max<long long>(1, std::min<long long>((t + 127) / 128, 8192)); };
+    brick_mask_kernel<<<blocks((long long)(hi[0] - lo[0]) * (hi[1] - lo[1]) * (hi[2] - lo[2])), 128, 0, s>>>(
+        grid, nx, ny, nz, lo[0], lo[1], lo[2], hi[0], hi[1], hi[2]);
+    // a brick's distance depends on the bricks up to kDistCap - 1 away along each axis
+    const int r = kDistCap, nb[3] = {n.nbx, n.nby, n.nbz};
+    int a[3], b[3], a2[3], b2[3];  // the bricks whose distance can change, and one reach beyond
+    for (int i = 0; i < 3; ++i) {
+        a[i] = std::max(0, lo[i] - r);
+        b[i] = std::min(nb[i], hi[i] + r);
+        a2[i] = std::max(0, lo[i] - 2 * r);
+        b2[i] = std::min(nb[i], hi[i] + 2 * r);
+    }
+    auto dist = [&](int pass, int ya, int yb, int za, int zb) {
+        brick_dist_kernel<<<blocks((long long)(b[0] - a[0]) * (yb - ya) * (zb - za)), 128, 0, s>>>(grid, nx, ny, nz, pass, a[0], ya, za,
+                                                                                                 b[0], yb, zb);
+    };
+    dist(0, a2[1], b2[1], a2[2], b2[2]);
+    dist(1, a[1], b[1], a2[2], b2[2]);
+    dist(2, a[1], b[1], a[2], b[2]);
+}
+
+}  // namespace mig

@@ -48,7 +48,7 @@ struct Request {
     mig_sensor sensor{};
     int mode = 0;
     HostPlan plan;
-    int steps_cap = 0;  // owned-voxel count: (node, yaw) pairs per chunk (0 = ray by ray)
+    StepsLayout steps{};  // owned-voxel count's region (cap 0 = ray by ray)
     int32_t *out_abs = nullptr, *out_marg = nullptr, *out_yaw = nullptr;
     const Camera *cam = nullptr;
     // device state while in flight
@@ -126,7 +126,8 @@ size_t request_bytes(const Request &r) {
     cv.take(12 * n);
     cv.take(4 * n);
     cv.take(4 * std::max(1, pl.n_internal) * WH);
-    cv.take(steps_region_bytes(r.steps_cap, WH));
+    cv.take(sizeof(uint2) * std::max(1, pl.n_internal) * hz_entries(r.sensor.width, r.sensor.height));
+    cv.take(r.steps.bytes);
     return cv.off;
 }
 
@@ -160,8 +161,9 @@ mig_status admit(mig_server *s, Request &r) {
     const size_t zero_end = cv.off;
     const size_t o_out = cv.take(12 * (size_t)n), o_sel = cv.take(4 * (size_t)n);
     const size_t o_arena = cv.take(4 * (size_t)std::max(1, pl.n_internal) * WH);
+    const size_t o_dpyr = cv.take(sizeof(uint2) * (size_t)std::max(1, pl.n_internal) * hz_entries(r.sensor.width, r.sensor.height));
     const size_t o_pcnt = pano ? cv.take(8 * (size_t)n * r.cam->pano_A) : 0;
-    const size_t o_steps = cv.take(steps_region_bytes(r.steps_cap, WH));
+    const size_t o_steps = cv.take(r.steps.bytes);
     r.dev_bytes = cv.off;
     r.dev = (char *)ctx->alloc.alloc(r.dev_bytes, ctx->stream);
     if (!r.dev) return fail(MIG_ENOMEM, "server: request allocation failed");
@@ -223,10 +225,9 @@ mig_status admit(mig_server *s, Request &r) {
     p.stats = nullptr;
     p.max_anc = std::max(1, pl.max_depth);
     if (pano) set_pano_params(p, r.cam, (int32_t *)(r.dev + o_pcnt));
-    p.steps = r.steps_cap ? (uint16_t *)(r.dev + o_steps) : nullptr;
-    p.vctr = steps_counter((uint16_t *)(r.dev + o_steps), r.steps_cap, WH);
+    if (r.steps.cap) set_steps(p, r.dev + o_steps, r.steps);
+    p.dpyr = (uint2 *)(r.dev + o_dpyr);
     p.voxel_pass = ctx->voxel_pass;
-    p.steps_cap = r.steps_cap;
     r.level = 0;
     return MIG_OK;
 }
@@ -287,7 +288,7 @@ mig_status run_step(mig_server *s) {
     cudaStream_t s0 = ctx->stream;
     MIG_CUDA_TRY(cudaEventRecord(s->fork, s0));
     for (int i = 0; i < S; ++i) MIG_CUDA_TRY(cudaStreamWaitEvent(s->pool[i], s->fork, 0));
-    const int cap = ctx->num_sms * 16, count_cap = ctx->num_sms * ctx->count_ctas;
+    const int count_cap = ctx->num_sms * ctx->count_ctas;
     const Clock::time_point now = Clock::now();
     for (int i = 0; i < R; ++i) {
         Request &r = *s->inflight[i];
@@ -300,7 +301,7 @@ mig_status run_step(mig_server *s) {
         const int Ld = pl.level_off[d + 1] - pl.level_off[d];
         launch_level_count(ctx, p, Ld, count_cap, st);
         launch_select(p, std::max(1, std::min((Ld + 127) / 128, 1024)), st);
-        if (pl.level_int[d] > 0 && d < pl.max_depth) launch_render(p, std::min(pl.level_int[d] * render_tiles(p.W, p.H), cap), st);
+        if (pl.level_int[d] > 0 && d < pl.max_depth) launch_render(p, pl.level_int[d], ctx->num_sms, st);
     }
     MIG_CUDA_TRY(cudaGetLastError());
     for (int i = 0; i < S; ++i) {
@@ -468,7 +469,7 @@ extern "C" mig_status mig_server_submit(mig_server *s, const mig_tree_desc *d, u
         int Lmax = 1;
         for (int lv = 0; lv <= r->plan.max_depth; ++lv)
             Lmax = std::max(Lmax, r->plan.level_off[lv + 1] - r->plan.level_off[lv]);
-        r->steps_cap = steps_cap_for(s->ctx, Lmax, d->sensor.yaw_bins, d->sensor.width, d->sensor.height, d->mode);
+        r->steps = steps_for(s->ctx, Lmax, d->sensor, d->map->voxel, d->mode);
     }
     r->out_abs = d->abs_gain;
     r->out_marg = d->marg_gain;

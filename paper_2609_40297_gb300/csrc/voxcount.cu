@@ -1,8 +1,7 @@
 // Owned-voxel count of one tree level (Sec. IV-B, the counts of Eq. 1 and Eq. 2 by depth
-// buffers), in two kernels per chunk of (node, yaw) pairs:
-//   cast_kernel  - every pixel ray of every pair runs the DDA to its first occupied voxel within
-//                  range and stores that voxel's step index (uint16 per ray; kNoHit if none);
-//   voxel_kernel - for every pair, the voxels within range of the node are enumerated slice by
+// buffers), per chunk of (node, yaw) pairs: the cast and the per-node count are in nodecount.cu;
+//   voxel_kernel - the count of single (node, yaw) pairs, for chunks that do not hold whole nodes
+//                  (or when asked for): for every pair, the voxels within range of the node are enumerated slice by
 //                  slice (z), rows clipped to the camera frustum; each unknown voxel goes to the
 //                  pixel that owns it (its centre's projection) and counts as absolute gain iff
 //                  that pixel's DDA reaches it before the range and before its first occupied
@@ -26,46 +25,10 @@ namespace {
 
 using namespace dev;
 
-constexpr int kCastWarps = 8;   // 256-thread CTAs, one ray per thread
 constexpr int kVoxWarps = 8;
 
 __device__ __forceinline__ int level_pairs(const LevelParams &p) {
     return (p.level_off[p.lvl + 1] - p.level_off[p.lvl]) * p.K;
-}
-
-// ------------------------------------------------------------------------------ cast kernel
-// Warp work item = (pair q of the chunk, 8x4 pixel tile); one ray per lane.
-
-template <bool STATS>
-__global__ void __launch_bounds__(kCastWarps * 32) cast_kernel(const LevelParams p) {
-    const int lane = threadIdx.x & 31;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *p.vctr = 0;  // the voxel pass that follows hands out work from 0
-    const int l0 = p.level_off[p.lvl];
-    const int q1 = min(p.q1, level_pairs(p));
-    if (p.q0 >= q1) return;
-    const int tx = (p.W + kCastTileW - 1) / kCastTileW, ty = (p.H + kCastTileH - 1) / kCastTileH;
-    const long long items = (long long)(q1 - p.q0) * tx * ty;
-    const size_t WH = (size_t)p.W * p.H;
-    const uint8_t *bocc = p.grid.g + bocc_offset(p.grid.nx, p.grid.ny, p.grid.nz);
-    const uint8_t *sbocc = p.grid.g + sbocc_offset(p.grid.nx, p.grid.ny, p.grid.nz);
-    uint32_t st_rays = 0, st_fine = 0, st_skip = 0;
-    for (long long it = (long long)blockIdx.x * kCastWarps + (threadIdx.x >> 5); it < items;
-         it += (long long)gridDim.x * kCastWarps) {
-        const int tile = (int)(it % (tx * ty));
-        const int ql = (int)(it / (tx * ty));
-        cast_item<STATS>(p, bocc, sbocc, l0, p.q0 + ql, tile, tx, p.steps + (size_t)ql * WH, lane, st_rays, st_fine,
-                         st_skip);
-    }
-    if constexpr (STATS) {
-        st_rays = __reduce_add_sync(0xffffffffu, st_rays);
-        st_fine = __reduce_add_sync(0xffffffffu, st_fine);
-        st_skip = __reduce_add_sync(0xffffffffu, st_skip);
-        if (lane == 0) {
-            atomicAdd(p.stats + 8, (unsigned long long)st_rays);
-            atomicAdd(p.stats + 9, (unsigned long long)st_fine);
-            atomicAdd(p.stats + 10, (unsigned long long)st_skip);
-        }
-    }
 }
 
 // ----------------------------------------------------------------------------- voxel kernel
@@ -283,80 +246,6 @@ __global__ void __launch_bounds__(kVoxWarps * 32, 3) voxel_kernel(const LevelPar
     }
 }
 
-// ------------------------------------------------------------------------ per-node voxel kernel
-// The same counts with each voxel taken once per node for all yaws: the ancestor test of Sec. IV-B
-// does not depend on the node's own yaw, and a voxel lies in several yaws' frusta. Warp work item
-// = (node of the chunk, slice z of its range ball, 32-row block of the slice), run by node_run
-// (voxitems.cuh); the warp's per-yaw counters go to the level's counters when its node changes.
-template <bool STATS>
-__global__ void __launch_bounds__(kVoxWarps * 32, 4) node_kernel(const LevelParams p) {
-    extern __shared__ __align__(16) unsigned char s_dyn[];
-    __shared__ NodeWarp s_nw[kVoxWarps];
-    __shared__ int s_yi[kNodeMaxK * 12];    // yaw rows: ck sk mu mv mz -
-    __shared__ float s_yf[kNodeMaxK * 9];   // mu mv mz / 2^16
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int K = p.K;
-    AncRec *anc = reinterpret_cast<AncRec *>(s_dyn) + warp * p.max_anc;
-    NodeWarp &Q = s_nw[warp];
-    const int l0 = p.level_off[p.lvl];
-    const int Ld = p.level_off[p.lvl + 1] - l0;
-    const int nb0 = p.q0 / K, nb1 = min(p.q1 / K, Ld);
-    if (nb0 >= nb1) return;
-    for (int t = threadIdx.x; t < 12 * K; t += blockDim.x) s_yi[t] = p.yawtab[t];
-    for (int t = threadIdx.x; t < 9 * K; t += blockDim.x) s_yf[t] = (float)p.yawtab[(t / 9) * 12 + 2 + t % 9] * (1.0f / 65536.0f);
-    for (int t = lane; t < 2 * K; t += 32) Q.cnt[t] = 0;
-    __syncthreads();
-    const int slices = 2 * ((int)(p.Tq >> 16) + 2) + 1;
-    const int nn = nb1 - nb0;
-    const int yb_n = node_row_blocks(p.Tq);
-    const int items = nn * slices * yb_n;
-    const size_t WH = (size_t)p.W * p.H;
-    NodeStats st;
-    int cur_node = -1, na = 0;
-    // items are handed out one at a time from the launch's counter, in groups of nodes whose step
-    // counts stay in L2 together; within a group every node's slice at its own height first (the
-    // fullest), then outwards alternately above and below, and within a slice the 32-row blocks from
-    // the middle outwards. The warp's counters hold node cur_node's counts until the node changes.
-    const int per_node = slices * yb_n;
-    const int grp = (int)max((size_t)1, min((size_t)nn, kStepsGroupBytes / ((size_t)K * WH * sizeof(uint16_t))));
-    for (;;) {
-        int it = 0;
-        if (lane == 0) it = atomicAdd(p.vctr, 1);
-        it = __shfl_sync(0xffffffffu, it, 0);
-        if (it >= items) break;
-        const int g = it / (grp * per_node), r = it - g * grp * per_node;
-        const int gsz = min(grp, nn - g * grp);
-        const int rzy = r / gsz, ln = g * grp + r % gsz;
-        const int rank = rzy / yb_n, rb = rzy - rank * yb_n;
-        const int n = p.level_nodes[l0 + nb0 + ln];
-        NodeSlice S;
-        if (!node_slice(p, n, rank, rb, yb_n, S)) continue;
-        if (n != cur_node) {
-            if (cur_node >= 0) node_flush(p, cur_node, Q, lane);
-            na = node_ancestors(p, n, anc, lane);
-            cur_node = n;
-        }
-        node_run<STATS>(p, S, s_yi, s_yf, p.steps + (size_t)ln * K * WH, Q, anc, na, lane, st);
-    }
-    if (cur_node >= 0) node_flush(p, cur_node, Q, lane);
-    if constexpr (STATS) {
-        st.cand = __reduce_add_sync(0xffffffffu, st.cand);
-        st.unk = __reduce_add_sync(0xffffffffu, st.unk);
-        st.visit = __reduce_add_sync(0xffffffffu, st.visit);
-        st.anc = __reduce_add_sync(0xffffffffu, st.anc);
-        st.reads = __reduce_add_sync(0xffffffffu, st.reads);
-        st.smp = __reduce_add_sync(0xffffffffu, st.smp);
-        if (lane == 0) {
-            atomicAdd(p.stats + 11, (unsigned long long)st.cand);
-            atomicAdd(p.stats + 12, (unsigned long long)st.unk);
-            atomicAdd(p.stats + 13, (unsigned long long)st.visit);
-            atomicAdd(p.stats + 14, (unsigned long long)st.smp);
-            atomicAdd(p.stats + 15, (unsigned long long)st.anc);
-            atomicAdd(p.stats + 16, (unsigned long long)st.reads);
-        }
-    }
-}
-
 // ------------------------------------------------------------------------- brick occupancy
 // Recomputes the occupancy byte of every brick in [b0, b1) (brick coordinates).
 __global__ void bocc_kernel(uint8_t *grid, int nx, int ny, int nz, int bx0, int by0, int bz0, int bx1, int by1,
@@ -417,26 +306,10 @@ int vox_ctas_per_sm() {
     return std::max(1, std::min(a, b));
 }
 
-int cast_ctas_per_sm() {
-    int a = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, cast_kernel<false>, kCastWarps * 32, 0);
-    cudaGetLastError();
-    return std::max(1, a);
-}
-
 size_t steps_pairs(long long pairs, int W, int H, size_t budget_bytes) {
     const size_t per = (size_t)W * H * sizeof(uint16_t);
     const size_t cap = std::max<size_t>(1, budget_bytes / per);
     return (size_t)std::max<long long>(1, std::min<long long>(pairs, (long long)cap));
-}
-
-void launch_cast_chunk(const LevelParams &c, int num_sms, cudaStream_t s) {
-    const long long cast_warps =
-        (long long)(c.q1 - c.q0) * ((c.W + kCastTileW - 1) / kCastTileW) * ((c.H + kCastTileH - 1) / kCastTileH);
-    const int cg = (int)std::max<long long>(1, std::min<long long>((cast_warps + kCastWarps - 1) / kCastWarps,
-                                                                    (long long)num_sms * 64));
-    if (c.stats) cast_kernel<true><<<cg, kCastWarps * 32, 0, s>>>(c);
-    else cast_kernel<false><<<cg, kCastWarps * 32, 0, s>>>(c);
 }
 
 void launch_voxel_chunk(const LevelParams &c, int num_sms, int vox_ctas, cudaStream_t s) {
@@ -448,45 +321,16 @@ void launch_voxel_chunk(const LevelParams &c, int num_sms, int vox_ctas, cudaStr
     else voxel_kernel<false><<<vg, kVoxWarps * 32, smem, s>>>(c);
 }
 
-size_t node_dyn_smem(int max_anc) { return (size_t)kVoxWarps * std::max(1, max_anc) * sizeof(AncRec); }
-
-int node_ctas_per_sm() {
-    int a = 0, b = 0;
-    const size_t smem = node_dyn_smem(MIG_MAX_DEPTH);
-    cudaFuncSetAttribute(node_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaFuncSetAttribute(node_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, node_kernel<false>, kVoxWarps * 32, node_dyn_smem(16));
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, node_kernel<true>, kVoxWarps * 32, node_dyn_smem(16));
-    cudaGetLastError();
-    return std::max(1, std::min(a, b));
-}
-
-// The per-node pass, when it applies: whole nodes in a chunk, at most kNodeMaxK yaws and a frustum
-// band. By default it is taken when a voxel lies in at least 3 yaws' frusta on average (K times the
-// azimuth half-width over pi; 4 at paper scale, 9 on the large workload, where it runs 1.2x and 1.3x
-// faster than the per-pair pass).
-bool node_pass(const LevelParams &p) {
-    if (!(p.az_half > 0.f && p.K <= kNodeMaxK && p.steps_cap >= p.K) || p.voxel_pass == MIG_COUNT_PAIRS) return false;
-    return p.voxel_pass == MIG_COUNT_NODES || (float)p.K * p.az_half >= 3.0f * 3.14159265f;
-}
-
-void launch_node_chunk(const LevelParams &c, int num_sms, int node_ctas, cudaStream_t s) {
-    const int slices = 2 * ((int)(c.Tq >> 16) + 2) + 1;
-    const long long items = (long long)((c.q1 - c.q0) / c.K) * slices * node_row_blocks(c.Tq);
-    const int g = (int)std::max<long long>(1, std::min<long long>((items + kVoxWarps - 1) / kVoxWarps,
-                                                                   (long long)num_sms * node_ctas));
-    const size_t smem = node_dyn_smem(c.max_anc);
-    if (c.stats) node_kernel<true><<<g, kVoxWarps * 32, smem, s>>>(c);
-    else node_kernel<false><<<g, kVoxWarps * 32, smem, s>>>(c);
-}
+// The per-node pass, when a chunk holds whole nodes (all their yaws).
+bool node_pass(const LevelParams &p) { return p.steps_cap >= p.K && p.voxel_pass != MIG_COUNT_PAIRS; }
 
 // Pairs per launch: within the step-count buffer, and few enough that the launch's work items
-// (pairs x slices, or nodes x slices x row blocks) stay below 2^30 for the 32-bit work counter.
+// (pairs x slices, or nodes x macro blocks) stay below 2^30 for the 32-bit work counter.
 int vox_chunk_pairs(const LevelParams &p) {
     const long long slices = 2 * ((long long)(p.Tq >> 16) + 2) + 1;
     const long long lim = 1ll << 30;
     if (node_pass(p)) {
-        const long long nodes = std::min<long long>(p.steps_cap / p.K, lim / (slices * node_row_blocks(p.Tq)));
+        const long long nodes = std::min<long long>(p.steps_cap / p.K, lim / node_items(p.Tq));
         return (int)std::max<long long>(1, nodes) * p.K;
     }
     return (int)std::max<long long>(1, std::min<long long>(p.steps_cap, lim / slices));

@@ -13,15 +13,21 @@ namespace mig {
 // (node, yaw) pairs per chunk of the owned-voxel count: all `pairs` of a level, or as many as a
 // step-count buffer of budget_bytes holds (W * H uint16 per pair), at least 1.
 size_t steps_pairs(long long pairs, int W, int H, size_t budget_bytes);
-// Device bytes of a step-count region for steps_cap pairs of W * H rays: the counts, then (256-byte
-// aligned) the work counter of the voxel pass; steps_counter gives that counter's address.
-inline size_t steps_region_bytes(int steps_cap, size_t WH) {
-    return (((size_t)steps_cap * WH * sizeof(uint16_t) + 255) & ~(size_t)255) + 256;
-}
-inline int32_t *steps_counter(uint16_t *steps, int steps_cap, size_t WH) {
-    return reinterpret_cast<int32_t *>(reinterpret_cast<char *>(steps) +
-                                       (((size_t)steps_cap * WH * sizeof(uint16_t) + 255) & ~(size_t)255));
-}
+// Entries of one image's tile bounds (bricks.cuh, Pyramid).
+size_t hz_entries(int W, int H);
+// The device region of an owned-voxel count for levels of at most max_nodes nodes: the step counts of
+// `cap` pairs, the counters, the counts' tile bounds and the per-node pass's queue.
+struct SensorDims {
+    int W, H, K;
+    int64_t Tq;
+};
+struct StepsLayout {
+    int cap;        // pairs per chunk (0: the ray-by-ray count, an empty region)
+    int queue_cap;  // records
+    size_t o_ctr, o_hz, o_queue, bytes;
+};
+StepsLayout steps_layout(const SensorDims &d, int max_nodes, size_t budget_bytes, bool node_pass);
+void set_steps(LevelParams &p, void *base, const StepsLayout &L);  // the region's fields
 // Step-count buffer budget per evaluation (device bytes).
 constexpr size_t kStepsBudget = (size_t)1 << 30;
 // One level's count for the sample modes (marginal, single parent, absolute): for each chunk of
@@ -35,11 +41,13 @@ void launch_vox_level(const LevelParams &p, long long pairs, int num_sms, int vo
 void launch_cast_chunk(const LevelParams &c, int num_sms, cudaStream_t s);
 void launch_voxel_chunk(const LevelParams &c, int num_sms, int vox_ctas, cudaStream_t s);
 void launch_node_chunk(const LevelParams &c, int num_sms, int node_ctas, cudaStream_t s);
-bool node_pass(const LevelParams &p);  // whole nodes per chunk and a frustum band: the per-node pass
+bool node_pass(const LevelParams &p);  // whole nodes per chunk: the per-node pass
 int vox_chunk_pairs(const LevelParams &p);  // pairs per chunk (a multiple of K for the per-node pass)
 int node_ctas_per_sm();
 int vox_ctas_per_sm();
-int cast_ctas_per_sm();
+long long node_items(int64_t Tq);  // work items of one node of the per-node pass
+// Recomputes the masks of the 4x4x4 bricks overlapping a box of voxels and the distances around them.
+void launch_brick_update(uint8_t *grid, int nx, int ny, int nz, int x0, int y0, int z0, int dx, int dy, int dz, cudaStream_t s);
 // Recomputes the brick occupancy bytes of the bricks overlapping a box of voxels.
 void launch_bocc(uint8_t *grid, int nx, int ny, int nz, int x0, int y0, int z0, int dx, int dy, int dz, cudaStream_t s);
 
