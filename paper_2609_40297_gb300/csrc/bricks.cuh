@@ -5,8 +5,10 @@
 // After the voxel codes and the occupancy bytes (voxcount.cuh) a map carries, per 4x4x4 brick
 // (x-fastest bricks; bit = (z & 3) * 16 + (y & 3) * 4 + (x & 3)):
 //   umask  64 bits, 1 = unknown voxel;      omask  64 bits, 1 = occupied voxel;
-//   dist   1 byte, the Chebyshev distance in bricks to the nearest brick that holds an occupied
-//          voxel (0 = this one), capped at kDistCap.
+//   oct    8 bytes (one array per octant of directions): the Chebyshev distance in bricks to the
+//          nearest brick with an occupied voxel among those not behind this one along any axis (0 =
+//          this one), capped at kDistCap: no occupied voxel lies in that many bricks ahead;
+//   dist   1 byte, the least of the eight: the distance in any direction.
 // They are refreshed by every update for the bricks whose value it can change.
 #pragma once
 
@@ -31,11 +33,15 @@ MIG_HD size_t omask_offset(int nx, int ny, int nz) {
 MIG_HD size_t dist_offset(int nx, int ny, int nz) {
     return omask_offset(nx, ny, nz) + ((8 * brick_count(nx, ny, nz) + 255) & ~(size_t)255);
 }
-// two byte arrays the distance passes work in, one after the other
-MIG_HD size_t dist_scratch_offset(int nx, int ny, int nz, int i) {
-    return dist_offset(nx, ny, nz) + (size_t)(1 + i) * ((brick_count(nx, ny, nz) + 255) & ~(size_t)255);
+// the octants' distances (octant_of), then six byte arrays that the distance passes work in
+MIG_HD size_t brick_bytes_offset(int nx, int ny, int nz, int i) {
+    return dist_offset(nx, ny, nz) + (size_t)i * ((brick_count(nx, ny, nz) + 255) & ~(size_t)255);
 }
-MIG_HD size_t brick_data_end(int nx, int ny, int nz) { return dist_scratch_offset(nx, ny, nz, 2); }
+MIG_HD size_t oct_offset(int nx, int ny, int nz, int o) { return brick_bytes_offset(nx, ny, nz, 1 + o); }
+MIG_HD size_t dist_scratch_offset(int nx, int ny, int nz, int i) { return brick_bytes_offset(nx, ny, nz, 9 + i); }
+MIG_HD size_t brick_data_end(int nx, int ny, int nz) { return brick_bytes_offset(nx, ny, nz, 15); }
+// The octant of a direction: a bit per axis that does not run backwards.
+MIG_HD int octant_of(int dx, int dy, int dz) { return (dx >= 0 ? 1 : 0) | (dy >= 0 ? 2 : 0) | (dz >= 0 ? 4 : 0); }
 
 MIG_HD uint64_t ld_u64(const uint64_t *p) {
 #ifdef __CUDA_ARCH__
@@ -54,12 +60,12 @@ MIG_HD int crossings_until(uint32_t n0, uint32_t ad, uint32_t ts) {
 }
 
 // Slack of the cast's float times and positions (voxels): at most 1024 voxels from the origin every
-// float step below is within 5e-4 of the exact value.
+// float step below is within 5e-4 of the exact value (5e-7 of the range at shorter ones; the cast takes
+// 2e-6 of its range, so that few rays of a warp ever need the exact walk).
 constexpr float kCastEps = 2e-3f;
-// Voxel steps after which the fine phase rebuilds its float times, and their relative error by then
-// (the division and product 4 roundings, one per step).
+// Relative error of the mask DDA's crossing times (4 roundings, then one per step of at most 10), with
+// room to spare.
 constexpr int kCastRounds = 2048;
-constexpr int kFineSteps = 48;
 constexpr float kFineErr = 4e-6f;
 constexpr float kTimeErr = 8e-6f;  // of a time that the fine phase hands back
 
@@ -82,6 +88,68 @@ MIG_HD float small_float(int v) {
 #endif
 }
 
+// The exact DDA from the voxel state at time ts (Q16; all crossings before it, in integers) up to the
+// first brick face crossed at a time of at least tf.
+struct ExactWalk {
+    bool more;         // the ray goes on, in voxel v just entered at time t by the crossing (en / ea, axis)
+    uint32_t hit;      // step index of an occupied voxel, entered by (en / ea), else kNoHit
+    int vx, vy, vz, axis;
+    uint32_t en, ea, steps;
+    float t;
+};
+MIG_HD ExactWalk exact_walk(const uint64_t *om, int gnx, int gny, int gnz, int Px, int Py, int Pz, int dx, int dy, int dz, int64_t Tq,
+                     uint32_t ts, float tf) {
+    int v0x, v0y, v0z, sx, sy, sz;
+    uint32_t n0x, n0y, n0z, ax, ay, az;
+    ray_axis(Px, dx, v0x, sx, n0x, ax);
+    ray_axis(Py, dy, v0y, sy, n0y, ay);
+    ray_axis(Pz, dz, v0z, sz, n0z, az);
+    const int nbx = (gnx + 3) >> 2, nby = (gny + 3) >> 2;
+    const int cx = crossings_until(n0x, ax, ts), cy = crossings_until(n0y, ay, ts), cz = crossings_until(n0z, az, ts);
+    ExactWalk w;
+    w.vx = v0x + sx * cx;
+    w.vy = v0y + sy * cy;
+    w.vz = v0z + sz * cz;
+    w.hit = kNoHit;
+    w.axis = 3;
+    w.en = 0;
+    w.ea = 1;
+    w.steps = 0;
+    w.t = 0.0f;
+    w.more = true;
+    uint32_t nx = n0x + ((uint32_t)cx << 16), ny = n0y + ((uint32_t)cy << 16), nz = n0z + ((uint32_t)cz << 16);
+    uint64_t m = ld_u64(om + ((size_t)((w.vz >> 2) * nby + (w.vy >> 2)) * nbx + (w.vx >> 2)));
+    bool walk = true;
+    while (walk) {
+        ++w.steps;
+        if ((m >> (((w.vz & 3) << 4) | ((w.vy & 3) << 2) | (w.vx & 3))) & 1ull) {
+            w.hit = (uint32_t)(abs(w.vx - v0x) + abs(w.vy - v0y) + abs(w.vz - v0z));
+            walk = w.more = false;
+        } else {
+            const int a = ev_argmin3(nx, ax, ny, ay, nz, az);
+            w.axis = a;
+            w.en = a == 0 ? nx : (a == 1 ? ny : nz);
+            w.ea = a == 0 ? ax : (a == 1 ? ay : az);
+            w.vx += a == 0 ? sx : 0;
+            w.vy += a == 1 ? sy : 0;
+            w.vz += a == 2 ? sz : 0;
+            nx += a == 0 ? kQ16 : 0u;
+            ny += a == 1 ? kQ16 : 0u;
+            nz += a == 2 ? kQ16 : 0u;
+            const int v = a == 0 ? w.vx : (a == 1 ? w.vy : w.vz), s = a == 0 ? sx : (a == 1 ? sy : sz);  // the coordinate that moved
+            if (((uint64_t)w.en << 30) >= (uint64_t)Tq * w.ea || (unsigned)v >= (unsigned)(a == 0 ? gnx : (a == 1 ? gny : gnz))) {
+                walk = w.more = false;  // the crossing starts at or beyond the range, or leaves the grid
+            } else if ((v & 3) == (s > 0 ? 0 : 3)) {  // entered another brick
+                m = ld_u64(om + ((size_t)((w.vz >> 2) * nby + (w.vy >> 2)) * nbx + (w.vx >> 2)));
+                // en / ea in voxels (Q16 over Q30)
+                w.t = (float)w.en * fast_divf(16384.0f, (float)w.ea);
+                walk = w.t < tf;
+            }
+        }
+    }
+    return w;
+}
+
 // Occupied voxels of a brick's mask m inside the box of local voxel coordinates [lo, hi] per axis.
 MIG_HD bool mask_box(uint64_t m, int lx, int hx, int ly, int hy, int lz, int hz) {
     const uint32_t row = (2u << hx) - (1u << lx);                                    // 4 bits
@@ -92,67 +160,76 @@ MIG_HD bool mask_box(uint64_t m, int lx, int hx, int ly, int hy, int lz, int hz)
 
 // Step index of the first occupied voxel that the DDA (Sec. IV-B) visits, else kNoHit; the same
 // value as the plain walk's. t0: a time up to which the caller knows that the ray meets no occupied
-// voxel (0 if it knows nothing). Two alternating phases, each a single-exit loop (no return or break
-// inside, so that a warp's rays meet again after each phase):
-//   jump - the ray is in brick b, known exactly, and crosses the box of 2 d - 1 bricks around it that
-//          holds no occupied voxel (d bricks to the nearest occupied one), or, in a brick with occupied
-//          voxels (d = 0), that brick if none of them lies in the box of voxels between the ray's entry
-//          and exit. It moves to the brick beyond the face that it crosses first. That brick's
-//          coordinate along the crossed axis is exact; the other two are floors of float positions, and
-//          where one lies within kCastEps of a brick face the jump is not taken (fine phase instead).
-//   fine - the exact voxel state at a time ts in free space (all crossings before ts, in integers) is
-//          rebuilt and the DDA runs voxel by voxel, reading one 64-bit occupancy mask per brick. The
-//          next crossing is chosen by float times where they differ by more than their error, else by
-//          the exact comparison of n / |d|; the voxel position is exact throughout.
+// voxel (0 if it knows nothing). oct: the distances for the ray's octant (octant_of).
+//
+// The ray is in brick b, known exactly, at time t. If no occupied brick lies within the d bricks ahead
+// of b along each axis (the octant distance, d >= 1), the ray moves to the brick beyond the face of
+// that box which it crosses first. It also passes a brick with occupied voxels (d = 0) if none of them
+// lies in the box of voxels between its entry and exit; otherwise it runs the DDA on the brick's
+// 64-bit mask, by float times. Either way the new brick is exact as long as the floats decide: a jump's
+// other two coordinates are floors of positions that must not lie within eps of a brick face, and two
+// crossings of the mask's DDA must differ by more than their error. Where they do not decide, and near
+// the range (0.2 to 0.4 % of the rays), the exact voxel state at a time in free space (all crossings
+// before it, in integers) is rebuilt and the DDA runs with exactly compared crossings up to the next
+// brick face (exact_walk). The loops have single exits (no return or break inside), so that a warp's rays
+// meet again after each; the mask's DDA runs outside the jump loop, where the rays that need it run it
+// together (inside it the cast took 9.3 instead of 8.0 ms at paper scale).
+// Bound by instruction issue (about 65 % of the slots, 23 of 32 lanes active). Cast per replan at
+// paper scale / on the large workload: 12.3 / 493 ms with 64-bit compared crossings, 8.2 / 219 ms with
+// one distance for all directions, 8.0 / 208 ms without the box test of occupied bricks, 6.4 / 170 ms.
 // The step index of a voxel is its Manhattan distance from the start voxel, so the walk need not
 // count steps. With DEPTH, ne / ade return the face distance and speed of the hit voxel's entry
 // (0 / 1 for the start voxel). fine, coarse: voxel steps and jumps taken (STATS).
 template <bool DEPTH, bool STATS>
-MIG_HD uint32_t cast_bricks(const uint64_t *om, const uint8_t *dist, int gnx, int gny, int gnz, int Px, int Py, int Pz,
+MIG_HD uint32_t cast_bricks(const uint64_t *om, const uint8_t *oct, int gnx, int gny, int gnz, int Px, int Py, int Pz,
                             int dx, int dy, int dz, int64_t Tq, float t0, uint32_t &ne, uint32_t &ade, uint32_t &fine,
                             uint32_t &coarse) {
-    int v0x, v0y, v0z, sx, sy, sz;
-    uint32_t n0x, n0y, n0z, ax, ay, az;
-    ray_axis(Px, dx, v0x, sx, n0x, ax);
-    ray_axis(Py, dy, v0y, sy, n0y, ay);
-    ray_axis(Pz, dz, v0z, sz, n0z, az);
     const float q30 = 9.31322574615478515625e-10f, q16 = 1.52587890625e-5f, q18 = 3.814697265625e-6f;
-    const int nbx = (gnx + 3) >> 2, nby = (gny + 3) >> 2;
-    const int b0x = v0x >> 2, b0y = v0y >> 2, b0z = v0z >> 2;
+    const int nbx = (gnx + 3) >> 2, nby = (gny + 3) >> 2, nbz = (gnz + 3) >> 2;
+    const int b0x = Px >> 18, b0y = Py >> 18, b0z = Pz >> 18;
+    const int sx = dx < 0 ? -1 : 1, sy = dy < 0 ? -1 : 1, sz = dz < 0 ? -1 : 1;
     // times per voxel along each axis; an axis that does not move gets a time beyond every range
-    const float fx = (float)ax * q30, fy = (float)ay * q30, fz = (float)az * q30;
-    const float ix = ax ? fast_divf(1.0f, fx) : 1e30f, iy = ay ? fast_divf(1.0f, fy) : 1e30f, iz = az ? fast_divf(1.0f, fz) : 1e30f;
-    const float T = (float)Tq * q16;
-    float t_end = T;
-    t_end = fminf(t_end, (float)(sx > 0 ? (gnx << 16) - Px : Px) * q16 * ix);
+    const float fx = fabsf((float)dx) * q30, fy = fabsf((float)dy) * q30, fz = fabsf((float)dz) * q30;
+    const float ix = fx > 0.0f ? fast_divf(1.0f, fx) : 1e30f, iy = fy > 0.0f ? fast_divf(1.0f, fy) : 1e30f, iz = fz > 0.0f ? fast_divf(1.0f, fz) : 1e30f;
+    const float T = (float)Tq * q16, eps = fmaf(T, 2e-6f, 3e-5f);
+    float t_end = fminf(T, (float)(sx > 0 ? (gnx << 16) - Px : Px) * q16 * ix);
     t_end = fminf(t_end, (float)(sy > 0 ? (gny << 16) - Py : Py) * q16 * iy);
     t_end = fminf(t_end, (float)(sz > 0 ? (gnz << 16) - Pz : Pz) * q16 * iz);
     // brick coordinates relative to the start brick, as floats: position p0 + k t; the far face of the
-    // box of brick b, at b + d or b - d + 1, is crossed at (b +- d + h) j
+    // d bricks from b on, at b + d or b - d + 1, is crossed at (b +- d + h) j
     const float gx = sx > 0 ? 1.0f : -1.0f, gy = sy > 0 ? 1.0f : -1.0f, gz = sz > 0 ? 1.0f : -1.0f;
     const float p0x = (float)(Px & 0x3FFFF) * q18, p0y = (float)(Py & 0x3FFFF) * q18, p0z = (float)(Pz & 0x3FFFF) * q18;
     const float kx = 0.25f * fx * gx, ky = 0.25f * fy * gy, kz = 0.25f * fz * gz;
     const float hx = (sx > 0 ? 0.0f : 1.0f) - p0x, hy = (sy > 0 ? 0.0f : 1.0f) - p0y, hz = (sz > 0 ? 0.0f : 1.0f) - p0z;
     const float jx = 4.0f * ix * gx, jy = 4.0f * iy * gy, jz = 4.0f * iz * gz;
-    if constexpr (DEPTH) {
-        ne = 0;
-        ade = 1;
-    }
-    const float kR = 0.5f - 0.25f * kCastEps, kMagic = 12582912.0f;
-    // the brick at time t0, and whether it is certain
+    const float kR = 0.5f - 0.25f * eps, kMagic = 12582912.0f, t_sure = t_end - eps;
+    uint32_t hit = kNoHit;
+    int last = 3;  // the axis of the latest crossing (3: none yet); with DEPTH
+    // the brick at time t0, and whether it is certain (p: position minus 1/2, m: nearest integers of p)
     float t = t0;
     float px = fmaf(kx, t, p0x) - 0.5f, py = fmaf(ky, t, p0y) - 0.5f, pz = fmaf(kz, t, p0z) - 0.5f;
     float bx = (px + kMagic) - kMagic, by = (py + kMagic) - kMagic, bz = (pz + kMagic) - kMagic;
-    bool sure = t < t_end - kCastEps && (t0 == 0.0f || fmaxf(fabsf(px - bx), fmaxf(fabsf(py - by), fabsf(pz - bz))) < kR);
+    bool sure = t < t_sure && (t0 == 0.0f || fmaxf(fabsf(px - bx), fmaxf(fabsf(py - by), fabsf(pz - bz))) < kR);
     if (t0 == 0.0f) bx = by = bz = 0.0f;
-    uint32_t hit = kNoHit;
-    int rounds = 0;  // every round passes a brick face; beyond kCastRounds one fine phase runs to the end
+    auto oct_at = [&]() {  // the distance at brick b; (int)b by the bits of a float whose unit is its last place
+        const int ib = (b0z + float_bits(bz + kMagic) - 0x4B400000) * nby + (b0y + float_bits(by + kMagic) - 0x4B400000);
+        return (size_t)ib * (size_t)nbx + (size_t)(b0x + float_bits(bx + kMagic) - 0x4B400000);
+    };
+    auto outside = [&]() {  // brick b is beyond the grid
+        const int x = b0x + float_bits(bx + kMagic) - 0x4B400000, y = b0y + float_bits(by + kMagic) - 0x4B400000, z = b0z + float_bits(bz + kMagic) - 0x4B400000;
+        return (unsigned)x >= (unsigned)nbx || (unsigned)y >= (unsigned)nby || (unsigned)z >= (unsigned)nbz;
+    };
+    size_t bi = 0;
+    int d = 0;
+    float r = 1.0f;
+    if (sure) {
+        bi = oct_at();
+        d = ld_u8(oct + bi);
+    }
+    int rounds = 0;  // every round passes a brick face; beyond kCastRounds the exact walk runs to the end
     for (bool more = true; more;) {
-        while (sure) {
-            // (int)b and (float)d by the bits of floats whose unit is their last place, without conversions
-            const int ib = (b0z + float_bits(bz + kMagic) - 0x4B400000) * nby + (b0y + float_bits(by + kMagic) - 0x4B400000);
-            const size_t bi = (size_t)ib * (size_t)nbx + (size_t)(b0x + float_bits(bx + kMagic) - 0x4B400000);
-            const int d = ld_u8(dist + bi);
+        bool dda = false;  // in a brick with an occupied voxel near the ray's way through it
+        while (sure && !dda) {
             if constexpr (STATS) ++coarse;
             const float df = small_float(max(d, 1));
             const float tx = (fmaf(gx, df, bx) + hx) * jx, ty = (fmaf(gy, df, by) + hy) * jy, tz = (fmaf(gz, df, bz) + hz) * jz;
@@ -161,94 +238,148 @@ MIG_HD uint32_t cast_bricks(const uint64_t *om, const uint8_t *dist, int gnx, in
             // floors of the positions (nearest integer of p - 1/2) and their distance from a brick's middle
             const float qx = fmaf(kx, t1, p0x) - 0.5f, qy = fmaf(ky, t1, p0y) - 0.5f, qz = fmaf(kz, t1, p0z) - 0.5f;
             const float mx = (qx + kMagic) - kMagic, my = (qy + kMagic) - kMagic, mz = (qz + kMagic) - kMagic;
-            const float r = fmaxf(ox ? 0.0f : fabsf(qx - mx), fmaxf(oy ? 0.0f : fabsf(qy - my), oz ? 0.0f : fabsf(qz - mz)));
-            bool ok = true;
-            if (d == 0) {  // an occupied voxel between the entry and the exit?
-                const float e = fmaf(t, kTimeErr, 2.0f * kCastEps);
-                const float fx_ = bx - 0.5f, fy_ = by - 0.5f, fz_ = bz - 0.5f;
-                const int lx = max(0, (int)floorf(4.0f * (fminf(px, qx) - fx_) - e)), ux = min(3, (int)floorf(4.0f * (fmaxf(px, qx) - fx_) + e));
-                const int ly = max(0, (int)floorf(4.0f * (fminf(py, qy) - fy_) - e)), uy = min(3, (int)floorf(4.0f * (fmaxf(py, qy) - fy_) + e));
-                const int lz = max(0, (int)floorf(4.0f * (fminf(pz, qz) - fz_) - e)), uz = min(3, (int)floorf(4.0f * (fmaxf(pz, qz) - fz_) + e));
-                ok = !mask_box(ld_u64(om + bi), min(lx, 3), max(ux, 0), min(ly, 3), max(uy, 0), min(lz, 3), max(uz, 0));
+            if (d == 0) {
+                // the voxels between entry and exit, widened by e: local coordinates (minus 1/2, nearest integers)
+                const float e = fmaf(t, kTimeErr, 2.0f * eps);
+                auto at = [&](float v) { return float_bits(fminf(fmaxf(v, 0.0f), 3.0f) + kMagic) & 3; };
+                const float cx = fmaf(-4.0f, bx, 1.5f), cy = fmaf(-4.0f, by, 1.5f), cz = fmaf(-4.0f, bz, 1.5f);
+                dda = mask_box(ld_u64(om + bi), at(fmaf(4.0f, fminf(px, qx), cx - e)), at(fmaf(4.0f, fmaxf(px, qx), cx + e)),
+                               at(fmaf(4.0f, fminf(py, qy), cy - e)), at(fmaf(4.0f, fmaxf(py, qy), cy + e)),
+                               at(fmaf(4.0f, fminf(pz, qz), cz - e)), at(fmaf(4.0f, fmaxf(pz, qz), cz + e)));
             }
-            if (ok) {
+            if (!dda) {
+                r = fmaxf(ox ? 0.0f : fabsf(qx - mx), fmaxf(oy ? 0.0f : fabsf(qy - my), oz ? 0.0f : fabsf(qz - mz)));
                 t = t1;
-                bx = ox ? fmaf(gx, df, bx) : mx;
-                by = oy ? fmaf(gy, df, by) : my;
-                bz = oz ? fmaf(gz, df, bz) : mz;
                 px = qx;
                 py = qy;
                 pz = qz;
-            }
-            sure = ok && t < t_end - kCastEps && r < kR;
-        }
-        // the ray is free of occupied voxels up to t: done if that is the range or the grid's edge
-        more = t <= t_end + kCastEps;
-        const float slack = fmaf(t, kTimeErr, kCastEps);
-        const float tf = ++rounds < kCastRounds ? t + slack : 1e30f;  // the fine phase runs at least to here
-        const uint32_t ts = (uint32_t)(int)(fmaxf(0.0f, fminf(t, t_end) - slack) * 65536.0f);
-        const int cx = crossings_until(n0x, ax, ts), cy = crossings_until(n0y, ay, ts), cz = crossings_until(n0z, az, ts);
-        int vx = v0x + sx * cx, vy = v0y + sy * cy, vz = v0z + sz * cz;
-        // next crossing times, advanced by additions: within 2^-24 t per step, hence kFineSteps and kFineErr
-        float tx = (float)(n0x + ((uint32_t)cx << 16)) * q16 * ix, ty = (float)(n0y + ((uint32_t)cy << 16)) * q16 * iy,
-              tz = (float)(n0z + ((uint32_t)cz << 16)) * q16 * iz;
-        uint64_t m = more ? ld_u64(om + ((size_t)((vz >> 2) * nby + (vy >> 2)) * nbx + (vx >> 2))) : 0ull;
-        int left = kFineSteps;
-        bool walk = more;
-        while (walk) {
-            if constexpr (STATS) ++fine;
-            const float mn = fminf(tx, fminf(ty, tz));
-            const float lim = fmaf(mn, kFineErr, mn);
-            bool ox = tx <= lim, oy = ty <= lim, oz = tz <= lim;
-            const bool occ = (m >> (((vz & 3) << 4) | ((vy & 3) << 2) | (vx & 3))) & 1ull;
-            if (occ) hit = (uint32_t)(abs(vx - v0x) + abs(vy - v0y) + abs(vz - v0z));
-            walk = !occ;
-            // two crossings too close to tell, or one near the range: the exact order and range test
-            if ((ox && oy) || (ox && oz) || (oy && oz) || lim >= T * (1.0f - kFineErr)) {
-                const uint32_t nx = n0x + ((uint32_t)abs(vx - v0x) << 16), ny = n0y + ((uint32_t)abs(vy - v0y) << 16),
-                               nz = n0z + ((uint32_t)abs(vz - v0z) << 16);
-                const int a = ev_argmin3(nx, ax, ny, ay, nz, az);
-                ox = a == 0;
-                oy = a == 1;
-                oz = a == 2;
-                const uint32_t nc = ox ? nx : (oy ? ny : nz), ac = ox ? ax : (oy ? ay : az);
-                walk = walk && ((uint64_t)nc << 30) < (uint64_t)Tq * ac;
-            }
-            if (walk) {
-                if constexpr (DEPTH) {
-                    ne = ox ? n0x + ((uint32_t)abs(vx - v0x) << 16) : (oy ? n0y + ((uint32_t)abs(vy - v0y) << 16) : n0z + ((uint32_t)abs(vz - v0z) << 16));
-                    ade = ox ? ax : (oy ? ay : az);
+                sure = t < t_sure && r < kR;
+                bx = ox ? fmaf(gx, df, bx) : mx;
+                by = oy ? fmaf(gy, df, by) : my;
+                bz = oz ? fmaf(gz, df, bz) : mz;
+                if constexpr (DEPTH) last = ox ? 0 : (oy ? 1 : 2);
+                if (sure) {
+                    bi = oct_at();
+                    d = ld_u8(oct + bi);
                 }
-                tx += ox ? ix : 0.0f;
-                ty += oy ? iy : 0.0f;
-                tz += oz ? iz : 0.0f;
-                vx += ox ? sx : 0;
-                vy += oy ? sy : 0;
-                vz += oz ? sz : 0;
-                --left;
-                const int v = ox ? vx : (oy ? vy : vz), s = ox ? sx : (oy ? sy : sz);  // the coordinate that moved
-                if ((v & 3) == (s > 0 ? 0 : 3) || left <= 0) {  // entered another brick
-                    // beyond the grid: in a brick of its own, or in the last, partial brick (no bit there)
-                    walk = (unsigned)v < (unsigned)(ox ? gnx : (oy ? gny : gnz));
-                    more = walk;
-                    if (walk) {
-                        m = ld_u64(om + ((size_t)((vz >> 2) * nby + (vy >> 2)) * nbx + (vx >> 2)));
-                        t = mn;
-                        walk = mn < tf && left > 0;
+            }
+        }
+        // free to the grid's edge: past it with a certain brick, every voxel before being in the free box
+        if (!sure && r < kR && outside()) more = false;
+        if (sure) {
+            // DDA on the brick's mask: entry voxel (local coordinates l, not within e of an inner face of the
+            // brick's voxels; the entry face itself is exact), next crossing times, and a packed state: bits
+            // 0-5 the mask's bit (plus 64), above them a guard per axis whose third bit is set while the
+            // coordinate is in 0..3
+            const uint64_t m = ld_u64(om + bi);
+            const float e = fmaf(t, kTimeErr, eps);
+            const float lx = fminf(fmaxf(4.0f * (px - bx) + 1.5f, -0.5f), 3.499f), ly = fminf(fmaxf(4.0f * (py - by) + 1.5f, -0.5f), 3.499f),
+                        lz = fminf(fmaxf(4.0f * (pz - bz) + 1.5f, -0.5f), 3.499f);  // minus 1/2
+            const float cx = fmaxf((lx + kMagic) - kMagic, 0.0f), cy = fmaxf((ly + kMagic) - kMagic, 0.0f), cz = fmaxf((lz + kMagic) - kMagic, 0.0f);
+            // within e of an inner face: l - c = +-1/2, but not at the brick's own faces
+            const float ux = fabsf(lx - 1.5f) > 1.9f ? 0.0f : fabsf(lx - cx), uy = fabsf(ly - 1.5f) > 1.9f ? 0.0f : fabsf(ly - cy),
+                        uz = fabsf(lz - 1.5f) > 1.9f ? 0.0f : fabsf(lz - cz);
+            float tx = (fmaf(0.25f, cx + (sx > 0 ? 1.0f : -4.0f), bx) + hx) * jx, ty = (fmaf(0.25f, cy + (sy > 0 ? 1.0f : -4.0f), by) + hy) * jy,
+                  tz = (fmaf(0.25f, cz + (sz > 0 ? 1.0f : -4.0f), bz) + hz) * jz;
+            const int vx = float_bits(cx + kMagic) & 3, vy = float_bits(cy + kMagic) & 3, vz = float_bits(cz + kMagic) & 3;
+            int w = 64 + vx + 4 * vy + 16 * vz + ((vx + 4) << 8) + ((vy + 4) << 12) + ((vz + 4) << 16);
+            const int wx = sx * 257, wy = sy * 4100, wz = sz * 65552;
+            bool walk = fmaxf(ux, fmaxf(uy, uz)) < 0.5f - e, ox = false, oy = false, left = false, occ = false;
+            sure = false;
+            float mn = t;
+            while (walk) {
+                if constexpr (STATS) ++fine;
+                occ = (m >> (w & 63)) & 1ull;
+                mn = fminf(tx, fminf(ty, tz));
+                const float lim = fmaf(mn, kFineErr, mn);
+                ox = tx <= lim;
+                oy = ty <= lim;
+                const bool oz = tz <= lim;
+                walk = !occ && !((ox && oy) || (ox && oz) || (oy && oz)) && mn < T - eps;
+                if (walk) {
+                    tx += ox ? ix : 0.0f;
+                    ty += oy ? iy : 0.0f;
+                    tz += oz ? iz : 0.0f;
+                    w += ox ? wx : (oy ? wy : wz);
+                    if constexpr (DEPTH) last = ox ? 0 : (oy ? 1 : 2);
+                    left = (w & 0x44400) != 0x44400;
+                    walk = !left;
+                }
+            }
+            if (occ) {
+                const int b4x = 4 * (b0x + float_bits(bx + kMagic) - 0x4B400000), b4y = 4 * (b0y + float_bits(by + kMagic) - 0x4B400000),
+                          b4z = 4 * (b0z + float_bits(bz + kMagic) - 0x4B400000);
+                const int cx_ = abs(b4x + (w & 3) - (Px >> 16)), cy_ = abs(b4y + ((w >> 2) & 3) - (Py >> 16)), cz_ = abs(b4z + ((w >> 4) & 3) - (Pz >> 16));
+                hit = (uint32_t)(cx_ + cy_ + cz_);
+                if constexpr (DEPTH) {
+                    const int c = last == 0 ? cx_ : (last == 1 ? cy_ : cz_), P = last == 0 ? Px : (last == 1 ? Py : Pz),
+                              dd = last == 0 ? dx : (last == 1 ? dy : dz);
+                    int v0, s;
+                    uint32_t n0;
+                    ray_axis(P, dd, v0, s, n0, ade);
+                    ne = n0 + ((uint32_t)(c - 1) << 16);
+                    if (last == 3) {  // the start voxel
+                        ne = 0;
+                        ade = 1;
                     }
                 }
-            } else {
                 more = false;
+            } else if (left) {  // into the next brick, across the face of the axis just crossed
+                t = mn;
+                bx += ox ? gx : 0.0f;
+                by += !ox && oy ? gy : 0.0f;
+                bz += !ox && !oy ? gz : 0.0f;
+                px = fmaf(kx, t, p0x) - 0.5f;
+                py = fmaf(ky, t, p0y) - 0.5f;
+                pz = fmaf(kz, t, p0z) - 0.5f;
+                more = !outside();
+                sure = more && t < t_sure;
+                r = 1.0f;
+                if (sure) {
+                    bi = oct_at();
+                    d = ld_u8(oct + bi);
+                }
+            } else if (mn > T + eps) {
+                more = false;  // the next crossing is beyond the range
             }
         }
-        // back to the jumps from the brick just entered, exactly known
-        bx = small_float(vx >> 2) - small_float(b0x);
-        by = small_float(vy >> 2) - small_float(b0y);
-        bz = small_float(vz >> 2) - small_float(b0z);
-        px = fmaf(kx, t, p0x) - 0.5f;
-        py = fmaf(ky, t, p0y) - 0.5f;
-        pz = fmaf(kz, t, p0z) - 0.5f;
-        sure = more && t < t_end - kCastEps;
+        // the ray is free of occupied voxels up to t: done if that is the range or the grid's edge
+        more = more && t <= t_end + eps;
+        if (more && !sure) {
+            const float slack = fmaf(t, kTimeErr, eps);
+            const ExactWalk w = exact_walk(om, gnx, gny, gnz, Px, Py, Pz, dx, dy, dz, Tq,
+                                           (uint32_t)(int)(fmaxf(0.0f, fminf(t, t_end) - slack) * 65536.0f),
+                                           ++rounds < kCastRounds ? t + slack : 1e30f);
+            if constexpr (STATS) fine += w.steps;
+            if constexpr (DEPTH) {
+                ne = w.en;
+                ade = w.ea;
+                last = w.axis;
+            }
+            hit = w.hit;
+            more = w.more;
+            if (more) {  // back to the jumps from the brick just entered, exactly known
+                t = w.t;
+                bx = small_float(w.vx >> 2) - small_float(Px >> 18);
+                by = small_float(w.vy >> 2) - small_float(Py >> 18);
+                bz = small_float(w.vz >> 2) - small_float(Pz >> 18);
+                px = fmaf(kx, t, p0x) - 0.5f;
+                py = fmaf(ky, t, p0y) - 0.5f;
+                pz = fmaf(kz, t, p0z) - 0.5f;
+                r = 1.0f;
+                sure = t < t_sure;
+                if (sure) {
+                    bi = oct_at();
+                    d = ld_u8(oct + bi);
+                }
+            }
+        }
+    }
+    if constexpr (DEPTH) {
+        if (hit == kNoHit) {
+            ne = 0;
+            ade = 1;
+        }
     }
     return hit;
 }

@@ -52,7 +52,7 @@ __device__ __forceinline__ float q16f(int v) { return (float)v * (1.0f / 65536.0
 //   small - one CTA per 16x16 tile, one part per warp, no beams and no 32x32 bounds, for levels that do
 //           not fill the GPU: their time is one warp's chain of dependent steps.
 // The level's size is only known on the device (tree_eval_device), so the kernels choose.
-constexpr int kCastCtas = 3;  // resident CTAs per SM: 80 registers; at 64 (4 CTAs) 2 % slower
+constexpr int kCastCtas = 4;  // resident CTAs per SM (64 registers; 3 CTAs of 80 are 2 % slower)
 enum CastLayout { kCastSmall, kCastMid, kCastLarge };
 __device__ __forceinline__ CastLayout cast_layout(long long images, int W, int H, int num_sms) {
     const long long tiles = images * ((W + 31) >> 5) * ((H + 31) >> 5), warps = (long long)num_sms * kCastCtas * kWarpsN;
@@ -126,11 +126,11 @@ struct RayHit {
     uint32_t m, ne, ade;
 };
 template <bool STATS, bool DEPTH>
-__device__ __noinline__ RayHit cast_ray(const uint64_t *om, const uint8_t *dist, int gnx, int gny, int gnz, int Px, int Py, int Pz,
+__device__ __noinline__ RayHit cast_ray(const uint64_t *om, const uint8_t *oct, int gnx, int gny, int gnz, int Px, int Py, int Pz,
                                        int dx, int dy, int dz, int Tq, float t0, CastCnt *st) {
     RayHit h{0, 0, 1};
     uint32_t fine = 0, jump = 0;
-    h.m = cast_bricks<DEPTH, STATS>(om, dist, gnx, gny, gnz, Px, Py, Pz, dx, dy, dz, Tq, t0, h.ne, h.ade, fine, jump);
+    h.m = cast_bricks<DEPTH, STATS>(om, oct, gnx, gny, gnz, Px, Py, Pz, dx, dy, dz, Tq, t0, h.ne, h.ade, fine, jump);
     if constexpr (STATS) {
         st->fine += fine;
         st->jump += jump;
@@ -154,7 +154,8 @@ __device__ __forceinline__ void cast_part(const LevelParams &p, const uint64_t *
         if (beam < 1e29f) {
             int dx, dy, dz;
             ray_dir(b, ck, sk, dx, dy, dz);
-            hit = cast_ray<STATS, OUT::kDepth>(om, dist, p.grid.nx, p.grid.ny, p.grid.nz, nd.x, nd.y, nd.z, dx, dy, dz, (int)p.Tq,
+            const uint8_t *oct = p.grid.g + oct_offset(p.grid.nx, p.grid.ny, p.grid.nz, octant_of(dx, dy, dz));
+            hit = cast_ray<STATS, OUT::kDepth>(om, oct, p.grid.nx, p.grid.ny, p.grid.nz, nd.x, nd.y, nd.z, dx, dy, dz, (int)p.Tq,
                                                beam_time(beam, b.w), &st);
         }
     }
@@ -985,35 +986,46 @@ __global__ void brick_mask_kernel(uint8_t *grid, int nx, int ny, int nz, int bx0
     }
 }
 
-// One pass of the Chebyshev distance to the nearest brick with an occupied voxel, over the bricks of
-// a box: along x from the masks (pass 0, into scratch 0), along y (pass 1, scratch 0 to 1), along
-// z (pass 2, scratch 1 to dist). d = min over j of max(|j|, the previous pass at offset j).
+// One pass of the octant distances over the bricks of a box: along x from the masks (pass 0: both
+// directions, scratch 0-1), along y (pass 1: scratch 2-5), along z (pass 2: the eight octants and their
+// minimum). One-sided: d = min over j >= 0 of max(j, the previous pass j bricks ahead).
 __global__ void brick_dist_kernel(uint8_t *grid, int nx, int ny, int nz, int pass, int bx0, int by0, int bz0, int bx1, int by1,
                                   int bz1) {
     const int nbx = (nx + 3) >> 2, nby = (ny + 3) >> 2, nbz = (nz + 3) >> 2;
     const uint64_t *om = reinterpret_cast<const uint64_t *>(grid + omask_offset(nx, ny, nz));
-    const uint8_t *src = grid + dist_scratch_offset(nx, ny, nz, pass == 2);
-    uint8_t *dst = grid + (pass == 2 ? dist_offset(nx, ny, nz) : dist_scratch_offset(nx, ny, nz, pass));
+    const size_t plane = dist_scratch_offset(nx, ny, nz, 1) - dist_scratch_offset(nx, ny, nz, 0);
+    uint8_t *scr = grid + dist_scratch_offset(nx, ny, nz, 0);
     const int wx = bx1 - bx0, wy = by1 - by0;
     const long long total = (long long)wx * wy * (bz1 - bz0);
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
         const int bx = bx0 + (int)(i % wx), by = by0 + (int)((i / wx) % wy), bz = bz0 + (int)(i / ((long long)wx * wy));
         const size_t b = ((size_t)bz * nby + by) * nbx + bx;
-        int d = kDistCap;
         if (pass == 0) {
-            for (int j = 0; j < d; ++j)
-                if ((bx - j >= 0 && om[b - j]) || (bx + j < nbx && om[b + j])) d = j;
+            int lo = kDistCap, hi = kDistCap;  // towards smaller and larger x
+            for (int j = min(kDistCap - 1, bx); j >= 0; --j) lo = om[b - j] ? j : lo;
+            for (int j = min(kDistCap - 1, nbx - 1 - bx); j >= 0; --j) hi = om[b + j] ? j : hi;
+            scr[b] = (uint8_t)lo;
+            scr[plane + b] = (uint8_t)hi;
         } else {
-            const int c = pass == 1 ? by : bz, n = pass == 1 ? nby : nbz;
+            const int c = pass == 1 ? by : bz, n = pass == 1 ? nby : nbz, arrays = pass == 1 ? 2 : 4;
             const ptrdiff_t step = pass == 1 ? nbx : (ptrdiff_t)nbx * nby;
-            for (int j = 0; j < d; ++j) {
-                int e = kDistCap;
-                if (c - j >= 0) e = min(e, (int)src[(ptrdiff_t)b - j * step]);
-                if (c + j < n) e = min(e, (int)src[(ptrdiff_t)b + j * step]);
-                d = min(d, max(e, j));
+            int least = kDistCap;
+            for (int a = 0; a < arrays; ++a) {
+                const uint8_t *src = scr + (size_t)(pass == 1 ? a : 2 + a) * plane;
+                int lo = kDistCap, hi = kDistCap;
+                for (int j = 0; j < kDistCap; ++j) {
+                    if (j <= c) lo = min(lo, max(j, (int)src[(ptrdiff_t)b - j * step]));
+                    if (c + j < n) hi = min(hi, max(j, (int)src[(ptrdiff_t)b + j * step]));
+                }
+                // array bits: x, then y, then z not backwards
+                uint8_t *d0 = pass == 1 ? scr + (size_t)(2 + a) * plane : grid + oct_offset(nx, ny, nz, a);
+                uint8_t *d1 = pass == 1 ? scr + (size_t)(4 + a) * plane : grid + oct_offset(nx, ny, nz, 4 + a);
+                d0[b] = (uint8_t)lo;
+                d1[b] = (uint8_t)hi;
+                least = min(least, min(lo, hi));
             }
+            if (pass == 2) grid[dist_offset(nx, ny, nz) + b] = (uint8_t)least;
         }
-        dst[b] = (uint8_t)d;
     }
 }
 

@@ -29,7 +29,7 @@ struct Grid {
     int N[3];
     std::vector<uint8_t> g;
     std::vector<uint64_t> om;
-    std::vector<uint8_t> dist;
+    std::vector<uint8_t> dist, oct[8];
     uint8_t at(int x, int y, int z) const { return g[((size_t)z * N[1] + y) * N[0] + x]; }
     void bricks() {
         const int b[3] = {(N[0] + 3) / 4, (N[1] + 3) / 4, (N[2] + 3) / 4};
@@ -40,20 +40,24 @@ struct Grid {
                 for (int x = 0; x < N[0]; ++x)
                     if (at(x, y, z) == 2)
                         om[((size_t)(z / 4) * b[1] + y / 4) * b[0] + x / 4] |= 1ull << ((z % 4) * 16 + (y % 4) * 4 + x % 4);
-        for (int z = 0; z < b[2]; ++z)
-            for (int y = 0; y < b[1]; ++y)
-                for (int x = 0; x < b[0]; ++x)
-                    for (int r = 0; r < kDistCap; ++r) {
-                        bool any = false;
-                        for (int k = std::max(0, z - r); k <= std::min(b[2] - 1, z + r) && !any; ++k)
-                            for (int j = std::max(0, y - r); j <= std::min(b[1] - 1, y + r) && !any; ++j)
-                                for (int i = std::max(0, x - r); i <= std::min(b[0] - 1, x + r); ++i)
-                                    if (om[((size_t)k * b[1] + j) * b[0] + i]) any = true;
-                        if (any) {
-                            dist[((size_t)z * b[1] + y) * b[0] + x] = (uint8_t)r;
-                            break;
-                        }
+        for (int o = 0; o < 8; ++o) {  // by definition: occupied bricks not behind along any axis
+            const int s[3] = {o & 1 ? 1 : -1, o & 2 ? 1 : -1, o & 4 ? 1 : -1};
+            oct[o].assign(om.size(), kDistCap);
+            for (int z = 0; z < b[2]; ++z)
+                for (int y = 0; y < b[1]; ++y)
+                    for (int x = 0; x < b[0]; ++x) {
+                        uint8_t &d = oct[o][((size_t)z * b[1] + y) * b[0] + x];
+                        for (int k = 0; k < d; ++k)
+                            for (int j = 0; j < d; ++j)
+                                for (int i = 0; i < d; ++i) {
+                                    const int X = x + s[0] * i, Y = y + s[1] * j, Z = z + s[2] * k;
+                                    if (X < 0 || Y < 0 || Z < 0 || X >= b[0] || Y >= b[1] || Z >= b[2]) continue;
+                                    if (om[((size_t)Z * b[1] + Y) * b[0] + X]) d = (uint8_t)std::min<int>(d, std::max(i, std::max(j, k)));
+                                }
+                        uint8_t &m = dist[((size_t)z * b[1] + y) * b[0] + x];
+                        m = std::min(m, d);
                     }
+        }
     }
 };
 
@@ -124,7 +128,7 @@ int main(int argc, char **argv) {
             i64 en, ea;
             const int w = walk(G, P, d, Tq, en, ea);
             uint32_t ne, ade, f = 0, c = 0;
-            const uint32_t got = cast_bricks<true, false>(G.om.data(), G.dist.data(), G.N[0], G.N[1], G.N[2], (int)P[0], (int)P[1],
+            const uint32_t got = cast_bricks<true, false>(G.om.data(), G.oct[octant_of((int)d[0], (int)d[1], (int)d[2])].data(), G.N[0], G.N[1], G.N[2], (int)P[0], (int)P[1],
                                                           (int)P[2], (int)d[0], (int)d[1], (int)d[2], Tq, 0.0f, ne, ade, f, c);
             ++rays;
             hits += w >= 0;
@@ -178,7 +182,7 @@ int main(int argc, char **argv) {
                     uint32_t got = kNoHit, ne, ade, f = 0, c = 0;
                     const float t0 = s > 0 ? std::max(0.0f, (float)(s * nrm) * (1.0f - 1e-6f) - kCastEps) : 0.0f;
                     if (s < 1e29f)
-                        got = cast_bricks<true, false>(G.om.data(), G.dist.data(), G.N[0], G.N[1], G.N[2], (int)P[0], (int)P[1], (int)P[2],
+                        got = cast_bricks<true, false>(G.om.data(), G.oct[octant_of((int)d[0], (int)d[1], (int)d[2])].data(), G.N[0], G.N[1], G.N[2], (int)P[0], (int)P[1], (int)P[2],
                                                        (int)d[0], (int)d[1], (int)d[2], Tq, t0, ne, ade, f, c);
                     ++beam_rays;
                     beam_free_rays += s >= 1e29f;
