@@ -204,7 +204,8 @@ mig_status mig_tree_score_device(mig_ctx *ctx, int n, const int32_t *parent, con
  * of the process; do not call cudaDeviceReset on that device afterwards (the array may move).
  * The yaw table travels in kernel parameters, not by a copy from host memory. Every call shares the one
  * array: calls whose work overlaps on the GPU (other streams, other contexts on the same
- * device) race and corrupt each other. It counts with the ray-by-ray kernel (identical results).
+ * device) race and corrupt each other. What the tree leaves of the array holds the step counts of as many
+ * nodes at a time as fit; a tree that leaves room for none is counted ray by ray (identical results).
  * --------------------------------------------------------------------------------------- */
 #define MIG_NOALLOC_SCRATCH_BYTES (64u << 20)
 mig_status mig_tree_eval_device_noalloc(mig_map *map, int n, const int32_t *parent, const float *pos_m,
@@ -320,12 +321,13 @@ typedef struct mig_kernel_times {
  * paper; all give identical results). Owned-voxel counting casts each pixel ray once to its first
  * occupied voxel, then tests every unknown voxel of the frustum against the ray of the pixel that
  * owns it (its centre's projection): MIG_COUNT_PAIRS enumerates each (node, yaw) frustum,
- * MIG_COUNT_NODES each node's voxels once for all yaws (at most 64 yaws; its ancestor test runs
- * once per voxel), MIG_COUNT_AUTO (the default) takes the per-node pass when a voxel lies in at least
- * 3 yaws' frusta on average. MIG_COUNT_RAYS walks every ray through every voxel it crosses and
+ * MIG_COUNT_NODES each node's voxels once for all yaws, whole 4x4x4 bricks at a time (its ancestor
+ * test runs once per voxel), MIG_COUNT_AUTO (the default) takes the per-node pass. Either falls back to
+ * the pairs when the buffer below does not hold all yaws of one node. MIG_COUNT_RAYS walks every ray through every voxel it crosses and
  * owner-tests the unknown ones. The owned-voxel kernels keep one uint16 step count per (node, yaw,
  * pixel) of a level in a buffer of at most steps_budget_bytes (0 = the default, 1 GiB); a level
- * that does not fit is counted in chunks. Errors: MIG_EINVAL (ctx NULL, unknown kernel). */
+ * that does not fit is counted in chunks. The per-node pass keeps a queue of undecided bricks beside it
+ * (at most 512 MiB). Errors: MIG_EINVAL (ctx NULL, unknown kernel). */
 #define MIG_COUNT_AUTO 0
 #define MIG_COUNT_RAYS 1
 #define MIG_COUNT_PAIRS 2

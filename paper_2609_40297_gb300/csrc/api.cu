@@ -197,6 +197,31 @@ void launch_level_count_timed(mig_ctx *ctx, const LevelParams &p, int Ld, int co
     }
 }
 
+// Steps of a tree whose levels' sizes only the device knows: every level may end in a partial chunk.
+int device_steps(int cap, int n, int K, int levels) { return cap >= K ? levels + n / (cap / K) : 0; }
+
+void launch_device_levels(mig_ctx *ctx, LevelParams p, int n, int levels, int2 *cursor, cudaStream_t s) {
+    const int count_cap = ctx->num_sms * std::min(ctx->count_ctas, std::max(1, (int)ctx->tiles.ctas_per_sm));
+    const int sel_grid = std::max(1, std::min((n + 127) / 128, 1024));
+    const bool steps = p.steps && node_pass(p);
+    const int count = steps ? device_steps(p.steps_cap, n, p.K, levels) : levels;
+    for (int i = 0; i < count; ++i) {
+        if (steps) {  // one chunk at a time, wherever the tree's levels end
+            p.cursor = cursor + i;
+            p.lvl = levels;
+            p.q0 = 0;
+            p.q1 = (int)std::min<long long>((long long)n * p.K, p.steps_cap);
+            timed_launch(ctx, kProfCast, [&] { launch_cast_chunk(p, ctx->num_sms, s); });
+            timed_launch(ctx, kProfVoxel, [&] { launch_node_chunk(p, ctx->num_sms, ctx->node_ctas, s); });
+        } else {
+            p.lvl = i;
+            launch_level_count_timed(ctx, p, n, count_cap);
+        }
+        timed_launch(ctx, kProfSelect, [&] { launch_select(p, sel_grid, s); });
+        timed_launch(ctx, kProfRender, [&] { launch_render(p, n, ctx->num_sms, s); });
+    }
+}
+
 StepsLayout steps_for(const mig_ctx *ctx, int Lmax, const mig_sensor &s, float voxel, int mode) {
     if (ctx->ray_count || mode == MIG_MODE_INTERVAL || mode == MIG_MODE_PANORAMIC) return StepsLayout{};
     return steps_layout(SensorDims{s.width, s.height, s.yaw_bins, range_q16(s.range_m, voxel)}, Lmax, ctx->steps_budget,
@@ -773,6 +798,9 @@ mig_status mig_tree_eval_device(mig_map *m, int n, const int32_t *parent, const 
     const size_t o_hasc = cv.take<int32_t>(n), o_slot = cv.take<int32_t>(1), o_roots = cv.take<int32_t>(1);
     const size_t o_err = cv.take<int32_t>(1), o_cnt = cv.take<int32_t>((size_t)n * K * 2);
     const size_t o_work = cv.take<int32_t>(L);
+    // level sizes are known on the device only: the step-count buffer is sized for n nodes
+    const StepsLayout steps = steps_for(ctx, n, *sensor, m->voxel, MIG_MODE_MARGINAL);
+    const size_t o_cursor = cv.take<int2>(device_steps(steps.cap, n, K, L) + 1);
     const size_t zero_bytes = cv.off;
     const size_t o_depth = cv.take<int32_t>(n), o_loff = cv.take<int32_t>(L + 1), o_lint = cv.take<int32_t>(L);
     const size_t o_lnodes = cv.take<int32_t>(n), o_ar = cv.take<int2>(n);
@@ -780,9 +808,6 @@ mig_status mig_tree_eval_device(mig_map *m, int n, const int32_t *parent, const 
     const size_t o_sel = cv.take<int32_t>(n);
     const size_t o_arena = cv.take<uint32_t>((size_t)n * WH);
     const size_t o_dpyr = cv.take<uint2>((size_t)n * hz_entries(cam->W, cam->H));
-    // level sizes are known on the device only: the step-count buffer is sized for n nodes (its
-    // chunks beyond a level's pairs return at once)
-    const StepsLayout steps = steps_for(ctx, n, *sensor, m->voxel, MIG_MODE_MARGINAL);
     const size_t o_steps = cv.take<char>(steps.bytes);
     char *dev = nullptr;
     st = ctx_workspace(ctx, cv.off, (void **)&dev);
@@ -837,14 +862,7 @@ mig_status mig_tree_eval_device(mig_map *m, int n, const int32_t *parent, const 
     p.max_anc = std::max(1, max_depth);
     if (steps.cap) set_steps(p, dev + o_steps, steps);
     p.dpyr = (uint2 *)(dev + o_dpyr);
-    const int count_cap = ctx->num_sms * std::min(ctx->count_ctas, std::max(1, (int)ctx->tiles.ctas_per_sm));
-    const int sel_grid = std::max(1, std::min((n + 127) / 128, 1024));
-    for (int d = 0; d < L; ++d) {
-        p.lvl = d;
-        launch_level_count_timed(ctx, p, n, count_cap);
-        timed_launch(ctx, kProfSelect, [&] { launch_select(p, sel_grid, ctx->stream); });
-        timed_launch(ctx, kProfRender, [&] { launch_render(p, n, ctx->num_sms, ctx->stream); });
-    }
+    launch_device_levels(ctx, p, n, L, (int2 *)(dev + o_cursor), ctx->stream);
     MIG_CUDA_TRY(cudaGetLastError());
     return MIG_OK;
 }

@@ -42,7 +42,7 @@ struct SegInfo {
 
 // Trees per persistent launch: their parameters travel in the kernel's parameter space (constant
 // bank, up to 32 KB), indexed by the warp-uniform tree number. Larger batches use several launches.
-constexpr int kBatchMaxTrees = 84;
+constexpr int kBatchMaxTrees = 80;
 // 8x4-pixel cast tiles per work item of a cast segment (one item per warp takes one atomic).
 #ifndef MIG_BATCH_CAST_TILES
 #define MIG_BATCH_CAST_TILES 16

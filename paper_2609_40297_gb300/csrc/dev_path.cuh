@@ -673,6 +673,28 @@ __device__ __forceinline__ void count_chunk(const LevelParams &p, const HOT &hp,
     }
 }
 
+// The level and the pairs [q0, q1) of it that a launch works on, clipped to the level's; ends: they are
+// the level's last.
+struct StepRange {
+    int lvl, l0, q0, q1;
+    bool ends;
+};
+__device__ __forceinline__ StepRange step_range(const LevelParams &p) {
+    StepRange r{p.lvl, 0, p.q0, p.q1, true};
+    if (p.cursor) {
+        const int2 c = *p.cursor;
+        if (c.x >= p.lvl) return StepRange{c.x, 0, 0, 0, false};  // past the last level
+        r.lvl = c.x;
+        r.q0 = c.y * p.K;
+        r.q1 = r.q0 + p.steps_cap;
+    }
+    r.l0 = p.level_off[r.lvl];
+    const int pairs = (p.level_off[r.lvl + 1] - r.l0) * p.K;
+    r.ends = r.q1 >= pairs;
+    r.q1 = min(r.q1, pairs);
+    return r;
+}
+
 // Yaw selection of node n (Sec. III-B): lowest k with the largest marginal count (absolute
 // count in the absolute mode, where both counts are equal); g_abs = max over yaws of the
 // absolute count.

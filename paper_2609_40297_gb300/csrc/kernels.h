@@ -75,6 +75,11 @@ struct LevelParams {
     // over pixel tiles, hz_entries(W, H) each; dpyr NULL: not kept
     uint32_t *hz;
     uint2 *dpyr;
+    // NULL, or the place in the tree where this step's launches begin: (level, first node of the level).
+    // The step takes one chunk of steps_cap pairs; a step that ends its level selects and renders it, and
+    // select writes the next step's place to cursor[1]. Used where the host does not know the levels'
+    // sizes: q0 and q1 are then taken from here (step_range), and lvl is the number of levels.
+    int2 *cursor;
     BrickRec *queue;  // per-node pass: undecided bricks of the chunk
     int queue_cap;
     // per-node pass: half a pixel at unit depth along the image axes, the depth below which the owner

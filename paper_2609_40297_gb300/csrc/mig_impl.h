@@ -171,6 +171,11 @@ void launch_level_count_timed(mig_ctx *ctx, const LevelParams &p, int Ld, int co
 // counts ray by ray or the mode does).
 struct StepsLayout;
 StepsLayout steps_for(const mig_ctx *ctx, int Lmax, const mig_sensor &s, float voxel, int mode);
+// The count, select and render launches of a device-planned tree of n nodes and at most `levels` levels.
+// With the per-node pass they go chunk by chunk through the levels, whose sizes only the device knows:
+// device_steps(..) steps and as many places + 1 in `cursor` (zeroed).
+int device_steps(int cap, int n, int K, int levels);
+void launch_device_levels(mig_ctx *ctx, LevelParams p, int n, int levels, int2 *cursor, cudaStream_t s);
 // records an event pair around launch() on the context stream when profiling is on
 void prof_begin(mig_ctx *ctx, int kind, cudaEvent_t *a);
 void prof_end(mig_ctx *ctx, int kind, cudaEvent_t a);

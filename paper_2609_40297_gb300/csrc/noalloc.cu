@@ -15,6 +15,7 @@
 
 #include "kernels.h"
 #include "mig_impl.h"
+#include "voxcount.h"
 
 // The shared scratch. In host code this name is a host-side stand-in, not a device address:
 // host code must pass the address obtained from cudaGetSymbolAddress (noalloc_scratch_ptr).
@@ -110,8 +111,16 @@ extern "C" mig_status mig_tree_eval_device_noalloc(mig_map *m, int n, const int3
     const size_t o_anc = cv.take(4 * std::max<size_t>(1, (size_t)n * max_depth)), o_node = cv.take(16 * (size_t)n);
     const size_t o_sel = cv.take(4 * (size_t)n), o_body = cv.take(16 * WH), o_yaw = cv.take(4 * (size_t)K * kYawRec);
     const size_t o_arena = cv.take(4 * (size_t)n * WH);
-    if (cv.off > (size_t)MIG_NOALLOC_SCRATCH_BYTES)
-        return fail(MIG_EINVAL, "tree_eval_device_noalloc: needs " + std::to_string(cv.off) + " bytes of scratch, above the " +
+    // what is left holds the depth buffers' bounds and the step counts of as many nodes as fit, for the
+    // owned-voxel count in chunks of nodes; a tree that leaves no room is counted ray by ray
+    const size_t need = cv.off, o_dpyr = cv.take(sizeof(uint2) * (size_t)n * hz_entries(W, H));
+    const size_t o_cursor = cv.take(sizeof(int2) * ((size_t)n + L + 1)), o_steps = cv.take(0);
+    const SensorDims dims{W, H, K, range_q16(sensor->range_m, m->voxel)};
+    const StepsLayout steps = o_steps < (size_t)MIG_NOALLOC_SCRATCH_BYTES
+                                  ? steps_layout_in(dims, n, (size_t)MIG_NOALLOC_SCRATCH_BYTES - o_steps)
+                                  : StepsLayout{};
+    if (need > (size_t)MIG_NOALLOC_SCRATCH_BYTES)
+        return fail(MIG_EINVAL, "tree_eval_device_noalloc: needs " + std::to_string(need) + " bytes of scratch, above the " +
                                     std::to_string((size_t)MIG_NOALLOC_SCRATCH_BYTES) +
                                     "-byte maximum (about nodes * width * height * 4 bytes of depth buffers)");
     // per-yaw rotation and projection rows from the host's libm, on the stack (no allocation); they
@@ -220,15 +229,18 @@ extern "C" mig_status mig_tree_eval_device_noalloc(mig_map *m, int n, const int3
     p.arena = (uint32_t *)(dev + o_arena);
     p.mode = MIG_MODE_MARGINAL;
     p.stats = nullptr;
-    p.max_anc = std::max(1, max_depth);
-    const int count_cap = ctx->num_sms * std::min(ctx->count_ctas, std::max(1, (int)ctx->tiles.ctas_per_sm));
-    const int sel_grid = std::max(1, std::min((n + 127) / 128, 1024));
-    for (int d = 0; d < L; ++d) {
-        p.lvl = d;
-        timed_launch(ctx, kProfCount, [&] { launch_count(p, count_cap, s); });
-        timed_launch(ctx, kProfSelect, [&] { launch_select(p, sel_grid, s); });
-        timed_launch(ctx, kProfRender, [&] { launch_render(p, n, ctx->num_sms, s); });
+    p.band_tlo = -1e30f;  // no elevation band: the camera test of the blocks stands alone
+    p.band_thi = 1e30f;
+    p.voxel_pass = MIG_COUNT_AUTO;
+    set_visit_params(p, sensor->hfov_deg, sensor->vfov_deg);
+    const bool rays = ctx->ray_count || ctx->voxel_pass == MIG_COUNT_PAIRS || steps.cap == 0;
+    if (!rays) {
+        set_steps(p, dev + o_steps, steps);
+        p.dpyr = (uint2 *)(dev + o_dpyr);
+        MIG_CUDA_TRY(cudaMemsetAsync(dev + o_cursor, 0, sizeof(int2), s));  // the first step's place
     }
+    p.max_anc = std::max(1, max_depth);
+    launch_device_levels(ctx, p, n, L, (int2 *)(dev + o_cursor), s);
     MIG_CUDA_TRY(cudaGetLastError());
     return MIG_OK;
 }

@@ -17,6 +17,8 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <climits>
+#include <cmath>
 #include <cstdint>
 
 #include "bricks.cuh"
@@ -285,10 +287,10 @@ __global__ void __launch_bounds__(kWarpsN * 32, kCastCtas) cast_kernel(const Lev
     __shared__ float s_beam[32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (blockIdx.x == 0 && threadIdx.x < 3) p.vctr[threadIdx.x] = 0;  // the counters of the passes that follow
-    const int l0 = p.level_off[p.lvl];
-    const int q1 = min(p.q1, (p.level_off[p.lvl + 1] - l0) * p.K);
-    if (p.q0 >= q1) return;
-    const CastLayout lay = cast_layout(q1 - p.q0, p.W, p.H, num_sms);
+    const StepRange step = step_range(p);
+    const int l0 = step.l0, q0 = step.q0, q1 = step.q1;
+    if (q0 >= q1) return;
+    const CastLayout lay = cast_layout(q1 - q0, p.W, p.H, num_sms);
     const int T = lay == kCastSmall ? 16 : 32;
     const int tx = (p.W + T - 1) / T, ty = (p.H + T - 1) / T;
     const size_t WH = (size_t)p.W * p.H;
@@ -296,11 +298,11 @@ __global__ void __launch_bounds__(kWarpsN * 32, kCastCtas) cast_kernel(const Lev
     const uint64_t *om = grid_omask(p.grid);
     const uint8_t *dist = p.grid.g + dist_offset(p.grid.nx, p.grid.ny, p.grid.nz);
     CastCnt st;
-    const long long items = (long long)(q1 - p.q0) * tx * ty;
+    const long long items = (long long)(q1 - q0) * tx * ty;
     const int per = lay == kCastLarge ? kWarpsN : 1, mine = lay == kCastLarge ? warp : 0;  // items at a time per CTA
     for (long long it = (long long)blockIdx.x * per + mine; it < items; it += (long long)gridDim.x * per) {
         const int tile = (int)(it % (tx * ty)), ql = (int)(it / (tx * ty));
-        const int q = p.q0 + ql;
+        const int q = q0 + ql;
         const int4 nd = p.node[p.level_nodes[l0 + q / p.K]];
         const int32_t *yk = p.yawtab + (q % p.K) * 12;
         const CastOut o{p.steps + (size_t)ql * WH, p.hz + (size_t)ql * y.n};
@@ -328,7 +330,13 @@ __global__ void __launch_bounds__(kWarpsN * 32, kCastCtas) render_kernel(const L
     __shared__ uint2 s_t[kWarpsN];
     __shared__ float s_beam[32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int l0 = p.level_off[p.lvl], Li = p.level_int[p.lvl];
+    int lvl = p.lvl;
+    if (p.cursor) {
+        const StepRange step = step_range(p);
+        if (!step.ends || step.q1 <= step.q0) return;
+        lvl = step.lvl;
+    }
+    const int l0 = p.level_off[lvl], Li = p.level_int[lvl];
     const CastLayout lay = cast_layout(Li, p.W, p.H, num_sms);
     const int T = lay == kCastSmall ? 16 : 32;
     const int tx = (p.W + T - 1) / T, ty = (p.H + T - 1) / T;
@@ -681,9 +689,8 @@ __global__ void __launch_bounds__(kWarpsN * 32, 3) node_kernel(const LevelParams
     const int K = p.K;
     YawRows *s_y = reinterpret_cast<YawRows *>(s_dyn);
     NodeAnc *anc = reinterpret_cast<NodeAnc *>(s_y + K) + warp * p.max_anc;
-    const int l0 = p.level_off[p.lvl];
-    const int Ld = p.level_off[p.lvl + 1] - l0;
-    const int nb0 = p.q0 / K, nn = min(p.q1 / K, Ld) - nb0;
+    const StepRange step = step_range(p);
+    const int l0 = step.l0, nb0 = step.q0 / K, nn = step.q1 / K - nb0;
     if (nn <= 0) return;
     for (int k = threadIdx.x; k < K; k += blockDim.x)
         s_y[k] = yaw_rows(p.yawtab + k * 12, p.W, p.H, p.vis_hu, p.vis_hv, p.ifx, p.ify);
@@ -915,9 +922,9 @@ __global__ void __launch_bounds__(kWarpsN * 32, 4) brick_kernel(const LevelParam
     const int K = p.K;
     YawRows *s_y = reinterpret_cast<YawRows *>(s_dyn);
     NodeAnc *anc = reinterpret_cast<NodeAnc *>(s_y + K) + warp * p.max_anc;
-    const int l0 = p.level_off[p.lvl];
-    const int nb0 = p.q0 / K;
-    if (min(p.q1 / K, p.level_off[p.lvl + 1] - l0) <= nb0) return;
+    const StepRange step = step_range(p);
+    const int l0 = step.l0, nb0 = step.q0 / K;
+    if (step.q1 <= step.q0) return;
     const int total = min(p.vctr[1], p.queue_cap);
     const int slice = max(1, min(64, total / (int)(gridDim.x * kWarpsN * 8)));
     if (blockIdx.x * kWarpsN * slice >= total) return;
@@ -1105,9 +1112,17 @@ static long long node_bricks(int64_t Tq) {
 constexpr double kQueueShare = 0.3;
 constexpr long long kQueueMax = 8ll << 20;  // records (512 MB)
 
+// The offsets of a region of L.cap pairs and L.queue_cap records.
+static void place(StepsLayout &L, const SensorDims &d) {
+    auto align = [](size_t b) { return (b + 255) & ~(size_t)255; };
+    L.o_ctr = align((size_t)L.cap * d.W * d.H * sizeof(uint16_t));
+    L.o_hz = L.o_ctr + 256;
+    L.o_queue = align(L.o_hz + (size_t)L.cap * hz_entries(d.W, d.H) * sizeof(uint32_t));
+    L.bytes = L.o_queue + (size_t)L.queue_cap * sizeof(BrickRec);
+}
+
 StepsLayout steps_layout(const SensorDims &d, int max_nodes, size_t budget_bytes, bool node_pass) {
     StepsLayout L{};
-    const size_t WH = (size_t)d.W * d.H;
     const long long pairs = (long long)std::max(1, max_nodes) * d.K;
     L.cap = (int)steps_pairs(pairs, d.W, d.H, budget_bytes);
     const long long per_node = (long long)(kQueueShare * (double)node_bricks(d.Tq)) + 1;
@@ -1116,11 +1131,23 @@ StepsLayout steps_layout(const SensorDims &d, int max_nodes, size_t budget_bytes
         L.cap = (int)nodes * d.K;
         L.queue_cap = (int)std::min(kQueueMax, std::max<long long>(nodes * per_node, 1ll << 16));
     }
-    auto align = [](size_t b) { return (b + 255) & ~(size_t)255; };
-    L.o_ctr = align((size_t)L.cap * WH * sizeof(uint16_t));
-    L.o_hz = L.o_ctr + 256;
-    L.o_queue = align(L.o_hz + (size_t)L.cap * hz_entries(d.W, d.H) * sizeof(uint32_t));
-    L.bytes = L.o_queue + (size_t)L.queue_cap * sizeof(BrickRec);
+    place(L, d);
+    return L;
+}
+
+StepsLayout steps_layout_in(const SensorDims &d, int max_nodes, size_t bytes) {
+    // per node: its step counts, their bounds and 0.7 of the usual queue (a full queue only slows the
+    // bricks beyond it), so that a fixed region holds more nodes at a time
+    const size_t recs = (size_t)(0.7 * kQueueShare * (double)node_bricks(d.Tq)) + 1;
+    const size_t node = (size_t)d.K * ((size_t)d.W * d.H * sizeof(uint16_t) + hz_entries(d.W, d.H) * sizeof(uint32_t)) +
+                        recs * sizeof(BrickRec);
+    const size_t fixed = 4 * 256;  // the counters and the alignment of the parts
+    StepsLayout L{};
+    if (bytes < fixed + node) return L;
+    const long long nodes = std::min<long long>(std::min<long long>(max_nodes, (1 << kRecNodeBits) - 1), (long long)((bytes - fixed) / node));
+    L.cap = (int)std::min<long long>(nodes, INT_MAX / d.K) * d.K;
+    L.queue_cap = (int)std::min<long long>(kQueueMax, (long long)(L.cap / d.K) * recs);
+    place(L, d);
     return L;
 }
 

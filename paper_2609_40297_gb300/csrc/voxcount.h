@@ -27,6 +27,8 @@ struct StepsLayout {
     size_t o_ctr, o_hz, o_queue, bytes;
 };
 StepsLayout steps_layout(const SensorDims &d, int max_nodes, size_t budget_bytes, bool node_pass);
+// The same for whole nodes within a region of at most `bytes` bytes (cap 0: not one node fits).
+StepsLayout steps_layout_in(const SensorDims &d, int max_nodes, size_t bytes);
 void set_steps(LevelParams &p, void *base, const StepsLayout &L);  // the region's fields
 // Step-count buffer budget per evaluation (device bytes).
 constexpr size_t kStepsBudget = (size_t)1 << 30;
