@@ -165,7 +165,7 @@ void set_pano_params(LevelParams &p, const Camera *cam, int32_t *pcnt) {
 
 void launch_level_count(const mig_ctx *ctx, const LevelParams &p, int Ld, int count_cap, cudaStream_t s) {
     const int items = Ld * p.K * p.tiles;
-    if (p.mode == MIG_MODE_INTERVAL) {
+    if (p.mode == MIG_MODE_INTERVAL && !p.steps) {
         launch_count_interval(p, std::max(1, std::min((items + 7) / 8, ctx->num_sms * ctx->interval_ctas)), s);
     } else if (p.mode == MIG_MODE_PANORAMIC) {
         const int pitems = Ld * p.pano_A;
@@ -179,7 +179,7 @@ void launch_level_count(const mig_ctx *ctx, const LevelParams &p, int Ld, int co
 }
 
 void launch_level_count_timed(mig_ctx *ctx, const LevelParams &p, int Ld, int count_cap) {
-    if (!p.steps || p.mode == MIG_MODE_INTERVAL || p.mode == MIG_MODE_PANORAMIC) {
+    if (!p.steps || p.mode == MIG_MODE_PANORAMIC) {
         timed_launch(ctx, kProfCount, [&] { launch_level_count(ctx, p, Ld, count_cap, ctx->stream); });
         return;
     }
@@ -223,9 +223,12 @@ void launch_device_levels(mig_ctx *ctx, LevelParams p, int n, int levels, int2 *
 }
 
 StepsLayout steps_for(const mig_ctx *ctx, int Lmax, const mig_sensor &s, float voxel, int mode) {
-    if (ctx->ray_count || mode == MIG_MODE_INTERVAL || mode == MIG_MODE_PANORAMIC) return StepsLayout{};
-    return steps_layout(SensorDims{s.width, s.height, s.yaw_bins, range_q16(s.range_m, voxel)}, Lmax, ctx->steps_budget,
-                        ctx->voxel_pass != MIG_COUNT_PAIRS);
+    if (ctx->ray_count || mode == MIG_MODE_PANORAMIC || (mode == MIG_MODE_INTERVAL && ctx->voxel_pass == MIG_COUNT_PAIRS))
+        return StepsLayout{};
+    const StepsLayout L = steps_layout(SensorDims{s.width, s.height, s.yaw_bins, range_q16(s.range_m, voxel)}, Lmax, ctx->steps_budget,
+                                       ctx->voxel_pass != MIG_COUNT_PAIRS, mode == MIG_MODE_INTERVAL);
+    // the interval mode has no pass per (node, yaw) pair: without room for whole nodes it counts ray by ray
+    return mode == MIG_MODE_INTERVAL && L.queue_cap == 0 ? StepsLayout{} : L;
 }
 
 void prof_begin(mig_ctx *ctx, int kind, cudaEvent_t *a) {

@@ -1,4 +1,4 @@
-// Interval-mode count pass: the paper's screen-space overlap test (Sec. IV-B, Eq. 5-7).
+// Interval-mode count pass, ray by ray (where the per-node pass of nodecount.cu does not apply): the paper's screen-space overlap test (Sec. IV-B, Eq. 5-7).
 //
 // For every candidate ray the 3D DDA (Sec. IV-B) visits voxels exactly as in the sample mode;
 // each owned unknown voxel (its centre projects into the ray's pixel) counts as absolute gain and
@@ -34,6 +34,7 @@
 #include <cstdint>
 
 #include "dev_path.cuh"
+#include "interval.cuh"
 #include "interval.h"
 #include "kernels.h"
 #include "mig.h"
@@ -51,179 +52,13 @@ using namespace dev;
 
 constexpr int kIvWarps = 8;
 constexpr int kIvThreads = kIvWarps * 32;
-constexpr float kZNear = 1.0f / 1024.0f;  // near end of the valid depth range, voxel units
-
-// an ancestor as the interval walk needs it: position (Q16), selected yaw, depth buffer
+// an ancestor as the interval walk needs it: position (Q16), selected yaw, the node in its camera's
+// coordinates (every ray's origin), depth buffer
 struct IvAnc {
     int px, py, pz, yaw;
+    float U0, V0, Z0;
     const uint32_t *D;
 };
-
-struct Seg {
-    float lo, hi;          // depth-clipped range of the ray fraction
-    float Za, Zb;          // camera z at lo, hi (voxel units)
-    float ua, va, ub, vb;  // projected clipped endpoints (pixels)
-    float wa, wb;          // inverse depths at the endpoints
-    float s0, s1;          // Liang-Barsky range of the screen parameter
-    float ru, rv;          // reciprocals of the segment's screen extent (0 when it is 0)
-};
-
-__device__ __forceinline__ float fadd(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ float fsub(float a, float b) { return __fsub_rn(a, b); }
-__device__ __forceinline__ float fmul(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ float fdiv(float a, float b) { return __fdiv_rn(a, b); }
-
-// steps 1-3 for the candidate ray from P to its range endpoint E (Q16) and the ancestor at Pa
-// with projection rows m (Q16: mu, mv, mz); false if nothing of the ray is in view, or if the
-// sample's ray fraction lam lies outside the depth-clipped range (seg_param would then reject it,
-// so the screen-space part is skipped with the same outcome)
-__device__ bool seg_setup(const int32_t *m, const int3 Pa, const int64_t P[3], const int64_t E[3], float zf, int W,
-                          int H, float lam, Seg &g) {
-    const int64_t r0x = P[0] - Pa.x, r0y = P[1] - Pa.y, r0z = P[2] - Pa.z;
-    const int64_t r1x = E[0] - Pa.x, r1y = E[1] - Pa.y, r1z = E[2] - Pa.z;
-    const float sc = 2.3283064365386963e-10f;  // 2^-32: Q32 -> voxel units
-    const float Z0 = fmul(__ll2float_rn((int64_t)m[6] * r0x + (int64_t)m[7] * r0y + (int64_t)m[8] * r0z), sc);
-    const float Z1 = fmul(__ll2float_rn((int64_t)m[6] * r1x + (int64_t)m[7] * r1y + (int64_t)m[8] * r1z), sc);
-    const float zn = kZNear;
-    const float dZ = fsub(Z1, Z0);
-    float lo = 0.0f, hi = 1.0f;
-    if (Z0 < zn) {
-        if (!(dZ > 0.0f)) return false;
-        lo = fdiv(fsub(zn, Z0), dZ);
-    }
-    if (Z1 < zn) {
-        if (!(dZ < 0.0f)) return false;
-        hi = fdiv(fsub(zn, Z0), dZ);
-    }
-    if (Z0 > zf) {
-        if (!(dZ < 0.0f)) return false;
-        const float l = fdiv(fsub(zf, Z0), dZ);
-        if (l > lo) lo = l;
-    }
-    if (Z1 > zf) {
-        if (!(dZ > 0.0f)) return false;
-        const float h = fdiv(fsub(zf, Z0), dZ);
-        if (h < hi) hi = h;
-    }
-    if (!(lo < hi)) return false;
-    if (!(lam >= lo && lam <= hi)) return false;
-    const float U0 = fmul(__ll2float_rn((int64_t)m[0] * r0x + (int64_t)m[1] * r0y + (int64_t)m[2] * r0z), sc);
-    const float V0 = fmul(__ll2float_rn((int64_t)m[3] * r0x + (int64_t)m[4] * r0y + (int64_t)m[5] * r0z), sc);
-    const float U1 = fmul(__ll2float_rn((int64_t)m[0] * r1x + (int64_t)m[1] * r1y + (int64_t)m[2] * r1z), sc);
-    const float V1 = fmul(__ll2float_rn((int64_t)m[3] * r1x + (int64_t)m[4] * r1y + (int64_t)m[5] * r1z), sc);
-    const float dU = fsub(U1, U0), dV = fsub(V1, V0);
-    const float Ua = fadd(U0, fmul(lo, dU)), Va = fadd(V0, fmul(lo, dV)), Za = fadd(Z0, fmul(lo, dZ));
-    const float Ub = fadd(U0, fmul(hi, dU)), Vb = fadd(V0, fmul(hi, dV)), Zb = fadd(Z0, fmul(hi, dZ));
-    if (!(Za > 0.0f && Zb > 0.0f)) return false;
-    g.lo = lo;
-    g.hi = hi;
-    g.Za = Za;
-    g.Zb = Zb;
-    // Eq. 5 with the inverse depths of Eq. 6: u = U w, v = V w
-    g.wa = fdiv(1.0f, Za);
-    g.wb = fdiv(1.0f, Zb);
-    g.ua = fmul(Ua, g.wa);
-    g.va = fmul(Va, g.wa);
-    g.ub = fmul(Ub, g.wb);
-    g.vb = fmul(Vb, g.wb);
-    // Liang-Barsky against 0 <= u <= W, 0 <= v <= H (edges in the order -u, +u, -v, +v); each
-    // edge's crossing is q times the reciprocal of p
-    const float du = fsub(g.ub, g.ua), dv = fsub(g.vb, g.va);
-    g.ru = du != 0.0f ? fdiv(1.0f, du) : 0.0f;
-    g.rv = dv != 0.0f ? fdiv(1.0f, dv) : 0.0f;
-    const float pe[4] = {-du, du, -dv, dv};
-    const float rp[4] = {-g.ru, g.ru, -g.rv, g.rv};
-    const float qe[4] = {g.ua, fsub(__int2float_rn(W), g.ua), g.va, fsub(__int2float_rn(H), g.va)};
-    float s0 = 0.0f, s1 = 1.0f;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        if (pe[e] == 0.0f) {
-            if (qe[e] < 0.0f) return false;
-            continue;
-        }
-        const float r = fmul(qe[e], rp[e]);
-        if (pe[e] < 0.0f) {
-            if (r > s1) return false;
-            if (r > s0) s0 = r;
-        } else {
-            if (r < s0) return false;
-            if (r < s1) s1 = r;
-        }
-    }
-    if (!(s0 < s1)) return false;
-    g.s0 = s0;
-    g.s1 = s1;
-    return true;
-}
-
-// screen parameter of the ray fraction lam (perspective-correct); false outside the clip
-__device__ __forceinline__ bool seg_param(const Seg &g, float lam, float &s) {
-    if (!(lam >= g.lo && lam <= g.hi)) return false;
-    const float mu = fdiv(fsub(lam, g.lo), fsub(g.hi, g.lo));
-    const float num = fmul(mu, g.Zb);
-    const float den = fadd(fmul(fsub(1.0f, mu), g.Za), num);
-    s = fdiv(num, den);
-    return s >= g.s0 && s < g.s1;
-}
-
-// a voxel's sample: midpoint of the ray's traversal of it (entry ne / ade, exit nx / adx capped at
-// the range) as a fraction of the range T (= Tq / 2^30 in crossing units)
-__device__ __forceinline__ float sample_lambda(uint32_t ne, uint32_t ade, uint32_t nx, uint32_t adx, float T) {
-    const float lin = fdiv(fdiv(__uint2float_rn(ne), __uint2float_rn(ade)), T);
-    float lout = fdiv(fdiv(__uint2float_rn(nx), __uint2float_rn(adx)), T);
-    if (lout > 1.0f) lout = 1.0f;
-    return fmul(fadd(lin, lout), 0.5f);
-}
-
-// Column (or row) crossings of the walk: boundary b_k = b0 + sgn k is crossed at screen parameter
-// x(k) = (b_k - a0) * r, the walk's own formula, non-decreasing in k. Counts the crossings at or
-// before s among k < kmax (crossing kmax leaves the buffer); lo / hi = the last crossing at or
-// before s and the next one. The count starts from a float estimate and is corrected exactly.
-__device__ __forceinline__ int count_crossings(float a0, float r, float d, int b0, int sgn, int kmax, float s,
-                                               float &lo, float &hi) {
-    const float est = (float)sgn * (s * d + a0 - (float)b0) + 1.0f;  // estimate only; corrected below
-    int k = !(est > 0.0f) ? 0 : (est >= (float)kmax ? kmax : (int)est);
-    auto x = [&](int kk) { return fmul(fsub(__int2float_rn(b0 + sgn * kk), a0), r); };
-    while (k > 0 && x(k - 1) > s) --k;
-    while (k < kmax && x(k) <= s) ++k;
-    lo = k > 0 ? x(k - 1) : __int_as_float(0xff800000);
-    hi = k < kmax ? x(k) : __int_as_float(0x7f800000);
-    return k;
-}
-
-// Step 4 for one screen parameter s in [s0, s1): the walk's portion containing s, found directly.
-// The walk crosses column and row boundaries in the order of their crossing parameters, so at s
-// it is in column i0 + si * (column crossings <= s) and row j0 + sj * (row crossings <= s), in the
-// portion from the latest crossing at or before s (s0 if none) to the next one (capped at s1).
-// True if that portion is observed; false if not, or if the walk leaves the buffer before s.
-__device__ bool seg_lookup(const Seg &g, int W, int H, const uint32_t *D, float s) {
-    const float du = fsub(g.ub, g.ua), dv = fsub(g.vb, g.va);
-    const float ru = g.ru, rv = g.rv;
-    const float fi = floorf(fadd(g.ua, fmul(g.s0, du))), fj = floorf(fadd(g.va, fmul(g.s0, dv)));
-    const int i0 = fi < 0.0f ? 0 : (fi > __int2float_rn(W - 1) ? W - 1 : __float2int_rz(fi));
-    const int j0 = fj < 0.0f ? 0 : (fj > __int2float_rn(H - 1) ? H - 1 : __float2int_rz(fj));
-    const int si = du > 0.0f ? 1 : (du < 0.0f ? -1 : 0), sj = dv > 0.0f ? 1 : (dv < 0.0f ? -1 : 0);
-    float xlo = __int_as_float(0xff800000), xhi = __int_as_float(0x7f800000), ylo = xlo, yhi = xhi;
-    int nx = 0, ny = 0;
-    if (si) {
-        const int kmax = si > 0 ? W - i0 : i0 + 1;
-        nx = count_crossings(g.ua, ru, du, si > 0 ? i0 + 1 : i0, si, kmax, s, xlo, xhi);
-        if (nx == kmax) return false;
-    }
-    if (sj) {
-        const int kmax = sj > 0 ? H - j0 : j0 + 1;
-        ny = count_crossings(g.va, rv, dv, sj > 0 ? j0 + 1 : j0, sj, kmax, s, ylo, yhi);
-        if (ny == kmax) return false;
-    }
-    const int i = i0 + si * nx, j = j0 + sj * ny;
-    const float s_in = (nx == 0 && ny == 0) ? g.s0 : (xlo > ylo ? xlo : ylo);
-    float s_out = xhi < yhi ? xhi : yhi;
-    if (g.s1 < s_out) s_out = g.s1;
-    const float sm = fmul(fadd(s_in, s_out), 0.5f);
-    const float wm = fadd(g.wa, fmul(sm, fsub(g.wb, g.wa)));
-    const float Dv = fmul(__uint2float_rn(__ldg(D + (size_t)j * W + i)), 1.52587890625e-05f);
-    return fmul(wm, Dv) >= 1.0f;  // z <= D in inverse depth
-}
 
 // A queued sample: the face distances of the crossings that enter and leave its voxel (Q16), and
 // which of the ray's direction components |d_x|, |d_y|, |d_z| each is divided by (code 3: the
@@ -239,7 +74,7 @@ __device__ __forceinline__ uint32_t speed_of(uint32_t code, uint32_t adx, uint32
 // Is the queued sample e (ray through pixel e.z >> 4, yaw ck / sk, origin P) inside an ancestor's
 // observed portions? Ancestors parent first; the ray's set-up is rebuilt per sample.
 template <bool STATS>
-__device__ bool iv_observed(const LevelParams &p, const IvAnc *anc, int na, const int64_t P[3], int ck, int sk,
+__device__ bool iv_observed(const LevelParams &p, const IvAnc *anc, int na, const int P[3], int ck, int sk,
                             float zf, float T, const uint4 e, uint32_t &st_seg) {
     const int pix = (int)(e.z >> 4);
     const int4 b = p.body[pix];
@@ -248,13 +83,14 @@ __device__ bool iv_observed(const LevelParams &p, const IvAnc *anc, int na, cons
     const uint32_t adx = (uint32_t)(dx < 0 ? -dx : dx), ady = (uint32_t)(dy < 0 ? -dy : dy),
                    adz = (uint32_t)(dz < 0 ? -dz : dz);
     const float lam = sample_lambda(e.x, speed_of(e.z & 3u, adx, ady, adz), e.y, speed_of((e.z >> 2) & 3u, adx, ady, adz), T);
-    const int64_t E[3] = {P[0] + (((int64_t)p.Tq * dx) >> 30), P[1] + (((int64_t)p.Tq * dy) >> 30),
-                          P[2] + (((int64_t)p.Tq * dz) >> 30)};
+    const int E[3] = {P[0] + (int)(((int64_t)p.Tq * dx) >> 30), P[1] + (int)(((int64_t)p.Tq * dy) >> 30),
+                      P[2] + (int)(((int64_t)p.Tq * dz) >> 30)};
     for (int a = 0; a < na; ++a) {
         const IvAnc &A = anc[a];
         Seg g;
         if constexpr (STATS) ++st_seg;
-        if (!seg_setup(p.yawtab + A.yaw * 12 + 2, make_int3(A.px, A.py, A.pz), P, E, zf, p.W, p.H, lam, g)) continue;
+        const int32_t *m = p.yawtab + A.yaw * 12 + 2;
+        if (!seg_setup(m, A.U0, A.V0, A.Z0, make_int3(E[0] - A.px, E[1] - A.py, E[2] - A.pz), zf, p.W, p.H, lam, g)) continue;
         float s;
         if (seg_param(g, lam, s) && seg_lookup(g, p.W, p.H, A.D, s)) return true;
     }
@@ -295,13 +131,18 @@ __global__ void __launch_bounds__(kIvThreads, MIG_IV_MINB) interval_count_kernel
             rec.py = an.y;
             rec.pz = an.z;
             rec.yaw = p.sel_yaw[a];
+            const int32_t *m = p.yawtab + rec.yaw * 12 + 2;
+            const int rx = nd.x - an.x, ry = nd.y - an.y, rz = nd.z - an.z;
+            rec.U0 = seg_coord(m, rx, ry, rz);
+            rec.V0 = seg_coord(m + 3, rx, ry, rz);
+            rec.Z0 = seg_coord(m + 6, rx, ry, rz);
             rec.D = p.arena + (size_t)an.w * p.W * p.H;
             anc[t] = rec;
         }
         __syncwarp();
         const int32_t *yk = p.yawtab + k * 12;
         const int ck = yk[0], sk = yk[1];
-        const int64_t P[3] = {nd.x, nd.y, nd.z};
+        const int P[3] = {nd.x, nd.y, nd.z};
         const int tx0 = (tile % p.tiles_x) * p.tile_w, ty0 = (tile / p.tiles_x) * p.tile_h;
         const int tile_rays = p.tile_w * p.tile_h;
         int next = 0, ti = 0, tj = 0, qn = 0, c_abs = 0, c_mrg = 0;

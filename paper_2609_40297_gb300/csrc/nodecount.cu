@@ -22,6 +22,7 @@
 #include <cstdint>
 
 #include "bricks.cuh"
+#include "interval.cuh"
 #include "kernels.h"
 #include "mig.h"
 #include "voxcount.h"
@@ -383,6 +384,7 @@ struct NodeAnc {
     int px, py, pz, yaw;
     const uint32_t *D;
     const uint2 *pyr;
+    float U0, V0, Z0, pad;  // interval mode: the node in the ancestor's camera coordinates
 };
 
 struct NodeCnt {  // statistics
@@ -494,6 +496,7 @@ __device__ __forceinline__ VoxConst vox_const(const LevelParams &p) {
 }
 
 // The ancestors of node n that the mode tests (Sec. IV-B), parent first; returns their number.
+template <bool INTERVAL>
 __device__ __forceinline__ int node_ancestors(const LevelParams &p, int n, NodeAnc *anc, size_t WH, int pyr_n, int lane) {
     const int2 ar = p.anc_range[n];
     int na = p.mode == MIG_MODE_ABSOLUTE ? 0 : (p.mode == MIG_MODE_SINGLE_PARENT ? min(ar.y, 1) : ar.y);
@@ -502,16 +505,92 @@ __device__ __forceinline__ int node_ancestors(const LevelParams &p, int n, NodeA
     for (int t = lane; t < na; t += 32) {
         const int a = p.anc[ar.x + t];
         const int4 an = p.node[a];
-        anc[t] = NodeAnc{an.x, an.y, an.z, p.sel_yaw[a], p.arena + (size_t)an.w * WH, p.dpyr + (size_t)an.w * pyr_n};
+        NodeAnc A{an.x, an.y, an.z, p.sel_yaw[a], p.arena + (size_t)an.w * WH, p.dpyr + (size_t)an.w * pyr_n, 0.f, 0.f, 0.f, 0.f};
+        if (INTERVAL) {
+            const int32_t *m = p.yawtab + A.yaw * 12 + 2;
+            const int4 nd = p.node[n];
+            const int rx = nd.x - an.x, ry = nd.y - an.y, rz = nd.z - an.z;
+            A.U0 = seg_coord(m, rx, ry, rz);
+            A.V0 = seg_coord(m + 3, rx, ry, rz);
+            A.Z0 = seg_coord(m + 6, rx, ry, rz);
+        }
+        anc[t] = A;
     }
     __syncwarp();
     return na;
 }
 
+// Interval mode: no sample in the box of half extents (hx, hy, hz) about the offset (cx, cy, cz) from
+// ancestor A's camera can fall in an observed portion of its buffer. A sample inside a portion
+// projects into the image within the float error of seg_setup and seg_param, whose screen coordinates
+// reach |U| / kZNear where the ray passes the camera plane: 6e-7 of that, plus one pixel, widens the
+// image here; its depth is at most the range.
+__device__ __forceinline__ bool iv_box_out(const YawRows &r, const NodeAnc &A, const int4 nd, float cx, float cy, float cz, float hx,
+                                           float hy, float hz, float W, float H, float Tv) {
+    const float reach = fmaxf(fmaxf(fabsf(q16f(A.px - nd.x)), fabsf(q16f(A.py - nd.y))), fabsf(q16f(A.pz - nd.z))) + Tv + 2.0f;
+    const float mu = fmaf(6.2e-4f * r.u.w, reach, 1.0f), mv = fmaf(6.2e-4f * r.v.w, reach, 1.0f);
+    const float Z = row_dot(r.z, cx, cy, cz), U = row_dot(r.u, cx, cy, cz), V = row_dot(r.v, cx, cy, cz);
+    const float eZ = row_ext(r.z.x, r.z.y, r.z.z, hx, hy, hz) + 0.05f;
+    // a half-space a Z + s m . r > 0: its value at the centre plus its largest change over the box
+    auto out = [&](float a, float s, const float4 &m, float v) {
+        return fmaf(a, Z, s * v) + row_ext(fmaf(a, r.z.x, s * m.x), fmaf(a, r.z.y, s * m.y), fmaf(a, r.z.z, s * m.z), hx, hy, hz) +
+                   kBoxErr * fmaf(fabsf(a), r.z.w, m.w) <
+               0.0f;
+    };
+    return Z + eZ < 0.0f || Z - eZ > Tv || out(mu, 1.0f, r.u, U) || out(W + mu, -1.0f, r.u, U) || out(mv, 1.0f, r.v, V) ||
+           out(H + mv, -1.0f, r.v, V);
+}
+
+// Interval mode: is the sample of voxel (x, y, z) on its owner ray (body-frame ray b, yaw cos ck, sin sk)
+// observed by one of the ancestors `left`? The ray's crossings that enter and leave the voxel are the
+// last entering and the first leaving event in the DDA's order (visit_index).
+__device__ __forceinline__ bool iv_observed(const LevelParams &p, const NodeAnc *anc, uint64_t left, const int4 nd, const int4 b, int ck,
+                                            int sk, int x, int y, int z) {
+    int dx, dy, dz;
+    ray_dir(b, ck, sk, dx, dy, dz);
+    uint32_t n[3], ad[3], en = 0, eA = 1, xn = 0, xA = 1;
+    int c[3], ea = -1;
+    {
+        const int P[3] = {nd.x, nd.y, nd.z}, d[3] = {dx, dy, dz}, v[3] = {x, y, z};
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            int v0, s;
+            ray_axis(P[a], d[a], v0, s, n[a], ad[a]);
+            c[a] = s * (v[a] - v0);
+            if (c[a] >= 1) {
+                const uint32_t na = n[a] + ((uint32_t)(c[a] - 1) << 16);
+                if (ea < 0 || ev_lt(en, eA, ea, na, ad[a], a)) {
+                    ea = a;
+                    en = na;
+                    eA = ad[a];
+                }
+            }
+        }
+        const uint32_t l0 = n[0] + ((uint32_t)c[0] << 16), l1 = n[1] + ((uint32_t)c[1] << 16), l2 = n[2] + ((uint32_t)c[2] << 16);
+        const int a = ev_argmin3(l0, ad[0], l1, ad[1], l2, ad[2]);
+        xn = a == 0 ? l0 : (a == 1 ? l1 : l2);
+        xA = a == 0 ? ad[0] : (a == 1 ? ad[1] : ad[2]);
+    }
+    const float zf = fmul(__ll2float_rn(p.Tq), 1.52587890625e-05f);     // range, voxel units
+    const float T = fmul(__ll2float_rn(p.Tq), 9.313225746154785e-10f);  // range, crossing units
+    const float lam = sample_lambda(en, eA, xn, xA, T);
+    const int Ex = nd.x + (int)(((int64_t)p.Tq * dx) >> 30), Ey = nd.y + (int)(((int64_t)p.Tq * dy) >> 30),
+              Ez = nd.z + (int)(((int64_t)p.Tq * dz) >> 30);
+    bool obs = false;
+    for (; left && !obs; left &= left - 1) {
+        const NodeAnc &A = anc[__ffsll((long long)left) - 1];
+        Seg g;
+        float s;
+        obs = seg_setup(p.yawtab + A.yaw * 12 + 2, A.U0, A.V0, A.Z0, make_int3(Ex - A.px, Ey - A.py, Ez - A.pz), zf, p.W, p.H, lam, g) &&
+              seg_param(g, lam, s) && seg_lookup(g, p.W, p.H, A.D, s);
+    }
+    return obs;
+}
+
 // One undecided brick (warp-uniform record r; lane = voxel of its lower and upper half): the
 // ancestor tests left, then each yaw's counts into c_abs / c_mrg of lane (yaw - first) % 32, slot
 // (yaw - first) / 32.
-template <bool STATS>
+template <bool STATS, bool INTERVAL>
 __device__ __forceinline__ void count_brick(const LevelParams &p, const VoxConst &vc, const YawRows *s_y, const NodeAnc *anc,
                                             const int4 nd, const uint16_t *steps, const BrickRec &r, int lane, int c_abs[2],
                                             int c_mrg[2], NodeCnt &st) {
@@ -526,7 +605,7 @@ __device__ __forceinline__ void count_brick(const LevelParams &p, const VoxConst
     // error of a row product per unit of the row's norm, for every voxel of the brick
     const float verr = 5e-7f * (__uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(rinf))) + 1.0f);
     // ---- the ancestors that were not decided for the whole brick
-    for (uint64_t as = r.anc; as; as &= as - 1) {
+    for (uint64_t as = INTERVAL ? 0ull : r.anc; as; as &= as - 1) {
         const NodeAnc A = anc[__ffsll((long long)as) - 1];
         const float4 ru = s_y[A.yaw].u, rv = s_y[A.yaw].v, rz = s_y[A.yaw].z;
         const int32_t *row = p.yawtab + A.yaw * 12;
@@ -563,8 +642,8 @@ __device__ __forceinline__ void count_brick(const LevelParams &p, const VoxConst
         }
         O |= (uint64_t)__ballot_sync(0xffffffffu, obs[0]) | ((uint64_t)__ballot_sync(0xffffffffu, obs[1]) << 32);
     }
-    // ---- yaws that count every unknown voxel
-    {
+    // ---- yaws that count every unknown voxel (interval mode: their samples differ by yaw, see below)
+    if (!INTERVAL) {
         const int cu = __popcll(U), cm = __popcll(U & ~O);
 #pragma unroll
         for (int i = 0; i < 2; ++i)
@@ -589,13 +668,14 @@ __device__ __forceinline__ void count_brick(const LevelParams &p, const VoxConst
         man[h] = mxy + abs(z0 + 2 * h - v0z);
     }
     const uint64_t rv64 = r.rch | r.vis;
-    for (uint64_t ks = r.part; ks; ks &= ks - 1) {
+    for (uint64_t ks = INTERVAL ? r.part | r.all : r.part; ks; ks &= ks - 1) {
         const int j = __ffsll((long long)ks) - 1, k = kb + j;
         const float4 ru = s_y[k].u, rv = s_y[k].v, rz = s_y[k].z;
         const float Zxy = fmaf(rz.x, ex, rz.y * ey), Uxy = fmaf(ru.x, ex, ru.y * ey), Vxy = fmaf(rv.x, ex, rv.y * ey);
         const int32_t *row = p.yawtab + k * 12;
         bool c[2] = {false, false};
-        if (!((rv64 >> j) & 1)) {
+        int pix[2] = {0, 0};
+        if (!INTERVAL && !((rv64 >> j) & 1)) {
             // every voxel is reached and visited: only the image test, without the pixel
             const float cz = verr * rz.w, cu = verr * ru.w, cv = verr * rv.w, cr = fmaf(vc.fW, cz, cu), cb = fmaf(vc.fH, cz, cv);
 #pragma unroll
@@ -612,7 +692,6 @@ __device__ __forceinline__ void count_brick(const LevelParams &p, const VoxConst
             const PixelErr pe{2.0f * verr * fmaf(vc.fW, rz.w, ru.w), 2.0f * verr * fmaf(vc.fH, rz.w, rv.w), vc.bu, vc.bv};
             const bool nr = (r.rch >> j) & 1, nv = (r.vis >> j) & 1;
             const uint16_t *stp = steps + (size_t)k * WH;
-            int pix[2];
             float Zf[2];
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
@@ -648,6 +727,17 @@ __device__ __forceinline__ void count_brick(const LevelParams &p, const VoxConst
                     }
             }
         }
+        if (INTERVAL && r.anc) {  // the sample on this yaw's owner ray
+            bool obs[2] = {false, false};
+#pragma unroll 1
+            for (int h = 0; h < 2; ++h) {
+                bool o = false;
+                if (h ? c[1] : c[0]) o = iv_observed(p, anc, r.anc, nd, p.body[h ? pix[1] : pix[0]], row[0], row[1], x, y, z0 + 2 * h);
+                obs[0] = h ? obs[0] : o;
+                obs[1] = h ? o : obs[1];
+            }
+            O = (uint64_t)__ballot_sync(0xffffffffu, obs[0]) | ((uint64_t)__ballot_sync(0xffffffffu, obs[1]) << 32);
+        }
         const unsigned m0 = __ballot_sync(0xffffffffu, c[0]), m1 = __ballot_sync(0xffffffffu, c[1]);
         if (lane == (j & 31)) {
             const int a = __popc(m0) + __popc(m1), m = __popc(m0 & ~(unsigned)O) + __popc(m1 & ~(unsigned)(O >> 32));
@@ -682,7 +772,7 @@ __device__ __forceinline__ void add_stats(const LevelParams &p, const NodeCnt &s
     }
 }
 
-template <bool STATS>
+template <bool STATS, bool INTERVAL>
 __global__ void __launch_bounds__(kWarpsN * 32, 3) node_kernel(const LevelParams p, int num_sms) {
     extern __shared__ __align__(16) unsigned char s_dyn[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -749,7 +839,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, 3) node_kernel(const LevelParams
         if (todo && n != cur) {
             if (cur >= 0) flush_counts<STATS>(p, cur, cur_kb, lane, c_abs, c_mrg, st);
             cur = n;
-            na = node_ancestors(p, n, anc, WH, pyr.n, lane);
+            na = node_ancestors<INTERVAL>(p, n, anc, WH, pyr.n, lane);
         }
         const uint32_t *hz = p.hz + (size_t)ln * K * pyr.n;
 #pragma unroll 1
@@ -840,11 +930,15 @@ __global__ void __launch_bounds__(kWarpsN * 32, 3) node_kernel(const LevelParams
                         const NodeAnc A = anc[ab + lane];
                         const float ox = q16f(((4 * X + 8) << 16) - A.px), oy = q16f(((4 * Y + 8) << 16) - A.py),
                                     oz = q16f(((4 * Z + 4) << 16) - A.pz);
-                        const BoxView b = box_view<false>(s_y[A.yaw], ox, oy, oz, 7.5f, 7.5f, 3.5f, W, H);
-                        rel = b.in >= 0;
-                        if (rel && box_lookup(b)) {
-                            const uint2 D = depth_box(A.pyr, pyr, b);
-                            rel = b.zlo * (65536.0f * (1.0f - 1e-6f)) <= (float)D.y + 1.5f;
+                        if (INTERVAL) {
+                            rel = !iv_box_out(s_y[A.yaw], A, nd, ox, oy, oz, 8.0f, 8.0f, 4.0f, vc.fW, vc.fH, vc.Tv);
+                        } else {
+                            const BoxView b = box_view<false>(s_y[A.yaw], ox, oy, oz, 7.5f, 7.5f, 3.5f, W, H);
+                            rel = b.in >= 0;
+                            if (rel && box_lookup(b)) {
+                                const uint2 D = depth_box(A.pyr, pyr, b);
+                                rel = b.zlo * (65536.0f * (1.0f - 1e-6f)) <= (float)D.y + 1.5f;
+                            }
                         }
                     }
 #pragma unroll 1
@@ -854,15 +948,20 @@ __global__ void __launch_bounds__(kWarpsN * 32, 3) node_kernel(const LevelParams
                             const NodeAnc A = anc[a];
                             const float ox = q16f(((4 * bx + 2) << 16) - A.px), oy = q16f(((4 * by + 2) << 16) - A.py),
                                         oz = q16f(((4 * bz + 2) << 16) - A.pz);
-                            const BoxView b = box_view<true>(s_y[A.yaw], ox, oy, oz, 1.5f, 1.5f, 1.5f, W, H);
-                            bool vox = b.in >= 0;
-                            if (vox && box_lookup(b)) {
-                                const uint2 D = depth_box(A.pyr, pyr, b);
-                                if (b.zlo * (65536.0f * (1.0f - 1e-6f)) > (float)D.y + 1.5f) {
-                                    vox = false;
-                                } else if (b.in > 0 && b.zhi * (65536.0f * (1.0f + 1e-6f)) < (float)D.x) {
-                                    O = U;
-                                    vox = false;
+                            bool vox;
+                            if (INTERVAL) {
+                                vox = !iv_box_out(s_y[A.yaw], A, nd, ox, oy, oz, 2.0f, 2.0f, 2.0f, vc.fW, vc.fH, vc.Tv);
+                            } else {
+                                const BoxView b = box_view<true>(s_y[A.yaw], ox, oy, oz, 1.5f, 1.5f, 1.5f, W, H);
+                                vox = b.in >= 0;
+                                if (vox && box_lookup(b)) {
+                                    const uint2 D = depth_box(A.pyr, pyr, b);
+                                    if (b.zlo * (65536.0f * (1.0f - 1e-6f)) > (float)D.y + 1.5f) {
+                                        vox = false;
+                                    } else if (b.in > 0 && b.zhi * (65536.0f * (1.0f + 1e-6f)) < (float)D.x) {
+                                        O = U;
+                                        vox = false;
+                                    }
                                 }
                             }
                             if (vox) left |= 1ull << a;
@@ -904,7 +1003,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, 3) node_kernel(const LevelParams
                         const int s = __ffs(full) - 1;
                         BrickRec q{shfl64(r.U, s), shfl64(r.O, s), shfl64(r.anc, s), shfl64(r.all, s), shfl64(r.part, s),
                                    shfl64(r.rch, s), shfl64(r.vis, s), __shfl_sync(0xffffffffu, r.brick, s), r.node};
-                        count_brick<STATS>(p, vc, s_y, anc, nd, p.steps + (size_t)ln * K * WH, q, lane, c_abs, c_mrg, st);
+                        count_brick<STATS, INTERVAL>(p, vc, s_y, anc, nd, p.steps + (size_t)ln * K * WH, q, lane, c_abs, c_mrg, st);
                     }
                 }
             }
@@ -915,7 +1014,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, 3) node_kernel(const LevelParams
 }
 
 // The queue's records, one warp each, in slices of consecutive records (mostly of one node).
-template <bool STATS>
+template <bool STATS, bool INTERVAL>
 __global__ void __launch_bounds__(kWarpsN * 32, 4) brick_kernel(const LevelParams p) {
     extern __shared__ __align__(16) unsigned char s_dyn[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -952,9 +1051,9 @@ __global__ void __launch_bounds__(kWarpsN * 32, 4) brick_kernel(const LevelParam
                 cur = r.node;
                 n = p.level_nodes[l0 + nb0 + (int)(cur & ((1u << kRecNodeBits) - 1))];
                 nd = p.node[n];
-                node_ancestors(p, n, anc, WH, pyr_n, lane);
+                node_ancestors<INTERVAL>(p, n, anc, WH, pyr_n, lane);
             }
-            count_brick<STATS>(p, vc, s_y, anc, nd, p.steps + (size_t)(cur & ((1u << kRecNodeBits) - 1)) * K * WH, r, lane, c_abs,
+            count_brick<STATS, INTERVAL>(p, vc, s_y, anc, nd, p.steps + (size_t)(cur & ((1u << kRecNodeBits) - 1)) * K * WH, r, lane, c_abs,
                                c_mrg, st);
         }
     }
@@ -1075,12 +1174,14 @@ void launch_render(const LevelParams &p, int nodes, int num_sms, cudaStream_t s)
 int node_ctas_per_sm() {
     // the most yaws and the deepest tree: 112 KB
     const int smem = (int)node_dyn_smem(MIG_MAX_YAW_BINS, MIG_MAX_DEPTH);
-    cudaFuncSetAttribute(node_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    cudaFuncSetAttribute(node_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    cudaFuncSetAttribute(brick_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    cudaFuncSetAttribute(brick_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaFuncSetAttribute(node_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaFuncSetAttribute(node_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaFuncSetAttribute(node_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaFuncSetAttribute(brick_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaFuncSetAttribute(brick_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaFuncSetAttribute(brick_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     int a = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, node_kernel<false>, kWarpsN * 32, node_dyn_smem(36, 16));
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, node_kernel<false, false>, kWarpsN * 32, node_dyn_smem(36, 16));
     cudaGetLastError();
     return std::max(1, a);
 }
@@ -1093,12 +1194,15 @@ void launch_node_chunk(const LevelParams &c, int num_sms, int node_ctas, cudaStr
     const int g = (int)std::max<long long>(1, std::min<long long>((items + kWarpsN - 1) / kWarpsN, (long long)num_sms * node_ctas));
     const size_t smem = node_dyn_smem(c.K, c.max_anc);
     const int gb = num_sms * 4;
-    if (c.stats) {
-        node_kernel<true><<<g, kWarpsN * 32, smem, s>>>(c, num_sms);
-        brick_kernel<true><<<gb, kWarpsN * 32, smem, s>>>(c);
+    if (c.mode == MIG_MODE_INTERVAL) {
+        node_kernel<false, true><<<g, kWarpsN * 32, smem, s>>>(c, num_sms);
+        brick_kernel<false, true><<<gb, kWarpsN * 32, smem, s>>>(c);
+    } else if (c.stats) {
+        node_kernel<true, false><<<g, kWarpsN * 32, smem, s>>>(c, num_sms);
+        brick_kernel<true, false><<<gb, kWarpsN * 32, smem, s>>>(c);
     } else {
-        node_kernel<false><<<g, kWarpsN * 32, smem, s>>>(c, num_sms);
-        brick_kernel<false><<<gb, kWarpsN * 32, smem, s>>>(c);
+        node_kernel<false, false><<<g, kWarpsN * 32, smem, s>>>(c, num_sms);
+        brick_kernel<false, false><<<gb, kWarpsN * 32, smem, s>>>(c);
     }
 }
 
@@ -1110,6 +1214,7 @@ static long long node_bricks(int64_t Tq) {
     return (long long)(4.19 * r * r * r) + 1;
 }
 constexpr double kQueueShare = 0.3;
+constexpr double kQueueShareInterval = 0.7;  // there every counted brick that an ancestor looks at
 constexpr long long kQueueMax = 8ll << 20;  // records (512 MB)
 
 // The offsets of a region of L.cap pairs and L.queue_cap records.
@@ -1121,11 +1226,11 @@ static void place(StepsLayout &L, const SensorDims &d) {
     L.bytes = L.o_queue + (size_t)L.queue_cap * sizeof(BrickRec);
 }
 
-StepsLayout steps_layout(const SensorDims &d, int max_nodes, size_t budget_bytes, bool node_pass) {
+StepsLayout steps_layout(const SensorDims &d, int max_nodes, size_t budget_bytes, bool node_pass, bool interval) {
     StepsLayout L{};
     const long long pairs = (long long)std::max(1, max_nodes) * d.K;
     L.cap = (int)steps_pairs(pairs, d.W, d.H, budget_bytes);
-    const long long per_node = (long long)(kQueueShare * (double)node_bricks(d.Tq)) + 1;
+    const long long per_node = (long long)((interval ? kQueueShareInterval : kQueueShare) * (double)node_bricks(d.Tq)) + 1;
     if (node_pass && L.cap >= d.K) {  // whole nodes, as many as the queue has room for
         const long long nodes = std::max<long long>(1, std::min<long long>(L.cap / d.K, kQueueMax / per_node));
         L.cap = (int)nodes * d.K;

@@ -26,7 +26,7 @@ struct StepsLayout {
     int queue_cap;  // records
     size_t o_ctr, o_hz, o_queue, bytes;
 };
-StepsLayout steps_layout(const SensorDims &d, int max_nodes, size_t budget_bytes, bool node_pass);
+StepsLayout steps_layout(const SensorDims &d, int max_nodes, size_t budget_bytes, bool node_pass, bool interval);
 // The same for whole nodes within a region of at most `bytes` bytes (cap 0: not one node fits).
 StepsLayout steps_layout_in(const SensorDims &d, int max_nodes, size_t bytes);
 void set_steps(LevelParams &p, void *base, const StepsLayout &L);  // the region's fields
