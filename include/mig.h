@@ -317,17 +317,19 @@ typedef struct mig_kernel_times {
     double cast_ms, voxel_ms;
     uint64_t cast_launches, voxel_launches;
 } mig_kernel_times;
-/* Count kernels of the sample modes (marginal, single parent, absolute; no counterpart in the
- * paper; all give identical results). Owned-voxel counting casts each pixel ray once to its first
- * occupied voxel, then tests every unknown voxel of the frustum against the ray of the pixel that
- * owns it (its centre's projection): MIG_COUNT_PAIRS enumerates each (node, yaw) frustum,
- * MIG_COUNT_NODES each node's voxels once for all yaws, whole 4x4x4 bricks at a time (its ancestor
- * test runs once per voxel), MIG_COUNT_AUTO (the default) takes the per-node pass. Either falls back to
- * the pairs when the buffer below does not hold all yaws of one node. MIG_COUNT_RAYS walks every ray through every voxel it crosses and
- * owner-tests the unknown ones. The owned-voxel kernels keep one uint16 step count per (node, yaw,
- * pixel) of a level in a buffer of at most steps_budget_bytes (0 = the default, 1 GiB); a level
- * that does not fit is counted in chunks. The per-node pass keeps a queue of undecided bricks beside it
- * (at most 512 MiB). Errors: MIG_EINVAL (ctx NULL, unknown kernel). */
+/* Count kernels (no counterpart in the paper; all give identical results). Owned-voxel counting casts
+ * each pixel ray once to its first occupied voxel, then tests every unknown voxel of the frustum
+ * against the ray of the pixel that owns it (its centre's projection): MIG_COUNT_PAIRS enumerates each
+ * (node, yaw) frustum, MIG_COUNT_NODES each node's voxels once for all yaws, whole 4x4x4 bricks at a
+ * time (its ancestor test runs once per voxel), MIG_COUNT_AUTO (the default) takes the per-node pass.
+ * In the marginal, single-parent and absolute modes either falls back to the pairs when the buffer
+ * below does not hold all yaws of one node. The interval and panoramic modes have no pass per pair:
+ * there, and with MIG_COUNT_PAIRS, they count like MIG_COUNT_RAYS, which walks every ray through every
+ * voxel it crosses and owner-tests the unknown ones. The owned-voxel kernels keep one uint16 step count
+ * per (node, yaw, pixel) of a level (panoramic mode: per node, column and row) in a buffer of at most
+ * steps_budget_bytes (0 = the default, 1 GiB); a level that does not fit is counted in chunks. The
+ * per-node pass keeps a queue of undecided bricks beside it (at most 512 MiB). Errors: MIG_EINVAL (ctx
+ * NULL, unknown kernel). */
 #define MIG_COUNT_AUTO 0
 #define MIG_COUNT_RAYS 1
 #define MIG_COUNT_PAIRS 2

@@ -161,6 +161,18 @@ void set_pano_params(LevelParams &p, const Camera *cam, int32_t *pcnt) {
     p.pano_dir = (const int4 *)cam->d_pano_dir;
     p.pano_row = (const int4 *)cam->d_pano_row;
     p.pano_cnt = pcnt;
+    set_pano_visit(p, cam->pano_A, cam->s.vfov_deg);
+}
+
+// f(the parameters of each chunk of `cap` of a level's `total` (node, yaw) pairs or nodes)
+template <class F>
+static void for_chunks(const LevelParams &p, long long total, int cap, F f) {
+    for (long long q0 = 0; q0 < total; q0 += cap) {
+        LevelParams c = p;
+        c.q0 = (int)q0;
+        c.q1 = (int)std::min<long long>(total, q0 + cap);
+        f(c);
+    }
 }
 
 void launch_level_count(const mig_ctx *ctx, const LevelParams &p, int Ld, int count_cap, cudaStream_t s) {
@@ -169,8 +181,13 @@ void launch_level_count(const mig_ctx *ctx, const LevelParams &p, int Ld, int co
         launch_count_interval(p, std::max(1, std::min((items + 7) / 8, ctx->num_sms * ctx->interval_ctas)), s);
     } else if (p.mode == MIG_MODE_PANORAMIC) {
         const int pitems = Ld * p.pano_A;
-        launch_pano_count(p, std::max(1, std::min((pitems + 7) / 8, ctx->num_sms * ctx->pano_ctas)), s);
-        launch_pano_window(p, std::max(1, std::min((Ld * p.K + 255) / 256, 1024)), s);
+        if (!p.steps) launch_pano_count(p, std::max(1, std::min((pitems + 7) / 8, ctx->num_sms * ctx->pano_ctas)), s);
+        else
+            for_chunks(p, Ld, p.steps_cap, [&](const LevelParams &c) {
+                launch_pano_cast_chunk(c, ctx->num_sms, s);
+                launch_pano_voxel_chunk(c, ctx->num_sms, s);
+            });
+        launch_pano_window(p, std::max(1, std::min((Ld * p.K + 7) / 8, ctx->num_sms * 8)), s);
     } else if (p.steps) {
         launch_vox_level(p, (long long)Ld * p.K, ctx->num_sms, ctx->vox_ctas, ctx->node_ctas, s);
     } else {
@@ -179,22 +196,25 @@ void launch_level_count(const mig_ctx *ctx, const LevelParams &p, int Ld, int co
 }
 
 void launch_level_count_timed(mig_ctx *ctx, const LevelParams &p, int Ld, int count_cap) {
-    if (!p.steps || p.mode == MIG_MODE_PANORAMIC) {
+    if (!p.steps) {
         timed_launch(ctx, kProfCount, [&] { launch_level_count(ctx, p, Ld, count_cap, ctx->stream); });
         return;
     }
-    const long long pairs = (long long)Ld * p.K;
-    const int cap = vox_chunk_pairs(p);
-    for (long long q0 = 0; q0 < pairs; q0 += cap) {
-        LevelParams c = p;
-        c.q0 = (int)q0;
-        c.q1 = (int)std::min<long long>(pairs, q0 + cap);
+    if (p.mode == MIG_MODE_PANORAMIC) {
+        for_chunks(p, Ld, p.steps_cap, [&](const LevelParams &c) {
+            timed_launch(ctx, kProfCast, [&] { launch_pano_cast_chunk(c, ctx->num_sms, ctx->stream); });
+            timed_launch(ctx, kProfVoxel, [&] { launch_pano_voxel_chunk(c, ctx->num_sms, ctx->stream); });
+        });
+        timed_launch(ctx, kProfVoxel, [&] { launch_pano_window(p, std::max(1, std::min((Ld * p.K + 7) / 8, ctx->num_sms * 8)), ctx->stream); });
+        return;
+    }
+    for_chunks(p, (long long)Ld * p.K, vox_chunk_pairs(p), [&](const LevelParams &c) {
         timed_launch(ctx, kProfCast, [&] { launch_cast_chunk(c, ctx->num_sms, ctx->stream); });
         timed_launch(ctx, kProfVoxel, [&] {
             if (node_pass(c)) launch_node_chunk(c, ctx->num_sms, ctx->node_ctas, ctx->stream);
             else launch_voxel_chunk(c, ctx->num_sms, ctx->vox_ctas, ctx->stream);
         });
-    }
+    });
 }
 
 // Steps of a tree whose levels' sizes only the device knows: every level may end in a partial chunk.
@@ -223,12 +243,18 @@ void launch_device_levels(mig_ctx *ctx, LevelParams p, int n, int levels, int2 *
 }
 
 StepsLayout steps_for(const mig_ctx *ctx, int Lmax, const mig_sensor &s, float voxel, int mode) {
-    if (ctx->ray_count || mode == MIG_MODE_PANORAMIC || (mode == MIG_MODE_INTERVAL && ctx->voxel_pass == MIG_COUNT_PAIRS))
-        return StepsLayout{};
-    const StepsLayout L = steps_layout(SensorDims{s.width, s.height, s.yaw_bins, range_q16(s.range_m, voxel)}, Lmax, ctx->steps_budget,
-                                       ctx->voxel_pass != MIG_COUNT_PAIRS, mode == MIG_MODE_INTERVAL);
-    // the interval mode has no pass per (node, yaw) pair: without room for whole nodes it counts ray by ray
-    return mode == MIG_MODE_INTERVAL && L.queue_cap == 0 ? StepsLayout{} : L;
+    const bool pano = mode == MIG_MODE_PANORAMIC, whole = pano || mode == MIG_MODE_INTERVAL;
+    // the interval and panoramic modes have no pass per (node, yaw) pair: without room for whole nodes they
+    // count ray by ray
+    if (ctx->ray_count || (whole && ctx->voxel_pass == MIG_COUNT_PAIRS)) return StepsLayout{};
+    SensorDims d{s.width, s.height, s.yaw_bins, range_q16(s.range_m, voxel)};
+    if (pano) {
+        d.W = pano_columns(s);
+        d.K = 1;
+        if ((size_t)d.W * d.H * sizeof(uint16_t) > ctx->steps_budget) return StepsLayout{};
+    }
+    const StepsLayout L = steps_layout(d, Lmax, ctx->steps_budget, ctx->voxel_pass != MIG_COUNT_PAIRS, mode);
+    return whole && L.queue_cap == 0 ? StepsLayout{} : L;
 }
 
 void prof_begin(mig_ctx *ctx, int kind, cudaEvent_t *a) {
@@ -348,6 +374,7 @@ mig_status mig_ctx_create(int device, void *stream, const mig_allocator *allocat
     ctx->count_ctas = count_ctas_per_sm();
     ctx->interval_ctas = count_interval_ctas_per_sm();
     ctx->pano_ctas = pano_ctas_per_sm();
+    pano_bricks_init();
     ctx->vox_ctas = vox_ctas_per_sm();
     ctx->node_ctas = node_ctas_per_sm();
     ctx->steps_budget = kStepsBudget;

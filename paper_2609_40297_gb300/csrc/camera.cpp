@@ -125,12 +125,15 @@ mig_status camera_build(const mig_sensor &s, Camera &c) {
 // column is no wider than a pinhole pixel at the image centre; yaw k's window is the
 // Wc = round(A hfov / 360) columns centred on its azimuth. Column c is a one-pixel-wide strip
 // camera looking along the wedge's centre azimuth with the pinhole's rows.
+int pano_columns(const mig_sensor &s) {
+    const double step = std::ceil(((double)s.width * 360.0) / ((double)s.hfov_deg * (double)s.yaw_bins));
+    return (int)std::min(std::max(step, 1.0) * s.yaw_bins, 2147483647.0);
+}
+
 mig_status pano_build(Camera &c) {
     const mig_sensor &s = c.s;
     if (s.pitch_deg != 0.0f) return fail(MIG_EINVAL, "panoramic mode: the camera must be level (pitch 0)");
-    int step = (int)std::ceil(((double)s.width * 360.0) / ((double)s.hfov_deg * (double)s.yaw_bins));
-    if (step < 1) step = 1;
-    const int A = step * s.yaw_bins, H = s.height;
+    const int A = pano_columns(s), step = A / s.yaw_bins, H = s.height;
     if (A > MIG_MAX_PANO_COLUMNS) return fail(MIG_EINVAL, "panoramic mode: too many azimuth columns");
     int Wc = (int)std::llrint(((double)A * (double)s.hfov_deg) / 360.0);
     if (Wc < 1) Wc = 1;

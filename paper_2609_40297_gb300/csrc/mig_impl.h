@@ -73,6 +73,7 @@ struct Camera {
     int32_t *d_pano_bc = nullptr, *d_pano_dir = nullptr, *d_pano_row = nullptr;
 };
 mig_status camera_build(const mig_sensor &s, Camera &out);
+int pano_columns(const mig_sensor &s);  // A
 mig_status pano_build(Camera &c);  // fills the pano_* host tables (MIG_EINVAL unless pitch is 0)
 mig_status sensor_check(const mig_sensor &s, float voxel);
 int64_t range_q16(float range_m, float voxel);

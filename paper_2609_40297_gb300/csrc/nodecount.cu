@@ -25,6 +25,7 @@
 #include "interval.cuh"
 #include "kernels.h"
 #include "mig.h"
+#include "nodecount.cuh"
 #include "voxcount.h"
 
 namespace mig {
@@ -32,255 +33,6 @@ namespace mig {
 namespace {
 
 using namespace dev;
-
-constexpr int kWarpsN = 8;  // warps per CTA of the kernels below
-
-__device__ __forceinline__ const uint64_t *grid_umask(const GridView &g) {
-    return reinterpret_cast<const uint64_t *>(g.g + umask_offset(g.nx, g.ny, g.nz));
-}
-__device__ __forceinline__ const uint64_t *grid_omask(const GridView &g) {
-    return reinterpret_cast<const uint64_t *>(g.g + omask_offset(g.nx, g.ny, g.nz));
-}
-
-__device__ __forceinline__ float q16f(int v) { return (float)v * (1.0f / 65536.0f); }
-
-// ------------------------------------------------------------------------- cast and render kernels
-// The rays of an image are cast 8x4 pixels at a time, one ray per lane. Before that, lanes follow one
-// such part each as a beam (beam_free): the part's rays start where the beam stopped, and are not
-// cast at all if it met nothing within the range (60 % of the parts on the large workload, 16 % at
-// paper scale). Three layouts, by the number of tiles of the level:
-//   large - one warp per 32x32 pixel tile, its 32 parts' beams on its 32 lanes;
-//   mid   - one CTA per 32x32 tile, the beams on its first warp, for levels of fewer tiles than keep every
-//           warp busy with several;
-//   small - one CTA per 16x16 tile, one part per warp, no beams and no 32x32 bounds, for levels that do
-//           not fill the GPU: their time is one warp's chain of dependent steps.
-// The level's size is only known on the device (tree_eval_device), so the kernels choose.
-constexpr int kCastCtas = 4;  // resident CTAs per SM (64 registers; 3 CTAs of 80 are 2 % slower)
-enum CastLayout { kCastSmall, kCastMid, kCastLarge };
-__device__ __forceinline__ CastLayout cast_layout(long long images, int W, int H, int num_sms) {
-    const long long tiles = images * ((W + 31) >> 5) * ((H + 31) >> 5), warps = (long long)num_sms * kCastCtas * kWarpsN;
-    return tiles >= 6 * warps ? kCastLarge : (2 * tiles >= warps ? kCastMid : kCastSmall);
-}
-
-// The beam of the 8x4 part at pixel (i0, j0).
-__device__ __forceinline__ float tile_beam(const LevelParams &p, const uint8_t *dist, const int4 nd, int ck, int sk, int i0, int j0) {
-    if (i0 >= p.W || j0 >= p.H) return 0.0f;
-    const int i1 = min(i0 + 7, p.W - 1), j1 = min(j0 + 3, p.H - 1);
-    const float q30 = 9.31322574615478515625e-10f, c = (float)ck * q30, s = (float)sk * q30;
-    float lo[3] = {1e30f, 1e30f, 1e30f}, hi[3] = {-1e30f, -1e30f, -1e30f};
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-        const int4 b = p.body[(t & 2 ? j1 : j0) * p.W + (t & 1 ? i1 : i0)];
-        const float z = __fdividef(1.0f, (float)b.w), x = (float)b.x * z, y = (float)b.y * z;
-        const float w[3] = {fmaf(c, x, -(s * y)), fmaf(s, x, c * y), (float)b.z * z};
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            lo[a] = fminf(lo[a], w[a]);
-            hi[a] = fmaxf(hi[a], w[a]);
-        }
-    }
-    // the largest camera depth of a unit ray: the part's pixel nearest the image centre on each axis
-    const float a0 = ((float)i0 + 0.5f - 0.5f * (float)p.W) * p.ifx, a1 = ((float)i1 + 0.5f - 0.5f * (float)p.W) * p.ifx;
-    const float b0 = ((float)j0 + 0.5f - 0.5f * (float)p.H) * p.ify, b1 = ((float)j1 + 0.5f - 0.5f * (float)p.H) * p.ify;
-    const float am = a0 * a1 <= 0.0f ? 0.0f : fminf(fabsf(a0), fabsf(a1)), bm = b0 * b1 <= 0.0f ? 0.0f : fminf(fabsf(b0), fabsf(b1));
-    const float s_end = q16f((int)p.Tq) * rsqrtf(1.0f + am * am + bm * bm) * 1.00001f;
-    return beam_free(dist, p.grid.nx, p.grid.ny, p.grid.nz, nd.x, nd.y, nd.z, lo, hi, s_end);
-}
-// The time before which a ray of camera depth cz (Q30, per unit length) of a beam free to depth s
-// meets no occupied voxel.
-__device__ __forceinline__ float beam_time(float s, int cz) {
-    return s > 0.0f ? fmaxf(0.0f, __fdividef(s * 1073741824.0f, (float)cz) * (1.0f - 1e-6f) - kCastEps) : 0.0f;
-}
-
-struct CastCnt {  // statistics
-    uint32_t rays = 0, fine = 0, jump = 0;
-};
-
-// What a pass keeps per ray and per tile: the cast the step index (16 bits, bounds packed as min |
-// ~max << 16), the render the depth.
-struct CastOut {
-    uint16_t *out;
-    uint32_t *hz;
-    static constexpr bool kDepth = false;
-    static constexpr uint32_t kMin = 0xFFFFu;
-    __device__ __forceinline__ uint32_t put(const LevelParams &, size_t i, int, uint32_t m, uint32_t, uint32_t) const {
-        out[i] = (uint16_t)m;
-        return m;
-    }
-    __device__ __forceinline__ void tile(size_t i, uint32_t lo, uint32_t hi) const { hz[i] = lo | ((hi ^ 0xFFFFu) << 16); }
-};
-struct RenderOut {
-    uint2 *pyr;  // NULL: not kept
-    int slot;
-    static constexpr bool kDepth = true;
-    static constexpr uint32_t kMin = 0xFFFFFFFFu;
-    __device__ __forceinline__ uint32_t put(const LevelParams &p, size_t i, int dzc, uint32_t m, uint32_t ne, uint32_t ade) const {
-        const uint32_t D = hit_depth(m != kNoHit, ne, ade, dzc, p.Tq);
-        arena_store(p.arena, p.arena_slots, slot, i, (size_t)p.W * p.H, D, p.bounds_err);
-        return D;
-    }
-    __device__ __forceinline__ void tile(size_t i, uint32_t lo, uint32_t hi) const {
-        if (pyr) pyr[i] = make_uint2(lo, hi);
-    }
-};
-
-// One ray, out of line: the layouts' loops keep their state in other registers than the walk's.
-struct RayHit {
-    uint32_t m, ne, ade;
-};
-template <bool STATS, bool DEPTH>
-__device__ __noinline__ RayHit cast_ray(const uint64_t *om, const uint8_t *oct, int gnx, int gny, int gnz, int Px, int Py, int Pz,
-                                       int dx, int dy, int dz, int Tq, float t0, CastCnt *st) {
-    RayHit h{0, 0, 1};
-    uint32_t fine = 0, jump = 0;
-    h.m = cast_bricks<DEPTH, STATS>(om, oct, gnx, gny, gnz, Px, Py, Pz, dx, dy, dz, Tq, t0, h.ne, h.ade, fine, jump);
-    if constexpr (STATS) {
-        st->fine += fine;
-        st->jump += jump;
-    }
-    return h;
-}
-
-// Casts the 8x4 part at pixel (i0, j0), lane l the pixel (l & 7, l >> 3); lo, hi gather its bounds.
-template <bool STATS, class OUT>
-__device__ __forceinline__ void cast_part(const LevelParams &p, const uint64_t *om, const uint8_t *dist, const int4 nd, int ck, int sk,
-                                          int i0, int j0, float beam, const OUT &o, int lane, uint32_t &lo, uint32_t &hi,
-                                          CastCnt &st) {
-    const int i = i0 + (lane & 7), j = j0 + (lane >> 3);
-    if (i >= p.W || j >= p.H) return;
-    const size_t at = (size_t)j * p.W + i;
-    RayHit hit{kNoHit, 0, 1};
-    int dzc = 0;
-    if (OUT::kDepth || beam < 1e29f) {
-        const int4 b = p.body[at];
-        dzc = b.w;
-        if (beam < 1e29f) {
-            int dx, dy, dz;
-            ray_dir(b, ck, sk, dx, dy, dz);
-            const uint8_t *oct = p.grid.g + oct_offset(p.grid.nx, p.grid.ny, p.grid.nz, octant_of(dx, dy, dz));
-            hit = cast_ray<STATS, OUT::kDepth>(om, oct, p.grid.nx, p.grid.ny, p.grid.nz, nd.x, nd.y, nd.z, dx, dy, dz, (int)p.Tq,
-                                               beam_time(beam, b.w), &st);
-        }
-    }
-    const uint32_t v = o.put(p, at, dzc, hit.m, hit.ne, hit.ade);
-    lo = min(lo, v);
-    hi = max(hi, v);
-    if constexpr (STATS) ++st.rays;
-}
-
-// The pixel of part t (0..7) of the 16x16 quadrant at (x0, y0): half t & 1 of 8x8 tile t >> 1.
-__device__ __forceinline__ int2 part_at(int x0, int y0, int t) {
-    return make_int2(x0 + ((t >> 1) & 1) * 8, y0 + (t >> 2) * 8 + (t & 1) * 4);
-}
-
-// One 16x16 quadrant by one warp, part t's beam in lane base + t of s; returns its bounds.
-template <bool STATS, class OUT>
-__device__ __forceinline__ uint2 cast_quad(const LevelParams &p, const uint64_t *om, const uint8_t *dist, const Pyramid &y,
-                                           const int4 nd, int ck, int sk, int x0, int y0, float s, int base, const OUT &o, int lane,
-                                           CastCnt &st) {
-    uint32_t lo = OUT::kMin, hi = 0u, lo16 = OUT::kMin, hi16 = 0u;
-#pragma unroll 1
-    for (int t = 0; t < 8; ++t) {
-        const int2 at = part_at(x0, y0, t);
-        const float beam = __shfl_sync(0xffffffffu, s, base + t);
-        cast_part<STATS>(p, om, dist, nd, ck, sk, at.x, at.y, beam, o, lane, lo, hi, st);
-        __syncwarp();
-        if (t & 1) {
-            lo = __reduce_min_sync(0xffffffffu, lo);
-            hi = __reduce_max_sync(0xffffffffu, hi);
-            if (lane == 0 && at.x < p.W && at.y - 4 < p.H) o.tile((size_t)(at.y >> 3) * y.w0 + (at.x >> 3), lo, hi);
-            lo16 = min(lo16, lo);
-            hi16 = max(hi16, hi);
-            lo = OUT::kMin;
-            hi = 0u;
-        }
-    }
-    if (lane == 0 && x0 < p.W && y0 < p.H) o.tile(y.o1 + (size_t)(y0 >> 4) * y.w1 + (x0 >> 4), lo16, hi16);
-    return make_uint2(lo16, hi16);
-}
-
-// One 32x32 tile at pixel (x0, y0) by one warp.
-template <bool STATS, class OUT>
-__device__ __forceinline__ void cast_large(const LevelParams &p, const uint64_t *om, const uint8_t *dist, const Pyramid &y,
-                                           const int4 nd, int ck, int sk, int x0, int y0, const OUT &o, int lane, CastCnt &st) {
-    const int2 at = part_at(x0 + ((lane >> 3) & 1) * 16, y0 + (lane >> 4) * 16, lane & 7);
-    const float s = tile_beam(p, dist, nd, ck, sk, at.x, at.y);
-    uint2 b = make_uint2(OUT::kMin, 0u);
-#pragma unroll 1
-    for (int q = 0; q < 4; ++q) {
-        const uint2 v = cast_quad<STATS>(p, om, dist, y, nd, ck, sk, x0 + (q & 1) * 16, y0 + (q >> 1) * 16, s, 8 * q, o, lane, st);
-        b = make_uint2(min(b.x, v.x), max(b.y, v.y));
-    }
-    if (lane == 0) o.tile(y.o2 + (size_t)(y0 >> 5) * y.w2 + (x0 >> 5), b.x, b.y);
-}
-
-// One 32x32 tile at pixel (x0, y0) by a CTA of 8 warps: warp w casts half of quadrant w >> 1.
-template <bool STATS, class OUT>
-__device__ __forceinline__ void cast_mid(const LevelParams &p, const uint64_t *om, const uint8_t *dist, const Pyramid &y,
-                                         const int4 nd, int ck, int sk, int x0, int y0, const OUT &o, uint2 *s_t, float *s_beam, int warp,
-                                         int lane, CastCnt &st) {
-    if (warp == 0) {
-        const int2 at = part_at(x0 + ((lane >> 3) & 1) * 16, y0 + (lane >> 4) * 16, lane & 7);
-        s_beam[lane] = tile_beam(p, dist, nd, ck, sk, at.x, at.y);
-    }
-    __syncthreads();
-    const int qx = x0 + ((warp >> 1) & 1) * 16, qy = y0 + (warp >> 2) * 16;
-    uint32_t lo = OUT::kMin, hi = 0u, lo2 = OUT::kMin, hi2 = 0u;
-#pragma unroll 1
-    for (int t = 4 * (warp & 1); t < 4 * (warp & 1) + 4; ++t) {
-        const int2 at = part_at(qx, qy, t);
-        cast_part<STATS>(p, om, dist, nd, ck, sk, at.x, at.y, s_beam[8 * (warp >> 1) + t], o, lane, lo, hi, st);
-        __syncwarp();
-        if (t & 1) {
-            lo = __reduce_min_sync(0xffffffffu, lo);
-            hi = __reduce_max_sync(0xffffffffu, hi);
-            if (lane == 0 && at.x < p.W && at.y - 4 < p.H) o.tile((size_t)(at.y >> 3) * y.w0 + (at.x >> 3), lo, hi);
-            lo2 = min(lo2, lo);
-            hi2 = max(hi2, hi);
-            lo = OUT::kMin;
-            hi = 0u;
-        }
-    }
-    if (lane == 0) s_t[warp] = make_uint2(lo2, hi2);
-    __syncthreads();
-    if (threadIdx.x < 4) {
-        const uint2 a = s_t[2 * threadIdx.x], b = s_t[2 * threadIdx.x + 1];
-        lo = min(a.x, b.x);
-        hi = max(a.y, b.y);
-        const int i0 = x0 + (threadIdx.x & 1) * 16, j0 = y0 + (threadIdx.x >> 1) * 16;
-        if (i0 < p.W && j0 < p.H) o.tile(y.o1 + (size_t)(j0 >> 4) * y.w1 + (i0 >> 4), lo, hi);
-        lo = __reduce_min_sync(0xfu, lo);
-        hi = __reduce_max_sync(0xfu, hi);
-        if (threadIdx.x == 0) o.tile(y.o2 + (size_t)(y0 >> 5) * y.w2 + (x0 >> 5), lo, hi);
-    }
-    __syncthreads();
-}
-
-// One 16x16 tile at pixel (x0, y0) by a CTA of 8 warps.
-template <bool STATS, class OUT>
-__device__ __forceinline__ void cast_small(const LevelParams &p, const uint64_t *om, const uint8_t *dist, const Pyramid &y,
-                                            const int4 nd, int ck, int sk, int x0, int y0, const OUT &o, uint2 *s_t, int warp, int lane,
-                                            CastCnt &st) {
-    uint32_t lo = OUT::kMin, hi = 0u;
-    const int2 at = part_at(x0, y0, warp);
-    cast_part<STATS>(p, om, dist, nd, ck, sk, at.x, at.y, 0.0f, o, lane, lo, hi, st);
-    __syncwarp();
-    lo = __reduce_min_sync(0xffffffffu, lo);
-    hi = __reduce_max_sync(0xffffffffu, hi);
-    if (lane == 0) s_t[warp] = make_uint2(lo, hi);
-    __syncthreads();
-    if (threadIdx.x < 4) {
-        const uint2 a = s_t[2 * threadIdx.x], b = s_t[2 * threadIdx.x + 1];
-        lo = min(a.x, b.x);
-        hi = max(a.y, b.y);
-        const int i0 = x0 + (threadIdx.x & 1) * 8, j0 = y0 + (threadIdx.x >> 1) * 8;
-        if (i0 < p.W && j0 < p.H) o.tile((size_t)(j0 >> 3) * y.w0 + (i0 >> 3), lo, hi);
-        lo = __reduce_min_sync(0xfu, lo);
-        hi = __reduce_max_sync(0xfu, hi);
-        if (threadIdx.x == 0) o.tile(y.o1 + (size_t)(y0 >> 4) * y.w1 + (x0 >> 4), lo, hi);
-    }
-    __syncthreads();
-}
 
 template <bool STATS>
 __global__ void __launch_bounds__(kWarpsN * 32, kCastCtas) cast_kernel(const LevelParams p, int num_sms) {
@@ -306,14 +58,15 @@ __global__ void __launch_bounds__(kWarpsN * 32, kCastCtas) cast_kernel(const Lev
         const int q = q0 + ql;
         const int4 nd = p.node[p.level_nodes[l0 + q / p.K]];
         const int32_t *yk = p.yawtab + (q % p.K) * 12;
+        const CameraRays rays{p, nd, yk[0], yk[1], p.W, p.H};
         const CastOut o{p.steps + (size_t)ql * WH, p.hz + (size_t)ql * y.n};
         const int x0 = tile % tx * T, y0 = tile / tx * T;
         if (lay == kCastLarge) {
-            cast_large<STATS>(p, om, dist, y, nd, yk[0], yk[1], x0, y0, o, lane, st);
+            cast_large<STATS>(p, om, dist, y, rays, x0, y0, o, lane, st);
         } else if (lay == kCastMid) {
-            cast_mid<STATS>(p, om, dist, y, nd, yk[0], yk[1], x0, y0, o, s_t, s_beam, warp, lane, st);
+            cast_mid<STATS>(p, om, dist, y, rays, x0, y0, o, s_t, s_beam, warp, lane, st);
         } else {
-            cast_small<STATS>(p, om, dist, y, nd, yk[0], yk[1], x0, y0, o, s_t, warp, lane, st);
+            cast_small<STATS>(p, om, dist, y, rays, x0, y0, o, s_t, warp, lane, st);
         }
     }
     if constexpr (STATS) {
@@ -353,14 +106,15 @@ __global__ void __launch_bounds__(kWarpsN * 32, kCastCtas) render_kernel(const L
         const int4 nd = p.node[n];
         if (nd.w < 0) continue;  // uniform over the warps of the item
         const int32_t *yk = p.yawtab + p.sel_yaw[n] * 12;
+        const CameraRays rays{p, nd, yk[0], yk[1], p.W, p.H};
         const RenderOut o{p.dpyr ? p.dpyr + (size_t)nd.w * y.n : nullptr, nd.w};
         const int x0 = tile % tx * T, y0 = tile / tx * T;
         if (lay == kCastLarge) {
-            cast_large<STATS>(p, om, dist, y, nd, yk[0], yk[1], x0, y0, o, lane, st);
+            cast_large<STATS>(p, om, dist, y, rays, x0, y0, o, lane, st);
         } else if (lay == kCastMid) {
-            cast_mid<STATS>(p, om, dist, y, nd, yk[0], yk[1], x0, y0, o, s_t, s_beam, warp, lane, st);
+            cast_mid<STATS>(p, om, dist, y, rays, x0, y0, o, s_t, s_beam, warp, lane, st);
         } else {
-            cast_small<STATS>(p, om, dist, y, nd, yk[0], yk[1], x0, y0, o, s_t, warp, lane, st);
+            cast_small<STATS>(p, om, dist, y, rays, x0, y0, o, s_t, warp, lane, st);
         }
     }
     if constexpr (STATS) {
@@ -376,171 +130,6 @@ __global__ void __launch_bounds__(kWarpsN * 32, kCastCtas) render_kernel(const L
 // one voxel of the brick's lower and upper half per lane. (As one kernel the two stages' code, 4300
 // instructions, did not fit the instruction cache, and a warp's block took 10 to 100 times as long as
 // another's: 338 ms on the large workload.)
-constexpr int kMacX = 16, kMacZ = 8;
-__host__ __device__ inline int mac_xy(int64_t Tq) { return (2 * ((int)(Tq >> 16) + 2)) / kMacX + 2; }
-__host__ __device__ inline int mac_z(int64_t Tq) { return (2 * ((int)(Tq >> 16) + 2)) / kMacZ + 2; }
-
-struct NodeAnc {
-    int px, py, pz, yaw;
-    const uint32_t *D;
-    const uint2 *pyr;
-    float U0, V0, Z0, pad;  // interval mode: the node in the ancestor's camera coordinates
-};
-
-struct NodeCnt {  // statistics
-    uint32_t cand = 0, unk = 0, visit = 0, anc = 0, reads = 0, smp = 0;
-};
-
-__device__ __forceinline__ uint64_t shfl64(uint64_t v, int src) {
-    return (uint64_t)__shfl_sync(0xffffffffu, (unsigned long long)v, src);
-}
-__device__ __forceinline__ uint64_t or64(uint64_t v) {  // over the warp
-    return (uint64_t)__reduce_or_sync(0xffffffffu, (unsigned)v) | ((uint64_t)__reduce_or_sync(0xffffffffu, (unsigned)(v >> 32)) << 32);
-}
-
-// Bounds of the step counts under a pixel box: min in the low half, ~max in the high half.
-__device__ __forceinline__ uint32_t hz_box(const uint32_t *hz, const Pyramid &y, int top, const BoxView &b) {
-    int sh, off, w;
-    pyramid_level(y, max(b.u1 - b.u0, b.v1 - b.v0), top, sh, off, w);
-    const uint32_t *t = hz + off;
-    uint32_t r = 0xFFFFFFFFu;
-#pragma unroll 1
-    for (int ty = b.v0 >> sh; ty <= (b.v1 >> sh); ++ty)
-#pragma unroll 1
-        for (int tx = b.u0 >> sh; tx <= (b.u1 >> sh); ++tx) r = __vminu2(r, __ldg(t + ty * w + tx));
-    return r;
-}
-// Bounds of the stored depths under a pixel box (the 32x32 level is not kept by every render).
-__device__ __forceinline__ uint2 depth_box(const uint2 *pyr, const Pyramid &y, const BoxView &b) {
-    int sh, off, w;
-    pyramid_level(y, max(b.u1 - b.u0, b.v1 - b.v0), 4, sh, off, w);
-    const uint2 *t = pyr + off;
-    uint2 r = make_uint2(0xFFFFFFFFu, 0u);
-#pragma unroll 1
-    for (int ty = b.v0 >> sh; ty <= (b.v1 >> sh); ++ty)
-#pragma unroll 1
-        for (int tx = b.u0 >> sh; tx <= (b.u1 >> sh); ++tx) {
-            const uint2 v = __ldg(t + ty * w + tx);
-            r.x = min(r.x, v.x);
-            r.y = max(r.y, v.y);
-        }
-    return r;
-}
-__device__ __forceinline__ bool box_lookup(const BoxView &b) {
-    return b.zlo >= 0.5f && b.u1 - b.u0 <= kPyramidSpan && b.v1 - b.v0 <= kPyramidSpan;
-}
-
-// Float pixel of a voxel centre at camera depth >= 1/2. c = 5e-7 (largest offset + 1) bounds a row
-// product's error per unit of the row's L1 norm, so eu = 2 c (norm_u + W norm_z) / Z + 1e-6 (W + 1)
-// bounds the error of u for every pixel inside the image, and of an outside one by less than its
-// distance to the image. su, sv: 2 c (norm + size norm_z).
-struct PixelErr {
-    float su, sv, bu, bv;
-};
-// 1: inside the image, pixel index pix; 0: outside; -1: undecided.
-__device__ __forceinline__ int pixel_float(const PixelErr &e, float Z, float U, float V, float fW, float fH, int &pix) {
-    const float kMagic = 12582912.0f;
-    const float zi = __fdividef(1.0f, Z);
-    const float u = fmaf(U, zi, -0.5f), v = fmaf(V, zi, -0.5f);
-    const float fu = (u + kMagic) - kMagic, fv = (v + kMagic) - kMagic;  // floors: nearest integers of u - 1/2
-    const bool sure = Z >= 0.5f && fmaf(zi, e.su, fabsf(u - fu)) <= e.bu && fmaf(zi, e.sv, fabsf(v - fv)) <= e.bv;
-    pix = __float_as_int(fmaf(fv, fW, fu) + 8388608.0f) & 0x7FFFFF;
-    if (!sure) return -1;
-    return fu >= 0.0f && fu < fW && fv >= 0.0f && fv < fH;
-}
-// The exact pixel index (Eq. 5) in integers, or -1 outside the image; Z (Q32).
-__device__ __forceinline__ int pixel_index(const int32_t *row, int rx, int ry, int rz, int W, int H, int64_t &Z) {
-    Z = (int64_t)row[8] * rx + (int64_t)row[9] * ry + (int64_t)row[10] * rz;
-    if (Z <= 0) return -1;
-    const int64_t U = (int64_t)row[2] * rx + (int64_t)row[3] * ry + (int64_t)row[4] * rz;
-    const int64_t V = (int64_t)row[5] * rx + (int64_t)row[6] * ry + (int64_t)row[7] * rz;
-    const float zi = __fdividef(1.0f, (float)Z);
-    int pu, pv;
-    if (!pixel_in(U, Z, (float)U * zi, W, pu) || !pixel_in(V, Z, (float)V * zi, H, pv)) return -1;
-    return pv * W + pu;
-}
-__device__ __noinline__ int pixel_exact(const int32_t *row, int rx, int ry, int rz, int W, int H) {
-    int64_t Z;
-    return pixel_index(row, rx, ry, rz, W, H, Z);
-}
-// The exact ancestor test (Sec. IV-B): inside the image and z <= D.
-__device__ __noinline__ bool observed_exact(const int32_t *row, int rx, int ry, int rz, int W, int H, const uint32_t *D) {
-    int64_t Z;
-    const int pix = pixel_index(row, rx, ry, rz, W, H, Z);
-    return pix >= 0 && Z < (((int64_t)__ldg(D + pix) + 1) << 16);
-}
-// The exact visit test of a voxel by its owner ray.
-__device__ __noinline__ bool visit_exact(int Px, int Py, int Pz, int bx, int by, int bz, int ck, int sk, int x, int y, int z,
-                                         int64_t Tq) {
-    int dx, dy, dz;
-    ray_dir(make_int4(bx, by, bz, 0), ck, sk, dx, dy, dz);
-    return visit_index(Px, Py, Pz, dx, dy, dz, x, y, z, Tq) >= 0;
-}
-
-// Per-launch constants of the voxel stage.
-struct VoxConst {
-    float fW, fH, bu, bv, Tv, out2, inf2, l22;
-};
-__device__ __forceinline__ VoxConst vox_const(const LevelParams &p) {
-    VoxConst c;
-    c.fW = (float)p.W;
-    c.fH = (float)p.H;
-    c.bu = 0.5f - 1.0e-6f * (c.fW + 1.0f);
-    c.bv = 0.5f - 1.0e-6f * (c.fH + 1.0f);
-    c.Tv = q16f((int)p.Tq);
-    // squared centre distances: no visit beyond out2; certain visits by the yaw's limit and by zl2
-    c.out2 = (c.Tv + 0.88f) * (c.Tv + 0.88f);
-    c.inf2 = fmaxf(c.Tv - 0.86f, 0.f) * fmaxf(c.Tv - 0.86f, 0.f);
-    c.l22 = fmaxf(c.Tv - 0.02f, 0.f) * fmaxf(c.Tv - 0.02f, 0.f);
-    return c;
-}
-
-// The ancestors of node n that the mode tests (Sec. IV-B), parent first; returns their number.
-template <bool INTERVAL>
-__device__ __forceinline__ int node_ancestors(const LevelParams &p, int n, NodeAnc *anc, size_t WH, int pyr_n, int lane) {
-    const int2 ar = p.anc_range[n];
-    int na = p.mode == MIG_MODE_ABSOLUTE ? 0 : (p.mode == MIG_MODE_SINGLE_PARENT ? min(ar.y, 1) : ar.y);
-    na = min(na, p.max_anc);
-    __syncwarp();
-    for (int t = lane; t < na; t += 32) {
-        const int a = p.anc[ar.x + t];
-        const int4 an = p.node[a];
-        NodeAnc A{an.x, an.y, an.z, p.sel_yaw[a], p.arena + (size_t)an.w * WH, p.dpyr + (size_t)an.w * pyr_n, 0.f, 0.f, 0.f, 0.f};
-        if (INTERVAL) {
-            const int32_t *m = p.yawtab + A.yaw * 12 + 2;
-            const int4 nd = p.node[n];
-            const int rx = nd.x - an.x, ry = nd.y - an.y, rz = nd.z - an.z;
-            A.U0 = seg_coord(m, rx, ry, rz);
-            A.V0 = seg_coord(m + 3, rx, ry, rz);
-            A.Z0 = seg_coord(m + 6, rx, ry, rz);
-        }
-        anc[t] = A;
-    }
-    __syncwarp();
-    return na;
-}
-
-// Interval mode: no sample in the box of half extents (hx, hy, hz) about the offset (cx, cy, cz) from
-// ancestor A's camera can fall in an observed portion of its buffer. A sample inside a portion
-// projects into the image within the float error of seg_setup and seg_param, whose screen coordinates
-// reach |U| / kZNear where the ray passes the camera plane: 6e-7 of that, plus one pixel, widens the
-// image here; its depth is at most the range.
-__device__ __forceinline__ bool iv_box_out(const YawRows &r, const NodeAnc &A, const int4 nd, float cx, float cy, float cz, float hx,
-                                           float hy, float hz, float W, float H, float Tv) {
-    const float reach = fmaxf(fmaxf(fabsf(q16f(A.px - nd.x)), fabsf(q16f(A.py - nd.y))), fabsf(q16f(A.pz - nd.z))) + Tv + 2.0f;
-    const float mu = fmaf(6.2e-4f * r.u.w, reach, 1.0f), mv = fmaf(6.2e-4f * r.v.w, reach, 1.0f);
-    const float Z = row_dot(r.z, cx, cy, cz), U = row_dot(r.u, cx, cy, cz), V = row_dot(r.v, cx, cy, cz);
-    const float eZ = row_ext(r.z.x, r.z.y, r.z.z, hx, hy, hz) + 0.05f;
-    // a half-space a Z + s m . r > 0: its value at the centre plus its largest change over the box
-    auto out = [&](float a, float s, const float4 &m, float v) {
-        return fmaf(a, Z, s * v) + row_ext(fmaf(a, r.z.x, s * m.x), fmaf(a, r.z.y, s * m.y), fmaf(a, r.z.z, s * m.z), hx, hy, hz) +
-                   kBoxErr * fmaf(fabsf(a), r.z.w, m.w) <
-               0.0f;
-    };
-    return Z + eZ < 0.0f || Z - eZ > Tv || out(mu, 1.0f, r.u, U) || out(W + mu, -1.0f, r.u, U) || out(mv, 1.0f, r.v, V) ||
-           out(H + mv, -1.0f, r.v, V);
-}
-
 // Interval mode: is the sample of voxel (x, y, z) on its owner ray (body-frame ray b, yaw cos ck, sin sk)
 // observed by one of the ancestors `left`? The ray's crossings that enter and leave the voxel are the
 // last entering and the first leaving event in the DDA's order (visit_index).
@@ -605,43 +194,7 @@ __device__ __forceinline__ void count_brick(const LevelParams &p, const VoxConst
     // error of a row product per unit of the row's norm, for every voxel of the brick
     const float verr = 5e-7f * (__uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(rinf))) + 1.0f);
     // ---- the ancestors that were not decided for the whole brick
-    for (uint64_t as = INTERVAL ? 0ull : r.anc; as; as &= as - 1) {
-        const NodeAnc A = anc[__ffsll((long long)as) - 1];
-        const float4 ru = s_y[A.yaw].u, rv = s_y[A.yaw].v, rz = s_y[A.yaw].z;
-        const int32_t *row = p.yawtab + A.yaw * 12;
-        const int ax = (x << 16) + 32768 - A.px, ay = (y << 16) + 32768 - A.py, az0 = (z0 << 16) + 32768 - A.pz;
-        const float ex = q16f(ax), ey = q16f(ay);
-        const float Zxy = fmaf(rz.x, ex, rz.y * ey), Uxy = fmaf(ru.x, ex, ru.y * ey), Vxy = fmaf(rv.x, ex, rv.y * ey);
-        const float c = verr + 5e-7f * fmaxf(fmaxf(fabsf(q16f(A.px - nd.x)), fabsf(q16f(A.py - nd.y))), fabsf(q16f(A.pz - nd.z)));
-        const PixelErr pe{2.0f * c * fmaf(vc.fW, rz.w, ru.w), 2.0f * c * fmaf(vc.fH, rz.w, rv.w), vc.bu, vc.bv};
-        const float e_z = c * rz.w;
-        const uint64_t rem = U & ~O;
-        bool obs[2] = {false, false};
-        int pix[2], in[2];
-        float Zf[2];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const float ez = q16f(az0 + (h << 17));
-            Zf[h] = fmaf(rz.z, ez, Zxy);
-            in[h] = pixel_float(pe, Zf[h], fmaf(ru.z, ez, Uxy), fmaf(rv.z, ez, Vxy), vc.fW, vc.fH, pix[h]);
-            if (!((uint32_t)(rem >> (32 * h)) >> lane & 1)) in[h] = 0;
-            if constexpr (STATS) st.anc += (uint32_t)(rem >> (32 * h)) >> lane & 1;
-        }
-        uint32_t D[2] = {0u, 0u};
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-            if (in[h] > 0) D[h] = __ldg(A.D + pix[h]);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            if constexpr (STATS) st.reads += in[h] > 0;
-            // z <= D  <=>  Z < (D + 1) / 2^16 (voxels); lim within 2^-23 of that
-            const float lim = ((float)D[h] + 1.0f) * (1.0f / 65536.0f);
-            obs[h] = in[h] > 0 && Zf[h] + e_z < lim * (1.0f - 2.4e-7f);
-            if (in[h] < 0 || (in[h] > 0 && !obs[h] && Zf[h] - e_z < lim * (1.0f + 2.4e-7f)))
-                obs[h] = observed_exact(row, ax, ay, az0 + (h << 17), W, H, A.D);
-        }
-        O |= (uint64_t)__ballot_sync(0xffffffffu, obs[0]) | ((uint64_t)__ballot_sync(0xffffffffu, obs[1]) << 32);
-    }
+    if (!INTERVAL) O = voxel_ancestors<STATS>(p, vc, s_y, anc, nd, r.anc, U, O, x, y, z0, verr, lane, st);
     // ---- yaws that count every unknown voxel (interval mode: their samples differ by yaw, see below)
     if (!INTERVAL) {
         const int cu = __popcll(U), cm = __popcll(U & ~O);
@@ -814,27 +367,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, 3) node_kernel(const LevelParams
         const int v0x = nd.x >> 16, v0y = nd.y >> 16, v0z = nd.z >> 16;
         // lane = macro block of the item: inside the grid, the ball and the elevation band?
         int mX = 0, mY = 0, mZ = 0;
-        bool live = false;
-        {
-            const int mi = g0 + lane;
-            if (lane < group && mi < mn) {
-                const int a = mi / mxy;
-                mX = ((v0x - Rv) >> 4) + (mi - a * mxy);
-                mZ = ((v0z - Rv) >> 3) + a / mxy;
-                mY = ((v0y - Rv) >> 4) + (a - (a / mxy) * mxy);
-                if (mX >= 0 && mY >= 0 && mZ >= 0 && 16 * mX < p.grid.nx && 16 * mY < p.grid.ny && 8 * mZ < p.grid.nz) {
-                    const float cx = q16f(((16 * mX + 8) << 16) - nd.x), cy = q16f(((16 * mY + 8) << 16) - nd.y),
-                                cz = q16f(((8 * mZ + 4) << 16) - nd.z);
-                    const float dx = fmaxf(fabsf(cx) - 7.5f, 0.f), dy = fmaxf(fabsf(cy) - 7.5f, 0.f),
-                                dz = fmaxf(fabsf(cz) - 3.5f, 0.f);
-                    const float rho = sqrtf(cx * cx + cy * cy), r0 = fmaxf(rho - 10.7f, 0.f), r1 = rho + 10.7f;
-                    const float eps = 0.01f * (r1 + fabsf(cz) + 4.f) + 0.05f;
-                    live = dx * dx + dy * dy + dz * dz <= R2 &&
-                           (p.band_thi >= 1e29f || cz - 3.5f <= p.band_thi * (p.band_thi > 0.f ? r1 : r0) + eps) &&
-                           (p.band_tlo <= -1e29f || cz + 3.5f >= p.band_tlo * (p.band_tlo < 0.f ? r1 : r0) - eps);
-                }
-            }
-        }
+        const bool live = lane < group && macro_block(p, nd, g0 + lane, mn, mxy, Rv, R2, mX, mY, mZ);
         unsigned todo = __ballot_sync(0xffffffffu, live);
         if (todo && n != cur) {
             if (cur >= 0) flush_counts<STATS>(p, cur, cur_kb, lane, c_abs, c_mrg, st);
@@ -923,51 +456,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, 3) node_kernel(const LevelParams
                 if (!__any_sync(0xffffffffu, want)) continue;
                 // ---- the ancestors' test (Sec. IV-B) of the bricks some yaw may count
                 uint64_t O = 0, left = 0;  // observed voxels; ancestors undecided for the brick
-#pragma unroll 1
-                for (int ab = 0; ab < na; ab += 32) {
-                    bool rel = false;  // lane = ancestor: does it look at the block, not behind its depths?
-                    if (ab + lane < na) {
-                        const NodeAnc A = anc[ab + lane];
-                        const float ox = q16f(((4 * X + 8) << 16) - A.px), oy = q16f(((4 * Y + 8) << 16) - A.py),
-                                    oz = q16f(((4 * Z + 4) << 16) - A.pz);
-                        if (INTERVAL) {
-                            rel = !iv_box_out(s_y[A.yaw], A, nd, ox, oy, oz, 8.0f, 8.0f, 4.0f, vc.fW, vc.fH, vc.Tv);
-                        } else {
-                            const BoxView b = box_view<false>(s_y[A.yaw], ox, oy, oz, 7.5f, 7.5f, 3.5f, W, H);
-                            rel = b.in >= 0;
-                            if (rel && box_lookup(b)) {
-                                const uint2 D = depth_box(A.pyr, pyr, b);
-                                rel = b.zlo * (65536.0f * (1.0f - 1e-6f)) <= (float)D.y + 1.5f;
-                            }
-                        }
-                    }
-#pragma unroll 1
-                    for (unsigned as = __ballot_sync(0xffffffffu, rel); as; as &= as - 1) {
-                        const int a = ab + __ffs(as) - 1;
-                        if (want && O != U) {
-                            const NodeAnc A = anc[a];
-                            const float ox = q16f(((4 * bx + 2) << 16) - A.px), oy = q16f(((4 * by + 2) << 16) - A.py),
-                                        oz = q16f(((4 * bz + 2) << 16) - A.pz);
-                            bool vox;
-                            if (INTERVAL) {
-                                vox = !iv_box_out(s_y[A.yaw], A, nd, ox, oy, oz, 2.0f, 2.0f, 2.0f, vc.fW, vc.fH, vc.Tv);
-                            } else {
-                                const BoxView b = box_view<true>(s_y[A.yaw], ox, oy, oz, 1.5f, 1.5f, 1.5f, W, H);
-                                vox = b.in >= 0;
-                                if (vox && box_lookup(b)) {
-                                    const uint2 D = depth_box(A.pyr, pyr, b);
-                                    if (b.zlo * (65536.0f * (1.0f - 1e-6f)) > (float)D.y + 1.5f) {
-                                        vox = false;
-                                    } else if (b.in > 0 && b.zhi * (65536.0f * (1.0f + 1e-6f)) < (float)D.x) {
-                                        O = U;
-                                        vox = false;
-                                    }
-                                }
-                            }
-                            if (vox) left |= 1ull << a;
-                        }
-                    }
-                }
+                block_ancestors<INTERVAL>(p, s_y, anc, na, nd, pyr, vc, X, Y, Z, bx, by, bz, U, want, lane, O, left);
                 if (O == U) left = 0;
                 if (kb != cur_kb) {
                     flush_counts<STATS>(p, cur, cur_kb, lane, c_abs, c_mrg, st);
@@ -1135,10 +624,6 @@ __global__ void brick_dist_kernel(uint8_t *grid, int nx, int ny, int nz, int pas
     }
 }
 
-size_t node_dyn_smem(int K, int max_anc) {
-    return (size_t)K * sizeof(YawRows) + (size_t)kWarpsN * std::max(1, max_anc) * sizeof(NodeAnc);
-}
-
 }  // namespace
 
 size_t hz_entries(int W, int H) { return (size_t)pyramid(W, H).n; }
@@ -1150,13 +635,6 @@ void set_visit_params(LevelParams &p, float hfov_deg, float vfov_deg) {
     p.vis_zl2 = l.zl2;
     p.ifx = (float)(std::tan(hfov_deg * 0.5 * (3.14159265358979323846 / 180.0)) / (p.W * 0.5));
     p.ify = (float)(std::tan(vfov_deg * 0.5 * (3.14159265358979323846 / 180.0)) / (p.H * 0.5));
-}
-
-// CTAs for a cast of `images` images (an upper bound of the level's): one per 16x16 tile, at most as
-// many as keep the kernel's loops short.
-static int cast_grid(long long images, int W, int H, int num_sms) {
-    const long long tiles = images * ((W + 15) / 16) * ((H + 15) / 16);
-    return (int)std::max<long long>(1, std::min<long long>(tiles, (long long)num_sms * 64));
 }
 
 void launch_cast_chunk(const LevelParams &c, int num_sms, cudaStream_t s) {
@@ -1215,7 +693,12 @@ static long long node_bricks(int64_t Tq) {
 }
 constexpr double kQueueShare = 0.3;
 constexpr double kQueueShareInterval = 0.7;  // there every counted brick that an ancestor looks at
+constexpr double kQueueSharePano = 0.5;      // every brick that a ray can reach
 constexpr long long kQueueMax = 8ll << 20;  // records (512 MB)
+
+static double queue_share(int mode) {
+    return mode == MIG_MODE_INTERVAL ? kQueueShareInterval : (mode == MIG_MODE_PANORAMIC ? kQueueSharePano : kQueueShare);
+}
 
 // The offsets of a region of L.cap pairs and L.queue_cap records.
 static void place(StepsLayout &L, const SensorDims &d) {
@@ -1226,11 +709,11 @@ static void place(StepsLayout &L, const SensorDims &d) {
     L.bytes = L.o_queue + (size_t)L.queue_cap * sizeof(BrickRec);
 }
 
-StepsLayout steps_layout(const SensorDims &d, int max_nodes, size_t budget_bytes, bool node_pass, bool interval) {
+StepsLayout steps_layout(const SensorDims &d, int max_nodes, size_t budget_bytes, bool node_pass, int mode) {
     StepsLayout L{};
     const long long pairs = (long long)std::max(1, max_nodes) * d.K;
     L.cap = (int)steps_pairs(pairs, d.W, d.H, budget_bytes);
-    const long long per_node = (long long)((interval ? kQueueShareInterval : kQueueShare) * (double)node_bricks(d.Tq)) + 1;
+    const long long per_node = (long long)(queue_share(mode) * (double)node_bricks(d.Tq)) + 1;
     if (node_pass && L.cap >= d.K) {  // whole nodes, as many as the queue has room for
         const long long nodes = std::max<long long>(1, std::min<long long>(L.cap / d.K, kQueueMax / per_node));
         L.cap = (int)nodes * d.K;

@@ -16,7 +16,8 @@ size_t steps_pairs(long long pairs, int W, int H, size_t budget_bytes);
 // Entries of one image's tile bounds (bricks.cuh, Pyramid).
 size_t hz_entries(int W, int H);
 // The device region of an owned-voxel count for levels of at most max_nodes nodes: the step counts of
-// `cap` pairs, the counters, the counts' tile bounds and the per-node pass's queue.
+// `cap` pairs, the counters, the counts' tile bounds and the per-node pass's queue. The panoramic mode
+// has one image of A x H per node: W = A, K = 1.
 struct SensorDims {
     int W, H, K;
     int64_t Tq;
@@ -26,7 +27,7 @@ struct StepsLayout {
     int queue_cap;  // records
     size_t o_ctr, o_hz, o_queue, bytes;
 };
-StepsLayout steps_layout(const SensorDims &d, int max_nodes, size_t budget_bytes, bool node_pass, bool interval);
+StepsLayout steps_layout(const SensorDims &d, int max_nodes, size_t budget_bytes, bool node_pass, int mode);
 // The same for whole nodes within a region of at most `bytes` bytes (cap 0: not one node fits).
 StepsLayout steps_layout_in(const SensorDims &d, int max_nodes, size_t bytes);
 void set_steps(LevelParams &p, void *base, const StepsLayout &L);  // the region's fields

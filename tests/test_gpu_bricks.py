@@ -69,6 +69,40 @@ def test_bricks_equal_rays(ctx, ci, mode):
         m.close()
 
 
+# few and many columns per brick, one row, one to 70 yaws, a node's brick around the seam
+PANO = CASES[:3] + CASES[5:] + [
+    ((30, 31, 14), 0.25, 0.05, 10, 4, Sensor(179, 60, 1, 1, 3.0, 1, 0.0)),
+    ((40, 37, 25), 0.2, 0.02, 12, 5, Sensor(20, 130, 90, 3, 5.0, 70, 0.0)),
+    ((67, 61, 30), 0.1, 0.003, 16, 6, Sensor(10, 60, 640, 40, 4.0, 16, 0.0)),
+    ((67, 61, 30), 0.1, 0.003, 30, 2, Sensor(87, 58, 100, 75, 5.0, 5, 0.0)),
+]
+
+
+@pytest.mark.parametrize("budget", [0, 1 << 18])
+@pytest.mark.parametrize("ci", range(len(PANO)))
+def test_panoramic_bricks_equal_rays(ctx, ci, budget):
+    """The panoramic mode, with the whole level and with few nodes at a time (or none: ray by ray)."""
+    (nx, ny, nz), v, occ, nodes, depth, s = PANO[ci]
+    sensor = Sensor(s.hfov_deg, s.vfov_deg, s.width, s.height, s.range_m, s.yaw_bins, 0.0)
+    p = synth.random_small(850 + ci, nx=nx, ny=ny, nz=nz, v=v, p_occ=occ, n_nodes=nodes, max_depth=depth, sensor=sensor)
+    p.tree.pos[1::2] = np.round(p.tree.pos[1::2] / v) * v  # every second node on voxel corners
+    p.tree.pos[2::4] = (np.floor(p.tree.pos[2::4] / v) + 0.5) * v  # and every fourth on a voxel centre
+    p.tree.pos = np.clip(p.tree.pos, 0, (np.array([nx, ny, nz]) - 0.5) * v).astype(np.float32)
+    m = mig.Map(ctx, p.map.grid, v, p.map.origin)
+    try:
+        rays = _eval(ctx, m, p, mig.MODE_PANORAMIC, mig.COUNT_RAYS)
+        assert rays["abs"].sum() > 0
+        ctx.set_count_kernel(mig.COUNT_AUTO, budget)
+        try:
+            got = mig.tree_eval(m, p.tree.parent, p.tree.pos, p.sensor, mode=mig.MODE_PANORAMIC, want_counts=True,
+                                want_depth=True)
+        finally:
+            ctx.set_count_kernel(mig.COUNT_AUTO, 0)
+        _same(got, rays, ci)
+    finally:
+        m.close()
+
+
 @pytest.mark.parametrize("mode", ["marginal", "interval"])
 def test_brick_data_follows_updates(ctx, mode):
     """Boxes of unknown, free and occupied voxels written over a sparse map whose sides are no multiple
