@@ -372,7 +372,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, 3) node_kernel(const LevelParams
         if (todo && n != cur) {
             if (cur >= 0) flush_counts<STATS>(p, cur, cur_kb, lane, c_abs, c_mrg, st);
             cur = n;
-            na = node_ancestors<INTERVAL>(p, n, anc, WH, pyr.n, lane);
+            na = node_ancestors(p, n, anc, WH, pyr.n, lane);
         }
         const uint32_t *hz = p.hz + (size_t)ln * K * pyr.n;
 #pragma unroll 1
@@ -540,7 +540,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, 4) brick_kernel(const LevelParam
                 cur = r.node;
                 n = p.level_nodes[l0 + nb0 + (int)(cur & ((1u << kRecNodeBits) - 1))];
                 nd = p.node[n];
-                node_ancestors<INTERVAL>(p, n, anc, WH, pyr_n, lane);
+                node_ancestors(p, n, anc, WH, pyr_n, lane);
             }
             count_brick<STATS, INTERVAL>(p, vc, s_y, anc, nd, p.steps + (size_t)(cur & ((1u << kRecNodeBits) - 1)) * K * WH, r, lane, c_abs,
                                c_mrg, st);

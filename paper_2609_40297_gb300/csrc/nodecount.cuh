@@ -304,7 +304,8 @@ struct NodeAnc {
     int px, py, pz, yaw;
     const uint32_t *D;
     const uint2 *pyr;
-    float U0, V0, Z0, pad;  // interval mode: the node in the ancestor's camera coordinates
+    float U0, V0, Z0;  // the node in the ancestor's camera coordinates
+    float err;         // 5e-7 of the node's largest offset from the ancestor
 };
 
 struct NodeCnt {  // statistics
@@ -416,25 +417,20 @@ __device__ __forceinline__ VoxConst vox_const(const LevelParams &p) {
 }
 
 // The ancestors of node n that the mode tests (Sec. IV-B), parent first; returns their number.
-template <bool INTERVAL>
 __device__ __forceinline__ int node_ancestors(const LevelParams &p, int n, NodeAnc *anc, size_t WH, int pyr_n, int lane) {
     const int2 ar = p.anc_range[n];
     int na = p.mode == MIG_MODE_ABSOLUTE ? 0 : (p.mode == MIG_MODE_SINGLE_PARENT ? min(ar.y, 1) : ar.y);
     na = min(na, p.max_anc);
+    const int4 nd = p.node[n];
     __syncwarp();
     for (int t = lane; t < na; t += 32) {
         const int a = p.anc[ar.x + t];
         const int4 an = p.node[a];
-        NodeAnc A{an.x, an.y, an.z, p.sel_yaw[a], p.arena + (size_t)an.w * WH, p.dpyr + (size_t)an.w * pyr_n, 0.f, 0.f, 0.f, 0.f};
-        if (INTERVAL) {
-            const int32_t *m = p.yawtab + A.yaw * 12 + 2;
-            const int4 nd = p.node[n];
-            const int rx = nd.x - an.x, ry = nd.y - an.y, rz = nd.z - an.z;
-            A.U0 = seg_coord(m, rx, ry, rz);
-            A.V0 = seg_coord(m + 3, rx, ry, rz);
-            A.Z0 = seg_coord(m + 6, rx, ry, rz);
-        }
-        anc[t] = A;
+        const int32_t *m = p.yawtab + p.sel_yaw[a] * 12 + 2;
+        const int rx = nd.x - an.x, ry = nd.y - an.y, rz = nd.z - an.z;
+        anc[t] = NodeAnc{an.x, an.y, an.z, p.sel_yaw[a], p.arena + (size_t)an.w * WH, p.dpyr + (size_t)an.w * pyr_n,
+                         seg_coord(m, rx, ry, rz), seg_coord(m + 3, rx, ry, rz), seg_coord(m + 6, rx, ry, rz),
+                         5e-7f * fmaxf(fmaxf(fabsf(q16f(rx)), fabsf(q16f(ry))), fabsf(q16f(rz)))};
     }
     __syncwarp();
     return na;
@@ -524,14 +520,14 @@ __device__ __forceinline__ uint64_t voxel_ancestors(const LevelParams &p, const 
                                                     const int4 nd, uint64_t left, uint64_t U, uint64_t O, int x, int y, int z0,
                                                     float verr, int lane, NodeCnt &st) {
     const int W = p.W, H = p.H;
-    for (uint64_t as = left; as; as &= as - 1) {
-        const NodeAnc A = anc[__ffsll((long long)as) - 1];
+    const float ex = q16f((x << 16) + 32768 - nd.x), ey = q16f((y << 16) + 32768 - nd.y), ez0 = q16f((z0 << 16) + 32768 - nd.z);
+    for (uint64_t as = left; as && (U & ~O); as &= as - 1) {
+        const NodeAnc &A = anc[__ffsll((long long)as) - 1];
         const float4 ru = s_y[A.yaw].u, rv = s_y[A.yaw].v, rz = s_y[A.yaw].z;
-        const int32_t *row = p.yawtab + A.yaw * 12;
-        const int ax = (x << 16) + 32768 - A.px, ay = (y << 16) + 32768 - A.py, az0 = (z0 << 16) + 32768 - A.pz;
-        const float ex = q16f(ax), ey = q16f(ay);
-        const float Zxy = fmaf(rz.x, ex, rz.y * ey), Uxy = fmaf(ru.x, ex, ru.y * ey), Vxy = fmaf(rv.x, ex, rv.y * ey);
-        const float c = verr + 5e-7f * fmaxf(fmaxf(fabsf(q16f(A.px - nd.x)), fabsf(q16f(A.py - nd.y))), fabsf(q16f(A.pz - nd.z)));
+        // camera coordinates: the node's plus the rotated offset from the node
+        const float Zxy = fmaf(rz.x, ex, fmaf(rz.y, ey, A.Z0)), Uxy = fmaf(ru.x, ex, fmaf(ru.y, ey, A.U0)),
+                    Vxy = fmaf(rv.x, ex, fmaf(rv.y, ey, A.V0));
+        const float c = verr + A.err;
         const PixelErr pe{2.0f * c * fmaf(vc.fW, rz.w, ru.w), 2.0f * c * fmaf(vc.fH, rz.w, rv.w), vc.bu, vc.bv};
         const float e_z = c * rz.w;
         const uint64_t rem = U & ~O;
@@ -540,7 +536,7 @@ __device__ __forceinline__ uint64_t voxel_ancestors(const LevelParams &p, const 
         float Zf[2];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const float ez = q16f(az0 + (h << 17));
+            const float ez = ez0 + (float)(2 * h);
             Zf[h] = fmaf(rz.z, ez, Zxy);
             in[h] = pixel_float(pe, Zf[h], fmaf(ru.z, ez, Uxy), fmaf(rv.z, ez, Vxy), vc.fW, vc.fH, pix[h]);
             if (!((uint32_t)(rem >> (32 * h)) >> lane & 1)) in[h] = 0;
@@ -557,7 +553,8 @@ __device__ __forceinline__ uint64_t voxel_ancestors(const LevelParams &p, const 
             const float lim = ((float)D[h] + 1.0f) * (1.0f / 65536.0f);
             obs[h] = in[h] > 0 && Zf[h] + e_z < lim * (1.0f - 2.4e-7f);
             if (in[h] < 0 || (in[h] > 0 && !obs[h] && Zf[h] - e_z < lim * (1.0f + 2.4e-7f)))
-                obs[h] = observed_exact(row, ax, ay, az0 + (h << 17), W, H, A.D);
+                obs[h] = observed_exact(p.yawtab + A.yaw * 12, (x << 16) + 32768 - A.px, (y << 16) + 32768 - A.py,
+                                        (z0 << 16) + 32768 + (h << 17) - A.pz, W, H, A.D);
         }
         O |= (uint64_t)__ballot_sync(0xffffffffu, obs[0]) | ((uint64_t)__ballot_sync(0xffffffffu, obs[1]) << 32);
     }

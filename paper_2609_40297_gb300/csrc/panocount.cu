@@ -329,7 +329,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, 3) pano_node_kernel(const LevelP
         unsigned todo = __ballot_sync(0xffffffffu, live);
         if (todo && n != cur) {
             cur = n;
-            na = node_ancestors<false>(p, n, anc, WH, pyr.n, lane);
+            na = node_ancestors(p, n, anc, WH, pyr.n, lane);
         }
         const uint32_t *hz = p.hz + (size_t)ln * ppyr.n;
 #pragma unroll 1
@@ -421,7 +421,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, 4) pano_brick_kernel(const Level
                 cur = r.node;
                 n = p.level_nodes[nr.l0 + nr.q0 + (int)cur];
                 nd = p.node[n];
-                node_ancestors<false>(p, n, anc, WH, pyr_n, lane);
+                node_ancestors(p, n, anc, WH, pyr_n, lane);
             }
             count_pano_brick(p, vc, pc, s_y, anc, n, nd, p.steps + (size_t)cur * AH, r, lane);
         }
