@@ -11,6 +11,7 @@
 #include "bricks.cuh"
 #include "dev_path.cuh"
 #include "kernels.h"
+#include "launch.cuh"
 #include "mig.h"
 #include "voxcount.h"
 
@@ -44,6 +45,7 @@ __global__ void __launch_bounds__(kWarps * 32, MIG_COUNT_MINB) count_kernel(cons
 // Yaw selection (Sec. III-B): lowest k with the largest marginal count (absolute count in the
 // absolute mode, where both counts are equal); g_abs = max over yaws of the absolute count.
 __global__ void select_kernel(const LevelParams p) {
+    wait_previous();
     int lvl = p.lvl;
     if (p.cursor) {
         const StepRange r = step_range(p);
@@ -208,7 +210,7 @@ int count_ctas_per_sm() {
     cudaGetLastError();
     return std::max(1, std::min(a, b));
 }
-void launch_select(const LevelParams &p, int grid, cudaStream_t s) { select_kernel<<<grid, 128, 0, s>>>(p); }
+void launch_select(const LevelParams &p, int grid, cudaStream_t s) { launch_behind(select_kernel, grid, 128, 0, s, p); }
 void launch_map_scatter(uint8_t *bricks, int nx, int ny, int nz, int nbx, int nby, const uint8_t *box, int x0, int y0,
                         int z0, int dx, int dy, int dz, cudaStream_t s) {
     const size_t total = (size_t)dx * dy * dz;

@@ -24,6 +24,7 @@
 #include "bricks.cuh"
 #include "interval.cuh"
 #include "kernels.h"
+#include "launch.cuh"
 #include "mig.h"
 #include "nodecount.cuh"
 #include "voxcount.h"
@@ -39,6 +40,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, kCastCtas) cast_kernel(const Lev
     __shared__ uint2 s_t[kWarpsN];
     __shared__ float s_beam[32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    wait_previous();
     if (blockIdx.x == 0 && threadIdx.x < 3) p.vctr[threadIdx.x] = 0;  // the counters of the passes that follow
     const StepRange step = step_range(p);
     const int l0 = step.l0, q0 = step.q0, q1 = step.q1;
@@ -84,6 +86,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, kCastCtas) render_kernel(const L
     __shared__ uint2 s_t[kWarpsN];
     __shared__ float s_beam[32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    wait_previous();
     int lvl = p.lvl;
     if (p.cursor) {
         const StepRange step = step_range(p);
@@ -332,12 +335,13 @@ __global__ void __launch_bounds__(kWarpsN * 32, 3) node_kernel(const LevelParams
     const int K = p.K;
     YawRows *s_y = reinterpret_cast<YawRows *>(s_dyn);
     NodeAnc *anc = reinterpret_cast<NodeAnc *>(s_y + K) + warp * p.max_anc;
+    for (int k = threadIdx.x; k < K; k += blockDim.x)
+        s_y[k] = yaw_rows(p.yawtab + k * 12, p.W, p.H, p.vis_hu, p.vis_hv, p.ifx, p.ify);
+    wait_previous();
+    __syncthreads();
     const StepRange step = step_range(p);
     const int l0 = step.l0, nb0 = step.q0 / K, nn = step.q1 / K - nb0;
     if (nn <= 0) return;
-    for (int k = threadIdx.x; k < K; k += blockDim.x)
-        s_y[k] = yaw_rows(p.yawtab + k * 12, p.W, p.H, p.vis_hu, p.vis_hv, p.ifx, p.ify);
-    __syncthreads();
     const int W = p.W, H = p.H;
     const size_t WH = (size_t)W * H;
     const Pyramid pyr = pyramid(W, H);
@@ -510,15 +514,16 @@ __global__ void __launch_bounds__(kWarpsN * 32, 4) brick_kernel(const LevelParam
     const int K = p.K;
     YawRows *s_y = reinterpret_cast<YawRows *>(s_dyn);
     NodeAnc *anc = reinterpret_cast<NodeAnc *>(s_y + K) + warp * p.max_anc;
+    for (int k = threadIdx.x; k < K; k += blockDim.x)
+        s_y[k] = yaw_rows(p.yawtab + k * 12, p.W, p.H, p.vis_hu, p.vis_hv, p.ifx, p.ify);
+    wait_previous();
+    __syncthreads();
     const StepRange step = step_range(p);
     const int l0 = step.l0, nb0 = step.q0 / K;
     if (step.q1 <= step.q0) return;
     const int total = min(p.vctr[1], p.queue_cap);
     const int slice = max(1, min(64, total / (int)(gridDim.x * kWarpsN * 8)));
     if (blockIdx.x * kWarpsN * slice >= total) return;
-    for (int k = threadIdx.x; k < K; k += blockDim.x)
-        s_y[k] = yaw_rows(p.yawtab + k * 12, p.W, p.H, p.vis_hu, p.vis_hv, p.ifx, p.ify);
-    __syncthreads();
     const size_t WH = (size_t)p.W * p.H;
     const int pyr_n = pyramid(p.W, p.H).n;
     const VoxConst vc = vox_const(p);
@@ -639,14 +644,14 @@ void set_visit_params(LevelParams &p, float hfov_deg, float vfov_deg) {
 
 void launch_cast_chunk(const LevelParams &c, int num_sms, cudaStream_t s) {
     const int g = cast_grid(c.q1 - c.q0, c.W, c.H, num_sms);
-    if (c.stats) cast_kernel<true><<<g, kWarpsN * 32, 0, s>>>(c, num_sms);
-    else cast_kernel<false><<<g, kWarpsN * 32, 0, s>>>(c, num_sms);
+    if (c.stats) launch_behind(cast_kernel<true>, g, kWarpsN * 32, 0, s, c, num_sms);
+    else launch_behind(cast_kernel<false>, g, kWarpsN * 32, 0, s, c, num_sms);
 }
 
 void launch_render(const LevelParams &p, int nodes, int num_sms, cudaStream_t s) {
     const int g = cast_grid(nodes, p.W, p.H, num_sms);
-    if (p.stats) render_kernel<true><<<g, kWarpsN * 32, 0, s>>>(p, num_sms);
-    else render_kernel<false><<<g, kWarpsN * 32, 0, s>>>(p, num_sms);
+    if (p.stats) launch_behind(render_kernel<true>, g, kWarpsN * 32, 0, s, p, num_sms);
+    else launch_behind(render_kernel<false>, g, kWarpsN * 32, 0, s, p, num_sms);
 }
 
 int node_ctas_per_sm() {
@@ -673,14 +678,14 @@ void launch_node_chunk(const LevelParams &c, int num_sms, int node_ctas, cudaStr
     const size_t smem = node_dyn_smem(c.K, c.max_anc);
     const int gb = num_sms * 4;
     if (c.mode == MIG_MODE_INTERVAL) {
-        node_kernel<false, true><<<g, kWarpsN * 32, smem, s>>>(c, num_sms);
-        brick_kernel<false, true><<<gb, kWarpsN * 32, smem, s>>>(c);
+        launch_behind(node_kernel<false, true>, g, kWarpsN * 32, smem, s, c, num_sms);
+        launch_behind(brick_kernel<false, true>, gb, kWarpsN * 32, smem, s, c);
     } else if (c.stats) {
-        node_kernel<true, false><<<g, kWarpsN * 32, smem, s>>>(c, num_sms);
-        brick_kernel<true, false><<<gb, kWarpsN * 32, smem, s>>>(c);
+        launch_behind(node_kernel<true, false>, g, kWarpsN * 32, smem, s, c, num_sms);
+        launch_behind(brick_kernel<true, false>, gb, kWarpsN * 32, smem, s, c);
     } else {
-        node_kernel<false, false><<<g, kWarpsN * 32, smem, s>>>(c, num_sms);
-        brick_kernel<false, false><<<gb, kWarpsN * 32, smem, s>>>(c);
+        launch_behind(node_kernel<false, false>, g, kWarpsN * 32, smem, s, c, num_sms);
+        launch_behind(brick_kernel<false, false>, gb, kWarpsN * 32, smem, s, c);
     }
 }
 

@@ -24,6 +24,7 @@
 
 #include "dev_path.cuh"
 #include "kernels.h"
+#include "launch.cuh"
 #include "mig.h"
 #include "pano.h"
 
@@ -160,6 +161,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) pano_count_kernel(const LevelP
 // starting at column k * step - Wc / 2 (mod A).
 // One warp per sum: a thread per sum is one chain of Wc loads.
 __global__ void pano_window_kernel(const LevelParams p) {
+    wait_previous();
     const int lane = threadIdx.x & 31;
     const int l0 = p.level_off[p.lvl];
     const int L = p.level_off[p.lvl + 1] - l0;
@@ -194,7 +196,7 @@ void launch_pano_count(const LevelParams &p, int grid, cudaStream_t s) {
 }
 
 void launch_pano_window(const LevelParams &p, int grid, cudaStream_t s) {
-    pano_window_kernel<<<grid, 256, 0, s>>>(p);
+    launch_behind(pano_window_kernel, grid, 256, 0, s, p);
 }
 
 int pano_ctas_per_sm() {

@@ -21,6 +21,7 @@
 #include <cmath>
 #include <cstdint>
 
+#include "launch.cuh"
 #include "nodecount.cuh"
 #include "pano.h"
 #include "voxcount.h"
@@ -78,6 +79,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, kCastCtas) pano_cast_kernel(cons
     __shared__ uint2 s_t[kWarpsN];
     __shared__ float s_beam[32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    wait_previous();
     if (blockIdx.x == 0 && threadIdx.x < 3) p.vctr[threadIdx.x] = 0;  // the counters of the passes that follow
     const NodeRange nr = node_range(p);
     if (nr.q0 >= nr.q1) return;
@@ -294,12 +296,13 @@ __global__ void __launch_bounds__(kWarpsN * 32, 3) pano_node_kernel(const LevelP
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     YawRows *s_y = reinterpret_cast<YawRows *>(s_dyn);
     NodeAnc *anc = reinterpret_cast<NodeAnc *>(s_y + p.K) + warp * p.max_anc;
+    for (int k = threadIdx.x; k < p.K; k += blockDim.x)
+        s_y[k] = yaw_rows(p.yawtab + k * 12, p.W, p.H, p.vis_hu, p.vis_hv, p.ifx, p.ify);
+    wait_previous();
+    __syncthreads();
     const NodeRange nr = node_range(p);
     const int nn = nr.q1 - nr.q0;
     if (nn <= 0) return;
-    for (int k = threadIdx.x; k < p.K; k += blockDim.x)
-        s_y[k] = yaw_rows(p.yawtab + k * 12, p.W, p.H, p.vis_hu, p.vis_hv, p.ifx, p.ify);
-    __syncthreads();
     const int A = p.pano_A, H = p.H;
     const size_t WH = (size_t)p.W * H, AH = (size_t)A * H;
     const Pyramid pyr = pyramid(p.W, H), ppyr = pyramid(A, H);
@@ -393,14 +396,15 @@ __global__ void __launch_bounds__(kWarpsN * 32, 4) pano_brick_kernel(const Level
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     YawRows *s_y = reinterpret_cast<YawRows *>(s_dyn);
     NodeAnc *anc = reinterpret_cast<NodeAnc *>(s_y + p.K) + warp * p.max_anc;
+    for (int k = threadIdx.x; k < p.K; k += blockDim.x)
+        s_y[k] = yaw_rows(p.yawtab + k * 12, p.W, p.H, p.vis_hu, p.vis_hv, p.ifx, p.ify);
+    wait_previous();
+    __syncthreads();
     const NodeRange nr = node_range(p);
     if (nr.q1 <= nr.q0) return;
     const int total = min(p.vctr[1], p.queue_cap);
     const int slice = max(1, min(64, total / (int)(gridDim.x * kWarpsN * 8)));
     if (blockIdx.x * kWarpsN * slice >= total) return;
-    for (int k = threadIdx.x; k < p.K; k += blockDim.x)
-        s_y[k] = yaw_rows(p.yawtab + k * 12, p.W, p.H, p.vis_hu, p.vis_hv, p.ifx, p.ify);
-    __syncthreads();
     const size_t WH = (size_t)p.W * p.H, AH = (size_t)p.pano_A * p.H;
     const int pyr_n = pyramid(p.W, p.H).n;
     const VoxConst vc = vox_const(p);
@@ -435,15 +439,15 @@ void set_pano_visit(LevelParams &p, int A, float vfov_deg) {
 }
 
 void launch_pano_cast_chunk(const LevelParams &c, int num_sms, cudaStream_t s) {
-    pano_cast_kernel<<<cast_grid(c.q1 - c.q0, c.pano_A, c.H, num_sms), kWarpsN * 32, 0, s>>>(c, num_sms);
+    launch_behind(pano_cast_kernel, cast_grid(c.q1 - c.q0, c.pano_A, c.H, num_sms), kWarpsN * 32, 0, s, c, num_sms);
 }
 
 void launch_pano_voxel_chunk(const LevelParams &c, int num_sms, cudaStream_t s) {
     const long long items = (long long)(c.q1 - c.q0) * node_items(c.Tq);
     const int g = (int)std::max<long long>(1, std::min<long long>((items + kWarpsN - 1) / kWarpsN, (long long)num_sms * 3));
     const size_t smem = node_dyn_smem(c.K, c.max_anc);
-    pano_node_kernel<<<g, kWarpsN * 32, smem, s>>>(c, num_sms);
-    pano_brick_kernel<<<num_sms * 4, kWarpsN * 32, smem, s>>>(c);
+    launch_behind(pano_node_kernel, g, kWarpsN * 32, smem, s, c, num_sms);
+    launch_behind(pano_brick_kernel, num_sms * 4, kWarpsN * 32, smem, s, c);
 }
 
 void pano_bricks_init() {
