@@ -222,7 +222,6 @@ int device_steps(int cap, int n, int K, int levels) { return cap >= K ? levels +
 
 void launch_device_levels(mig_ctx *ctx, LevelParams p, int n, int levels, int2 *cursor, cudaStream_t s) {
     const int count_cap = ctx->num_sms * std::min(ctx->count_ctas, std::max(1, (int)ctx->tiles.ctas_per_sm));
-    const int sel_grid = std::max(1, std::min((n + 127) / 128, 1024));
     const bool steps = p.steps && node_pass(p);
     const int count = steps ? device_steps(p.steps_cap, n, p.K, levels) : levels;
     for (int i = 0; i < count; ++i) {
@@ -237,8 +236,7 @@ void launch_device_levels(mig_ctx *ctx, LevelParams p, int n, int levels, int2 *
             p.lvl = i;
             launch_level_count_timed(ctx, p, n, count_cap);
         }
-        timed_launch(ctx, kProfSelect, [&] { launch_select(p, sel_grid, s); });
-        timed_launch(ctx, kProfRender, [&] { launch_render(p, n, ctx->num_sms, s); });
+        timed_launch(ctx, kProfRender, [&] { launch_select_render(p, n, ctx->num_sms, s); });
     }
 }
 
@@ -711,10 +709,9 @@ static mig_status eval_host(mig_map *m, int n, const int32_t *parent, const floa
         p.lvl = d;
         const int Ld = plan.level_off[d + 1] - plan.level_off[d];
         launch_level_count_timed(ctx, p, Ld, count_cap);
-        timed_launch(ctx, kProfSelect,
-                     [&] { launch_select(p, std::max(1, std::min((Ld + 127) / 128, 1024)), ctx->stream); });
         const int inner = plan.level_int[d];
-        if (inner > 0) timed_launch(ctx, kProfRender, [&] { launch_render(p, inner, ctx->num_sms, ctx->stream); });
+        if (inner > 0) timed_launch(ctx, kProfRender, [&] { launch_select_render(p, inner, ctx->num_sms, ctx->stream); });
+        else timed_launch(ctx, kProfSelect, [&] { launch_select(p, std::max(1, std::min((Ld + 127) / 128, 1024)), ctx->stream); });
         n_count++;
         n_render += inner > 0;
     }

@@ -737,8 +737,8 @@ mig_status batch_run_streams(mig_ctx *ctx, std::vector<BatchItem> &items) {
                 p.lvl = d;
                 const int Ld = pl.level_off[d + 1] - pl.level_off[d];
                 launch_level_count(ctx, p, Ld, count_cap, s);
-                launch_select(p, std::max(1, std::min((Ld + 127) / 128, 1024)), s);
-                if (pl.level_int[d] > 0) launch_render(p, pl.level_int[d], ctx->num_sms, s);
+                if (pl.level_int[d] > 0) launch_select_render(p, pl.level_int[d], ctx->num_sms, s);
+                else launch_select(p, std::max(1, std::min((Ld + 127) / 128, 1024)), s);
             }
             e = cudaGetLastError();
         }

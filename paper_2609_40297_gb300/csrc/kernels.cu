@@ -43,19 +43,11 @@ __global__ void __launch_bounds__(kWarps * 32, MIG_COUNT_MINB) count_kernel(cons
 
 // ------------------------------------------------------------------------------ select kernel
 // Yaw selection (Sec. III-B): lowest k with the largest marginal count (absolute count in the
-// absolute mode, where both counts are equal); g_abs = max over yaws of the absolute count.
+// absolute mode, where both counts are equal); g_abs = max over yaws of the absolute count. For levels
+// without internal nodes; the others select in the render's launch (launch_select_render).
 __global__ void select_kernel(const LevelParams p) {
     wait_previous();
-    int lvl = p.lvl;
-    if (p.cursor) {
-        const StepRange r = step_range(p);
-        // the next step: the level's next chunk, the next level, or (past the deepest node) here again
-        // with nothing to do
-        if (blockIdx.x == 0 && threadIdx.x == 0)
-            p.cursor[1] = r.q1 <= r.q0 ? make_int2(r.lvl, r.q0 / p.K) : (r.ends ? make_int2(r.lvl + 1, 0) : make_int2(r.lvl, r.q1 / p.K));
-        if (!r.ends || r.q1 <= r.q0) return;
-        lvl = r.lvl;
-    }
+    const int lvl = p.lvl;
     const int l0 = p.level_off[lvl];
     const int L = p.level_off[lvl + 1] - l0;
     for (int li = blockIdx.x * blockDim.x + threadIdx.x; li < L; li += gridDim.x * blockDim.x)

@@ -89,8 +89,9 @@ struct LevelParams {
 
 void launch_count(const LevelParams &p, int grid, cudaStream_t s);
 int count_ctas_per_sm();  // resident CTAs per SM of the count kernel
-void launch_select(const LevelParams &p, int grid, cudaStream_t s);
-void launch_render(const LevelParams &p, int nodes, int num_sms, cudaStream_t s);  // nodes: at least the level's internal ones
+void launch_select(const LevelParams &p, int grid, cudaStream_t s);  // a level without internal nodes
+// Selects the yaws of the level's nodes and renders its internal ones (`nodes`: at least their number).
+void launch_select_render(const LevelParams &p, int nodes, int num_sms, cudaStream_t s);
 void set_visit_params(LevelParams &p, float hfov_deg, float vfov_deg);  // the vis_* fields, from p.W and p.H
 // Writes a box of voxel codes into a grid of nx * ny * nz and refreshes the occupancy bytes, masks
 // and distances of the bricks it touches.

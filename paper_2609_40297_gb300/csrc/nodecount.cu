@@ -78,9 +78,33 @@ __global__ void __launch_bounds__(kWarpsN * 32, kCastCtas) cast_kernel(const Lev
     }
 }
 
-// Depth buffer of the selected yaw (Sec. IV-A): per pixel ray, camera z of the entry point of the
-// first occupied voxel, else of the range endpoint. Only nodes with children (the level's first
-// level_int nodes) are rendered; descendants read them in the ancestor test.
+// Yaw selection (select_node's rule) of one node by a warp; returns the yaw.
+__device__ __forceinline__ int select_warp(const LevelParams &p, int n, bool write, int lane) {
+    const int2 *c = reinterpret_cast<const int2 *>(p.cnt) + (size_t)n * p.K;  // (abs, marginal)
+    int best = 0x7fffffff, bm = -1, amax = 0;
+    for (int k = lane; k < p.K; k += 32) {
+        const int2 v = c[k];
+        best = v.y > bm ? k : best;
+        bm = max(bm, v.y);
+        amax = max(amax, v.x);
+    }
+    const int m = __reduce_max_sync(0xffffffffu, bm);
+    best = __reduce_min_sync(0xffffffffu, bm == m ? best : 0x7fffffff);
+    amax = __reduce_max_sync(0xffffffffu, amax);
+    if (write && lane == 0) {
+        p.sel_yaw[n] = best;
+        p.out_abs[n] = amax;
+        p.out_marg[n] = m;
+        p.out_yaw[n] = best;
+    }
+    return best;
+}
+
+// The yaw selection of the level's nodes, and the depth buffer of the selected yaw (Sec. IV-A): per
+// pixel ray, camera z of the entry point of the first occupied voxel, else of the range endpoint. Only
+// nodes with children (the level's first level_int nodes) are rendered; descendants read them in the
+// ancestor test. Each tile's warps select their node's yaw themselves (one load and three reductions),
+// which saves a level one launch of its chain: 4 to 5 us.
 template <bool STATS>
 __global__ void __launch_bounds__(kWarpsN * 32, kCastCtas) render_kernel(const LevelParams p, int num_sms) {
     __shared__ uint2 s_t[kWarpsN];
@@ -89,11 +113,17 @@ __global__ void __launch_bounds__(kWarpsN * 32, kCastCtas) render_kernel(const L
     wait_previous();
     int lvl = p.lvl;
     if (p.cursor) {
-        const StepRange step = step_range(p);
-        if (!step.ends || step.q1 <= step.q0) return;
-        lvl = step.lvl;
+        const StepRange r = step_range(p);
+        // the next step: the level's next chunk, the next level, or (past the deepest node) here again
+        // with nothing to do
+        if (blockIdx.x == 0 && threadIdx.x == 0)
+            p.cursor[1] = r.q1 <= r.q0 ? make_int2(r.lvl, r.q0 / p.K) : (r.ends ? make_int2(r.lvl + 1, 0) : make_int2(r.lvl, r.q1 / p.K));
+        if (!r.ends || r.q1 <= r.q0) return;
+        lvl = r.lvl;
     }
-    const int l0 = p.level_off[lvl], Li = p.level_int[lvl];
+    const int l0 = p.level_off[lvl], Li = p.level_int[lvl], L = p.level_off[lvl + 1] - l0;
+    for (int li = Li + blockIdx.x * kWarpsN + warp; li < L; li += gridDim.x * kWarpsN)
+        select_warp(p, p.level_nodes[l0 + li], true, lane);
     const CastLayout lay = cast_layout(Li, p.W, p.H, num_sms);
     const int T = lay == kCastSmall ? 16 : 32;
     const int tx = (p.W + T - 1) / T, ty = (p.H + T - 1) / T;
@@ -107,8 +137,8 @@ __global__ void __launch_bounds__(kWarpsN * 32, kCastCtas) render_kernel(const L
         const int tile = it % (tx * ty);
         const int n = p.level_nodes[l0 + it / (tx * ty)];
         const int4 nd = p.node[n];
+        const int32_t *yk = p.yawtab + select_warp(p, n, tile == 0 && (lay == kCastLarge || warp == 0), lane) * 12;
         if (nd.w < 0) continue;  // uniform over the warps of the item
-        const int32_t *yk = p.yawtab + p.sel_yaw[n] * 12;
         const CameraRays rays{p, nd, yk[0], yk[1], p.W, p.H};
         const RenderOut o{p.dpyr ? p.dpyr + (size_t)nd.w * y.n : nullptr, nd.w};
         const int x0 = tile % tx * T, y0 = tile / tx * T;
@@ -328,6 +358,7 @@ __device__ __forceinline__ void add_stats(const LevelParams &p, const NodeCnt &s
     }
 }
 
+constexpr int kNodeSplit = 8;  // parts of the yaws at most
 template <bool STATS, bool INTERVAL>
 __global__ void __launch_bounds__(kWarpsN * 32, 3) node_kernel(const LevelParams p, int num_sms) {
     extern __shared__ __align__(16) unsigned char s_dyn[];
@@ -354,8 +385,10 @@ __global__ void __launch_bounds__(kWarpsN * 32, 3) node_kernel(const LevelParams
     const int mxy = mac_xy(p.Tq), mn = mxy * mxy * mac_z(p.Tq);
     // macro blocks per work item: enough items for every warp to get several, at most one per lane
     const int group = (int)max(1ll, min(32ll, (long long)nn * mn / ((long long)gridDim.x * kWarpsN * 8)));
-    // too few blocks to fill the GPU: an item takes every split-th yaw of a block
-    const int split = (long long)nn * mn < 2ll * gridDim.x * kWarpsN ? min(K, 8) : 1;
+    // too few blocks to fill the GPU: an item takes every split-th yaw of a block, so that every warp gets
+    // one or two (node and brick pass of 9 levels of 11 nodes: 389 us with 8 parts below half that size
+    // and a warp per block, 313 so, 329 with twice, 343 with half as many)
+    const int split = (int)max(1ll, min((long long)min(K, kNodeSplit), 2ll * gridDim.x * kWarpsN / ((long long)nn * mn)));
     const int gpn = (mn + group - 1) / group * split;
     NodeCnt st;
     int cur = -1, cur_kb = 0, na = 0;
@@ -648,7 +681,7 @@ void launch_cast_chunk(const LevelParams &c, int num_sms, cudaStream_t s) {
     else launch_behind(cast_kernel<false>, g, kWarpsN * 32, 0, s, c, num_sms);
 }
 
-void launch_render(const LevelParams &p, int nodes, int num_sms, cudaStream_t s) {
+void launch_select_render(const LevelParams &p, int nodes, int num_sms, cudaStream_t s) {
     const int g = cast_grid(nodes, p.W, p.H, num_sms);
     if (p.stats) launch_behind(render_kernel<true>, g, kWarpsN * 32, 0, s, p, num_sms);
     else launch_behind(render_kernel<false>, g, kWarpsN * 32, 0, s, p, num_sms);
@@ -673,7 +706,8 @@ int node_ctas_per_sm() {
 long long node_items(int64_t Tq) { return (long long)mac_xy(Tq) * mac_xy(Tq) * mac_z(Tq); }
 
 void launch_node_chunk(const LevelParams &c, int num_sms, int node_ctas, cudaStream_t s) {
-    const long long items = (long long)((c.q1 - c.q0) / c.K) * node_items(c.Tq);
+    // a warp per macro block, or per block and eighth of the yaws where the blocks alone leave SMs idle (split)
+    const long long items = (long long)((c.q1 - c.q0) / c.K) * node_items(c.Tq) * std::min(c.K, kNodeSplit);
     const int g = (int)std::max<long long>(1, std::min<long long>((items + kWarpsN - 1) / kWarpsN, (long long)num_sms * node_ctas));
     const size_t smem = node_dyn_smem(c.K, c.max_anc);
     const int gb = num_sms * 4;

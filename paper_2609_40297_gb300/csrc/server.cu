@@ -300,8 +300,8 @@ mig_status run_step(mig_server *s) {
         const int d = r.level;
         const int Ld = pl.level_off[d + 1] - pl.level_off[d];
         launch_level_count(ctx, p, Ld, count_cap, st);
-        launch_select(p, std::max(1, std::min((Ld + 127) / 128, 1024)), st);
-        if (pl.level_int[d] > 0 && d < pl.max_depth) launch_render(p, pl.level_int[d], ctx->num_sms, st);
+        if (pl.level_int[d] > 0) launch_select_render(p, pl.level_int[d], ctx->num_sms, st);
+        else launch_select(p, std::max(1, std::min((Ld + 127) / 128, 1024)), st);
     }
     MIG_CUDA_TRY(cudaGetLastError());
     for (int i = 0; i < S; ++i) {
