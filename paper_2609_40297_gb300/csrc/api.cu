@@ -175,6 +175,12 @@ static void for_chunks(const LevelParams &p, long long total, int cap, F f) {
     }
 }
 
+void launch_tree_count(const mig_ctx *ctx, const LevelParams &p, int levels, cudaStream_t s) {
+    if (!p.steps || !p.tree) return;
+    if (p.mode == MIG_MODE_PANORAMIC) launch_pano_tree_cast(p, levels, ctx->num_sms, s);
+    else launch_tree_cast(p, levels, ctx->num_sms, s);
+}
+
 void launch_level_count(const mig_ctx *ctx, const LevelParams &p, int Ld, int count_cap, cudaStream_t s) {
     const int items = Ld * p.K * p.tiles;
     if (p.mode == MIG_MODE_INTERVAL && !p.steps) {
@@ -184,7 +190,7 @@ void launch_level_count(const mig_ctx *ctx, const LevelParams &p, int Ld, int co
         if (!p.steps) launch_pano_count(p, std::max(1, std::min((pitems + 7) / 8, ctx->num_sms * ctx->pano_ctas)), s);
         else
             for_chunks(p, Ld, p.steps_cap, [&](const LevelParams &c) {
-                launch_pano_cast_chunk(c, ctx->num_sms, s);
+                if (!p.tree) launch_pano_cast_chunk(c, ctx->num_sms, s);
                 launch_pano_voxel_chunk(c, ctx->num_sms, s);
             });
         launch_pano_window(p, std::max(1, std::min((Ld * p.K + 7) / 8, ctx->num_sms * 8)), s);
@@ -202,14 +208,14 @@ void launch_level_count_timed(mig_ctx *ctx, const LevelParams &p, int Ld, int co
     }
     if (p.mode == MIG_MODE_PANORAMIC) {
         for_chunks(p, Ld, p.steps_cap, [&](const LevelParams &c) {
-            timed_launch(ctx, kProfCast, [&] { launch_pano_cast_chunk(c, ctx->num_sms, ctx->stream); });
+            if (!p.tree) timed_launch(ctx, kProfCast, [&] { launch_pano_cast_chunk(c, ctx->num_sms, ctx->stream); });
             timed_launch(ctx, kProfVoxel, [&] { launch_pano_voxel_chunk(c, ctx->num_sms, ctx->stream); });
         });
         timed_launch(ctx, kProfVoxel, [&] { launch_pano_window(p, std::max(1, std::min((Ld * p.K + 7) / 8, ctx->num_sms * 8)), ctx->stream); });
         return;
     }
     for_chunks(p, (long long)Ld * p.K, vox_chunk_pairs(p), [&](const LevelParams &c) {
-        timed_launch(ctx, kProfCast, [&] { launch_cast_chunk(c, ctx->num_sms, ctx->stream); });
+        if (!p.tree) timed_launch(ctx, kProfCast, [&] { launch_cast_chunk(c, ctx->num_sms, ctx->stream); });
         timed_launch(ctx, kProfVoxel, [&] {
             if (node_pass(c)) launch_node_chunk(c, ctx->num_sms, ctx->node_ctas, ctx->stream);
             else launch_voxel_chunk(c, ctx->num_sms, ctx->vox_ctas, ctx->stream);
@@ -218,19 +224,22 @@ void launch_level_count_timed(mig_ctx *ctx, const LevelParams &p, int Ld, int co
 }
 
 // Steps of a tree whose levels' sizes only the device knows: every level may end in a partial chunk.
-int device_steps(int cap, int n, int K, int levels) { return cap >= K ? levels + n / (cap / K) : 0; }
+int device_steps(const StepsLayout &L, int n, int K, int levels) {
+    return L.tree ? levels : (L.cap >= K ? levels + n / (L.cap / K) : 0);
+}
 
 void launch_device_levels(mig_ctx *ctx, LevelParams p, int n, int levels, int2 *cursor, cudaStream_t s) {
     const int count_cap = ctx->num_sms * std::min(ctx->count_ctas, std::max(1, (int)ctx->tiles.ctas_per_sm));
     const bool steps = p.steps && node_pass(p);
-    const int count = steps ? device_steps(p.steps_cap, n, p.K, levels) : levels;
+    const int count = steps ? device_steps(StepsLayout{p.steps_cap, p.tree}, n, p.K, levels) : levels;
+    if (p.tree) timed_launch(ctx, kProfCast, [&] { launch_tree_count(ctx, p, levels, s); });
     for (int i = 0; i < count; ++i) {
         if (steps) {  // one chunk at a time, wherever the tree's levels end
             p.cursor = cursor + i;
             p.lvl = levels;
             p.q0 = 0;
             p.q1 = (int)std::min<long long>((long long)n * p.K, p.steps_cap);
-            timed_launch(ctx, kProfCast, [&] { launch_cast_chunk(p, ctx->num_sms, s); });
+            if (!p.tree) timed_launch(ctx, kProfCast, [&] { launch_cast_chunk(p, ctx->num_sms, s); });
             timed_launch(ctx, kProfVoxel, [&] { launch_node_chunk(p, ctx->num_sms, ctx->node_ctas, s); });
         } else {
             p.lvl = i;
@@ -240,18 +249,18 @@ void launch_device_levels(mig_ctx *ctx, LevelParams p, int n, int levels, int2 *
     }
 }
 
-StepsLayout steps_for(const mig_ctx *ctx, int Lmax, const mig_sensor &s, float voxel, int mode) {
+StepsLayout steps_for(const mig_ctx *ctx, int n, int Lmax, const mig_sensor &s, float voxel, int mode, int lean) {
     const bool pano = mode == MIG_MODE_PANORAMIC, whole = pano || mode == MIG_MODE_INTERVAL;
     // the interval and panoramic modes have no pass per (node, yaw) pair: without room for whole nodes they
     // count ray by ray
-    if (ctx->ray_count || (whole && ctx->voxel_pass == MIG_COUNT_PAIRS)) return StepsLayout{};
+    if (ctx->ray_count || lean == 2 || (whole && ctx->voxel_pass == MIG_COUNT_PAIRS)) return StepsLayout{};
     SensorDims d{s.width, s.height, s.yaw_bins, range_q16(s.range_m, voxel)};
     if (pano) {
         d.W = pano_columns(s);
         d.K = 1;
         if ((size_t)d.W * d.H * sizeof(uint16_t) > ctx->steps_budget) return StepsLayout{};
     }
-    const StepsLayout L = steps_layout(d, Lmax, ctx->steps_budget, ctx->voxel_pass != MIG_COUNT_PAIRS, mode);
+    const StepsLayout L = steps_layout(d, n, Lmax, ctx->steps_budget, lean == 0 ? kTreeSteps : 0, ctx->voxel_pass != MIG_COUNT_PAIRS, mode);
     return whole && L.queue_cap == 0 ? StepsLayout{} : L;
 }
 
@@ -645,19 +654,26 @@ static mig_status eval_host(mig_map *m, int n, const int32_t *parent, const floa
     const size_t o_cnt = cv.take<int32_t>((size_t)n * K * 2);
     const size_t o_work = cv.take<int32_t>(L);
     const size_t o_arena = cv.take<uint32_t>((size_t)std::max(1, plan.n_internal) * WH);
-    const size_t o_dpyr = cv.take<uint2>((size_t)std::max(1, plan.n_internal) * hz_entries(cam->W, cam->H));
     const size_t o_stats = cv.take<unsigned long long>(kStatsCounters);
     const size_t o_pcnt = cv.take<int32_t>(pano ? (size_t)n * cam->pano_A * 2 : 1);
     int Lmax = 1;
     for (int d = 0; d < L; ++d) Lmax = std::max(Lmax, plan.level_off[d + 1] - plan.level_off[d]);
-    const StepsLayout steps = steps_for(ctx, Lmax, *sensor, m->voxel, mode);
-    const size_t o_steps = cv.take<char>(steps.bytes);
-    // instrumented pass: the ray-by-ray count kernel is re-run into scratch counters afterwards,
-    // for the method's own work counts (rays, DDA steps, owner tests) and as a cross-check
-    const bool rerun = stats && steps.cap > 0;
-    const size_t o_cnt2 = cv.take<int32_t>(rerun ? (size_t)n * K * 2 + L : 1);
+    StepsLayout steps{};
+    size_t o_dpyr = 0, o_steps = 0, o_cnt2 = 0;
+    bool rerun = false;
     char *dev = nullptr;
-    st = ctx_workspace(ctx, cv.off, (void **)&dev);
+    for (int lean = 0; lean < 3; ++lean) {  // less memory where the allocator has not enough
+        Carver c = cv;
+        steps = steps_for(ctx, n, Lmax, *sensor, m->voxel, mode, lean);
+        o_dpyr = c.take<uint2>(steps.cap ? (size_t)std::max(1, plan.n_internal) * hz_entries(cam->W, cam->H) : 0);
+        o_steps = c.take<char>(steps.bytes);
+        // instrumented pass: the ray-by-ray count kernel is re-run into scratch counters afterwards,
+        // for the method's own work counts (rays, DDA steps, owner tests) and as a cross-check
+        rerun = stats && steps.cap > 0;
+        o_cnt2 = c.take<int32_t>(rerun ? (size_t)n * K * 2 + L : 1);
+        st = ctx_workspace(ctx, c.off, (void **)&dev);
+        if (st != MIG_ENOMEM) break;
+    }
     if (st != MIG_OK) return st;
     char *host = nullptr;
     st = ctx_pinned(ctx, std::max(up_bytes, 3 * (size_t)n * 4), (void **)&host);
@@ -698,13 +714,14 @@ static mig_status eval_host(mig_map *m, int n, const int32_t *parent, const floa
     MIG_CUDA_TRY(cudaMemsetAsync(p.bounds_err, 0, 4, ctx->stream));
 #endif
     if (steps.cap) set_steps(p, dev + o_steps, steps);
-    p.dpyr = (uint2 *)(dev + o_dpyr);
+    p.dpyr = steps.cap ? (uint2 *)(dev + o_dpyr) : nullptr;
     if (stats) {
         p.stats = (unsigned long long *)(dev + o_stats);
         MIG_CUDA_TRY(cudaMemsetAsync(p.stats, 0, kStatsCounters * sizeof(unsigned long long), ctx->stream));
     }
     const int count_cap = ctx->num_sms * std::min(ctx->count_ctas, std::max(1, (int)ctx->tiles.ctas_per_sm));
     uint64_t n_count = 0, n_render = 0;
+    if (p.tree) timed_launch(ctx, kProfCast, [&] { launch_tree_count(ctx, p, L, ctx->stream); });
     for (int d = 0; d < L; ++d) {
         p.lvl = d;
         const int Ld = plan.level_off[d + 1] - plan.level_off[d];
@@ -819,25 +836,31 @@ mig_status mig_tree_eval_device(mig_map *m, int n, const int32_t *parent, const 
     if (st != MIG_OK) return st;
     const int K = cam->K, L = max_depth + 1;
     const size_t WH = (size_t)cam->W * cam->H;
-    Carver cv;
-    // zero-initialised region first
-    const size_t o_lcnt = cv.take<int32_t>(L), o_licnt = cv.take<int32_t>(L), o_cur2 = cv.take<int32_t>(2 * L);
-    const size_t o_hasc = cv.take<int32_t>(n), o_slot = cv.take<int32_t>(1), o_roots = cv.take<int32_t>(1);
-    const size_t o_err = cv.take<int32_t>(1), o_cnt = cv.take<int32_t>((size_t)n * K * 2);
-    const size_t o_work = cv.take<int32_t>(L);
-    // level sizes are known on the device only: the step-count buffer is sized for n nodes
-    const StepsLayout steps = steps_for(ctx, n, *sensor, m->voxel, MIG_MODE_MARGINAL);
-    const size_t o_cursor = cv.take<int2>(device_steps(steps.cap, n, K, L) + 1);
-    const size_t zero_bytes = cv.off;
-    const size_t o_depth = cv.take<int32_t>(n), o_loff = cv.take<int32_t>(L + 1), o_lint = cv.take<int32_t>(L);
-    const size_t o_lnodes = cv.take<int32_t>(n), o_ar = cv.take<int2>(n);
-    const size_t o_anc = cv.take<int32_t>(std::max<size_t>(1, (size_t)n * max_depth)), o_node = cv.take<int4>(n);
-    const size_t o_sel = cv.take<int32_t>(n);
-    const size_t o_arena = cv.take<uint32_t>((size_t)n * WH);
-    const size_t o_dpyr = cv.take<uint2>((size_t)n * hz_entries(cam->W, cam->H));
-    const size_t o_steps = cv.take<char>(steps.bytes);
+    size_t o_lcnt, o_licnt, o_cur2, o_hasc, o_slot, o_roots, o_err, o_cnt, o_work, o_cursor, o_depth, o_loff,
+        o_lint, o_lnodes, o_ar, o_anc, o_node, o_sel, o_arena, o_dpyr, o_steps, zero_bytes;
+    StepsLayout steps{};
     char *dev = nullptr;
-    st = ctx_workspace(ctx, cv.off, (void **)&dev);
+    for (int lean = 0; lean < 3; ++lean) {  // less memory where the allocator has not enough
+        Carver cv;
+        // zero-initialised region first
+        o_lcnt = cv.take<int32_t>(L); o_licnt = cv.take<int32_t>(L); o_cur2 = cv.take<int32_t>(2 * L);
+        o_hasc = cv.take<int32_t>(n); o_slot = cv.take<int32_t>(1); o_roots = cv.take<int32_t>(1);
+        o_err = cv.take<int32_t>(1); o_cnt = cv.take<int32_t>((size_t)n * K * 2);
+        o_work = cv.take<int32_t>(L);
+        // level sizes are known on the device only: the step-count buffer is sized for n nodes
+        steps = steps_for(ctx, n, n, *sensor, m->voxel, MIG_MODE_MARGINAL, lean);
+        o_cursor = cv.take<int2>(device_steps(steps, n, K, L) + 1);
+        zero_bytes = cv.off;
+        o_depth = cv.take<int32_t>(n); o_loff = cv.take<int32_t>(L + 1); o_lint = cv.take<int32_t>(L);
+        o_lnodes = cv.take<int32_t>(n); o_ar = cv.take<int2>(n);
+        o_anc = cv.take<int32_t>(std::max<size_t>(1, (size_t)n * max_depth)); o_node = cv.take<int4>(n);
+        o_sel = cv.take<int32_t>(n);
+        o_arena = cv.take<uint32_t>((size_t)n * WH);
+        o_dpyr = cv.take<uint2>(steps.cap ? (size_t)n * hz_entries(cam->W, cam->H) : 0);
+        o_steps = cv.take<char>(steps.bytes);
+        st = ctx_workspace(ctx, cv.off, (void **)&dev);
+        if (st != MIG_ENOMEM) break;
+    }
     if (st != MIG_OK) return st;
     MIG_CUDA_TRY(cudaMemsetAsync(dev, 0, zero_bytes, ctx->stream));
     DevPlanParams dp{};
@@ -888,7 +911,7 @@ mig_status mig_tree_eval_device(mig_map *m, int n, const int32_t *parent, const 
     p.mode = MIG_MODE_MARGINAL;
     p.max_anc = std::max(1, max_depth);
     if (steps.cap) set_steps(p, dev + o_steps, steps);
-    p.dpyr = (uint2 *)(dev + o_dpyr);
+    p.dpyr = steps.cap ? (uint2 *)(dev + o_dpyr) : nullptr;
     launch_device_levels(ctx, p, n, L, (int2 *)(dev + o_cursor), ctx->stream);
     MIG_CUDA_TRY(cudaGetLastError());
     return MIG_OK;

@@ -640,19 +640,24 @@ mig_status batch_run_streams(mig_ctx *ctx, std::vector<BatchItem> &items) {
     for (int t = 0; t < T; ++t) order[t] = t;
     std::sort(order.begin(), order.end(), [&](int a, int c) { return items[a].plan.n > items[c].plan.n; });
     std::vector<StepsLayout> steps(T);
-    std::vector<size_t> stream_steps(S, 0);
-    for (int oi = 0; oi < T; ++oi) {
-        const int t = order[oi];
-        const HostPlan &pl = items[t].plan;
-        int Lmax = 1;
-        for (int d = 0; d <= pl.max_depth; ++d) Lmax = std::max(Lmax, pl.level_off[d + 1] - pl.level_off[d]);
-        steps[t] = steps_for(ctx, Lmax, items[t].sensor, items[t].map->voxel, items[t].mode);
-        stream_steps[oi % S] = std::max(stream_steps[oi % S], steps[t].bytes);
-    }
     std::vector<size_t> o_steps(S);
-    for (int i = 0; i < S; ++i) o_steps[i] = cv.take(std::max<size_t>(stream_steps[i], 1));
     char *dev = nullptr;
-    mig_status st = ctx_workspace(ctx, cv.off, (void **)&dev);
+    mig_status st = MIG_OK;
+    for (int lean = 0; lean < 3; ++lean) {  // less memory where the allocator has not enough
+        std::vector<size_t> stream_steps(S, 0);
+        for (int oi = 0; oi < T; ++oi) {
+            const int t = order[oi];
+            const HostPlan &pl = items[t].plan;
+            int Lmax = 1;
+            for (int d = 0; d <= pl.max_depth; ++d) Lmax = std::max(Lmax, pl.level_off[d + 1] - pl.level_off[d]);
+            steps[t] = steps_for(ctx, pl.n, Lmax, items[t].sensor, items[t].map->voxel, items[t].mode, lean);
+            stream_steps[oi % S] = std::max(stream_steps[oi % S], steps[t].bytes);
+        }
+        Carve c = cv;
+        for (int i = 0; i < S; ++i) o_steps[i] = c.take(std::max<size_t>(stream_steps[i], 1));
+        st = ctx_workspace(ctx, c.off, (void **)&dev);
+        if (st != MIG_ENOMEM) break;
+    }
     if (st != MIG_OK) return st;
     char *host = nullptr;
     st = ctx_pinned(ctx, std::max(up_bytes, down_bytes) + 256, (void **)&host);
@@ -733,6 +738,7 @@ mig_status batch_run_streams(mig_ctx *ctx, std::vector<BatchItem> &items) {
             cudaStream_t s = B->pool[oi % S];
             LevelParams p = lp[t];
             const HostPlan &pl = items[t].plan;
+            launch_tree_count(ctx, p, pl.max_depth + 1, s);
             for (int d = 0; d <= pl.max_depth; ++d) {
                 p.lvl = d;
                 const int Ld = pl.level_off[d + 1] - pl.level_off[d];

@@ -47,6 +47,7 @@ __global__ void __launch_bounds__(kWarps * 32, MIG_COUNT_MINB) count_kernel(cons
 // without internal nodes; the others select in the render's launch (launch_select_render).
 __global__ void select_kernel(const LevelParams p) {
     wait_previous();
+    if (p.tree && blockIdx.x == 0 && threadIdx.x < 3) p.vctr[threadIdx.x] = 0;  // for the next level's count
     const int lvl = p.lvl;
     const int l0 = p.level_off[lvl];
     const int L = p.level_off[lvl + 1] - l0;

@@ -82,6 +82,9 @@ struct LevelParams {
     int2 *cursor;
     BrickRec *queue;  // per-node pass: undecided bricks of the chunk
     int queue_cap;
+    // 0, or the tree's nodes: all of them were cast by one launch, and the step counts and bounds of the
+    // i-th of level_nodes are the buffers' i-th (else a chunk's nodes are, from 0)
+    int tree;
     // per-node pass: half a pixel at unit depth along the image axes, the depth below which the owner
     // ray certainly visits its voxel, and the reciprocal focal lengths (set_visit_params)
     float vis_hu, vis_hv, vis_zl2, ifx, ify;

@@ -164,18 +164,21 @@ void set_pano_params(LevelParams &p, const Camera *cam, int32_t *pcnt);
 // the level, or an upper bound of it for the sample modes' owned-voxel kernels, which read the
 // level's size on the device). The sample modes use the owned-voxel kernels when p.steps is set,
 // else the ray-by-ray count kernel. The panoramic mode also runs its window sums, so
-// launch_select may follow.
+// launch_select or launch_select_render may follow.
 void launch_level_count(const mig_ctx *ctx, const LevelParams &p, int Ld, int count_cap, cudaStream_t s);
+// What the counts of all levels share (the cast of a whole small tree); before the first level.
+void launch_tree_count(const mig_ctx *ctx, const LevelParams &p, int levels, cudaStream_t s);
 // The same on the context stream, each launch timed under its own kind (mig_ctx_profile).
 void launch_level_count_timed(mig_ctx *ctx, const LevelParams &p, int Ld, int count_cap);
-// The owned-voxel count's region for a tree whose widest level has Lmax nodes (empty when the context
-// counts ray by ray or the mode does).
+// The owned-voxel count's region for a tree of n nodes whose widest level has Lmax (empty when the context
+// counts ray by ray or the mode does). lean 0: the whole tree's step counts if small, 1: a level's, 2: none
+// (ray by ray); a caller whose allocation fails takes the next.
 struct StepsLayout;
-StepsLayout steps_for(const mig_ctx *ctx, int Lmax, const mig_sensor &s, float voxel, int mode);
-// The count, select and render launches of a device-planned tree of n nodes and at most `levels` levels.
+StepsLayout steps_for(const mig_ctx *ctx, int n, int Lmax, const mig_sensor &s, float voxel, int mode, int lean);
+// The count and select-and-render launches of a device-planned tree of n nodes and at most `levels` levels.
 // With the per-node pass they go chunk by chunk through the levels, whose sizes only the device knows:
 // device_steps(..) steps and as many places + 1 in `cursor` (zeroed).
-int device_steps(int cap, int n, int K, int levels);
+int device_steps(const StepsLayout &L, int n, int K, int levels);
 void launch_device_levels(mig_ctx *ctx, LevelParams p, int n, int levels, int2 *cursor, cudaStream_t s);
 // records an event pair around launch() on the context stream when profiling is on
 void prof_begin(mig_ctx *ctx, int kind, cudaEvent_t *a);

@@ -42,10 +42,17 @@ __global__ void __launch_bounds__(kWarpsN * 32, kCastCtas) cast_kernel(const Lev
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     wait_previous();
     if (blockIdx.x == 0 && threadIdx.x < 3) p.vctr[threadIdx.x] = 0;  // the counters of the passes that follow
-    const StepRange step = step_range(p);
-    const int l0 = step.l0, q0 = step.q0, q1 = step.q1;
+    int l0 = 0, q0 = 0, q1 = 0;
+    if (p.tree) {  // lvl: the number of levels
+        q1 = min(p.tree, p.level_off[p.lvl]) * p.K;
+    } else {
+        const StepRange step = step_range(p);
+        l0 = step.l0;
+        q0 = step.q0;
+        q1 = step.q1;
+    }
     if (q0 >= q1) return;
-    const CastLayout lay = cast_layout(q1 - q0, p.W, p.H, num_sms);
+    const CastLayout lay = cast_layout(p.tree ? (long long)p.tree * p.K : q1 - q0, p.W, p.H, num_sms);
     const int T = lay == kCastSmall ? 16 : 32;
     const int tx = (p.W + T - 1) / T, ty = (p.H + T - 1) / T;
     const size_t WH = (size_t)p.W * p.H;
@@ -111,6 +118,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, kCastCtas) render_kernel(const L
     __shared__ float s_beam[32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     wait_previous();
+    if (p.tree && blockIdx.x == 0 && threadIdx.x < 3) p.vctr[threadIdx.x] = 0;  // for the next level's count
     int lvl = p.lvl;
     if (p.cursor) {
         const StepRange r = step_range(p);
@@ -373,10 +381,11 @@ __global__ void __launch_bounds__(kWarpsN * 32, 3) node_kernel(const LevelParams
     const StepRange step = step_range(p);
     const int l0 = step.l0, nb0 = step.q0 / K, nn = step.q1 / K - nb0;
     if (nn <= 0) return;
+    const int base = p.tree ? l0 + nb0 : 0;  // the chunk's first node in the step counts and bounds
     const int W = p.W, H = p.H;
     const size_t WH = (size_t)W * H;
     const Pyramid pyr = pyramid(W, H);
-    const int top = cast_layout((long long)nn * K, W, H, num_sms) == kCastSmall ? 4 : 5;  // the bounds the cast kept
+    const int top = cast_layout((long long)(p.tree ? p.tree : nn) * K, W, H, num_sms) == kCastSmall ? 4 : 5;  // the bounds the cast kept
     const BrickDims bd = brick_dims(p.grid.nx, p.grid.ny, p.grid.nz);
     const uint64_t *umask = grid_umask(p.grid);
     const VoxConst vc = vox_const(p);
@@ -411,7 +420,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, 3) node_kernel(const LevelParams
             cur = n;
             na = node_ancestors(p, n, anc, WH, pyr.n, lane);
         }
-        const uint32_t *hz = p.hz + (size_t)ln * K * pyr.n;
+        const uint32_t *hz = p.hz + (size_t)(base + ln) * K * pyr.n;
 #pragma unroll 1
         for (; todo; todo &= todo - 1) {
             const int src = __ffs(todo) - 1;
@@ -529,7 +538,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, 3) node_kernel(const LevelParams
                         const int s = __ffs(full) - 1;
                         BrickRec q{shfl64(r.U, s), shfl64(r.O, s), shfl64(r.anc, s), shfl64(r.all, s), shfl64(r.part, s),
                                    shfl64(r.rch, s), shfl64(r.vis, s), __shfl_sync(0xffffffffu, r.brick, s), r.node};
-                        count_brick<STATS, INTERVAL>(p, vc, s_y, anc, nd, p.steps + (size_t)ln * K * WH, q, lane, c_abs, c_mrg, st);
+                        count_brick<STATS, INTERVAL>(p, vc, s_y, anc, nd, p.steps + (size_t)(base + ln) * K * WH, q, lane, c_abs, c_mrg, st);
                     }
                 }
             }
@@ -554,6 +563,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, 4) brick_kernel(const LevelParam
     const StepRange step = step_range(p);
     const int l0 = step.l0, nb0 = step.q0 / K;
     if (step.q1 <= step.q0) return;
+    const int base = p.tree ? l0 + nb0 : 0;
     const int total = min(p.vctr[1], p.queue_cap);
     const int slice = max(1, min(64, total / (int)(gridDim.x * kWarpsN * 8)));
     if (blockIdx.x * kWarpsN * slice >= total) return;
@@ -580,7 +590,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, 4) brick_kernel(const LevelParam
                 nd = p.node[n];
                 node_ancestors(p, n, anc, WH, pyr_n, lane);
             }
-            count_brick<STATS, INTERVAL>(p, vc, s_y, anc, nd, p.steps + (size_t)(cur & ((1u << kRecNodeBits) - 1)) * K * WH, r, lane, c_abs,
+            count_brick<STATS, INTERVAL>(p, vc, s_y, anc, nd, p.steps + (size_t)(base + (int)(cur & ((1u << kRecNodeBits) - 1))) * K * WH, r, lane, c_abs,
                                c_mrg, st);
         }
     }
@@ -681,6 +691,14 @@ void launch_cast_chunk(const LevelParams &c, int num_sms, cudaStream_t s) {
     else launch_behind(cast_kernel<false>, g, kWarpsN * 32, 0, s, c, num_sms);
 }
 
+void launch_tree_cast(const LevelParams &p, int levels, int num_sms, cudaStream_t s) {
+    LevelParams c = p;
+    c.lvl = levels;
+    c.q0 = 0;
+    c.q1 = p.tree * p.K;
+    launch_cast_chunk(c, num_sms, s);
+}
+
 void launch_select_render(const LevelParams &p, int nodes, int num_sms, cudaStream_t s) {
     const int g = cast_grid(nodes, p.W, p.H, num_sms);
     if (p.stats) launch_behind(render_kernel<true>, g, kWarpsN * 32, 0, s, p, num_sms);
@@ -748,7 +766,7 @@ static void place(StepsLayout &L, const SensorDims &d) {
     L.bytes = L.o_queue + (size_t)L.queue_cap * sizeof(BrickRec);
 }
 
-StepsLayout steps_layout(const SensorDims &d, int max_nodes, size_t budget_bytes, bool node_pass, int mode) {
+StepsLayout steps_layout(const SensorDims &d, int n, int max_nodes, size_t budget_bytes, size_t tree_bytes, bool node_pass, int mode) {
     StepsLayout L{};
     const long long pairs = (long long)std::max(1, max_nodes) * d.K;
     L.cap = (int)steps_pairs(pairs, d.W, d.H, budget_bytes);
@@ -757,6 +775,13 @@ StepsLayout steps_layout(const SensorDims &d, int max_nodes, size_t budget_bytes
         const long long nodes = std::max<long long>(1, std::min<long long>(L.cap / d.K, kQueueMax / per_node));
         L.cap = (int)nodes * d.K;
         L.queue_cap = (int)std::min(kQueueMax, std::max<long long>(nodes * per_node, 1ll << 16));
+        // all of a small tree's nodes, if one level's work items stay below 2^30
+        const double images = (double)n * d.K, bytes = images * d.W * d.H * sizeof(uint16_t);
+        if (bytes <= (double)std::min(budget_bytes, tree_bytes) && images * (double)hz_entries(d.W, d.H) <= (double)tree_bytes &&
+            nodes >= max_nodes && (double)n * (double)node_items(d.Tq) * d.K < (double)(1ll << 30)) {
+            L.tree = n;
+            L.cap = n * d.K;
+        }
     }
     place(L, d);
     return L;
@@ -774,6 +799,8 @@ StepsLayout steps_layout_in(const SensorDims &d, int max_nodes, size_t bytes) {
     const long long nodes = std::min<long long>(std::min<long long>(max_nodes, (1 << kRecNodeBits) - 1), (long long)((bytes - fixed) / node));
     L.cap = (int)std::min<long long>(nodes, INT_MAX / d.K) * d.K;
     L.queue_cap = (int)std::min<long long>(kQueueMax, (long long)(L.cap / d.K) * recs);
+    // room for the whole tree (max_nodes nodes): one cast
+    if (nodes == max_nodes && (double)nodes * (double)node_items(d.Tq) * d.K < (double)(1ll << 30)) L.tree = max_nodes;
     place(L, d);
     return L;
 }
@@ -786,6 +813,7 @@ void set_steps(LevelParams &p, void *base, const StepsLayout &L) {
     p.queue = reinterpret_cast<BrickRec *>(b + L.o_queue);
     p.queue_cap = L.queue_cap;
     p.steps_cap = L.cap;
+    p.tree = L.tree;
 }
 
 void launch_brick_update(uint8_t *grid, int nx, int ny, int nz, int x0, int y0, int z0, int dx, int dy, int dz, cudaStream_t s) {

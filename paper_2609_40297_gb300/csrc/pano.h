@@ -14,6 +14,7 @@ void launch_pano_window(const LevelParams &p, int grid, cudaStream_t s);
 // The same counts by owned voxels (panocount.cu), for the nodes [c.q0, c.q1) of the level, at most
 // steps_cap: the cast, then the per-node and the brick pass. The cast clears their column counts.
 void launch_pano_cast_chunk(const LevelParams &c, int num_sms, cudaStream_t s);
+void launch_pano_tree_cast(const LevelParams &p, int levels, int num_sms, cudaStream_t s);  // launch_tree_cast
 void launch_pano_voxel_chunk(const LevelParams &c, int num_sms, cudaStream_t s);
 void set_pano_visit(LevelParams &p, int A, float vfov_deg);  // vis_zl2 of a strip's cells
 void pano_bricks_init();  // lifts the kernels' dynamic shared-memory limit; call once

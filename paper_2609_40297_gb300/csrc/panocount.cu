@@ -34,7 +34,9 @@ namespace {
 struct NodeRange {
     int l0, q0, q1;
 };
-__device__ __forceinline__ NodeRange node_range(const LevelParams &p) {
+// (with p.tree: of the tree, in the cast, where lvl is the number of levels)
+__device__ __forceinline__ NodeRange node_range(const LevelParams &p, bool cast = false) {
+    if (p.tree && cast) return NodeRange{0, 0, min(p.tree, p.level_off[p.lvl])};
     const int l0 = p.level_off[p.lvl], n = p.level_off[p.lvl + 1] - l0;
     return NodeRange{l0, p.q0, min(p.q1, n)};
 }
@@ -81,10 +83,10 @@ __global__ void __launch_bounds__(kWarpsN * 32, kCastCtas) pano_cast_kernel(cons
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     wait_previous();
     if (blockIdx.x == 0 && threadIdx.x < 3) p.vctr[threadIdx.x] = 0;  // the counters of the passes that follow
-    const NodeRange nr = node_range(p);
+    const NodeRange nr = node_range(p, true);
     if (nr.q0 >= nr.q1) return;
     const int A = p.pano_A, H = p.H;
-    const CastLayout lay = cast_layout(nr.q1 - nr.q0, A, H, num_sms);
+    const CastLayout lay = cast_layout(p.tree ? p.tree : nr.q1 - nr.q0, A, H, num_sms);
     const int T = lay == kCastSmall ? 16 : 32;
     const int tx = (A + T - 1) / T, ty = (H + T - 1) / T;
     const size_t AH = (size_t)A * H;
@@ -303,10 +305,11 @@ __global__ void __launch_bounds__(kWarpsN * 32, 3) pano_node_kernel(const LevelP
     const NodeRange nr = node_range(p);
     const int nn = nr.q1 - nr.q0;
     if (nn <= 0) return;
+    const int base = p.tree ? nr.l0 + nr.q0 : 0;  // the chunk's first node in the step counts and bounds
     const int A = p.pano_A, H = p.H;
     const size_t WH = (size_t)p.W * H, AH = (size_t)A * H;
     const Pyramid pyr = pyramid(p.W, H), ppyr = pyramid(A, H);
-    const int top = cast_layout(nn, A, H, num_sms) == kCastSmall ? 4 : 5;  // the bounds the cast kept
+    const int top = cast_layout(p.tree ? p.tree : nn, A, H, num_sms) == kCastSmall ? 4 : 5;  // the bounds the cast kept
     const BrickDims bd = brick_dims(p.grid.nx, p.grid.ny, p.grid.nz);
     const uint64_t *umask = grid_umask(p.grid);
     const VoxConst vc = vox_const(p);
@@ -334,7 +337,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, 3) pano_node_kernel(const LevelP
             cur = n;
             na = node_ancestors(p, n, anc, WH, pyr.n, lane);
         }
-        const uint32_t *hz = p.hz + (size_t)ln * ppyr.n;
+        const uint32_t *hz = p.hz + (size_t)(base + ln) * ppyr.n;
 #pragma unroll 1
         for (; todo; todo &= todo - 1) {
             const int src = __ffs(todo) - 1;
@@ -384,7 +387,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, 3) pano_node_kernel(const LevelP
                 const int s = __ffs(full) - 1;
                 BrickRec q{shfl64(r.U, s), shfl64(r.O, s), shfl64(r.anc, s), shfl64(r.all, s), 0ull,
                            shfl64(r.rch, s), shfl64(r.vis, s), __shfl_sync(0xffffffffu, r.brick, s), r.node};
-                count_pano_brick(p, vc, pc, s_y, anc, n, nd, p.steps + (size_t)ln * AH, q, lane);
+                count_pano_brick(p, vc, pc, s_y, anc, n, nd, p.steps + (size_t)(base + ln) * AH, q, lane);
             }
         }
     }
@@ -402,6 +405,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, 4) pano_brick_kernel(const Level
     __syncthreads();
     const NodeRange nr = node_range(p);
     if (nr.q1 <= nr.q0) return;
+    const int base = p.tree ? nr.l0 + nr.q0 : 0;
     const int total = min(p.vctr[1], p.queue_cap);
     const int slice = max(1, min(64, total / (int)(gridDim.x * kWarpsN * 8)));
     if (blockIdx.x * kWarpsN * slice >= total) return;
@@ -427,7 +431,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, 4) pano_brick_kernel(const Level
                 nd = p.node[n];
                 node_ancestors(p, n, anc, WH, pyr_n, lane);
             }
-            count_pano_brick(p, vc, pc, s_y, anc, n, nd, p.steps + (size_t)cur * AH, r, lane);
+            count_pano_brick(p, vc, pc, s_y, anc, n, nd, p.steps + (size_t)(base + (int)cur) * AH, r, lane);
         }
     }
 }
@@ -440,6 +444,14 @@ void set_pano_visit(LevelParams &p, int A, float vfov_deg) {
 
 void launch_pano_cast_chunk(const LevelParams &c, int num_sms, cudaStream_t s) {
     launch_behind(pano_cast_kernel, cast_grid(c.q1 - c.q0, c.pano_A, c.H, num_sms), kWarpsN * 32, 0, s, c, num_sms);
+}
+
+void launch_pano_tree_cast(const LevelParams &p, int levels, int num_sms, cudaStream_t s) {
+    LevelParams c = p;
+    c.lvl = levels;
+    c.q0 = 0;
+    c.q1 = p.tree;
+    launch_pano_cast_chunk(c, num_sms, s);
 }
 
 void launch_pano_voxel_chunk(const LevelParams &c, int num_sms, cudaStream_t s) {

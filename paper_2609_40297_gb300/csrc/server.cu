@@ -48,6 +48,7 @@ struct Request {
     mig_sensor sensor{};
     int mode = 0;
     HostPlan plan;
+    int Lmax = 1;         // nodes of its largest level
     StepsLayout steps{};  // owned-voxel count's region (cap 0 = ray by ray)
     int32_t *out_abs = nullptr, *out_marg = nullptr, *out_yaw = nullptr;
     const Camera *cam = nullptr;
@@ -163,9 +164,14 @@ mig_status admit(mig_server *s, Request &r) {
     const size_t o_arena = cv.take(4 * (size_t)std::max(1, pl.n_internal) * WH);
     const size_t o_dpyr = cv.take(sizeof(uint2) * (size_t)std::max(1, pl.n_internal) * hz_entries(r.sensor.width, r.sensor.height));
     const size_t o_pcnt = pano ? cv.take(8 * (size_t)n * r.cam->pano_A) : 0;
-    const size_t o_steps = cv.take(r.steps.bytes);
-    r.dev_bytes = cv.off;
-    r.dev = (char *)ctx->alloc.alloc(r.dev_bytes, ctx->stream);
+    size_t o_steps = 0;
+    for (int lean = 0; lean < 3 && !r.dev; ++lean) {  // less memory where the allocator has not enough
+        if (lean) r.steps = steps_for(ctx, n, r.Lmax, r.sensor, r.map->voxel, r.mode, lean);
+        Carve c = cv;
+        o_steps = c.take(r.steps.bytes);
+        r.dev_bytes = c.off;
+        r.dev = (char *)ctx->alloc.alloc(r.dev_bytes, ctx->stream);
+    }
     if (!r.dev) return fail(MIG_ENOMEM, "server: request allocation failed");
     if (s->pinned_bytes < up) {
         if (s->pinned) {
@@ -299,6 +305,7 @@ mig_status run_step(mig_server *s) {
         const HostPlan &pl = r.plan;
         const int d = r.level;
         const int Ld = pl.level_off[d + 1] - pl.level_off[d];
+        if (d == 0) launch_tree_count(ctx, r.p, pl.max_depth + 1, st);
         launch_level_count(ctx, p, Ld, count_cap, st);
         if (pl.level_int[d] > 0) launch_select_render(p, pl.level_int[d], ctx->num_sms, st);
         else launch_select(p, std::max(1, std::min((Ld + 127) / 128, 1024)), st);
@@ -466,10 +473,13 @@ extern "C" mig_status mig_server_submit(mig_server *s, const mig_tree_desc *d, u
     r->sensor = d->sensor;
     r->mode = d->mode;
     {
-        int Lmax = 1;
         for (int lv = 0; lv <= r->plan.max_depth; ++lv)
-            Lmax = std::max(Lmax, r->plan.level_off[lv + 1] - r->plan.level_off[lv]);
-        r->steps = steps_for(s->ctx, Lmax, d->sensor, d->map->voxel, d->mode);
+            r->Lmax = std::max(r->Lmax, r->plan.level_off[lv + 1] - r->plan.level_off[lv]);
+        // the whole tree's step counts only where as many such requests as may be in flight fit the budget
+        for (int lean = 0; lean < 2; ++lean) {
+            r->steps = steps_for(s->ctx, r->plan.n, r->Lmax, d->sensor, d->map->voxel, d->mode, lean);
+            if (!r->steps.tree || request_bytes(*r) <= s->budget / (size_t)s->max_inflight) break;
+        }
     }
     r->out_abs = d->abs_gain;
     r->out_marg = d->marg_gain;

@@ -342,7 +342,7 @@ void launch_vox_level(const LevelParams &p, long long pairs, int num_sms, int vo
         LevelParams c = p;
         c.q0 = (int)q0;
         c.q1 = (int)std::min<long long>(pairs, q0 + cap);
-        launch_cast_chunk(c, num_sms, s);
+        if (!p.tree) launch_cast_chunk(c, num_sms, s);
         if (node_pass(p)) launch_node_chunk(c, num_sms, node_ctas, s);
         else launch_voxel_chunk(c, num_sms, vox_ctas, s);
     }

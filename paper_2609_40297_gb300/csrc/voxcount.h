@@ -15,7 +15,7 @@ namespace mig {
 size_t steps_pairs(long long pairs, int W, int H, size_t budget_bytes);
 // Entries of one image's tile bounds (bricks.cuh, Pyramid).
 size_t hz_entries(int W, int H);
-// The device region of an owned-voxel count for levels of at most max_nodes nodes: the step counts of
+// The device region of an owned-voxel count of a tree of n nodes with levels of at most max_nodes: the step counts of
 // `cap` pairs, the counters, the counts' tile bounds and the per-node pass's queue. The panoramic mode
 // has one image of A x H per node: W = A, K = 1.
 struct SensorDims {
@@ -24,15 +24,22 @@ struct SensorDims {
 };
 struct StepsLayout {
     int cap;        // pairs per chunk (0: the ray-by-ray count, an empty region)
+    int tree;       // 0, or the tree's nodes: the region holds all of them (cap = tree * K)
     int queue_cap;  // records
     size_t o_ctr, o_hz, o_queue, bytes;
 };
-StepsLayout steps_layout(const SensorDims &d, int max_nodes, size_t budget_bytes, bool node_pass, int mode);
+// tree_bytes: the most step counts for the whole tree (0: level by level)
+StepsLayout steps_layout(const SensorDims &d, int n, int max_nodes, size_t budget_bytes, size_t tree_bytes, bool node_pass, int mode);
 // The same for whole nodes within a region of at most `bytes` bytes (cap 0: not one node fits).
 StepsLayout steps_layout_in(const SensorDims &d, int max_nodes, size_t bytes);
 void set_steps(LevelParams &p, void *base, const StepsLayout &L);  // the region's fields
 // Step-count buffer budget per evaluation (device bytes).
 constexpr size_t kStepsBudget = (size_t)1 << 30;
+// A tree whose step counts stay below this is cast by one launch instead of level by level: a level's cast
+// needs nothing of the levels above it, and each level's cast ends with SMs idle. Cast times of 20 nodes
+// of 36x24x8: 89 -> 30 us, 100 of 48x28x8: 188 -> 76 us, 500 of 160x120x16 (307 MB, beyond L2): 6.4 -> 5.3
+// ms with an unchanged voxel stage. Larger trees have levels of several ms of cast each.
+constexpr size_t kTreeSteps = (size_t)512 << 20;
 // One level's count for the sample modes (marginal, single parent, absolute): for each chunk of
 // p.steps_cap pairs of the first `pairs` (node, yaw) pairs, a cast launch and a voxel launch. The
 // kernels read the level's true size from p.level_off and skip pairs beyond it, so `pairs` may be
@@ -42,6 +49,8 @@ constexpr size_t kStepsBudget = (size_t)1 << 30;
 void launch_vox_level(const LevelParams &p, long long pairs, int num_sms, int vox_ctas, int node_ctas, cudaStream_t s);
 // The launches of one chunk [c.q0, c.q1) (launch_vox_level runs them for every chunk).
 void launch_cast_chunk(const LevelParams &c, int num_sms, cudaStream_t s);
+// The cast of all nodes of a tree of `levels` levels (p.tree > 0), before its levels are counted.
+void launch_tree_cast(const LevelParams &p, int levels, int num_sms, cudaStream_t s);
 void launch_voxel_chunk(const LevelParams &c, int num_sms, int vox_ctas, cudaStream_t s);
 void launch_node_chunk(const LevelParams &c, int num_sms, int node_ctas, cudaStream_t s);
 bool node_pass(const LevelParams &p);  // whole nodes per chunk: the per-node pass

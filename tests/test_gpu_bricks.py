@@ -148,3 +148,66 @@ def test_noalloc_chunks(ctx, width, height, yaws):
             assert np.array_equal(a, b) and np.array_equal(a, rays[k]), k
     finally:
         m.close()
+
+
+@pytest.mark.parametrize("call", ["host", "panoramic", "interval", "device", "batch"])
+def test_less_memory(monkeypatch, call):
+    """An allocator that refuses the largest request: the tree's step counts, then the level's, then none
+    (ray by ray), with the same results."""
+    limit, asked = [1 << 62], []
+    real = mig._torch_allocator
+
+    def limited(device):
+        a = real(device)
+
+        def alloc(nbytes, stream, user):
+            asked.append(int(nbytes))
+            return None if nbytes > limit[0] else a.alloc(nbytes, stream, user)
+
+        b = mig.Allocator(mig.ALLOC_FN(alloc), a.free, None)
+        b.keep = (a, alloc)
+        return b
+
+    monkeypatch.setattr(mig, "_torch_allocator", limited)
+    p = synth.random_small(77, nx=60, ny=60, nz=30, v=0.1, p_occ=0.001, n_nodes=24, max_depth=6,
+                           sensor=Sensor(90, 60, 40, 30, 2.0, 8, 0.0))
+
+    def run(most):
+        c = mig.Context(0)
+        try:
+            m = mig.Map(c, p.map.grid, p.map.voxel_size, p.map.origin)
+            try:
+                if call == "panoramic":  # the camera's tables
+                    mig.tree_eval(m, p.tree.parent[:1], p.tree.pos[:1], p.sensor, mode=mig.MODE_PANORAMIC)
+                limit[0] = most
+                asked.clear()
+                if call == "device":
+                    par, pos = torch.from_numpy(p.tree.parent).cuda(), torch.from_numpy(p.tree.pos).cuda()
+                    o = [torch.empty(p.tree.n, dtype=torch.int32, device="cuda") for _ in range(3)]
+                    mig.tree_eval_device(m, par, pos, p.sensor, 6, *o)
+                    c.sync()
+                    return [t.cpu().numpy() for t in o]
+                if call == "batch":
+                    got = mig.tree_eval_batch(c, [(p.tree.parent, p.tree.pos, p.sensor)] * 2, [m, m])[1]
+                else:
+                    got = mig.tree_eval(m, p.tree.parent, p.tree.pos, p.sensor, mode=MODES.get(call, mig.MODE_MARGINAL)
+                                        if call != "panoramic" else mig.MODE_PANORAMIC)
+                return [got[k] for k in ("abs", "marg", "yaw")]
+            finally:
+                limit[0] = 1 << 62
+                m.close()
+        finally:
+            c.close()
+
+    want, steps, most = run(1 << 62), 0, 1 << 62
+    while True:
+        need = [b for b in asked if b <= most]
+        most = max(need) - 1
+        try:
+            got = run(most)
+        except mig.MigError:
+            break
+        steps += 1
+        assert all(np.array_equal(a, b) for a, b in zip(got, want)), steps
+    # the device call does not know its levels' sizes: there the level's step counts are the tree's
+    assert steps >= (1 if call == "device" else 2)
