@@ -85,6 +85,9 @@ struct LevelParams {
     // 0, or the tree's nodes: all of them were cast by one launch, and the step counts and bounds of the
     // i-th of level_nodes are the buffers' i-th (else a chunk's nodes are, from 0)
     int tree;
+    // NULL, or the depth buffers of all the tree's (node, yaw) pairs of internal nodes, stored by the cast:
+    // W * H per pair, in the step counts' order. The render then copies the selected yaw's.
+    uint32_t *depths;
     // per-node pass: half a pixel at unit depth along the image axes, the depth below which the owner
     // ray certainly visits its voxel, and the reciprocal focal lengths (set_visit_params)
     float vis_hu, vis_hv, vis_zl2, ifx, ify;

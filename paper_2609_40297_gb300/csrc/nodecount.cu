@@ -35,7 +35,7 @@ namespace {
 
 using namespace dev;
 
-template <bool STATS>
+template <bool STATS, bool DEPTH>
 __global__ void __launch_bounds__(kWarpsN * 32, kCastCtas) cast_kernel(const LevelParams p, int num_sms) {
     __shared__ uint2 s_t[kWarpsN];
     __shared__ float s_beam[32];
@@ -68,7 +68,8 @@ __global__ void __launch_bounds__(kWarpsN * 32, kCastCtas) cast_kernel(const Lev
         const int4 nd = p.node[p.level_nodes[l0 + q / p.K]];
         const int32_t *yk = p.yawtab + (q % p.K) * 12;
         const CameraRays rays{p, nd, yk[0], yk[1], p.W, p.H};
-        const CastOut o{p.steps + (size_t)ql * WH, p.hz + (size_t)ql * y.n};
+        const CastOut<DEPTH> o{p.steps + (size_t)ql * WH, p.hz + (size_t)ql * y.n,
+                               DEPTH && nd.w >= 0 ? p.depths + (size_t)ql * WH : nullptr};
         const int x0 = tile % tx * T, y0 = tile / tx * T;
         if (lay == kCastLarge) {
             cast_large<STATS>(p, om, dist, y, rays, x0, y0, o, lane, st);
@@ -145,10 +146,12 @@ __global__ void __launch_bounds__(kWarpsN * 32, kCastCtas) render_kernel(const L
         const int tile = it % (tx * ty);
         const int n = p.level_nodes[l0 + it / (tx * ty)];
         const int4 nd = p.node[n];
-        const int32_t *yk = p.yawtab + select_warp(p, n, tile == 0 && (lay == kCastLarge || warp == 0), lane) * 12;
+        const int k = select_warp(p, n, tile == 0 && (lay == kCastLarge || warp == 0), lane);
+        const int32_t *yk = p.yawtab + k * 12;
         if (nd.w < 0) continue;  // uniform over the warps of the item
         const CameraRays rays{p, nd, yk[0], yk[1], p.W, p.H};
-        const RenderOut o{p.dpyr ? p.dpyr + (size_t)nd.w * y.n : nullptr, nd.w};
+        const RenderOut o{p.dpyr ? p.dpyr + (size_t)nd.w * y.n : nullptr, nd.w,
+                          p.depths ? p.depths + ((size_t)(l0 + it / (tx * ty)) * p.K + k) * ((size_t)p.W * p.H) : nullptr};
         const int x0 = tile % tx * T, y0 = tile / tx * T;
         if (lay == kCastLarge) {
             cast_large<STATS>(p, om, dist, y, rays, x0, y0, o, lane, st);
@@ -687,8 +690,8 @@ void set_visit_params(LevelParams &p, float hfov_deg, float vfov_deg) {
 
 void launch_cast_chunk(const LevelParams &c, int num_sms, cudaStream_t s) {
     const int g = cast_grid(c.q1 - c.q0, c.W, c.H, num_sms);
-    if (c.stats) launch_behind(cast_kernel<true>, g, kWarpsN * 32, 0, s, c, num_sms);
-    else launch_behind(cast_kernel<false>, g, kWarpsN * 32, 0, s, c, num_sms);
+    if (c.stats) launch_behind(c.depths ? cast_kernel<true, true> : cast_kernel<true, false>, g, kWarpsN * 32, 0, s, c, num_sms);
+    else launch_behind(c.depths ? cast_kernel<false, true> : cast_kernel<false, false>, g, kWarpsN * 32, 0, s, c, num_sms);
 }
 
 void launch_tree_cast(const LevelParams &p, int levels, int num_sms, cudaStream_t s) {
@@ -763,7 +766,8 @@ static void place(StepsLayout &L, const SensorDims &d) {
     L.o_ctr = align((size_t)L.cap * d.W * d.H * sizeof(uint16_t));
     L.o_hz = L.o_ctr + 256;
     L.o_queue = align(L.o_hz + (size_t)L.cap * hz_entries(d.W, d.H) * sizeof(uint32_t));
-    L.bytes = L.o_queue + (size_t)L.queue_cap * sizeof(BrickRec);
+    L.o_depths = align(L.o_queue + (size_t)L.queue_cap * sizeof(BrickRec));
+    L.bytes = L.o_depths + (L.depths ? (size_t)L.cap * d.W * d.H * sizeof(uint32_t) : 0);
 }
 
 StepsLayout steps_layout(const SensorDims &d, int n, int max_nodes, size_t budget_bytes, size_t tree_bytes, bool node_pass, int mode) {
@@ -781,6 +785,7 @@ StepsLayout steps_layout(const SensorDims &d, int n, int max_nodes, size_t budge
             nodes >= max_nodes && (double)n * (double)node_items(d.Tq) * d.K < (double)(1ll << 30)) {
             L.tree = n;
             L.cap = n * d.K;
+            L.depths = mode != MIG_MODE_PANORAMIC && 2.0 * bytes <= (double)kTreeDepths;
         }
     }
     place(L, d);
@@ -814,6 +819,7 @@ void set_steps(LevelParams &p, void *base, const StepsLayout &L) {
     p.queue_cap = L.queue_cap;
     p.steps_cap = L.cap;
     p.tree = L.tree;
+    p.depths = L.depths ? reinterpret_cast<uint32_t *>(b + L.o_depths) : nullptr;
 }
 
 void launch_brick_update(uint8_t *grid, int nx, int ny, int nz, int x0, int y0, int z0, int dx, int dy, int dz, cudaStream_t s) {

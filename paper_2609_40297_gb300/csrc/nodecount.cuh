@@ -93,13 +93,18 @@ struct CastCnt {  // statistics
 
 // What a pass keeps per ray and per tile: the cast the step index (16 bits, bounds packed as min |
 // ~max << 16), the render the depth.
+template <bool DEPTH>
 struct CastOut {
     uint16_t *out;
     uint32_t *hz;
-    static constexpr bool kDepth = false;
+    uint32_t *depth;  // DEPTH: NULL for nodes that no descendant looks at
+    static constexpr bool kDepth = DEPTH;
     static constexpr uint32_t kMin = 0xFFFFu;
-    __device__ __forceinline__ uint32_t put(const LevelParams &, size_t i, int, uint32_t m, uint32_t, uint32_t) const {
+    __device__ __forceinline__ bool stored() const { return false; }
+    __device__ __forceinline__ uint32_t load(const LevelParams &, size_t) const { return 0u; }
+    __device__ __forceinline__ uint32_t put(const LevelParams &p, size_t i, int dzc, uint32_t m, uint32_t ne, uint32_t ade) const {
         out[i] = (uint16_t)m;
+        if (DEPTH && depth) depth[i] = hit_depth(m != kNoHit, ne, ade, dzc, p.Tq);
         return m;
     }
     __device__ __forceinline__ void tile(size_t i, uint32_t lo, uint32_t hi) const { hz[i] = lo | ((hi ^ 0xFFFFu) << 16); }
@@ -107,8 +112,15 @@ struct CastOut {
 struct RenderOut {
     uint2 *pyr;  // NULL: not kept
     int slot;
+    const uint32_t *src;  // NULL, or the depths that the cast stored
     static constexpr bool kDepth = true;
     static constexpr uint32_t kMin = 0xFFFFFFFFu;
+    __device__ __forceinline__ bool stored() const { return src != nullptr; }
+    __device__ __forceinline__ uint32_t load(const LevelParams &p, size_t i) const {
+        const uint32_t D = __ldg(src + i);
+        arena_store(p.arena, p.arena_slots, slot, i, (size_t)p.W * p.H, D, p.bounds_err);
+        return D;
+    }
     __device__ __forceinline__ uint32_t put(const LevelParams &p, size_t i, int dzc, uint32_t m, uint32_t ne, uint32_t ade) const {
         const uint32_t D = hit_depth(m != kNoHit, ne, ade, dzc, p.Tq);
         arena_store(p.arena, p.arena_slots, slot, i, (size_t)p.W * p.H, D, p.bounds_err);
@@ -144,20 +156,25 @@ __device__ __forceinline__ void cast_part(const LevelParams &p, const uint64_t *
     const int i = i0 + (lane & 7), j = j0 + (lane >> 3);
     if (i >= r.W || j >= r.H) return;
     const size_t at = (size_t)j * r.W + i;
-    RayHit hit{kNoHit, 0, 1};
-    int dzc = 0;
-    if (OUT::kDepth || beam < 1e29f) {
-        const int4 b = r.ray(i, j);
-        dzc = b.w;
-        if (beam < 1e29f) {
-            int dx, dy, dz;
-            r.dir(b, dx, dy, dz);
-            const uint8_t *oct = p.grid.g + oct_offset(p.grid.nx, p.grid.ny, p.grid.nz, octant_of(dx, dy, dz));
-            hit = cast_ray<STATS, OUT::kDepth>(om, oct, p.grid.nx, p.grid.ny, p.grid.nz, r.nd.x, r.nd.y, r.nd.z, dx, dy, dz, (int)p.Tq,
-                                               beam_time(beam, b.w), &st);
+    uint32_t v;
+    if (o.stored()) {
+        v = o.load(p, at);
+    } else {
+        RayHit hit{kNoHit, 0, 1};
+        int dzc = 0;
+        if (OUT::kDepth || beam < 1e29f) {
+            const int4 b = r.ray(i, j);
+            dzc = b.w;
+            if (beam < 1e29f) {
+                int dx, dy, dz;
+                r.dir(b, dx, dy, dz);
+                const uint8_t *oct = p.grid.g + oct_offset(p.grid.nx, p.grid.ny, p.grid.nz, octant_of(dx, dy, dz));
+                hit = cast_ray<STATS, OUT::kDepth>(om, oct, p.grid.nx, p.grid.ny, p.grid.nz, r.nd.x, r.nd.y, r.nd.z, dx, dy, dz, (int)p.Tq,
+                                                   beam_time(beam, b.w), &st);
+            }
         }
+        v = o.put(p, at, dzc, hit.m, hit.ne, hit.ade);
     }
-    const uint32_t v = o.put(p, at, dzc, hit.m, hit.ne, hit.ade);
     lo = min(lo, v);
     hi = max(hi, v);
     if constexpr (STATS) ++st.rays;

@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, kCastCtas) pano_cast_kernel(cons
         const int tile = (int)(it % (tx * ty)), ln = (int)(it / (tx * ty));
         const int n = p.level_nodes[nr.l0 + nr.q0 + ln];
         const PanoRays rays{p, p.node[n], A, H};
-        const CastOut o{p.steps + (size_t)ln * AH, p.hz + (size_t)ln * y.n};
+        const CastOut<false> o{p.steps + (size_t)ln * AH, p.hz + (size_t)ln * y.n, nullptr};
         const int x0 = tile % tx * T, y0 = tile / tx * T;
         if (y0 == 0) {  // the first row of tiles clears its columns' counts
             const int c = x0 + (lay == kCastLarge ? lane : (int)threadIdx.x);

@@ -26,7 +26,8 @@ struct StepsLayout {
     int cap;        // pairs per chunk (0: the ray-by-ray count, an empty region)
     int tree;       // 0, or the tree's nodes: the region holds all of them (cap = tree * K)
     int queue_cap;  // records
-    size_t o_ctr, o_hz, o_queue, bytes;
+    bool depths;    // the tree's depth buffers, all yaws
+    size_t o_ctr, o_hz, o_queue, o_depths, bytes;
 };
 // tree_bytes: the most step counts for the whole tree (0: level by level)
 StepsLayout steps_layout(const SensorDims &d, int n, int max_nodes, size_t budget_bytes, size_t tree_bytes, bool node_pass, int mode);
@@ -40,6 +41,11 @@ constexpr size_t kStepsBudget = (size_t)1 << 30;
 // of 36x24x8: 89 -> 30 us, 100 of 48x28x8: 188 -> 76 us, 500 of 160x120x16 (307 MB, beyond L2): 6.4 -> 5.3
 // ms with an unchanged voxel stage. Larger trees have levels of several ms of cast each.
 constexpr size_t kTreeSteps = (size_t)512 << 20;
+// A tree whose depth buffers, those of every yaw of its nodes, stay below this has them stored by the cast,
+// and its levels' renders are copies: 63 -> 34 us of render for 20 nodes of 36x24x8 (4 levels), 145 -> 74 for
+// 100 of 48x28x8 (9), the cast within 10 us. For larger trees the stores cost more than they save: the cast
+// of 500 nodes of 160x120x16 5.3 -> 5.9 ms, the render 0.43 -> 0.28.
+constexpr size_t kTreeDepths = (size_t)64 << 20;
 // One level's count for the sample modes (marginal, single parent, absolute): for each chunk of
 // p.steps_cap pairs of the first `pairs` (node, yaw) pairs, a cast launch and a voxel launch. The
 // kernels read the level's true size from p.level_off and skip pairs beyond it, so `pairs` may be
