@@ -249,11 +249,36 @@ void launch_device_levels(mig_ctx *ctx, LevelParams p, int n, int levels, int2 *
     }
 }
 
-StepsLayout steps_for(const mig_ctx *ctx, int n, int Lmax, const mig_sensor &s, float voxel, int mode, int lean) {
+// Microseconds of the two ways to count a tree, fitted to 150 timings (200 to 1200 nodes, range R = 60 to
+// 150 voxels, images of 16x12 to 192x144, 4 to 36 yaws, both kinds of world):
+//   ray by ray - a chain of voxel loads as long as the range per level, and each ray's walk:
+//                ch R levels + r R rays;
+//   by voxels  - each node's range ball between the image's elevations, and each yaw's frustum of it:
+//                R^3 n sin(vfov / 2) (a + b K hfov / 90).
+// Voxels that lie closer than the image's pixels are mostly on no ray at all, so that a coarse image over
+// a long range is walked sooner than enumerated: 1000 nodes, R = 150, 16 yaws of 56x42 count in 68 ms
+// ray by ray and 184 by voxels, of 128x96 in 251 and 201 (interval 147 and 387, 468 and 454; panoramic
+// 27 and 50, 88 and 51); the estimates' order was the timings' wherever these differed by a quarter.
+bool rays_cheaper(const mig_sensor &s, float voxel, int n, int levels, int mode) {
+    struct {
+        double chain, ray, a, b;
+    } c = {5.7, 10.5e-6, 20e-6, 5.7e-6};
+    double rays = (double)s.yaw_bins * s.width * s.height;
+    if (mode == MIG_MODE_INTERVAL) c = {14.7, 20e-6, 0.0, 15.4e-6};
+    if (mode == MIG_MODE_PANORAMIC) {
+        c = {2.3, 15e-6, 31e-6, 0.0};
+        rays = (double)pano_columns(s) * s.height;
+    }
+    const double R = s.range_m / voxel, ball = R * R * R * n * std::sin(s.vfov_deg * (M_PI / 360.0));
+    return c.chain * R * levels + c.ray * R * n * rays < ball * (c.a + c.b * s.yaw_bins * (s.hfov_deg / 90.0));
+}
+
+StepsLayout steps_for(const mig_ctx *ctx, int n, int levels, int Lmax, const mig_sensor &s, float voxel, int mode, int lean) {
     const bool pano = mode == MIG_MODE_PANORAMIC, whole = pano || mode == MIG_MODE_INTERVAL;
     // the interval and panoramic modes have no pass per (node, yaw) pair: without room for whole nodes they
     // count ray by ray
     if (ctx->ray_count || lean == 2 || (whole && ctx->voxel_pass == MIG_COUNT_PAIRS)) return StepsLayout{};
+    if (ctx->voxel_pass == MIG_COUNT_AUTO && rays_cheaper(s, voxel, n, levels, mode)) return StepsLayout{};
     SensorDims d{s.width, s.height, s.yaw_bins, range_q16(s.range_m, voxel)};
     if (pano) {
         d.W = pano_columns(s);
@@ -664,7 +689,7 @@ static mig_status eval_host(mig_map *m, int n, const int32_t *parent, const floa
     char *dev = nullptr;
     for (int lean = 0; lean < 3; ++lean) {  // less memory where the allocator has not enough
         Carver c = cv;
-        steps = steps_for(ctx, n, Lmax, *sensor, m->voxel, mode, lean);
+        steps = steps_for(ctx, n, L, Lmax, *sensor, m->voxel, mode, lean);
         o_dpyr = c.take<uint2>(steps.cap ? (size_t)std::max(1, plan.n_internal) * hz_entries(cam->W, cam->H) : 0);
         o_steps = c.take<char>(steps.bytes);
         // instrumented pass: the ray-by-ray count kernel is re-run into scratch counters afterwards,
@@ -848,7 +873,7 @@ mig_status mig_tree_eval_device(mig_map *m, int n, const int32_t *parent, const 
         o_err = cv.take<int32_t>(1); o_cnt = cv.take<int32_t>((size_t)n * K * 2);
         o_work = cv.take<int32_t>(L);
         // level sizes are known on the device only: the step-count buffer is sized for n nodes
-        steps = steps_for(ctx, n, n, *sensor, m->voxel, MIG_MODE_MARGINAL, lean);
+        steps = steps_for(ctx, n, L, n, *sensor, m->voxel, MIG_MODE_MARGINAL, lean);
         o_cursor = cv.take<int2>(device_steps(steps, n, K, L) + 1);
         zero_bytes = cv.off;
         o_depth = cv.take<int32_t>(n); o_loff = cv.take<int32_t>(L + 1); o_lint = cv.take<int32_t>(L);

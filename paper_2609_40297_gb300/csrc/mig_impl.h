@@ -171,10 +171,11 @@ void launch_tree_count(const mig_ctx *ctx, const LevelParams &p, int levels, cud
 // The same on the context stream, each launch timed under its own kind (mig_ctx_profile).
 void launch_level_count_timed(mig_ctx *ctx, const LevelParams &p, int Ld, int count_cap);
 // The owned-voxel count's region for a tree of n nodes whose widest level has Lmax (empty when the context
-// counts ray by ray or the mode does). lean 0: the whole tree's step counts if small, 1: a level's, 2: none
+// counts ray by ray, the mode does, or that is the cheaper way, rays_cheaper). lean 0: the whole tree's step counts if small, 1: a level's, 2: none
 // (ray by ray); a caller whose allocation fails takes the next.
 struct StepsLayout;
-StepsLayout steps_for(const mig_ctx *ctx, int n, int Lmax, const mig_sensor &s, float voxel, int mode, int lean);
+bool rays_cheaper(const mig_sensor &s, float voxel, int n, int levels, int mode);
+StepsLayout steps_for(const mig_ctx *ctx, int n, int levels, int Lmax, const mig_sensor &s, float voxel, int mode, int lean);
 // The count and select-and-render launches of a device-planned tree of n nodes and at most `levels` levels.
 // With the per-node pass they go chunk by chunk through the levels, whose sizes only the device knows:
 // device_steps(..) steps and as many places + 1 in `cursor` (zeroed).

@@ -64,7 +64,7 @@ def test_bricks_equal_rays(ctx, ci, mode):
     try:
         rays = _eval(ctx, m, p, MODES[mode], mig.COUNT_RAYS)
         assert rays["abs"].sum() > 0
-        _same(_eval(ctx, m, p, MODES[mode], mig.COUNT_AUTO), rays, (ci, mode))
+        _same(_eval(ctx, m, p, MODES[mode], mig.COUNT_NODES), rays, (ci, mode))
     finally:
         m.close()
 
@@ -92,7 +92,7 @@ def test_panoramic_bricks_equal_rays(ctx, ci, budget):
     try:
         rays = _eval(ctx, m, p, mig.MODE_PANORAMIC, mig.COUNT_RAYS)
         assert rays["abs"].sum() > 0
-        ctx.set_count_kernel(mig.COUNT_AUTO, budget)
+        ctx.set_count_kernel(mig.COUNT_NODES, budget)
         try:
             got = mig.tree_eval(m, p.tree.parent, p.tree.pos, p.sensor, mode=mig.MODE_PANORAMIC, want_counts=True,
                                 want_depth=True)
@@ -121,7 +121,7 @@ def test_brick_data_follows_updates(ctx, mode):
             g[z:z + d[2], y:y + d[1], x:x + d[0]] = box
             fresh = mig.Map(ctx, g, p.map.voxel_size, p.map.origin)
             try:
-                _same(_eval(ctx, m, p, MODES[mode], mig.COUNT_AUTO), _eval(ctx, fresh, p, MODES[mode], mig.COUNT_RAYS), i)
+                _same(_eval(ctx, m, p, MODES[mode], mig.COUNT_NODES), _eval(ctx, fresh, p, MODES[mode], mig.COUNT_RAYS), i)
             finally:
                 fresh.close()
     finally:
@@ -211,3 +211,38 @@ def test_less_memory(monkeypatch, call):
         assert all(np.array_equal(a, b) for a, b in zip(got, want)), steps
     # the device call does not know its levels' sizes: there the level's step counts are the tree's
     assert steps >= (1 if call == "device" else 2)
+
+
+@pytest.mark.parametrize("call", ["marginal", "interval", "panoramic", "device", "noalloc"])
+@pytest.mark.parametrize("width,height", [(6, 4), (160, 120)])
+def test_coarse_images_are_walked(ctx, call, width, height):
+    """An image whose pixels lie farther apart than the voxels over most of the range (the default counts it
+    ray by ray) and a fine one: equal to the count by voxels."""
+    p = synth.random_small(91, nx=130, ny=120, nz=50, v=0.1, p_occ=0.0003, n_nodes=200, max_depth=2,
+                           sensor=Sensor(90, 60, width, height, 9.0, 16 if width < 10 else 2, 0.0))
+    m = mig.Map(ctx, p.map.grid, p.map.voxel_size, p.map.origin)
+    dev = torch.device("cuda:0")
+    par, pos = torch.from_numpy(p.tree.parent).to(dev), torch.from_numpy(p.tree.pos).to(dev)
+    try:
+        outs = []
+        for kernel in (mig.COUNT_AUTO, mig.COUNT_NODES):
+            if call in ("device", "noalloc"):
+                ctx.set_count_kernel(kernel, 0)
+                o = [torch.full((p.tree.n,), -7, dtype=torch.int32, device=dev) for _ in range(3)]
+                try:
+                    (mig.tree_eval_device if call == "device" else mig.tree_eval_device_noalloc)(m, par, pos, p.sensor, 2, *o)
+                    ctx.sync()
+                finally:
+                    ctx.set_count_kernel(mig.COUNT_AUTO, 0)
+                outs.append(dict(zip(("abs", "marg", "yaw"), [t.cpu().numpy() for t in o])))
+            else:
+                outs.append(_eval(ctx, m, p, MODES.get(call, mig.MODE_PANORAMIC), kernel))
+        assert outs[0]["abs"].sum() > 0
+        for k in outs[0]:
+            if isinstance(outs[0][k], np.ndarray):
+                assert np.array_equal(outs[0][k], outs[1][k]), k
+        if call == "marginal":
+            st = mig.tree_eval_stats(m, p.tree.parent, p.tree.pos, p.sensor)[1]
+            assert st["voxel_pass"] == (mig.COUNT_RAYS if width < 10 else mig.COUNT_NODES)
+    finally:
+        m.close()
