@@ -146,11 +146,11 @@ def spread(xs):
 # -------------------------------------------------------------------- kernels and roofline
 # Source files whose code (comments and blank lines removed) an ncu summary is tied to.
 KERNEL_SOURCES = {
-    "cast_kernel": ("voxcount.cu", "voxcount.cuh", "voxitems.cuh", "dev_path.cuh", "kernels.h"),
-    "voxel_kernel": ("voxcount.cu", "voxcount.cuh", "voxitems.cuh", "dev_path.cuh", "kernels.h"),
-    "node_kernel": ("voxcount.cu", "voxcount.cuh", "voxitems.cuh", "dev_path.cuh", "kernels.h"),
+    "cast_kernel": ("nodecount.cu", "nodecount.cuh", "bricks.cuh", "dev_path.cuh", "kernels.h"),
+    "voxel_kernel": ("voxcount.cu", "voxcount.cuh", "dev_path.cuh", "kernels.h"),
+    "node_kernel": ("nodecount.cu", "nodecount.cuh", "bricks.cuh", "interval.cuh", "dev_path.cuh", "kernels.h"),
     "count_kernel": ("kernels.cu", "kernels.h", "dev_path.cuh"),
-    "render_kernel": ("kernels.cu", "kernels.h", "dev_path.cuh"),
+    "render_kernel": ("nodecount.cu", "nodecount.cuh", "bricks.cuh", "dev_path.cuh", "kernels.h"),
 }
 
 
@@ -187,15 +187,19 @@ def profiled(kernel, workload):
 
 
 # Algorithmic bytes per unit of work (the roofline's per-unit figures, applied to the units each
-# kernel processes): a voxel step or a brick jump reads 1 B; a cast ray reads its 16 B ray-table
-# entry and writes its 2 B step count; an enumerated voxel reads 1 B; a counted sample reads its
-# owner pixel's 2 B step count and 16 B ray entry; an ancestor test that reaches the buffer reads
-# a 4 B depth texel; a rendered pixel writes a 4 B texel.
+# kernel processes): a voxel step or a jump reads 1 B; a cast ray reads its 16 B ray-table entry and
+# writes its 2 B step count; the per-pair pass reads 1 B per enumerated voxel and, per counted sample,
+# its owner pixel's 2 B step count and 16 B ray entry; the per-node pass reads a 4 B tile bound per
+# (64-voxel brick, yaw) pair; an ancestor test that reaches the buffer reads a 4 B depth texel; a
+# rendered pixel writes a 4 B texel.
 def kernel_units(kernel, st):
     if kernel == "cast_kernel":
         return (st["cast_steps"] + st["cast_jumps"] + 18 * st["cast_rays"],
                 "voxel steps + brick jumps (1 B each) + cast rays (16 B ray entry + 2 B step count)")
-    if kernel in ("voxel_kernel", "node_kernel"):
+    if kernel == "node_kernel":
+        return (st["voxel_candidates"] // 64 * 4 + 4 * st["voxel_depth_reads"],
+                "(4x4x4 brick, yaw) pairs (4 B tile bound) + depth reads (4 B); node and brick kernel together")
+    if kernel == "voxel_kernel":
         return (st["voxel_candidates"] + 18 * st["owned_samples"] + 4 * st["voxel_depth_reads"],
                 "enumerated voxels (1 B) + counted samples (2 B step count + 16 B ray entry) + depth reads (4 B)")
     if kernel == "count_kernel":
@@ -339,7 +343,8 @@ def measure_single(workload, steps, warmup, with_modes=False, count_pass="auto",
     prof = profiled(kernel, workload)
     count_pass_ms = (kms["cast"] + kms["voxel"] + kms["count"]) / steps
     n_launches = int(ktimes["count_launches"] + ktimes["select_launches"] + ktimes["render_launches"] +
-                     ktimes["plan_launches"] * 4 + ktimes["cast_launches"] + ktimes["voxel_launches"])
+                     ktimes["plan_launches"] * 4 + ktimes["cast_launches"] +
+                     ktimes["voxel_launches"] * (2 if stats.get("voxel_pass") == 3 else 1))
     sm_count = torch.cuda.get_device_properties(dev).multi_processor_count
     res = {
         "metric": METRIC, "value": value, "unit": "rays/s", "n_gpus": ws, "steps": steps, "warmup": warmup,
@@ -363,8 +368,8 @@ def measure_single(workload, steps, warmup, with_modes=False, count_pass="auto",
                      "avg_launch_ms": avg_launch_s * 1e3, "launches_per_step": lps,
                      "units": unit_desc, "peak_source": f"{peak_kind} HBM copy bandwidth (MEASURED_PEAKS.json hbm_gbs)",
                      "ncu": prof,
-                     "note": "the kernel is bound by integer issue and L2-served gathers, not by HBM: its data "
-                             "(map, step counts, depth buffers) stays L2-resident between its loads"},
+                     "note": "the kernel is bound by instruction issue, not by HBM: most voxels are decided as "
+                             "whole bricks, and its data (masks, bounds, depth buffers) stays L2-resident"},
         "method_work": {"bytes_per_step": method_bytes(stats),
                         "gb_per_s_over_count_pass": method_bytes(stats) / (count_pass_ms / 1e3) / 1e9,
                         "count_pass_ms": count_pass_ms,

@@ -1,4 +1,5 @@
-// Interval-mode count pass, ray by ray (where the per-node pass of nodecount.cu does not apply): the paper's screen-space overlap test (Sec. IV-B, Eq. 5-7).
+// Interval-mode count pass, ray by ray (where the per-node pass of nodecount.cu does not apply or is the
+// slower one): the paper's screen-space overlap test (Sec. IV-B, Eq. 5-7).
 //
 // For every candidate ray the 3D DDA (Sec. IV-B) visits voxels exactly as in the sample mode;
 // each owned unknown voxel (its centre projects into the ray's pixel) counts as absolute gain and
