@@ -45,7 +45,7 @@ struct LevelParams {
     int32_t *sel_yaw;           // device, n (written by select)
     uint32_t *arena;            // device, slots * W * H depth buffers
     int32_t *cnt;               // device, n*K*2 (abs, excl) counts
-    int32_t *work;              // device, levels: count-pass work counters (zeroed)
+    int32_t *work;              // device, levels: count-pass work counters (zeroed); [0] also the cast's
     int32_t *out_abs, *out_marg, *out_yaw;  // device, n
     int mode;                   // mig_mode
     int lvl;

@@ -34,10 +34,10 @@ __device__ __forceinline__ float q16f(int v) { return (float)v * (1.0f / 65536.0
 // The rays of an image are cast 8x4 pixels at a time, one ray per lane. Before that, lanes follow one
 // such part each as a beam (beam_free): the part's rays start where the beam stopped, and are not
 // cast at all if it met nothing within the range (60 % of the parts on the large workload, 16 % at
-// paper scale). Three layouts, by the number of tiles of the level:
-//   large - one warp per 32x32 pixel tile, its 32 parts' beams on its 32 lanes;
-//   mid   - one CTA per 32x32 tile, the beams on its first warp, for levels of fewer tiles than keep every
-//           warp busy with several;
+// paper scale). Three layouts, by the number of tiles of the launch:
+//   large - one warp per 32x32 pixel tile, its 32 parts' beams on its 32 lanes, from 3 tiles per resident
+//           warp on (6 and 1.5 measured the same or slower, 1.5 by a fifth in the smallest launches);
+//   mid   - one CTA per 32x32 tile, the beams on its first warp;
 //   small - one CTA per 16x16 tile, one part per warp, no beams and no 32x32 bounds, for levels that do
 //           not fill the GPU: their time is one warp's chain of dependent steps.
 // The level's size is only known on the device (tree_eval_device), so the kernels choose.
@@ -45,7 +45,7 @@ constexpr int kCastCtas = 4;  // resident CTAs per SM (64 registers; 3 CTAs of 8
 enum CastLayout { kCastSmall, kCastMid, kCastLarge };
 __device__ __forceinline__ CastLayout cast_layout(long long images, int W, int H, int num_sms) {
     const long long tiles = images * ((W + 31) >> 5) * ((H + 31) >> 5), warps = (long long)num_sms * kCastCtas * kWarpsN;
-    return tiles >= 6 * warps ? kCastLarge : (2 * tiles >= warps ? kCastMid : kCastSmall);
+    return tiles >= 3 * warps ? kCastLarge : (2 * tiles >= warps ? kCastMid : kCastSmall);
 }
 
 // The rays of a yaw's image from node nd.
@@ -580,9 +580,9 @@ __device__ __forceinline__ uint64_t voxel_ancestors(const LevelParams &p, const 
 
 // CTAs for a cast of `images` images (an upper bound of the level's): one per 16x16 tile, at most as
 // many as keep the kernel's loops short.
-inline int cast_grid(long long images, int W, int H, int num_sms) {
+inline int cast_grid(long long images, int W, int H, int num_sms, int per_sm) {
     const long long tiles = images * ((W + 15) / 16) * ((H + 15) / 16);
-    return (int)std::max<long long>(1, std::min<long long>(tiles, (long long)num_sms * 64));
+    return (int)std::max<long long>(1, std::min<long long>(tiles, (long long)num_sms * per_sm));
 }
 
 // Shared memory of a CTA: the yaws' rows and each warp's ancestors.

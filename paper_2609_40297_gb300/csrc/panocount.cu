@@ -97,8 +97,11 @@ __global__ void __launch_bounds__(kWarpsN * 32, kCastCtas) pano_cast_kernel(cons
     const uint8_t *dist = p.grid.g + dist_offset(p.grid.nx, p.grid.ny, p.grid.nz);
     CastCnt st;
     const long long items = (long long)(nr.q1 - nr.q0) * tx * ty;
-    const int per = lay == kCastLarge ? kWarpsN : 1, mine = lay == kCastLarge ? warp : 0;  // items at a time per CTA
-    for (long long it = (long long)blockIdx.x * per + mine; it < items; it += (long long)gridDim.x * per) {
+    const bool dyn = lay == kCastLarge;  // tile by tile, as in cast_kernel
+    long long it = dyn ? __shfl_sync(0xffffffffu, lane == 0 ? atomicAdd(p.work, 1) : 0, 0) : (long long)blockIdx.x;
+    while (it < items) {
+        int more = 0;
+        if (dyn && lane == 0) more = atomicAdd(p.work, 1);
         const int tile = (int)(it % (tx * ty)), ln = (int)(it / (tx * ty));
         const int n = p.level_nodes[nr.l0 + nr.q0 + ln];
         const PanoRays rays{p, p.node[n], A, H};
@@ -115,6 +118,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, kCastCtas) pano_cast_kernel(cons
         } else {
             cast_small<false>(p, om, dist, y, rays, x0, y0, o, s_t, warp, lane, st);
         }
+        it = dyn ? __shfl_sync(0xffffffffu, more, 0) : it + gridDim.x;
     }
 }
 
@@ -303,6 +307,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, 3) pano_node_kernel(const LevelP
     for (int k = threadIdx.x; k < p.K; k += blockDim.x)
         s_y[k] = yaw_rows(p.yawtab + k * 12, p.W, p.H, p.vis_hu, p.vis_hv, p.ifx, p.ify);
     wait_previous();
+    if (blockIdx.x == 0 && threadIdx.x == 0) p.work[0] = 0;  // the next cast's tiles
     __syncthreads();
     const NodeRange nr = node_range(p);
     const int nn = nr.q1 - nr.q0;
@@ -445,7 +450,7 @@ void set_pano_visit(LevelParams &p, int A, float vfov_deg) {
 }
 
 void launch_pano_cast_chunk(const LevelParams &c, int num_sms, cudaStream_t s) {
-    launch_behind(pano_cast_kernel, cast_grid(c.q1 - c.q0, c.pano_A, c.H, num_sms), kWarpsN * 32, 0, s, c, num_sms);
+    launch_behind(pano_cast_kernel, cast_grid(c.q1 - c.q0, c.pano_A, c.H, num_sms, 64), kWarpsN * 32, 0, s, c, num_sms);
 }
 
 void launch_pano_tree_cast(const LevelParams &p, int levels, int num_sms, cudaStream_t s) {

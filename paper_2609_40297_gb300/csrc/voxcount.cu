@@ -51,6 +51,7 @@ __global__ void __launch_bounds__(kVoxWarps * 32, 3) voxel_kernel(const LevelPar
     const unsigned lt_mask = (1u << lane) - 1u;
     AncRec *anc = s_anc_dyn + warp * p.max_anc;
     VoxQueues &Q = s_vq[warp];
+    if (blockIdx.x == 0 && threadIdx.x == 0) p.work[0] = 0;  // the next cast's tiles
     const int l0 = p.level_off[p.lvl];
     const int q1 = min(p.q1, level_pairs(p));
     if (p.q0 >= q1) return;
