@@ -12,7 +12,7 @@ from test_kernel_helpers_host import HERE, ROOT, _nvcc
 
 
 @pytest.fixture(scope="module")
-def checker(tmp_path_factory):
+def program(tmp_path_factory):
     nvcc = _nvcc()
     if nvcc is None:
         pytest.skip("nvcc not found")
@@ -25,8 +25,8 @@ def checker(tmp_path_factory):
 
 
 @pytest.mark.parametrize("seed", [1, 2])
-def test_brick_steps_agree_with_their_definitions(checker, seed):
-    r = subprocess.run([checker, str(seed)], capture_output=True, text=True, timeout=600)
+def test_brick_steps_agree_with_their_definitions(program, seed):
+    r = subprocess.run([program, str(seed)], capture_output=True, text=True, timeout=600)
     c = {k: int(v) for k, v in re.findall(r"(\w+) (\d+)", r.stdout)}
     assert r.returncode == 0, r.stdout[-2000:]
     assert c["hits"] > 10_000 and c["inside"] > 10_000 and c["outside"] > 10_000 and c["sure"] > 1_000_000
