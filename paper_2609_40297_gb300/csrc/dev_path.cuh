@@ -57,6 +57,16 @@ __device__ __forceinline__ bool in_bounds(int32_t *err, bool ok, int bit) {
 #endif
 }
 
+// A value that the kernels before this one (launch.cuh) or other CTAs of this kernel (batch.cu) store: step
+// counts, tile bounds, depths. The reader's lifetime overlaps the writer's, and __ldg is only defined for
+// memory that nothing writes while the kernel runs (the map and the camera tables), so these are ordinary
+// global loads, ordered by the wait or fence before them.
+template <class T>
+__device__ __forceinline__ T ld_written(const T *p) {
+    __builtin_assume(__isGlobal(p));
+    return *p;
+}
+
 __device__ __forceinline__ uint32_t grid_cells(int nx, int ny, int nz) {
 #if MIG_LAYOUT == 1
     return (uint32_t)nx * (uint32_t)ny * (uint32_t)nz;
@@ -302,7 +312,7 @@ __device__ __forceinline__ bool observed(const HOT &p, const AncRec *anc, int na
         const float vf = fmaf(A.m[3], rx, fmaf(A.m[4], ry, A.m[5] * rz)) * zi;
         int pu, pv;
         if (!pixel_in(Ua, Za, uf, p.W(), pu) || !pixel_in(Va, Za, vf, p.H(), pv)) continue;
-        const uint32_t D = __ldg(A.D + pv * p.W() + pu);
+        const uint32_t D = ld_written(A.D + pv * p.W() + pu);
         if constexpr (STATS) ++st_reads;
         if (Za < (((int64_t)D + 1) << 16)) return true;  // z <= D
     }

@@ -173,7 +173,7 @@ __device__ __forceinline__ bool seg_lookup(const Seg &g, int W, int H, const uin
     if (g.s1 < s_out) s_out = g.s1;
     const float sm = fmul(fadd(s_in, s_out), 0.5f);
     const float wm = fadd(g.wa, fmul(sm, fsub(g.wb, g.wa)));
-    const float Dv = fmul(__uint2float_rn(__ldg(D + (size_t)j * W + i)), 1.52587890625e-05f);
+    const float Dv = fmul(__uint2float_rn(ld_written(D + (size_t)j * W + i)), 1.52587890625e-05f);
     return fmul(wm, Dv) >= 1.0f;  // z <= D in inverse depth
 }
 

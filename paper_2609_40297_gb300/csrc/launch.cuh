@@ -3,9 +3,12 @@
 // sets up what does not depend on it, and waits on the device for its end: a small level's time is its
 // chain of launches, and this takes the launch and the first CTAs' start out of the chain (338 -> 311 us
 // for 24 launches over a 20-node tree, 10.3 -> 10.0 ms for 60 at paper scale).
-// Every such kernel calls wait_previous() before its first access to memory that a kernel before it
+// Every such kernel calls wait_previous() before its first access to memory that a kernel of the chain
 // writes or reads, in all threads and on every way to its end, so that the end of a kernel implies the
-// end of all before it.
+// end of all before it. What it reads before that is the camera's yaw table, which no kernel of the chain
+// writes: the copy or the kernels (noalloc.cu) that fill it come before the chain's first launch and never
+// let a launch start early. Two neighbours' lifetimes overlap, so what one of the chain wrote is read by
+// ld_written (dev_path.cuh), never through __ldg.
 #pragma once
 
 #include <cuda_runtime.h>

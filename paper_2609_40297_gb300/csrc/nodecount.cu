@@ -316,7 +316,7 @@ __device__ __forceinline__ void count_brick(const LevelParams &p, const VoxConst
                 int m[2] = {0, 0};
 #pragma unroll
                 for (int h = 0; h < 2; ++h)
-                    if (c[h]) m[h] = __ldg(stp + pix[h]);
+                    if (c[h]) m[h] = ld_written(stp + pix[h]);
                 c[0] = man[0] < m[0];
                 c[1] = man[1] < m[1];
             }

@@ -117,7 +117,7 @@ struct RenderOut {
     static constexpr uint32_t kMin = 0xFFFFFFFFu;
     __device__ __forceinline__ bool stored() const { return src != nullptr; }
     __device__ __forceinline__ uint32_t load(const LevelParams &p, size_t i) const {
-        const uint32_t D = __ldg(src + i);
+        const uint32_t D = ld_written(src + i);
         arena_store(p.arena, p.arena_slots, slot, i, (size_t)p.W * p.H, D, p.bounds_err);
         return D;
     }
@@ -345,7 +345,7 @@ __device__ __forceinline__ uint32_t hz_box(const uint32_t *hz, const Pyramid &y,
 #pragma unroll 1
     for (int ty = b.v0 >> sh; ty <= (b.v1 >> sh); ++ty)
 #pragma unroll 1
-        for (int tx = b.u0 >> sh; tx <= (b.u1 >> sh); ++tx) r = __vminu2(r, __ldg(t + ty * w + tx));
+        for (int tx = b.u0 >> sh; tx <= (b.u1 >> sh); ++tx) r = __vminu2(r, ld_written(t + ty * w + tx));
     return r;
 }
 // Bounds of the stored depths under a pixel box (the 32x32 level is not kept by every render).
@@ -358,7 +358,7 @@ __device__ __forceinline__ uint2 depth_box(const uint2 *pyr, const Pyramid &y, c
     for (int ty = b.v0 >> sh; ty <= (b.v1 >> sh); ++ty)
 #pragma unroll 1
         for (int tx = b.u0 >> sh; tx <= (b.u1 >> sh); ++tx) {
-            const uint2 v = __ldg(t + ty * w + tx);
+            const uint2 v = ld_written(t + ty * w + tx);
             r.x = min(r.x, v.x);
             r.y = max(r.y, v.y);
         }
@@ -405,7 +405,7 @@ __device__ __noinline__ int pixel_exact(const int32_t *row, int rx, int ry, int 
 __device__ __noinline__ bool observed_exact(const int32_t *row, int rx, int ry, int rz, int W, int H, const uint32_t *D) {
     int64_t Z;
     const int pix = pixel_index(row, rx, ry, rz, W, H, Z);
-    return pix >= 0 && Z < (((int64_t)__ldg(D + pix) + 1) << 16);
+    return pix >= 0 && Z < (((int64_t)ld_written(D + pix) + 1) << 16);
 }
 // The exact visit test of a voxel by its owner ray.
 __device__ __noinline__ bool visit_exact(int Px, int Py, int Pz, int bx, int by, int bz, int ck, int sk, int x, int y, int z,
@@ -562,7 +562,7 @@ __device__ __forceinline__ uint64_t voxel_ancestors(const LevelParams &p, const 
         uint32_t D[2] = {0u, 0u};
 #pragma unroll
         for (int h = 0; h < 2; ++h)
-            if (in[h] > 0) D[h] = __ldg(A.D + pix[h]);
+            if (in[h] > 0) D[h] = ld_written(A.D + pix[h]);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             if constexpr (STATS) st.reads += in[h] > 0;

@@ -272,7 +272,7 @@ __device__ __forceinline__ void count_pano_brick(const LevelParams &p, const Vox
                 else row = row_exact(m0, m1, rx, ry, rz0 + (h << 17), H);
                 in = row >= 0;
             }
-            if (in && r.rch) in = mxy + abs(z0 + 2 * h - (nd.z >> 16)) < (int)__ldg(steps + (size_t)row * A + col);
+            if (in && r.rch) in = mxy + abs(z0 + 2 * h - (nd.z >> 16)) < (int)ld_written(steps + (size_t)row * A + col);
             if (in && r.vis && !(Z >= 0.5f && r2 < vc.l22 && Z < p.vis_zl2)) {
                 const int4 d = p.pano_dir[(size_t)col * H + row];
                 const float q30 = 9.31322574615478515625e-10f;

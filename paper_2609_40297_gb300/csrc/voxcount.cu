@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(kVoxWarps * 32, 3) voxel_kernel(const LevelPar
                     if (pixel_in(U, Z, uf, p.W, pu) && pixel_in(V, Z, vf, p.H, pv)) {
                         pix = pv * p.W + pu;
                         const int man = abs(x - v0x) + abs(y - v0y) + abs(z - v0z);
-                        keep = man < (int)__ldg(steps + pix);
+                        keep = man < (int)ld_written(steps + pix);
                     }
                 }
             }

@@ -78,7 +78,7 @@ __device__ __forceinline__ bool observed_fast(const LevelParams &p, const AncRec
         if (in == 0) continue;
         const int4 *row = reinterpret_cast<const int4 *>(p.yawtab + A.yaw * 12);
         if (in > 0) {
-            const uint32_t D = __ldg(A.D + pv * p.W + pu);
+            const uint32_t D = ld_written(A.D + pv * p.W + pu);
             if constexpr (STATS) ++st_reads;
             // z <= D  <=>  Z < (D + 1) / 2^16 (voxels); lim within relative 2^-23 of that
             const float lim = ((float)D + 1.0f) * (1.0f / 65536.0f);
@@ -99,7 +99,7 @@ __device__ __forceinline__ bool observed_fast(const LevelParams &p, const AncRec
         const float uf = fmaf(A.m[0], ex, fmaf(A.m[1], ey, A.m[2] * ez)) * zi;
         const float vf = fmaf(A.m[3], ex, fmaf(A.m[4], ey, A.m[5] * ez)) * zi;
         if (!pixel_in(Ua, Za, uf, p.W, pu) || !pixel_in(Va, Za, vf, p.H, pv)) continue;
-        const uint32_t D = __ldg(A.D + pv * p.W + pu);
+        const uint32_t D = ld_written(A.D + pv * p.W + pu);
         if constexpr (STATS) ++st_reads;
         if (Za < (((int64_t)D + 1) << 16)) return true;
     }
@@ -325,7 +325,7 @@ __device__ __forceinline__ void node_run(const LevelParams &p, const NodeSlice &
                 }
                 if (in) {
                     pix = pv * p.W + pu;
-                    if (man < (int)__ldg(steps + (size_t)k * WH + pix)) {  // before the owner ray's hit
+                    if (man < (int)ld_written(steps + (size_t)k * WH + pix)) {  // before the owner ray's hit
                         if constexpr (STATS) ++st.visit;
                         int dx, dy, dz;
                         ray_dir(p.body[pix], rw[0], rw[1], dx, dy, dz);
