@@ -328,8 +328,9 @@ typedef struct mig_kernel_times {
  * voxel it crosses and owner-tests the unknown ones. The owned-voxel kernels keep one uint16 step count
  * per (node, yaw, pixel) of a level (panoramic mode: per node, column and row) in a buffer of at most
  * steps_budget_bytes (0 = the default, 1 GiB); a level that does not fit is counted in chunks. The
- * per-node pass keeps a queue of undecided bricks beside it (at most 512 MiB). Errors: MIG_EINVAL (ctx
- * NULL, unknown kernel). */
+ * per-node pass keeps a queue of undecided bricks beside it (at most 512 MiB). A server's requests keep
+ * the kernel and budget that were set when they were submitted. Errors: MIG_EINVAL (ctx NULL, unknown
+ * kernel). */
 #define MIG_COUNT_AUTO 0
 #define MIG_COUNT_RAYS 1
 #define MIG_COUNT_PAIRS 2

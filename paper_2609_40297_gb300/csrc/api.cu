@@ -273,19 +273,19 @@ bool rays_cheaper(const mig_sensor &s, float voxel, int n, int levels, int mode)
     return c.chain * R * levels + c.ray * R * n * rays < ball * (c.a + c.b * s.yaw_bins * (s.hfov_deg / 90.0));
 }
 
-StepsLayout steps_for(const mig_ctx *ctx, int n, int levels, int Lmax, const mig_sensor &s, float voxel, int mode, int lean) {
+StepsLayout steps_for(const CountChoice &c, int n, int levels, int Lmax, const mig_sensor &s, float voxel, int mode, int lean) {
     const bool pano = mode == MIG_MODE_PANORAMIC, whole = pano || mode == MIG_MODE_INTERVAL;
     // the interval and panoramic modes have no pass per (node, yaw) pair: without room for whole nodes they
     // count ray by ray
-    if (ctx->ray_count || lean == 2 || (whole && ctx->voxel_pass == MIG_COUNT_PAIRS)) return StepsLayout{};
-    if (ctx->voxel_pass == MIG_COUNT_AUTO && rays_cheaper(s, voxel, n, levels, mode)) return StepsLayout{};
+    if (c.rays || lean == 2 || (whole && c.pass == MIG_COUNT_PAIRS)) return StepsLayout{};
+    if (c.pass == MIG_COUNT_AUTO && rays_cheaper(s, voxel, n, levels, mode)) return StepsLayout{};
     SensorDims d{s.width, s.height, s.yaw_bins, range_q16(s.range_m, voxel)};
     if (pano) {
         d.W = pano_columns(s);
         d.K = 1;
-        if ((size_t)d.W * d.H * sizeof(uint16_t) > ctx->steps_budget) return StepsLayout{};
+        if ((size_t)d.W * d.H * sizeof(uint16_t) > c.steps_budget) return StepsLayout{};
     }
-    const StepsLayout L = steps_layout(d, n, Lmax, ctx->steps_budget, lean == 0 ? kTreeSteps : 0, ctx->voxel_pass != MIG_COUNT_PAIRS, mode);
+    const StepsLayout L = steps_layout(d, n, Lmax, c.steps_budget, lean == 0 ? kTreeSteps : 0, c.pass != MIG_COUNT_PAIRS, mode);
     return whole && L.queue_cap == 0 ? StepsLayout{} : L;
 }
 
@@ -367,7 +367,7 @@ static LevelParams level_params(const mig_map *m, const Camera *cam, const mig_c
     p.tiles_x = (p.W + p.tile_w - 1) / p.tile_w;
     p.tiles = p.tiles_x * ((p.H + p.tile_h - 1) / p.tile_h);
     set_band(p, cam);
-    p.voxel_pass = ctx->voxel_pass;
+    p.voxel_pass = ctx->count.pass;
     return p;
 }
 
@@ -409,7 +409,7 @@ mig_status mig_ctx_create(int device, void *stream, const mig_allocator *allocat
     pano_bricks_init();
     ctx->vox_ctas = vox_ctas_per_sm();
     ctx->node_ctas = node_ctas_per_sm();
-    ctx->steps_budget = kStepsBudget;
+    ctx->count.steps_budget = kStepsBudget;
     ctx->d_err = (int32_t *)ctx->alloc.alloc(256, ctx->stream);
     if (!ctx->d_err) return fail(MIG_ENOMEM, "ctx_create: allocation failed");
     MIG_CUDA_TRY(cudaMemsetAsync(ctx->d_err, 0, 256, ctx->stream));
@@ -472,9 +472,10 @@ mig_status mig_ctx_set_count_kernel(mig_ctx *ctx, int kernel, uint64_t steps_bud
     if (!ctx) return fail(MIG_EINVAL, "ctx is NULL");
     if (kernel < MIG_COUNT_AUTO || kernel > MIG_COUNT_NODES) return fail(MIG_EINVAL, "set_count_kernel: unknown kernel");
     std::lock_guard<std::mutex> lk(ctx->mu);
-    ctx->ray_count = kernel == MIG_COUNT_RAYS;
-    ctx->voxel_pass = kernel == MIG_COUNT_RAYS ? MIG_COUNT_AUTO : kernel;
-    ctx->steps_budget = steps_budget_bytes ? (size_t)steps_budget_bytes : kStepsBudget;
+    std::lock_guard<std::mutex> ck(ctx->count_mu);
+    ctx->count.rays = kernel == MIG_COUNT_RAYS;
+    ctx->count.pass = kernel == MIG_COUNT_RAYS ? MIG_COUNT_AUTO : kernel;
+    ctx->count.steps_budget = steps_budget_bytes ? (size_t)steps_budget_bytes : kStepsBudget;
     return MIG_OK;
 }
 
@@ -689,7 +690,7 @@ static mig_status eval_host(mig_map *m, int n, const int32_t *parent, const floa
     char *dev = nullptr;
     for (int lean = 0; lean < 3; ++lean) {  // less memory where the allocator has not enough
         Carver c = cv;
-        steps = steps_for(ctx, n, L, Lmax, *sensor, m->voxel, mode, lean);
+        steps = steps_for(ctx->count, n, L, Lmax, *sensor, m->voxel, mode, lean);
         o_dpyr = c.take<uint2>(steps.cap ? (size_t)std::max(1, plan.n_internal) * hz_entries(cam->W, cam->H) : 0);
         o_steps = c.take<char>(steps.bytes);
         // instrumented pass: the ray-by-ray count kernel is re-run into scratch counters afterwards,
@@ -873,7 +874,7 @@ mig_status mig_tree_eval_device(mig_map *m, int n, const int32_t *parent, const 
         o_err = cv.take<int32_t>(1); o_cnt = cv.take<int32_t>((size_t)n * K * 2);
         o_work = cv.take<int32_t>(L);
         // level sizes are known on the device only: the step-count buffer is sized for n nodes
-        steps = steps_for(ctx, n, L, n, *sensor, m->voxel, MIG_MODE_MARGINAL, lean);
+        steps = steps_for(ctx->count, n, L, n, *sensor, m->voxel, MIG_MODE_MARGINAL, lean);
         o_cursor = cv.take<int2>(device_steps(steps, n, K, L) + 1);
         zero_bytes = cv.off;
         o_depth = cv.take<int32_t>(n); o_loff = cv.take<int32_t>(L + 1); o_lint = cv.take<int32_t>(L);

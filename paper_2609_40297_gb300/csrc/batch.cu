@@ -650,7 +650,7 @@ mig_status batch_run_streams(mig_ctx *ctx, std::vector<BatchItem> &items) {
             const HostPlan &pl = items[t].plan;
             int Lmax = 1;
             for (int d = 0; d <= pl.max_depth; ++d) Lmax = std::max(Lmax, pl.level_off[d + 1] - pl.level_off[d]);
-            steps[t] = steps_for(ctx, pl.n, pl.max_depth + 1, Lmax, items[t].sensor, items[t].map->voxel, items[t].mode, lean);
+            steps[t] = steps_for(ctx->count, pl.n, pl.max_depth + 1, Lmax, items[t].sensor, items[t].map->voxel, items[t].mode, lean);
             stream_steps[oi % S] = std::max(stream_steps[oi % S], steps[t].bytes);
         }
         Carve c = cv;
@@ -713,7 +713,7 @@ mig_status batch_run_streams(mig_ctx *ctx, std::vector<BatchItem> &items) {
     for (int oi = 0; oi < T; ++oi) {
         const int t = order[oi];
         if (steps[t].cap) set_steps(lp[t], dev + o_steps[oi % S], steps[t]);
-        lp[t].voxel_pass = ctx->voxel_pass;
+        lp[t].voxel_pass = ctx->count.pass;
     }
     if (!ctx->batch) ctx->batch = new mig_ctx::Batch();
     mig_ctx::Batch *B = ctx->batch;
@@ -873,7 +873,7 @@ extern "C" mig_status mig_tree_eval_batch(mig_ctx *ctx, int n_trees, const mig_t
     // the persistent kernel runs the per-node owned-voxel pass of the sample modes; batches holding an
     // interval or panoramic tree, a sensor outside the per-node pass (more than kNodeMaxK yaws, a
     // frustum without an azimuth window) or a context counting ray by ray run on the stream chains
-    bool per_level_kernels = ctx->ray_count;
+    bool per_level_kernels = ctx->count.rays;
     for (auto &it : items) {
         mig_status st = ctx_camera(ctx, it.sensor, &it.cam);
         if (st != MIG_OK) return st;

@@ -107,6 +107,13 @@ struct Profiler {
     uint64_t launches[kProfKinds] = {};
 };
 
+// mig_ctx_set_count_kernel's choice.
+struct CountChoice {
+    bool rays = false;          // count with the ray-by-ray kernel instead of the owned-voxel kernels
+    int pass = MIG_COUNT_AUTO;  // owned-voxel pass: per (node, yaw) pair, per node, or chosen
+    size_t steps_budget = 0;    // owned-voxel step-count buffer per evaluation (bytes; set at creation)
+};
+
 }  // namespace mig
 
 // ----------------------------------------------------------------------------- public objects
@@ -120,9 +127,8 @@ struct mig_ctx {
     int pano_ctas = 1;         // resident panoramic count CTAs per SM
     int vox_ctas = 1;          // resident owned-voxel count CTAs per SM
     int node_ctas = 1;         // resident per-node voxel-pass CTAs per SM
-    bool ray_count = false;    // count with the ray-by-ray kernel instead of the owned-voxel kernels
-    int voxel_pass = MIG_COUNT_AUTO;  // owned-voxel pass: per (node, yaw) pair, per node, or chosen
-    size_t steps_budget = 0;   // owned-voxel step-count buffer per evaluation (bytes; set at creation)
+    mig::CountChoice count;    // written with mu and count_mu held, read with either
+    std::mutex count_mu;       // for readers that do not wait for the device (mig_server_submit)
     std::vector<std::unique_ptr<mig::Camera>> cameras;
     mig::DevBuf ws;          // per-call workspace (plan, counters, outputs, arena)
     void *pinned = nullptr;  // pinned host staging
@@ -175,7 +181,7 @@ void launch_level_count_timed(mig_ctx *ctx, const LevelParams &p, int Ld, int co
 // (ray by ray); a caller whose allocation fails takes the next.
 struct StepsLayout;
 bool rays_cheaper(const mig_sensor &s, float voxel, int n, int levels, int mode);
-StepsLayout steps_for(const mig_ctx *ctx, int n, int levels, int Lmax, const mig_sensor &s, float voxel, int mode, int lean);
+StepsLayout steps_for(const CountChoice &c, int n, int levels, int Lmax, const mig_sensor &s, float voxel, int mode, int lean);
 // The count and select-and-render launches of a device-planned tree of n nodes and at most `levels` levels.
 // With the per-node pass they go chunk by chunk through the levels, whose sizes only the device knows:
 // device_steps(..) steps and as many places + 1 in `cursor` (zeroed).

@@ -233,8 +233,8 @@ extern "C" mig_status mig_tree_eval_device_noalloc(mig_map *m, int n, const int3
     p.band_thi = 1e30f;
     p.voxel_pass = MIG_COUNT_AUTO;
     set_visit_params(p, sensor->hfov_deg, sensor->vfov_deg);
-    const bool rays = ctx->ray_count || ctx->voxel_pass == MIG_COUNT_PAIRS || steps.cap == 0 ||
-                      (ctx->voxel_pass == MIG_COUNT_AUTO && rays_cheaper(*sensor, m->voxel, n, L, MIG_MODE_MARGINAL));
+    const bool rays = ctx->count.rays || ctx->count.pass == MIG_COUNT_PAIRS || steps.cap == 0 ||
+                      (ctx->count.pass == MIG_COUNT_AUTO && rays_cheaper(*sensor, m->voxel, n, L, MIG_MODE_MARGINAL));
     if (!rays) {
         set_steps(p, dev + o_steps, steps);
         p.dpyr = (uint2 *)(dev + o_dpyr);

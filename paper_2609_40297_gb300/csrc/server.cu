@@ -49,6 +49,7 @@ struct Request {
     int mode = 0;
     HostPlan plan;
     int Lmax = 1;         // nodes of its largest level
+    CountChoice count;    // the count kernel at submission, for the region and the launches alike
     StepsLayout steps{};  // owned-voxel count's region (cap 0 = ray by ray)
     int32_t *out_abs = nullptr, *out_marg = nullptr, *out_yaw = nullptr;
     const Camera *cam = nullptr;
@@ -166,7 +167,7 @@ mig_status admit(mig_server *s, Request &r) {
     const size_t o_pcnt = pano ? cv.take(8 * (size_t)n * r.cam->pano_A) : 0;
     size_t o_steps = 0;
     for (int lean = 0; lean < 3 && !r.dev; ++lean) {  // less memory where the allocator has not enough
-        if (lean) r.steps = steps_for(ctx, n, L, r.Lmax, r.sensor, r.map->voxel, r.mode, lean);
+        if (lean) r.steps = steps_for(r.count, n, L, r.Lmax, r.sensor, r.map->voxel, r.mode, lean);
         Carve c = cv;
         o_steps = c.take(r.steps.bytes);
         r.dev_bytes = c.off;
@@ -233,7 +234,7 @@ mig_status admit(mig_server *s, Request &r) {
     if (pano) set_pano_params(p, r.cam, (int32_t *)(r.dev + o_pcnt));
     if (r.steps.cap) set_steps(p, r.dev + o_steps, r.steps);
     p.dpyr = (uint2 *)(r.dev + o_dpyr);
-    p.voxel_pass = ctx->voxel_pass;
+    p.voxel_pass = r.count.pass;
     r.level = 0;
     return MIG_OK;
 }
@@ -473,13 +474,15 @@ extern "C" mig_status mig_server_submit(mig_server *s, const mig_tree_desc *d, u
     r->sensor = d->sensor;
     r->mode = d->mode;
     {
-        for (int lv = 0; lv <= r->plan.max_depth; ++lv)
-            r->Lmax = std::max(r->Lmax, r->plan.level_off[lv + 1] - r->plan.level_off[lv]);
-        // the whole tree's step counts only where as many such requests as may be in flight fit the budget
-        for (int lean = 0; lean < 2; ++lean) {
-            r->steps = steps_for(s->ctx, r->plan.n, r->plan.max_depth + 1, r->Lmax, d->sensor, d->map->voxel, d->mode, lean);
-            if (!r->steps.tree || request_bytes(*r) <= s->budget / (size_t)s->max_inflight) break;
-        }
+        std::lock_guard<std::mutex> ck(s->ctx->count_mu);
+        r->count = s->ctx->count;
+    }
+    for (int lv = 0; lv <= r->plan.max_depth; ++lv)
+        r->Lmax = std::max(r->Lmax, r->plan.level_off[lv + 1] - r->plan.level_off[lv]);
+    // the whole tree's step counts only where as many such requests as may be in flight fit the budget
+    for (int lean = 0; lean < 2; ++lean) {
+        r->steps = steps_for(r->count, r->plan.n, r->plan.max_depth + 1, r->Lmax, d->sensor, d->map->voxel, d->mode, lean);
+        if (!r->steps.tree || request_bytes(*r) <= s->budget / (size_t)s->max_inflight) break;
     }
     r->out_abs = d->abs_gain;
     r->out_marg = d->marg_gain;
