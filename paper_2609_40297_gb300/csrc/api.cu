@@ -354,7 +354,7 @@ static mig_status check_codes(const uint8_t *v, size_t n) {
 
 static LevelParams level_params(const mig_map *m, const Camera *cam, const mig_ctx *ctx) {
     LevelParams p{};
-    p.grid = GridView{m->d_grid, m->nx, m->ny, m->nz, m->nbx, m->nby};
+    p.grid = GridView{m->d_grid, m->nx, m->ny, m->nz};
     p.body = (const int4 *)cam->d_body;
     p.yawtab = cam->d_yaw;
     p.yawf = cam->d_yawf;
@@ -533,7 +533,7 @@ mig_status mig_map_create(mig_ctx *ctx, int nx, int ny, int nz, float voxel_size
     m->nx = nx;
     m->ny = ny;
     m->nz = nz;
-    m->grid_bytes = map_layout_bytes(nx, ny, nz, &m->nbx, &m->nby, &m->nbz);
+    m->grid_bytes = map_layout_bytes(nx, ny, nz);
     if (map_codes_bytes(nx, ny, nz) >= ((size_t)1 << 32)) return fail(MIG_EINVAL, "map_create: padded grid above 2^32 voxels");
     m->voxel = voxel_size_m;
     for (int a = 0; a < 3; ++a) m->origin[a] = origin_m ? origin_m[a] : 0.f;
@@ -554,7 +554,7 @@ mig_status mig_map_create(mig_ctx *ctx, int nx, int ny, int nz, float voxel_size
             return fail(MIG_ENOMEM, "map_create: staging allocation failed");
         }
         MIG_CUDA_TRY(cudaMemcpyAsync(tmp, host_voxels, nvox, cudaMemcpyHostToDevice, ctx->stream));
-        launch_map_scatter(m->d_grid, m->nx, m->ny, m->nz, m->nbx, m->nby, tmp, 0, 0, 0, nx, ny, nz, ctx->stream);
+        launch_map_scatter(m->d_grid, m->nx, m->ny, m->nz, tmp, 0, 0, 0, nx, ny, nz, ctx->stream);
         MIG_CUDA_TRY(cudaGetLastError());
         ctx->alloc.free(tmp, nvox, ctx->stream);
     } else {
@@ -579,7 +579,7 @@ mig_status mig_map_update(mig_map *m, int x0, int y0, int z0, int dx, int dy, in
     uint8_t *tmp = (uint8_t *)ctx->alloc.alloc(nvox, ctx->stream);
     if (!tmp) return fail(MIG_ENOMEM, "map_update: staging allocation failed");
     MIG_CUDA_TRY(cudaMemcpyAsync(tmp, host_voxels, nvox, cudaMemcpyHostToDevice, ctx->stream));
-    launch_map_scatter(m->d_grid, m->nx, m->ny, m->nz, m->nbx, m->nby, tmp, x0, y0, z0, dx, dy, dz, ctx->stream);
+    launch_map_scatter(m->d_grid, m->nx, m->ny, m->nz, tmp, x0, y0, z0, dx, dy, dz, ctx->stream);
     MIG_CUDA_TRY(cudaGetLastError());
     ctx->alloc.free(tmp, nvox, ctx->stream);
     MIG_CUDA_TRY(cudaStreamSynchronize(ctx->stream));  // the host buffer may be reused on return
@@ -593,12 +593,7 @@ mig_status mig_map_read(mig_map *m, uint8_t *host_out) {
     const size_t nvox = (size_t)m->nx * m->ny * m->nz;
     std::lock_guard<std::mutex> lk(ctx->mu);
     MIG_CUDA_TRY(cudaSetDevice(ctx->device));
-    uint8_t *tmp = (uint8_t *)ctx->alloc.alloc(nvox, ctx->stream);
-    if (!tmp) return fail(MIG_ENOMEM, "map_read: staging allocation failed");
-    launch_map_gather(m->d_grid, m->nbx, m->nby, tmp, m->nx, m->ny, m->nz, ctx->stream);
-    MIG_CUDA_TRY(cudaGetLastError());
-    MIG_CUDA_TRY(cudaMemcpyAsync(host_out, tmp, nvox, cudaMemcpyDeviceToHost, ctx->stream));
-    ctx->alloc.free(tmp, nvox, ctx->stream);
+    MIG_CUDA_TRY(cudaMemcpyAsync(host_out, m->d_grid, nvox, cudaMemcpyDeviceToHost, ctx->stream));
     MIG_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
     return MIG_OK;
 }

@@ -450,7 +450,7 @@ mig_status batch_run(mig_ctx *ctx, std::vector<BatchItem> &items) {
         std::memcpy(host + to[t].lnodes, pl.level_nodes.data(), 4 * (size_t)n);
         LevelParams p{};
         mig_map *m = it.map;
-        p.grid = GridView{m->d_grid, m->nx, m->ny, m->nz, m->nbx, m->nby};
+        p.grid = GridView{m->d_grid, m->nx, m->ny, m->nz};
         p.body = (const int4 *)it.cam->d_body;
         p.yawtab = it.cam->d_yaw;
         p.yawf = it.cam->d_yawf;
@@ -678,7 +678,7 @@ mig_status batch_run_streams(mig_ctx *ctx, std::vector<BatchItem> &items) {
         std::memcpy(host + to[t].lnodes, pl.level_nodes.data(), 4 * (size_t)n);
         LevelParams p{};
         mig_map *m = it.map;
-        p.grid = GridView{m->d_grid, m->nx, m->ny, m->nz, m->nbx, m->nby};
+        p.grid = GridView{m->d_grid, m->nx, m->ny, m->nz};
         p.body = (const int4 *)it.cam->d_body;
         p.yawtab = it.cam->d_yaw;
         p.yawf = it.cam->d_yawf;

@@ -13,11 +13,6 @@
 #include "kernels.h"
 #include "mig.h"
 
-// Voxel layout of the device grid: 0 = 8x8x8 bricks of 512 B (z-major inside a brick),
-// 1 = x-fastest rows (the host order), stepped with an incremental address.
-#ifndef MIG_LAYOUT
-#define MIG_LAYOUT 1
-#endif
 // 1 = the chunk's own-camera constants (projection rows, yaw cos/sin, node position) are read
 // from the warp's shared-memory slot at each use instead of being held in registers.
 #ifndef MIG_CAM_SMEM
@@ -68,11 +63,7 @@ __device__ __forceinline__ T ld_written(const T *p) {
 }
 
 __device__ __forceinline__ uint32_t grid_cells(int nx, int ny, int nz) {
-#if MIG_LAYOUT == 1
     return (uint32_t)nx * (uint32_t)ny * (uint32_t)nz;
-#else
-    return (uint32_t)((nx + 7) >> 3) * (uint32_t)((ny + 7) >> 3) * (uint32_t)((nz + 7) >> 3) * 512u;
-#endif
 }
 
 // The code of the ray's current voxel (an occupied code for a checked build's skipped access).
@@ -89,15 +80,6 @@ __device__ __forceinline__ void arena_store(uint32_t *arena, int slots, int slot
 }
 constexpr int kUnknown = 0;
 constexpr uint32_t kQ16 = 65536;
-
-__device__ __forceinline__ uint32_t voxel_addr(const GridView &G, int x, int y, int z) {
-#if MIG_LAYOUT == 1
-    return ((uint32_t)z * (uint32_t)G.ny + (uint32_t)y) * (uint32_t)G.nx + (uint32_t)x;
-#else
-    const uint32_t b = ((uint32_t)(z >> 3) * (uint32_t)G.nby + (uint32_t)(y >> 3)) * (uint32_t)G.nbx + (uint32_t)(x >> 3);
-    return (b << 9) | ((uint32_t)(z & 7) << 6) | ((uint32_t)(y & 7) << 3) | (uint32_t)(x & 7);
-#endif
-}
 
 // Per-axis DDA set-up (Sec. IV-B, Amanatides-Woo). n = distance to the next face (Q16),
 // ad = |d| (Q30), s = step sign, l = face limit: crossing k along this axis is at n + k 2^16 and
@@ -129,56 +111,34 @@ __device__ __forceinline__ void axis_init(int P, int d, int N, int64_t Tq, int &
     l = n + ((uint32_t)min((int64_t)grid_rem, range_rem) << 16);
 }
 
-// DDA state of one ray. The current voxel is not stored: along an axis with step sign s, the
+// DDA state of one ray, stepped with an incremental address (the grid's rows are x-fastest). The current voxel is not stored: along an axis with step sign s, the
 // centre of the current voxel lies s (n - 2^15) (Q16) from the ray origin, because n is the
 // distance from the origin to the voxel's far face along the ray's direction of travel.
 struct RayIn {
     uint32_t nx, ny, nz, adx, ady, adz, lx, ly, lz;
     int sx, sy, sz;
-#if MIG_LAYOUT == 1
     uint32_t addr;
     int dax, day, daz;  // signed address strides of one step along each axis
-#else
-    int vx, vy, vz;
-#endif
 };
 
 // Q16 offset, along one axis, of the current voxel's centre from the ray origin.
 __device__ __forceinline__ int voxel_offset(uint32_t n, int s) { return s * (int)(n - 32768u); }
 
-__device__ __forceinline__ void ray_init_dims(RayIn &r, int gnx, int gny, int gnz, const GridView &G, int Px, int Py,
-                                              int Pz, int dx, int dy, int dz, int64_t Tq) {
+__device__ __forceinline__ void ray_init_dims(RayIn &r, int gnx, int gny, int gnz, int Px, int Py, int Pz,
+                                               int dx, int dy, int dz, int64_t Tq) {
     int vx, vy, vz;
     axis_init(Px, dx, gnx, Tq, vx, r.nx, r.adx, r.sx, r.lx);
     axis_init(Py, dy, gny, Tq, vy, r.ny, r.ady, r.sy, r.ly);
     axis_init(Pz, dz, gnz, Tq, vz, r.nz, r.adz, r.sz, r.lz);
-#if MIG_LAYOUT == 1
-    (void)G;
     r.addr = ((uint32_t)vz * (uint32_t)gny + (uint32_t)vy) * (uint32_t)gnx + (uint32_t)vx;
     r.dax = r.sx;
     r.day = r.sy * gnx;
     r.daz = r.sz * gnx * gny;
-#else
-    (void)gnx;
-    (void)gny;
-    r.vx = vx;
-    r.vy = vy;
-    r.vz = vz;
-#endif
 }
 
 __device__ __forceinline__ void ray_init(RayIn &r, const GridView &G, int Px, int Py, int Pz, int dx, int dy, int dz,
                                          int64_t Tq) {
-    ray_init_dims(r, G.nx, G.ny, G.nz, G, Px, Py, Pz, dx, dy, dz, Tq);
-}
-
-__device__ __forceinline__ uint32_t ray_addr(const RayIn &r, const GridView &G) {
-#if MIG_LAYOUT == 1
-    (void)G;
-    return r.addr;
-#else
-    return voxel_addr(G, r.vx, r.vy, r.vz);
-#endif
+    ray_init_dims(r, G.nx, G.ny, G.nz, Px, Py, Pz, dx, dy, dz, Tq);
 }
 
 // World direction of (yaw k, pixel): yaw rotation of the body-frame ray, floored (Q30).
@@ -211,13 +171,7 @@ __device__ __forceinline__ bool ray_step(RayIn &r, uint32_t &ne, uint32_t &ade) 
     r.nx += bx ? kQ16 : 0u;
     r.ny += by ? kQ16 : 0u;
     r.nz += bz ? kQ16 : 0u;
-#if MIG_LAYOUT == 1
     r.addr += bx ? r.dax : (by ? r.day : r.daz);
-#else
-    r.vx += bx ? r.sx : 0;
-    r.vy += by ? r.sy : 0;
-    r.vz += bz ? r.sz : 0;
-#endif
     return true;
 }
 
@@ -477,10 +431,10 @@ __device__ __forceinline__ void count_chunk(const LevelParams &p, const HOT &hp,
 #if MIG_CAM_SMEM
                     const int4 c3 = lds128(cam + 3), c0 = lds128(cam);
                     ray_dir(b, c3.x, c3.y, dx, dy, dz);
-                    ray_init_dims(r, hp.nx(), hp.ny(), hp.nz(), p.grid, c0.x, c0.y, c0.z, dx, dy, dz, hp.Tq());
+                    ray_init_dims(r, hp.nx(), hp.ny(), hp.nz(), c0.x, c0.y, c0.z, dx, dy, dz, hp.Tq());
 #else
                     ray_dir(b, ck, sk, dx, dy, dz);
-                    ray_init_dims(r, hp.nx(), hp.ny(), hp.nz(), p.grid, nd.x, nd.y, nd.z, dx, dy, dz, hp.Tq());
+                    ray_init_dims(r, hp.nx(), hp.ny(), hp.nz(), nd.x, nd.y, nd.z, dx, dy, dz, hp.Tq());
 #endif
                     have = true;
                     if constexpr (STATS) ++st_rays;
@@ -491,7 +445,7 @@ __device__ __forceinline__ void count_chunk(const LevelParams &p, const HOT &hp,
 #pragma unroll
         for (int sidx = 0; sidx < kCountBlock; ++sidx) {
             if (have) {
-                const uint8_t code = load_code(hp.g(), ray_addr(r, p.grid), p.grid, p.bounds_err);
+                const uint8_t code = load_code(hp.g(), r.addr, p.grid, p.bounds_err);
                 if constexpr (STATS) ++st_steps;
                 if (code == kOcc) {
                     have = false;
@@ -579,10 +533,10 @@ __device__ __forceinline__ void count_chunk(const LevelParams &p, const HOT &hp,
 #if MIG_CAM_SMEM
                     const int4 c3 = lds128(cam + 3), c0 = lds128(cam);
                     ray_dir(b, c3.x, c3.y, dx, dy, dz);
-                    ray_init_dims(r, hp.nx(), hp.ny(), hp.nz(), p.grid, c0.x, c0.y, c0.z, dx, dy, dz, hp.Tq());
+                    ray_init_dims(r, hp.nx(), hp.ny(), hp.nz(), c0.x, c0.y, c0.z, dx, dy, dz, hp.Tq());
 #else
                     ray_dir(b, ck, sk, dx, dy, dz);
-                    ray_init_dims(r, hp.nx(), hp.ny(), hp.nz(), p.grid, nd.x, nd.y, nd.z, dx, dy, dz, hp.Tq());
+                    ray_init_dims(r, hp.nx(), hp.ny(), hp.nz(), nd.x, nd.y, nd.z, dx, dy, dz, hp.Tq());
 #endif
                     have = true;
                     if constexpr (STATS) ++st_rays;
@@ -596,7 +550,7 @@ __device__ __forceinline__ void count_chunk(const LevelParams &p, const HOT &hp,
         bool owned = false;
         unsigned long long samp = 0;
         if (have) {
-            const uint8_t code = load_code(hp.g(), ray_addr(r, p.grid), p.grid, p.bounds_err);
+            const uint8_t code = load_code(hp.g(), r.addr, p.grid, p.bounds_err);
             if constexpr (STATS) ++st_steps;
             if (code == kOcc) {
                 have = false;
@@ -737,7 +691,7 @@ __device__ __forceinline__ uint32_t render_pixel(const LevelParams &p, int n, co
     uint32_t ne = 0, ade = 1, steps = 0;
     bool hit = false;
     for (;;) {
-        const uint8_t code = load_code(p.grid.g, ray_addr(r, p.grid), p.grid, p.bounds_err);
+        const uint8_t code = load_code(p.grid.g, r.addr, p.grid, p.bounds_err);
         ++steps;
         if (code == kOcc) {
             hit = true;
@@ -789,7 +743,7 @@ __device__ __forceinline__ void render_chunk(const LevelParams &p, int n, int ti
             continue;
         }
         if (have) {
-            const uint8_t code = load_code(p.grid.g, ray_addr(r, p.grid), p.grid, p.bounds_err);
+            const uint8_t code = load_code(p.grid.g, r.addr, p.grid, p.bounds_err);
             const bool hit = code == kOcc;
             if (hit || !ray_step<true>(r, ne, ade)) {
                 arena_store(p.arena, p.arena_slots, nd.w, (size_t)tj * p.W + ti, (size_t)p.W * p.H,

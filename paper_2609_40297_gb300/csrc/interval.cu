@@ -178,7 +178,7 @@ __global__ void __launch_bounds__(kIvThreads, MIG_IV_MINB) interval_count_kernel
             bool owned = false;
             uint4 key = make_uint4(0u, 0u, 0u, 0u);
             if (have) {
-                const uint8_t code = load_code(p.grid.g, ray_addr(r, p.grid), p.grid, p.bounds_err);
+                const uint8_t code = load_code(p.grid.g, r.addr, p.grid, p.bounds_err);
                 if constexpr (STATS) ++st_steps;
                 if (code == kOcc) {
                     have = false;

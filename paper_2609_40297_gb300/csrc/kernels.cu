@@ -1,5 +1,5 @@
 // Device kernels: fused per-level count (3D DDA + owner test + ancestor depth test + integer
-// reductions), yaw selection, map scatter/gather, device planning.
+// reductions), yaw selection, map scatter, device planning.
 //
 // All result-deciding arithmetic is integer (the fixed-point reading of Sec. IV-A..C):
 // positions Q16 voxel units, ray directions Q30, projection rows Q16, depths Q16.16.
@@ -56,27 +56,14 @@ __global__ void select_kernel(const LevelParams p) {
 }
 
 // ------------------------------------------------------------------------------- map kernels
-__global__ void map_scatter_kernel(uint8_t *bricks, int nx, int ny, int nbx, int nby, const uint8_t *box, int x0,
-                                   int y0, int z0, int dx, int dy, int dz) {
+__global__ void map_scatter_kernel(uint8_t *grid, int nx, int ny, const uint8_t *box, int x0, int y0, int z0, int dx, int dy,
+                                   int dz) {
     const size_t total = (size_t)dx * dy * dz;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
         const int x = (int)(i % dx) + x0;
         const int y = (int)((i / dx) % dy) + y0;
         const int z = (int)(i / ((size_t)dx * dy)) + z0;
-        const GridView G{nullptr, nx, ny, 0, nbx, nby};
-        bricks[voxel_addr(G, x, y, z)] = box[i];
-    }
-}
-
-__global__ void map_gather_kernel(const uint8_t *bricks, int nbx, int nby, uint8_t *lin, int nx, int ny, int nz) {
-    // (the layout's address of voxel (x, y, z); identity for x-fastest rows)
-    const size_t total = (size_t)nx * ny * nz;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const int x = (int)(i % nx);
-        const int y = (int)((i / nx) % ny);
-        const int z = (int)(i / ((size_t)nx * ny));
-        const GridView G{nullptr, nx, ny, 0, nbx, nby};
-        lin[i] = bricks[voxel_addr(G, x, y, z)];
+        grid[((size_t)z * ny + y) * nx + x] = box[i];
     }
 }
 
@@ -180,18 +167,9 @@ void launch_count(const LevelParams &p, int grid, cudaStream_t s) {
 
 size_t map_codes_bytes(int nx, int ny, int nz) { return occ_summary_end(nx, ny, nz); }
 
-size_t map_layout_bytes(int nx, int ny, int nz, int *nbx, int *nby, int *nbz) {
-    *nbx = (nx + 7) / 8;
-    *nby = (ny + 7) / 8;
-    *nbz = (nz + 7) / 8;
-#if MIG_LAYOUT == 1
-    // voxel codes, then (each 256-byte aligned) one occupancy byte per 8x8x8 brick and one per 32x32x32
-    // super-brick, and the masks and distances of the 4x4x4 bricks
-    return brick_data_end(nx, ny, nz);
-#else
-    return (size_t)*nbx * *nby * *nbz * 512;
-#endif
-}
+// voxel codes, then (each 256-byte aligned) one occupancy byte per 8x8x8 brick and one per 32x32x32
+// super-brick, and the masks and distances of the 4x4x4 bricks
+size_t map_layout_bytes(int nx, int ny, int nz) { return brick_data_end(nx, ny, nz); }
 
 int count_ctas_per_sm() {
     int a = 0, b = 0;
@@ -204,22 +182,13 @@ int count_ctas_per_sm() {
     return std::max(1, std::min(a, b));
 }
 void launch_select(const LevelParams &p, int grid, cudaStream_t s) { launch_behind(select_kernel, grid, 128, 0, s, p); }
-void launch_map_scatter(uint8_t *bricks, int nx, int ny, int nz, int nbx, int nby, const uint8_t *box, int x0, int y0,
-                        int z0, int dx, int dy, int dz, cudaStream_t s) {
+void launch_map_scatter(uint8_t *grid, int nx, int ny, int nz, const uint8_t *box, int x0, int y0, int z0, int dx, int dy,
+                        int dz, cudaStream_t s) {
     const size_t total = (size_t)dx * dy * dz;
-    const int grid = (int)std::min<size_t>((total + 255) / 256, 4096);
-    map_scatter_kernel<<<grid, 256, 0, s>>>(bricks, nx, ny, nbx, nby, box, x0, y0, z0, dx, dy, dz);
-#if MIG_LAYOUT == 1
-    launch_bocc(bricks, nx, ny, nz, x0, y0, z0, dx, dy, dz, s);  // the summaries of the bricks it touched
-    launch_brick_update(bricks, nx, ny, nz, x0, y0, z0, dx, dy, dz, s);
-#else
-    (void)nz;
-#endif
-}
-void launch_map_gather(const uint8_t *bricks, int nbx, int nby, uint8_t *lin, int nx, int ny, int nz, cudaStream_t s) {
-    const size_t total = (size_t)nx * ny * nz;
-    const int grid = (int)std::min<size_t>((total + 255) / 256, 4096);
-    map_gather_kernel<<<grid, 256, 0, s>>>(bricks, nbx, nby, lin, nx, ny, nz);
+    const int blocks = (int)std::min<size_t>((total + 255) / 256, 4096);
+    map_scatter_kernel<<<blocks, 256, 0, s>>>(grid, nx, ny, box, x0, y0, z0, dx, dy, dz);
+    launch_bocc(grid, nx, ny, nz, x0, y0, z0, dx, dy, dz, s);  // the summaries of the bricks it touched
+    launch_brick_update(grid, nx, ny, nz, x0, y0, z0, dx, dy, dz, s);
 }
 void launch_plan(const DevPlanParams &p, cudaStream_t s) {
     const int grid = std::max(1, std::min((p.n + 255) / 256, 1024));

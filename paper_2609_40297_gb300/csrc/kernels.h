@@ -10,9 +10,8 @@ namespace mig {
 constexpr int kStatsCounters = 20;
 
 struct GridView {
-    const uint8_t *g;  // voxel codes in the traversal layout (x-fastest rows or 8x8x8 bricks)
+    const uint8_t *g;  // voxel codes (x-fastest rows), then what bricks.cuh lists
     int nx, ny, nz;
-    int nbx, nby;
 };
 
 // A brick that the per-node pass leaves to its voxel stage: unknown voxels, those an ancestor is known
@@ -101,13 +100,12 @@ void launch_select_render(const LevelParams &p, int nodes, int num_sms, cudaStre
 void set_visit_params(LevelParams &p, float hfov_deg, float vfov_deg);  // the vis_* fields, from p.W and p.H
 // Writes a box of voxel codes into a grid of nx * ny * nz and refreshes the occupancy bytes, masks
 // and distances of the bricks it touches.
-void launch_map_scatter(uint8_t *bricks, int nx, int ny, int nz, int nbx, int nby, const uint8_t *box, int x0, int y0,
+void launch_map_scatter(uint8_t *grid, int nx, int ny, int nz, const uint8_t *box, int x0, int y0,
                         int z0, int dx, int dy, int dz, cudaStream_t s);
 // device bytes of an nx*ny*nz grid's voxel codes and occupancy bytes
 size_t map_codes_bytes(int nx, int ny, int nz);
-// device bytes of an nx*ny*nz grid in the traversal layout (and its brick counts)
-size_t map_layout_bytes(int nx, int ny, int nz, int *nbx, int *nby, int *nbz);
-void launch_map_gather(const uint8_t *bricks, int nbx, int nby, uint8_t *lin, int nx, int ny, int nz, cudaStream_t s);
+// device bytes of an nx*ny*nz grid with the masks and distances of its bricks
+size_t map_layout_bytes(int nx, int ny, int nz);
 
 // Device planning (tree on the device): depth, levels, ancestors, slots, quantised positions.
 struct DevPlanParams {

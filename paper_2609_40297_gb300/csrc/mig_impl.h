@@ -19,8 +19,6 @@ namespace mig {
 
 constexpr int64_t kOneQ16 = 65536;
 constexpr int64_t kOneQ30 = int64_t(1) << 30;
-constexpr int kBrickShift = 3;  // 8x8x8 bricks of uint8 codes, 512 B each
-constexpr int kBrick = 1 << kBrickShift;
 constexpr int kYawRec = 12;  // per yaw: ck, sk, mu[3], mv[3], mz[3], pad
 
 // ---------------------------------------------------------------------------------- errors
@@ -147,10 +145,9 @@ struct mig_ctx {
 struct mig_map {
     mig_ctx *ctx = nullptr;
     int nx = 0, ny = 0, nz = 0;
-    int nbx = 0, nby = 0, nbz = 0;  // bricks per axis
     float voxel = 0.f;
     float origin[3] = {0.f, 0.f, 0.f};
-    uint8_t *d_grid = nullptr;       // bricked codes, nbx*nby*nbz*512 bytes
+    uint8_t *d_grid = nullptr;       // voxel codes, summaries, brick data (bricks.cuh)
     size_t grid_bytes = 0;
     uint64_t version = 0;
 };

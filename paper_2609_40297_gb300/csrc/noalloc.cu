@@ -203,7 +203,7 @@ extern "C" mig_status mig_tree_eval_device_noalloc(mig_map *m, int n, const int3
     dp.out_yaw = best_yaw;
     launch_plan(dp, s);
     LevelParams p{};
-    p.grid = GridView{m->d_grid, m->nx, m->ny, m->nz, m->nbx, m->nby};
+    p.grid = GridView{m->d_grid, m->nx, m->ny, m->nz};
     p.body = (const int4 *)(dev + o_body);
     p.yawtab = (const int32_t *)(dev + o_yaw);
     p.W = W;

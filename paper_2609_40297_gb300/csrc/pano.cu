@@ -86,7 +86,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) pano_count_kernel(const LevelP
             bool owned = false;
             unsigned long long samp = 0;
             if (have) {
-                const uint8_t code = load_code(p.grid.g, ray_addr(r, p.grid), p.grid, p.bounds_err);
+                const uint8_t code = load_code(p.grid.g, r.addr, p.grid, p.bounds_err);
                 if constexpr (STATS) ++st_steps;
                 if (code == kOcc) {
                     have = false;

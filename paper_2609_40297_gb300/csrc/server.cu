@@ -202,7 +202,7 @@ mig_status admit(mig_server *s, Request &r) {
     r.grid->users++;
     LevelParams &p = r.p;
     mig_map *m = r.map;
-    p.grid = GridView{r.grid->ptr, m->nx, m->ny, m->nz, m->nbx, m->nby};
+    p.grid = GridView{r.grid->ptr, m->nx, m->ny, m->nz};
     p.body = (const int4 *)r.cam->d_body;
     p.yawtab = r.cam->d_yaw;
     p.yawf = r.cam->d_yawf;
@@ -279,7 +279,7 @@ mig_status apply_update(mig_server *s, Update &u) {
     uint8_t *tmp = (uint8_t *)ctx->alloc.alloc(nv, ctx->stream);
     if (!tmp) return fail(MIG_ENOMEM, "server: update staging allocation failed");
     MIG_CUDA_TRY(cudaMemcpyAsync(tmp, u.voxels.data(), nv, cudaMemcpyHostToDevice, ctx->stream));
-    launch_map_scatter(m->d_grid, m->nx, m->ny, m->nz, m->nbx, m->nby, tmp, u.x0, u.y0, u.z0, u.dx, u.dy, u.dz, ctx->stream);
+    launch_map_scatter(m->d_grid, m->nx, m->ny, m->nz, tmp, u.x0, u.y0, u.z0, u.dx, u.dy, u.dz, ctx->stream);
     MIG_CUDA_TRY(cudaGetLastError());
     ctx->alloc.free(tmp, nv, ctx->stream);
     MIG_CUDA_TRY(cudaStreamSynchronize(ctx->stream));  // the host voxels are freed with the update
