@@ -33,13 +33,19 @@ MIG_HD size_t omask_offset(int nx, int ny, int nz) {
 MIG_HD size_t dist_offset(int nx, int ny, int nz) {
     return omask_offset(nx, ny, nz) + ((8 * brick_count(nx, ny, nz) + 255) & ~(size_t)255);
 }
-// the octants' distances (octant_of), then six byte arrays that the distance passes work in
+// the octants' distances (octant_of), then what only updates use: the distances within a z layer (four
+// bytes a brick) and a bit per brick with an occupied voxel, rows of bits_words words
 MIG_HD size_t brick_bytes_offset(int nx, int ny, int nz, int i) {
     return dist_offset(nx, ny, nz) + (size_t)i * ((brick_count(nx, ny, nz) + 255) & ~(size_t)255);
 }
 MIG_HD size_t oct_offset(int nx, int ny, int nz, int o) { return brick_bytes_offset(nx, ny, nz, 1 + o); }
-MIG_HD size_t dist_scratch_offset(int nx, int ny, int nz, int i) { return brick_bytes_offset(nx, ny, nz, 9 + i); }
-MIG_HD size_t brick_data_end(int nx, int ny, int nz) { return brick_bytes_offset(nx, ny, nz, 15); }
+MIG_HD size_t dist_xy_offset(int nx, int ny, int nz) { return brick_bytes_offset(nx, ny, nz, 9); }
+MIG_HD size_t bits_offset(int nx, int ny, int nz) { return brick_bytes_offset(nx, ny, nz, 13); }
+MIG_HD int bits_words(int nbx) { return (nbx + 31) >> 5; }
+MIG_HD size_t brick_data_end(int nx, int ny, int nz) {
+    const BrickDims n = brick_dims(nx, ny, nz);
+    return bits_offset(nx, ny, nz) + (size_t)n.nby * n.nbz * bits_words(n.nbx) * 4;
+}
 // The octant of a direction: a bit per axis that does not run backwards.
 MIG_HD int octant_of(int dx, int dy, int dz) { return (dx >= 0 ? 1 : 0) | (dy >= 0 ? 2 : 0) | (dz >= 0 ? 4 : 0); }
 

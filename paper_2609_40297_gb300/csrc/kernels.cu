@@ -1,5 +1,5 @@
 // Device kernels: fused per-level count (3D DDA + owner test + ancestor depth test + integer
-// reductions), yaw selection, map scatter, device planning.
+// reductions), yaw selection, device planning.
 //
 // All result-deciding arithmetic is integer (the fixed-point reading of Sec. IV-A..C):
 // positions Q16 voxel units, ray directions Q30, projection rows Q16, depths Q16.16.
@@ -8,12 +8,10 @@
 #include <algorithm>
 #include <cstdint>
 
-#include "bricks.cuh"
 #include "dev_path.cuh"
 #include "kernels.h"
 #include "launch.cuh"
 #include "mig.h"
-#include "voxcount.h"
 
 namespace mig {
 
@@ -53,18 +51,6 @@ __global__ void select_kernel(const LevelParams p) {
     const int L = p.level_off[lvl + 1] - l0;
     for (int li = blockIdx.x * blockDim.x + threadIdx.x; li < L; li += gridDim.x * blockDim.x)
         select_node(p, p.level_nodes[l0 + li]);
-}
-
-// ------------------------------------------------------------------------------- map kernels
-__global__ void map_scatter_kernel(uint8_t *grid, int nx, int ny, const uint8_t *box, int x0, int y0, int z0, int dx, int dy,
-                                   int dz) {
-    const size_t total = (size_t)dx * dy * dz;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const int x = (int)(i % dx) + x0;
-        const int y = (int)((i / dx) % dy) + y0;
-        const int z = (int)(i / ((size_t)dx * dy)) + z0;
-        grid[((size_t)z * ny + y) * nx + x] = box[i];
-    }
 }
 
 // ----------------------------------------------------------------------------- device plan
@@ -165,12 +151,6 @@ void launch_count(const LevelParams &p, int grid, cudaStream_t s) {
     else count_kernel<false><<<grid, kWarps * 32, smem, s>>>(p);
 }
 
-size_t map_codes_bytes(int nx, int ny, int nz) { return occ_summary_end(nx, ny, nz); }
-
-// voxel codes, then (each 256-byte aligned) one occupancy byte per 8x8x8 brick and one per 32x32x32
-// super-brick, and the masks and distances of the 4x4x4 bricks
-size_t map_layout_bytes(int nx, int ny, int nz) { return brick_data_end(nx, ny, nz); }
-
 int count_ctas_per_sm() {
     int a = 0, b = 0;
     const size_t smem = count_dyn_smem(MIG_MAX_DEPTH);  // the worst case
@@ -182,14 +162,6 @@ int count_ctas_per_sm() {
     return std::max(1, std::min(a, b));
 }
 void launch_select(const LevelParams &p, int grid, cudaStream_t s) { launch_behind(select_kernel, grid, 128, 0, s, p); }
-void launch_map_scatter(uint8_t *grid, int nx, int ny, int nz, const uint8_t *box, int x0, int y0, int z0, int dx, int dy,
-                        int dz, cudaStream_t s) {
-    const size_t total = (size_t)dx * dy * dz;
-    const int blocks = (int)std::min<size_t>((total + 255) / 256, 4096);
-    map_scatter_kernel<<<blocks, 256, 0, s>>>(grid, nx, ny, box, x0, y0, z0, dx, dy, dz);
-    launch_bocc(grid, nx, ny, nz, x0, y0, z0, dx, dy, dz, s);  // the summaries of the bricks it touched
-    launch_brick_update(grid, nx, ny, nz, x0, y0, z0, dx, dy, dz, s);
-}
 void launch_plan(const DevPlanParams &p, cudaStream_t s) {
     const int grid = std::max(1, std::min((p.n + 255) / 256, 1024));
     plan_depth_kernel<<<grid, 256, 0, s>>>(p);

@@ -16,13 +16,13 @@
 namespace mig {
 
 template <class... P, class... A>
-inline void launch_behind(void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t s, const A &...args) {
+inline void launch_behind(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const A &...args) {
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t c{};
-    c.gridDim = dim3((unsigned)grid);
-    c.blockDim = dim3((unsigned)block);
+    c.gridDim = grid;
+    c.blockDim = block;
     c.dynamicSmemBytes = smem;
     c.stream = s;
     c.attrs = &at;

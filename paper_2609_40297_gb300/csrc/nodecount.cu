@@ -614,80 +614,6 @@ __global__ void __launch_bounds__(kWarpsN * 32, 4) brick_kernel(const LevelParam
     add_stats<STATS>(p, st);
 }
 
-// ---------------------------------------------------------------------------- brick data update
-// Masks of the bricks [b0, b1) from the voxel codes: one thread per brick. A row of four codes is
-// one 32-bit load where rows are 4-byte aligned; the codes 0 / 1 / 2 differ in their two low bits.
-__device__ __forceinline__ uint32_t nibble(uint32_t v) { return ((v & 0x01010101u) * 0x01020408u) >> 24; }
-
-__global__ void brick_mask_kernel(uint8_t *grid, int nx, int ny, int nz, int bx0, int by0, int bz0, int bx1, int by1, int bz1) {
-    const int nbx = (nx + 3) >> 2, nby = (ny + 3) >> 2;
-    uint64_t *um = reinterpret_cast<uint64_t *>(grid + umask_offset(nx, ny, nz));
-    uint64_t *om = reinterpret_cast<uint64_t *>(grid + omask_offset(nx, ny, nz));
-    const int wx = bx1 - bx0, wy = by1 - by0;
-    const long long total = (long long)wx * wy * (bz1 - bz0);
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-        const int bx = bx0 + (int)(i % wx), by = by0 + (int)((i / wx) % wy), bz = bz0 + (int)(i / ((long long)wx * wy));
-        const int w = min(4, nx - 4 * bx);
-        uint64_t u = 0, o = 0;
-        for (int z = 0; z < 4 && 4 * bz + z < nz; ++z)
-            for (int y = 0; y < 4 && 4 * by + y < ny; ++y) {
-                const uint8_t *r = grid + ((size_t)(4 * bz + z) * ny + (4 * by + y)) * nx + 4 * bx;
-                uint32_t c = 0x01010101u;  // beyond the grid: neither unknown nor occupied
-                if ((nx & 3) == 0) c = *reinterpret_cast<const uint32_t *>(r);
-                else
-                    for (int x = 0; x < w; ++x) c = (c & ~(0xFFu << (8 * x))) | ((uint32_t)r[x] << (8 * x));
-                u |= (uint64_t)nibble(~(c | (c >> 1))) << (16 * z + 4 * y);
-                o |= (uint64_t)nibble(c >> 1) << (16 * z + 4 * y);
-            }
-        const size_t b = ((size_t)bz * nby + by) * nbx + bx;
-        um[b] = u;
-        om[b] = o;
-    }
-}
-
-// One pass of the octant distances over the bricks of a box: along x from the masks (pass 0: both
-// directions, scratch 0-1), along y (pass 1: scratch 2-5), along z (pass 2: the eight octants and their
-// minimum). One-sided: d = min over j >= 0 of max(j, the previous pass j bricks ahead).
-__global__ void brick_dist_kernel(uint8_t *grid, int nx, int ny, int nz, int pass, int bx0, int by0, int bz0, int bx1, int by1,
-                                  int bz1) {
-    const int nbx = (nx + 3) >> 2, nby = (ny + 3) >> 2, nbz = (nz + 3) >> 2;
-    const uint64_t *om = reinterpret_cast<const uint64_t *>(grid + omask_offset(nx, ny, nz));
-    const size_t plane = dist_scratch_offset(nx, ny, nz, 1) - dist_scratch_offset(nx, ny, nz, 0);
-    uint8_t *scr = grid + dist_scratch_offset(nx, ny, nz, 0);
-    const int wx = bx1 - bx0, wy = by1 - by0;
-    const long long total = (long long)wx * wy * (bz1 - bz0);
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-        const int bx = bx0 + (int)(i % wx), by = by0 + (int)((i / wx) % wy), bz = bz0 + (int)(i / ((long long)wx * wy));
-        const size_t b = ((size_t)bz * nby + by) * nbx + bx;
-        if (pass == 0) {
-            int lo = kDistCap, hi = kDistCap;  // towards smaller and larger x
-            for (int j = min(kDistCap - 1, bx); j >= 0; --j) lo = om[b - j] ? j : lo;
-            for (int j = min(kDistCap - 1, nbx - 1 - bx); j >= 0; --j) hi = om[b + j] ? j : hi;
-            scr[b] = (uint8_t)lo;
-            scr[plane + b] = (uint8_t)hi;
-        } else {
-            const int c = pass == 1 ? by : bz, n = pass == 1 ? nby : nbz, arrays = pass == 1 ? 2 : 4;
-            const ptrdiff_t step = pass == 1 ? nbx : (ptrdiff_t)nbx * nby;
-            int least = kDistCap;
-            for (int a = 0; a < arrays; ++a) {
-                const uint8_t *src = scr + (size_t)(pass == 1 ? a : 2 + a) * plane;
-                int lo = kDistCap, hi = kDistCap;
-                for (int j = 0; j < kDistCap; ++j) {
-                    if (j <= c) lo = min(lo, max(j, (int)src[(ptrdiff_t)b - j * step]));
-                    if (c + j < n) hi = min(hi, max(j, (int)src[(ptrdiff_t)b + j * step]));
-                }
-                // array bits: x, then y, then z not backwards
-                uint8_t *d0 = pass == 1 ? scr + (size_t)(2 + a) * plane : grid + oct_offset(nx, ny, nz, a);
-                uint8_t *d1 = pass == 1 ? scr + (size_t)(4 + a) * plane : grid + oct_offset(nx, ny, nz, 4 + a);
-                d0[b] = (uint8_t)lo;
-                d1[b] = (uint8_t)hi;
-                least = min(least, min(lo, hi));
-            }
-            if (pass == 2) grid[dist_offset(nx, ny, nz) + b] = (uint8_t)least;
-        }
-    }
-}
-
 }  // namespace
 
 size_t hz_entries(int W, int H) { return (size_t)pyramid(W, H).n; }
@@ -833,30 +759,6 @@ void set_steps(LevelParams &p, void *base, const StepsLayout &L) {
     p.steps_cap = L.cap;
     p.tree = L.tree;
     p.depths = L.depths ? reinterpret_cast<uint32_t *>(b + L.o_depths) : nullptr;
-}
-
-void launch_brick_update(uint8_t *grid, int nx, int ny, int nz, int x0, int y0, int z0, int dx, int dy, int dz, cudaStream_t s) {
-    const BrickDims n = brick_dims(nx, ny, nz);
-    const int lo[3] = {x0 >> 2, y0 >> 2, z0 >> 2}, hi[3] = {(x0 + dx + 3) >> 2, (y0 + dy + 3) >> 2, (z0 + dz + 3) >> 2};
-    auto blocks = [](long long t) { return (int)std::max<long long>(1, std::min<long long>((t + 127) / 128, 8192)); };
-    brick_mask_kernel<<<blocks((long long)(hi[0] - lo[0]) * (hi[1] - lo[1]) * (hi[2] - lo[2])), 128, 0, s>>>(
-        grid, nx, ny, nz, lo[0], lo[1], lo[2], hi[0], hi[1], hi[2]);
-    // a brick's distance depends on the bricks up to kDistCap - 1 away along each axis
-    const int r = kDistCap, nb[3] = {n.nbx, n.nby, n.nbz};
-    int a[3], b[3], a2[3], b2[3];  // the bricks whose distance can change, and one reach beyond
-    for (int i = 0; i < 3; ++i) {
-        a[i] = std::max(0, lo[i] - r);
-        b[i] = std::min(nb[i], hi[i] + r);
-        a2[i] = std::max(0, lo[i] - 2 * r);
-        b2[i] = std::min(nb[i], hi[i] + 2 * r);
-    }
-    auto dist = [&](int pass, int ya, int yb, int za, int zb) {
-        brick_dist_kernel<<<blocks((long long)(b[0] - a[0]) * (yb - ya) * (zb - za)), 128, 0, s>>>(grid, nx, ny, nz, pass, a[0], ya, za,
-                                                                                                 b[0], yb, zb);
-    };
-    dist(0, a2[1], b2[1], a2[2], b2[2]);
-    dist(1, a[1], b[1], a2[2], b2[2]);
-    dist(2, a[1], b[1], a[2], b[2]);
 }
 
 }  // namespace mig

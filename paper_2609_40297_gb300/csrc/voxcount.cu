@@ -247,51 +247,6 @@ __global__ void __launch_bounds__(kVoxWarps * 32, 3) voxel_kernel(const LevelPar
     }
 }
 
-// ------------------------------------------------------------------------- brick occupancy
-// Recomputes the occupancy byte of every brick in [b0, b1) (brick coordinates).
-__global__ void bocc_kernel(uint8_t *grid, int nx, int ny, int nz, int bx0, int by0, int bz0, int bx1, int by1,
-                            int bz1) {
-    const int nbx = (nx + 7) >> 3, nby = (ny + 7) >> 3;
-    uint8_t *bocc = grid + bocc_offset(nx, ny, nz);
-    const int wx = bx1 - bx0, wy = by1 - by0;
-    const long long total = (long long)wx * wy * (bz1 - bz0);
-    const int lane = threadIdx.x & 31;
-    // one warp per brick: lane l checks rows (y, z) = (l & 7, l >> 3) and (l & 7, (l >> 3) + 4)
-    for (long long b = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); b < total;
-         b += (long long)gridDim.x * (blockDim.x >> 5)) {
-        const int bx = bx0 + (int)(b % wx), by = by0 + (int)((b / wx) % wy), bz = bz0 + (int)(b / ((long long)wx * wy));
-        bool occ = false;
-        for (int h = 0; h < 2; ++h) {
-            const int y = (by << 3) + (lane & 7), z = (bz << 3) + (lane >> 3) + 4 * h;
-            if (y >= ny || z >= nz) continue;
-            const uint8_t *row = grid + ((size_t)z * ny + y) * nx;
-            for (int x = bx << 3; x < min(nx, (bx << 3) + 8); ++x) occ |= row[x] == kOcc;
-        }
-        occ = __any_sync(0xffffffffu, occ);
-        if (lane == 0) bocc[((size_t)bz * nby + by) * nbx + bx] = occ ? 1 : 0;
-    }
-}
-
-// Recomputes the occupancy byte of every super-brick in [s0, s1) (super-brick coordinates) from its
-// bricks' bytes.
-__global__ void sbocc_kernel(uint8_t *grid, int nx, int ny, int nz, int sx0, int sy0, int sz0, int sx1, int sy1,
-                             int sz1) {
-    const int nbx = (nx + 7) >> 3, nby = (ny + 7) >> 3, nbz = (nz + 7) >> 3;
-    const int nsx = (nx + 31) >> 5, nsy = (ny + 31) >> 5;
-    const uint8_t *bocc = grid + bocc_offset(nx, ny, nz);
-    uint8_t *sbocc = grid + sbocc_offset(nx, ny, nz);
-    const int wx = sx1 - sx0, wy = sy1 - sy0;
-    const long long total = (long long)wx * wy * (sz1 - sz0);
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-        const int sx = sx0 + (int)(i % wx), sy = sy0 + (int)((i / wx) % wy), sz = sz0 + (int)(i / ((long long)wx * wy));
-        uint8_t occ = 0;
-        for (int bz = 4 * sz; bz < min(4 * sz + 4, nbz); ++bz)
-            for (int by = 4 * sy; by < min(4 * sy + 4, nby); ++by)
-                for (int bx = 4 * sx; bx < min(4 * sx + 4, nbx); ++bx) occ |= bocc[((size_t)bz * nby + by) * nbx + bx];
-        sbocc[((size_t)sz * nsy + sy) * nsx + sx] = occ ? 1 : 0;
-    }
-}
-
 }  // namespace
 
 size_t vox_dyn_smem(int max_anc) { return (size_t)kVoxWarps * (size_t)std::max(1, max_anc) * sizeof(AncRec); }
@@ -347,20 +302,6 @@ void launch_vox_level(const LevelParams &p, long long pairs, int num_sms, int vo
         if (node_pass(p)) launch_node_chunk(c, num_sms, node_ctas, s);
         else launch_voxel_chunk(c, num_sms, vox_ctas, s);
     }
-}
-
-void launch_bocc(uint8_t *grid, int nx, int ny, int nz, int x0, int y0, int z0, int dx, int dy, int dz, cudaStream_t s) {
-    const int bx0 = x0 >> 3, by0 = y0 >> 3, bz0 = z0 >> 3;
-    const int bx1 = (x0 + dx + 7) >> 3, by1 = (y0 + dy + 7) >> 3, bz1 = (z0 + dz + 7) >> 3;
-    const long long total = (long long)(bx1 - bx0) * (by1 - by0) * (bz1 - bz0);
-    const int grid_ = (int)std::max<long long>(1, std::min<long long>((total + 7) / 8, 4096));
-    bocc_kernel<<<grid_, 256, 0, s>>>(grid, nx, ny, nz, bx0, by0, bz0, bx1, by1, bz1);
-    // the super-bricks holding those bricks
-    const int sx0 = bx0 >> 2, sy0 = by0 >> 2, sz0 = bz0 >> 2;
-    const int sx1 = (bx1 + 3) >> 2, sy1 = (by1 + 3) >> 2, sz1 = (bz1 + 3) >> 2;
-    const long long stotal = (long long)(sx1 - sx0) * (sy1 - sy0) * (sz1 - sz0);
-    const int sgrid = (int)std::max<long long>(1, std::min<long long>((stotal + 255) / 256, 1024));
-    sbocc_kernel<<<sgrid, 256, 0, s>>>(grid, nx, ny, nz, sx0, sy0, sz0, sx1, sy1, sz1);
 }
 
 }  // namespace mig

@@ -64,9 +64,5 @@ int vox_chunk_pairs(const LevelParams &p);  // pairs per chunk (a multiple of K 
 int node_ctas_per_sm();
 int vox_ctas_per_sm();
 long long node_items(int64_t Tq);  // work items of one node of the per-node pass
-// Recomputes the masks of the 4x4x4 bricks overlapping a box of voxels and the distances around them.
-void launch_brick_update(uint8_t *grid, int nx, int ny, int nz, int x0, int y0, int z0, int dx, int dy, int dz, cudaStream_t s);
-// Recomputes the brick occupancy bytes of the bricks overlapping a box of voxels.
-void launch_bocc(uint8_t *grid, int nx, int ny, int nz, int x0, int y0, int z0, int dx, int dy, int dz, cudaStream_t s);
 
 }  // namespace mig
