@@ -714,6 +714,7 @@ mig_status batch_run_streams(mig_ctx *ctx, std::vector<BatchItem> &items) {
         const int t = order[oi];
         if (steps[t].cap) set_steps(lp[t], dev + o_steps[oi % S], steps[t]);
         lp[t].voxel_pass = ctx->count.pass;
+        lp[t].crowd = (int)S;
     }
     if (!ctx->batch) ctx->batch = new mig_ctx::Batch();
     mig_ctx::Batch *B = ctx->batch;

@@ -90,6 +90,7 @@ struct LevelParams {
     // per-node pass: half a pixel at unit depth along the image axes, the depth below which the owner
     // ray certainly visits its voxel, and the reciprocal focal lengths (set_visit_params)
     float vis_hu, vis_hv, vis_zl2, ifx, ify;
+    int crowd;  // trees whose launches run beside these (batches, servers), with this one; 0: alone
 };
 
 void launch_count(const LevelParams &p, int grid, cudaStream_t s);

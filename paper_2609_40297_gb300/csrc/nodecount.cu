@@ -665,12 +665,32 @@ int node_ctas_per_sm() {
 // Macro blocks of a node's range ball (its bounding box): the node pass's items per node.
 long long node_items(int64_t Tq) { return (long long)mac_xy(Tq) * mac_xy(Tq) * mac_z(Tq); }
 
+// Bricks that a node's range ball can touch.
+static long long node_bricks(int64_t Tq) {
+    const double r = ((double)Tq / 65536.0 + 1.0) / 4.0 + 1.74;
+    return (long long)(4.19 * r * r * r) + 1;
+}
+
+// The CTAs of a node pass of `items` work items, and of the brick pass that follows it for `nodes` nodes (and
+// groups of 64 yaws). A tree alone takes every SM it can use, down to one item per warp. Among others a
+// small level takes several items per warp instead, since its CTAs that find little to do, and the next
+// launch's that wait for it, keep the others' from the SMs: 9 trees of 10 to 78 nodes of 43x24x8 in one batch
+// 995 -> 750 us (935 row by row), while one of them alone takes 325 us with one item per warp, 329 with 8.
+int node_grid(long long items, int most, int crowd) {
+    const long long per_cta = kWarpsN * std::max(1, std::min(crowd, 8));
+    return (int)std::max<long long>(1, std::min<long long>((items + per_cta - 1) / per_cta, most));
+}
+int brick_grid(long long nodes, int64_t Tq, int num_sms, int crowd) {
+    const long long most = num_sms * 4;
+    return (int)(crowd > 1 ? std::max<long long>(1, std::min<long long>(most, nodes * node_bricks(Tq) / (4 * kWarpsN))) : most);
+}
+
 void launch_node_chunk(const LevelParams &c, int num_sms, int node_ctas, cudaStream_t s) {
     // a warp per macro block, or per block and eighth of the yaws where the blocks alone leave SMs idle (split)
-    const long long items = (long long)((c.q1 - c.q0) / c.K) * node_items(c.Tq) * std::min(c.K, kNodeSplit);
-    const int g = (int)std::max<long long>(1, std::min<long long>((items + kWarpsN - 1) / kWarpsN, (long long)num_sms * node_ctas));
+    const int nodes = (c.q1 - c.q0) / c.K;
+    const int g = node_grid((long long)nodes * node_items(c.Tq) * std::min(c.K, kNodeSplit), num_sms * node_ctas, c.crowd);
     const size_t smem = node_dyn_smem(c.K, c.max_anc);
-    const int gb = num_sms * 4;
+    const int gb = brick_grid((long long)nodes * ((c.K + 63) / 64), c.Tq, num_sms, c.crowd);
     if (c.mode == MIG_MODE_INTERVAL) {
         launch_behind(node_kernel<false, true>, g, kWarpsN * 32, smem, s, c, num_sms);
         launch_behind(brick_kernel<false, true>, gb, kWarpsN * 32, smem, s, c);
@@ -683,13 +703,8 @@ void launch_node_chunk(const LevelParams &c, int num_sms, int node_ctas, cudaStr
     }
 }
 
-// Bricks that a node's range ball can touch, and the records a chunk's queue has room for per node
-// (measured: up to 0.27 of them are left undecided as a whole; a fuller queue only sends its last
-// bricks through the slower path inside node_kernel).
-static long long node_bricks(int64_t Tq) {
-    const double r = ((double)Tq / 65536.0 + 1.0) / 4.0 + 1.74;
-    return (long long)(4.19 * r * r * r) + 1;
-}
+// The share of them that a chunk's queue has room for (measured: up to 0.27 of a node's bricks are left
+// undecided as a whole; a fuller queue only sends its last bricks through the slower path inside node_kernel).
 constexpr double kQueueShare = 0.3;
 constexpr double kQueueShareInterval = 0.7;  // there every counted brick that an ancestor looks at
 constexpr double kQueueSharePano = 0.5;      // every brick that a ray can reach

@@ -462,11 +462,10 @@ void launch_pano_tree_cast(const LevelParams &p, int levels, int num_sms, cudaSt
 }
 
 void launch_pano_voxel_chunk(const LevelParams &c, int num_sms, cudaStream_t s) {
-    const long long items = (long long)(c.q1 - c.q0) * node_items(c.Tq);
-    const int g = (int)std::max<long long>(1, std::min<long long>((items + kWarpsN - 1) / kWarpsN, (long long)num_sms * 3));
+    const int g = node_grid((long long)(c.q1 - c.q0) * node_items(c.Tq), num_sms * 3, c.crowd);
     const size_t smem = node_dyn_smem(c.K, c.max_anc);
     launch_behind(pano_node_kernel, g, kWarpsN * 32, smem, s, c, num_sms);
-    launch_behind(pano_brick_kernel, num_sms * 4, kWarpsN * 32, smem, s, c);
+    launch_behind(pano_brick_kernel, brick_grid(c.q1 - c.q0, c.Tq, num_sms, c.crowd), kWarpsN * 32, smem, s, c);
 }
 
 void pano_bricks_init() {

@@ -303,6 +303,7 @@ mig_status run_step(mig_server *s) {
         cudaStream_t st = s->pool[i % S];
         LevelParams p = r.p;
         p.lvl = r.level;
+        p.crowd = R;
         const HostPlan &pl = r.plan;
         const int d = r.level;
         const int Ld = pl.level_off[d + 1] - pl.level_off[d];

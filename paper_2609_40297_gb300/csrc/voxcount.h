@@ -63,6 +63,8 @@ bool node_pass(const LevelParams &p);  // whole nodes per chunk: the per-node pa
 int vox_chunk_pairs(const LevelParams &p);  // pairs per chunk (a multiple of K for the per-node pass)
 int node_ctas_per_sm();
 int vox_ctas_per_sm();
+int node_grid(long long items, int most, int crowd);  // CTAs of the node and the brick pass
+int brick_grid(long long nodes, int64_t Tq, int num_sms, int crowd);
 long long node_items(int64_t Tq);  // work items of one node of the per-node pass
 
 }  // namespace mig
