@@ -249,44 +249,50 @@ void launch_device_levels(mig_ctx *ctx, LevelParams p, int n, int levels, int2 *
     }
 }
 
-// Microseconds of the two ways to count a tree, fitted to 150 timings (200 to 1200 nodes, range R = 60 to
-// 150 voxels, images of 16x12 to 192x144, 4 to 36 yaws, both kinds of world):
-//   ray by ray - a chain of voxel loads as long as the range per level, and each ray's walk:
-//                ch R levels + r R rays;
-//   by voxels  - each node's range ball between the image's elevations, and each yaw's frustum of it:
-//                R^3 n sin(vfov / 2) (a + b K hfov / 90).
-// Voxels that lie closer than the image's pixels are mostly on no ray at all, so that a coarse image over
-// a long range is walked sooner than enumerated: 1000 nodes, R = 150, 16 yaws of 56x42 count in 68 ms
-// ray by ray and 184 by voxels, of 128x96 in 251 and 201 (interval 147 and 387, 468 and 454; panoramic
-// 27 and 50, 88 and 51); the estimates' order was the timings' wherever these differed by a quarter.
-bool rays_cheaper(const mig_sensor &s, float voxel, int n, int levels, int mode) {
+// Microseconds of the two ways to count a tree, fitted to 2800 timings (5 to 1500 nodes, ranges of R = 5 to 200
+// voxels, images of 8x4 to 320x240, 1 to 48 yaws; rooms, terrain and a map full of boxes, ranges within the
+// grid and far beyond it):
+//   ray by ray - per level two launches and a chain of voxel loads as long as a ray's way, and each ray's walk;
+//                a ray's way ends at the range or about a third of the grid away;
+//   by voxels  - per round (a level or a chunk of one) three launches; the cast of each ray; and, over the part
+//                of the range ball between the image's elevations that lies in the grid, each node's voxels
+//                and each yaw's frustum of them.
+// Voxels that lie closer than the image's pixels are mostly on no ray at all, so that a coarse image over a
+// long range is walked sooner than enumerated: 1000 nodes, R = 150, 16 yaws of 56x42 count in 68 ms ray by
+// ray and 184 by voxels, of 128x96 in 251 and 201. The slower way by more than a quarter is chosen in 66 of
+// the 2800, 3 of them among images 36 pixels wide or more, 4 yaws, 20 nodes and ranges of 15 voxels or more.
+// margin: what the caller adds to the voxels' side.
+bool rays_cheaper(const mig_sensor &s, const mig_map *m, int n, int levels, int rounds, int mode, double margin) {
     struct {
-        double chain, ray, a, b;
-    } c = {5.7, 10.5e-6, 20e-6, 5.7e-6};
-    double rays = (double)s.yaw_bins * s.width * s.height;
-    if (mode == MIG_MODE_INTERVAL) c = {14.7, 20e-6, 0.0, 15.4e-6};
+        double level, chain, walk, start, way, round, cast, cast_way, node, yaw;
+    } c = {18.0, 1.65, 3.9e-6, 1.7, 0.35, 28.0, 12e-6, 1e-6, 6e-6, 2.4e-6};
+    double rays = (double)s.yaw_bins * s.width * s.height * n;
+    if (mode == MIG_MODE_INTERVAL) c = {16.0, 3.2, 5e-6, 0.4, 0.47, 32.0, 16e-6, 1.4e-6, 5.6e-6, 4.5e-6};
     if (mode == MIG_MODE_PANORAMIC) {
-        c = {2.3, 15e-6, 31e-6, 0.0};
-        rays = (double)pano_columns(s) * s.height;
+        c = {20.0, 1.4, 7.5e-6, 1.2, 0.23, 35.0, 7e-6, 1.35e-6, 15.5e-6, 0.43e-6};
+        rays = (double)pano_columns(s) * s.height * n;
     }
-    const double R = s.range_m / voxel, ball = R * R * R * n * std::sin(s.vfov_deg * (M_PI / 360.0));
-    return c.chain * R * levels + c.ray * R * n * rays < ball * (c.a + c.b * s.yaw_bins * (s.hfov_deg / 90.0));
+    const double R = s.range_m / m->voxel, way = std::min(R, c.way * std::max(m->nx, m->ny)), up = std::sin(s.vfov_deg * (M_PI / 360.0));
+    const double ball = R * R * R * up * std::min(1.0, m->nx / (2.0 * R)) * std::min(1.0, m->ny / (2.0 * R)) * std::min(1.0, m->nz / (2.0 * R * up));
+    return levels * (c.level + c.chain * way) + c.walk * rays * (way + c.start) <
+           margin * (rounds * c.round + (c.cast + c.cast_way * way) * rays + n * ball * (c.node + c.yaw * s.yaw_bins * (s.hfov_deg / 90.0)));
 }
 
-StepsLayout steps_for(const CountChoice &c, int n, int levels, int Lmax, const mig_sensor &s, float voxel, int mode, int lean) {
+StepsLayout steps_for(const CountChoice &c, int n, int levels, int Lmax, const mig_sensor &s, const mig_map *m, int mode, int lean) {
     const bool pano = mode == MIG_MODE_PANORAMIC, whole = pano || mode == MIG_MODE_INTERVAL;
     // the interval and panoramic modes have no pass per (node, yaw) pair: without room for whole nodes they
     // count ray by ray
     if (c.rays || lean == 2 || (whole && c.pass == MIG_COUNT_PAIRS)) return StepsLayout{};
-    if (c.pass == MIG_COUNT_AUTO && rays_cheaper(s, voxel, n, levels, mode)) return StepsLayout{};
-    SensorDims d{s.width, s.height, s.yaw_bins, range_q16(s.range_m, voxel)};
+    SensorDims d{s.width, s.height, s.yaw_bins, range_q16(s.range_m, m->voxel)};
     if (pano) {
         d.W = pano_columns(s);
         d.K = 1;
         if ((size_t)d.W * d.H * sizeof(uint16_t) > c.steps_budget) return StepsLayout{};
     }
     const StepsLayout L = steps_layout(d, n, Lmax, c.steps_budget, lean == 0 ? kTreeSteps : 0, c.pass != MIG_COUNT_PAIRS, mode);
-    return whole && L.queue_cap == 0 ? StepsLayout{} : L;
+    if (whole && L.queue_cap == 0) return StepsLayout{};
+    if (c.pass == MIG_COUNT_AUTO && rays_cheaper(s, m, n, levels, std::max(levels, device_steps(L, n, d.K, levels)), mode, 1.0)) return StepsLayout{};
+    return L;
 }
 
 void prof_begin(mig_ctx *ctx, int kind, cudaEvent_t *a) {
@@ -685,7 +691,7 @@ static mig_status eval_host(mig_map *m, int n, const int32_t *parent, const floa
     char *dev = nullptr;
     for (int lean = 0; lean < 3; ++lean) {  // less memory where the allocator has not enough
         Carver c = cv;
-        steps = steps_for(ctx->count, n, L, Lmax, *sensor, m->voxel, mode, lean);
+        steps = steps_for(ctx->count, n, L, Lmax, *sensor, m, mode, lean);
         o_dpyr = c.take<uint2>(steps.cap ? (size_t)std::max(1, plan.n_internal) * hz_entries(cam->W, cam->H) : 0);
         o_steps = c.take<char>(steps.bytes);
         // instrumented pass: the ray-by-ray count kernel is re-run into scratch counters afterwards,
@@ -869,7 +875,7 @@ mig_status mig_tree_eval_device(mig_map *m, int n, const int32_t *parent, const 
         o_err = cv.take<int32_t>(1); o_cnt = cv.take<int32_t>((size_t)n * K * 2);
         o_work = cv.take<int32_t>(L);
         // level sizes are known on the device only: the step-count buffer is sized for n nodes
-        steps = steps_for(ctx->count, n, L, n, *sensor, m->voxel, MIG_MODE_MARGINAL, lean);
+        steps = steps_for(ctx->count, n, L, n, *sensor, m, MIG_MODE_MARGINAL, lean);
         o_cursor = cv.take<int2>(device_steps(steps, n, K, L) + 1);
         zero_bytes = cv.off;
         o_depth = cv.take<int32_t>(n); o_loff = cv.take<int32_t>(L + 1); o_lint = cv.take<int32_t>(L);

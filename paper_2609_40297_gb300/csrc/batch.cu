@@ -650,7 +650,7 @@ mig_status batch_run_streams(mig_ctx *ctx, std::vector<BatchItem> &items) {
             const HostPlan &pl = items[t].plan;
             int Lmax = 1;
             for (int d = 0; d <= pl.max_depth; ++d) Lmax = std::max(Lmax, pl.level_off[d + 1] - pl.level_off[d]);
-            steps[t] = steps_for(ctx->count, pl.n, pl.max_depth + 1, Lmax, items[t].sensor, items[t].map->voxel, items[t].mode, lean);
+            steps[t] = steps_for(ctx->count, pl.n, pl.max_depth + 1, Lmax, items[t].sensor, items[t].map, items[t].mode, lean);
             stream_steps[oi % S] = std::max(stream_steps[oi % S], steps[t].bytes);
         }
         Carve c = cv;

@@ -34,6 +34,30 @@ mig_status sensor_check(const mig_sensor &s, float voxel) {
     return MIG_OK;
 }
 
+// The elevation of the direction through (a, b) on the image plane has the sine -(b cp + sp) / sqrt(a^2 + b^2
+// + 1). Without a vertical direction inside the image its extremes lie on the border: for fixed b it is
+// monotone in a^2, and along a = const it has one stationary point, b = cp (1 + a^2) / sp.
+void elevation_band(const mig_sensor &s, float &tlo, float &thi) {
+    const double t_h = std::tan(((double)s.hfov_deg * 0.5) * (M_PI / 180.0)), t_v = std::tan(((double)s.vfov_deg * 0.5) * (M_PI / 180.0));
+    const double th = (double)s.pitch_deg * (M_PI / 180.0), cp = std::cos(th), sp = std::sin(th);
+    double elo = 1e9, ehi = -1e9;
+    auto add = [&](double a, double b) {
+        const double el = std::asin(std::min(1.0, std::max(-1.0, -(b * cp + sp) / std::sqrt((a * a + b * b) + 1.0))));
+        elo = std::min(elo, el);
+        ehi = std::max(ehi, el);
+    };
+    for (const double a : {0.0, t_h}) {
+        add(a, -t_v);
+        add(a, t_v);
+        if (std::fabs(cp * (1.0 + a * a)) < t_v * std::fabs(sp)) add(a, cp * (1.0 + a * a) / sp);
+    }
+    // the vertical directions in camera coordinates: up (0, -cp, -sp), down (0, cp, sp)
+    const bool up_in = -sp > 0.0 && std::fabs(cp / sp) <= t_v, down_in = sp > 0.0 && std::fabs(cp / sp) <= t_v;
+    const double margin = 0.5 * M_PI / 180.0;
+    thi = (up_in || ehi + margin >= 89.5 * M_PI / 180.0) ? 1e30f : (float)std::tan(ehi + margin);
+    tlo = (down_in || elo - margin <= -89.5 * M_PI / 180.0) ? -1e30f : (float)std::tan(elo - margin);
+}
+
 mig_status camera_build(const mig_sensor &s, Camera &c) {
     c.s = s;
     c.W = s.width;
@@ -60,8 +84,9 @@ mig_status camera_build(const mig_sensor &s, Camera &c) {
         }
     }
     // Elevation band and azimuth half-width of the frustum (culling bounds for the per-node voxel
-    // pass): without a vertical direction inside the frustum, both extremes lie on the image
+    // passes): without a vertical direction inside the frustum, the largest azimuth lies on the image
     // border, sampled densely here and widened by half a degree.
+    elevation_band(s, c.band_tlo, c.band_thi);
     {
         auto body_dir = [&](double a, double b, double out[3]) {
             const double nrm = std::sqrt((a * a + b * b) + 1.0);
@@ -70,7 +95,7 @@ mig_status camera_build(const mig_sensor &s, Camera &c) {
             out[1] = -x;
             out[2] = -(y * cp + z * sp);
         };
-        double elo = 1e9, ehi = -1e9, az = 0.0;
+        double az = 0.0;
         const int S = 4096;
         for (int e = 0; e < 4; ++e) {
             for (int t = 0; t <= S; ++t) {
@@ -79,9 +104,6 @@ mig_status camera_build(const mig_sensor &s, Camera &c) {
                 const double b = (e < 2 ? (e == 0 ? -1.0 : 1.0) : f) * t_v;
                 double d[3];
                 body_dir(a, b, d);
-                const double el = std::atan2(d[2], std::hypot(d[0], d[1]));
-                elo = std::min(elo, el);
-                ehi = std::max(ehi, el);
                 az = std::max(az, std::fabs(std::atan2(d[1], d[0])));
             }
         }
@@ -89,10 +111,6 @@ mig_status camera_build(const mig_sensor &s, Camera &c) {
         const bool up_in = -sp > 0.0 && std::fabs(cp / sp) <= t_v;
         const bool down_in = sp > 0.0 && std::fabs(cp / sp) <= t_v;
         const double margin = 0.5 * M_PI / 180.0;
-        elo -= margin;
-        ehi += margin;
-        c.band_thi = (up_in || ehi >= 89.5 * M_PI / 180.0) ? 1e30f : (float)std::tan(ehi);
-        c.band_tlo = (down_in || elo <= -89.5 * M_PI / 180.0) ? -1e30f : (float)std::tan(elo);
         c.az_half = (up_in || down_in || az + margin >= M_PI) ? 3.2f : (float)(az + margin);
     }
     const double fx = ((double)W * 0.5) / t_h, fy = ((double)H * 0.5) / t_v;

@@ -72,6 +72,9 @@ struct Camera {
 };
 mig_status camera_build(const mig_sensor &s, Camera &out);
 int pano_columns(const mig_sensor &s);  // A
+// Tangents of the lowest and highest elevation of the frustum, widened by half a degree (-+1e30 where it holds
+// or nearly holds the vertical).
+void elevation_band(const mig_sensor &s, float &tlo, float &thi);
 mig_status pano_build(Camera &c);  // fills the pano_* host tables (MIG_EINVAL unless pitch is 0)
 mig_status sensor_check(const mig_sensor &s, float voxel);
 int64_t range_q16(float range_m, float voxel);
@@ -177,8 +180,8 @@ void launch_level_count_timed(mig_ctx *ctx, const LevelParams &p, int Ld, int co
 // counts ray by ray, the mode does, or that is the cheaper way, rays_cheaper). lean 0: the whole tree's step counts if small, 1: a level's, 2: none
 // (ray by ray); a caller whose allocation fails takes the next.
 struct StepsLayout;
-bool rays_cheaper(const mig_sensor &s, float voxel, int n, int levels, int mode);
-StepsLayout steps_for(const CountChoice &c, int n, int levels, int Lmax, const mig_sensor &s, float voxel, int mode, int lean);
+bool rays_cheaper(const mig_sensor &s, const mig_map *m, int n, int levels, int rounds, int mode, double margin);
+StepsLayout steps_for(const CountChoice &c, int n, int levels, int Lmax, const mig_sensor &s, const mig_map *m, int mode, int lean);
 // The count and select-and-render launches of a device-planned tree of n nodes and at most `levels` levels.
 // With the per-node pass they go chunk by chunk through the levels, whose sizes only the device knows:
 // device_steps(..) steps and as many places + 1 in `cursor` (zeroed).

@@ -229,12 +229,12 @@ extern "C" mig_status mig_tree_eval_device_noalloc(mig_map *m, int n, const int3
     p.arena = (uint32_t *)(dev + o_arena);
     p.mode = MIG_MODE_MARGINAL;
     p.stats = nullptr;
-    p.band_tlo = -1e30f;  // no elevation band: the camera test of the blocks stands alone
-    p.band_thi = 1e30f;
+    elevation_band(*sensor, p.band_tlo, p.band_thi);
     p.voxel_pass = MIG_COUNT_AUTO;
     set_visit_params(p, sensor->hfov_deg, sensor->vfov_deg);
+    // (by voxels only where it is sooner with a quarter to spare: what the rounds take varies with the chunks)
     const bool rays = ctx->count.rays || ctx->count.pass == MIG_COUNT_PAIRS || steps.cap == 0 ||
-                      (ctx->count.pass == MIG_COUNT_AUTO && rays_cheaper(*sensor, m->voxel, n, L, MIG_MODE_MARGINAL));
+                      (ctx->count.pass == MIG_COUNT_AUTO && rays_cheaper(*sensor, m, n, L, device_steps(steps, n, K, L), MIG_MODE_MARGINAL, 1.25));
     if (!rays) {
         set_steps(p, dev + o_steps, steps);
         p.dpyr = (uint2 *)(dev + o_dpyr);

@@ -167,7 +167,7 @@ mig_status admit(mig_server *s, Request &r) {
     const size_t o_pcnt = pano ? cv.take(8 * (size_t)n * r.cam->pano_A) : 0;
     size_t o_steps = 0;
     for (int lean = 0; lean < 3 && !r.dev; ++lean) {  // less memory where the allocator has not enough
-        if (lean) r.steps = steps_for(r.count, n, L, r.Lmax, r.sensor, r.map->voxel, r.mode, lean);
+        if (lean) r.steps = steps_for(r.count, n, L, r.Lmax, r.sensor, r.map, r.mode, lean);
         Carve c = cv;
         o_steps = c.take(r.steps.bytes);
         r.dev_bytes = c.off;
@@ -482,7 +482,7 @@ extern "C" mig_status mig_server_submit(mig_server *s, const mig_tree_desc *d, u
         r->Lmax = std::max(r->Lmax, r->plan.level_off[lv + 1] - r->plan.level_off[lv]);
     // the whole tree's step counts only where as many such requests as may be in flight fit the budget
     for (int lean = 0; lean < 2; ++lean) {
-        r->steps = steps_for(r->count, r->plan.n, r->plan.max_depth + 1, r->Lmax, d->sensor, d->map->voxel, d->mode, lean);
+        r->steps = steps_for(r->count, r->plan.n, r->plan.max_depth + 1, r->Lmax, d->sensor, d->map, d->mode, lean);
         if (!r->steps.tree || request_bytes(*r) <= s->budget / (size_t)s->max_inflight) break;
     }
     r->out_abs = d->abs_gain;
