@@ -273,7 +273,8 @@ mig_status mig_batch_trace_read(mig_ctx *ctx, mig_trace_rec *out, int cap, int *
 
 /* ---------------------------------------------------------------------------------------
  * Serving: continuous batching of replanning requests. Submitted trees wait in an admission
- * queue until their device bytes (depth-buffer arena nodes * W * H * 4, counters, step counts) plus
+ * queue until their device bytes (depth-buffer arena nodes * W * H * 4, counters, and their share of the
+ * budget, budget / max_inflight, or at most the step counts of their largest level where that is more) plus
  * the bytes already held (requests in flight and map snapshots) fit the budget, then
  * join the device work of the requests already running; each request's results are the same
  * as a lone mig_tree_eval on the map contents at submission time. The descriptor's host arrays

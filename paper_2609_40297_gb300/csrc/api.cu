@@ -278,17 +278,18 @@ bool rays_cheaper(const mig_sensor &s, const mig_map *m, int n, int levels, int 
            margin * (rounds * c.round + (c.cast + c.cast_way * way) * rays + n * ball * (c.node + c.yaw * s.yaw_bins * (s.hfov_deg / 90.0)));
 }
 
+SensorDims steps_dims(const mig_sensor &s, const mig_map *m, int mode) {
+    const bool pano = mode == MIG_MODE_PANORAMIC;
+    return SensorDims{pano ? pano_columns(s) : s.width, s.height, pano ? 1 : s.yaw_bins, range_q16(s.range_m, m->voxel)};
+}
+
 StepsLayout steps_for(const CountChoice &c, int n, int levels, int Lmax, const mig_sensor &s, const mig_map *m, int mode, int lean) {
     const bool pano = mode == MIG_MODE_PANORAMIC, whole = pano || mode == MIG_MODE_INTERVAL;
     // the interval and panoramic modes have no pass per (node, yaw) pair: without room for whole nodes they
     // count ray by ray
     if (c.rays || lean == 2 || (whole && c.pass == MIG_COUNT_PAIRS)) return StepsLayout{};
-    SensorDims d{s.width, s.height, s.yaw_bins, range_q16(s.range_m, m->voxel)};
-    if (pano) {
-        d.W = pano_columns(s);
-        d.K = 1;
-        if ((size_t)d.W * d.H * sizeof(uint16_t) > c.steps_budget) return StepsLayout{};
-    }
+    const SensorDims d = steps_dims(s, m, mode);
+    if (pano && (size_t)d.W * d.H * sizeof(uint16_t) > c.steps_budget) return StepsLayout{};
     const StepsLayout L = steps_layout(d, n, Lmax, c.steps_budget, lean == 0 ? kTreeSteps : 0, c.pass != MIG_COUNT_PAIRS, mode);
     if (whole && L.queue_cap == 0) return StepsLayout{};
     if (c.pass == MIG_COUNT_AUTO && rays_cheaper(s, m, n, levels, std::max(levels, device_steps(L, n, d.K, levels)), mode, 1.0)) return StepsLayout{};

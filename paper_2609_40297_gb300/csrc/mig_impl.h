@@ -180,6 +180,8 @@ void launch_level_count_timed(mig_ctx *ctx, const LevelParams &p, int Ld, int co
 // counts ray by ray, the mode does, or that is the cheaper way, rays_cheaper). lean 0: the whole tree's step counts if small, 1: a level's, 2: none
 // (ray by ray); a caller whose allocation fails takes the next.
 struct StepsLayout;
+struct SensorDims;
+SensorDims steps_dims(const mig_sensor &s, const mig_map *m, int mode);  // the images of one node
 bool rays_cheaper(const mig_sensor &s, const mig_map *m, int n, int levels, int rounds, int mode, double margin);
 StepsLayout steps_for(const CountChoice &c, int n, int levels, int Lmax, const mig_sensor &s, const mig_map *m, int mode, int lean);
 // The count and select-and-render launches of a device-planned tree of n nodes and at most `levels` levels.

@@ -117,7 +117,7 @@ extern "C" mig_status mig_tree_eval_device_noalloc(mig_map *m, int n, const int3
     const size_t o_cursor = cv.take(sizeof(int2) * ((size_t)n + L + 1)), o_steps = cv.take(0);
     const SensorDims dims{W, H, K, range_q16(sensor->range_m, m->voxel)};
     const StepsLayout steps = o_steps < (size_t)MIG_NOALLOC_SCRATCH_BYTES
-                                  ? steps_layout_in(dims, n, (size_t)MIG_NOALLOC_SCRATCH_BYTES - o_steps)
+                                  ? steps_layout_in(dims, n, n, (size_t)MIG_NOALLOC_SCRATCH_BYTES - o_steps)
                                   : StepsLayout{};
     if (need > (size_t)MIG_NOALLOC_SCRATCH_BYTES)
         return fail(MIG_EINVAL, "tree_eval_device_noalloc: needs " + std::to_string(need) + " bytes of scratch, above the " +

@@ -746,7 +746,7 @@ StepsLayout steps_layout(const SensorDims &d, int n, int max_nodes, size_t budge
     return L;
 }
 
-StepsLayout steps_layout_in(const SensorDims &d, int max_nodes, size_t bytes) {
+StepsLayout steps_layout_in(const SensorDims &d, int n, int max_nodes, size_t bytes) {
     // per node: its step counts, their bounds and 0.7 of the usual queue (a full queue only slows the
     // bricks beyond it), so that a fixed region holds more nodes at a time
     const size_t recs = (size_t)(0.7 * kQueueShare * (double)node_bricks(d.Tq)) + 1;
@@ -758,8 +758,17 @@ StepsLayout steps_layout_in(const SensorDims &d, int max_nodes, size_t bytes) {
     const long long nodes = std::min<long long>(std::min<long long>(max_nodes, (1 << kRecNodeBits) - 1), (long long)((bytes - fixed) / node));
     L.cap = (int)std::min<long long>(nodes, INT_MAX / d.K) * d.K;
     L.queue_cap = (int)std::min<long long>(kQueueMax, (long long)(L.cap / d.K) * recs);
-    // room for the whole tree (max_nodes nodes): one cast
-    if (nodes == max_nodes && (double)nodes * (double)node_items(d.Tq) * d.K < (double)(1ll << 30)) L.tree = max_nodes;
+    // room for the whole tree: one cast
+    if (nodes == n && (double)nodes * (double)node_items(d.Tq) * d.K < (double)(1ll << 30)) L.tree = n;
+    place(L, d);
+    return L;
+}
+
+StepsLayout steps_pairs_in(const SensorDims &d, int max_nodes, size_t bytes) {
+    const size_t pair = (size_t)d.W * d.H * sizeof(uint16_t) + hz_entries(d.W, d.H) * sizeof(uint32_t), fixed = 4 * 256;
+    StepsLayout L{};
+    if (bytes < fixed + pair) return L;
+    L.cap = (int)std::min<long long>((long long)std::min<size_t>((bytes - fixed) / pair, INT_MAX), (long long)max_nodes * d.K);
     place(L, d);
     return L;
 }

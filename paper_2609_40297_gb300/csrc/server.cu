@@ -112,6 +112,12 @@ struct mig_server {
 
 namespace {
 
+// Bounds of a request's depth buffers: read by the per-node passes, which have a queue.
+size_t depth_bounds(const Request &r) {
+    return sizeof(uint2) * std::max(1, r.plan.n_internal) * hz_entries(r.sensor.width, r.sensor.height);
+}
+size_t dpyr_bytes(const Request &r) { return r.steps.queue_cap ? depth_bounds(r) : 0; }
+
 size_t request_bytes(const Request &r) {
     const HostPlan &pl = r.plan;
     const size_t n = pl.n, L = pl.max_depth + 1, K = r.sensor.yaw_bins;
@@ -128,9 +134,36 @@ size_t request_bytes(const Request &r) {
     cv.take(12 * n);
     cv.take(4 * n);
     cv.take(4 * std::max(1, pl.n_internal) * WH);
-    cv.take(sizeof(uint2) * std::max(1, pl.n_internal) * hz_entries(r.sensor.width, r.sensor.height));
+    cv.take(dpyr_bytes(r));
     cv.take(r.steps.bytes);
     return cv.off;
+}
+
+// The device region of a request's count: the largest that leaves as many requests in flight as the budget
+// can hold. Its own share of the budget always does; beyond that a request takes no more than the step counts
+// of its largest level (marginal, single parent and absolute mode), without room for anything else: bounds and
+// queue then come out of it, for fewer nodes at a time (a full queue only slows the bricks beyond it).
+void choose_region(const mig_server *s, Request &r) {
+    const HostPlan &pl = r.plan;
+    const size_t share = s->budget / (size_t)s->max_inflight;
+    const SensorDims d = steps_dims(r.sensor, r.map, r.mode);
+    const bool sample = r.mode != MIG_MODE_INTERVAL && r.mode != MIG_MODE_PANORAMIC;
+    size_t counts = 0;
+    if (sample)
+        counts = (steps_pairs((long long)r.Lmax * d.K, d.W, d.H, r.count.steps_budget) * d.W * d.H * sizeof(uint16_t) + 511) & ~(size_t)255;
+    r.steps = StepsLayout{};
+    const size_t bare = request_bytes(r), most = std::max(share, bare + counts);
+    for (int lean = 0; lean < 2; ++lean) {
+        r.steps = steps_for(r.count, pl.n, pl.max_depth + 1, r.Lmax, r.sensor, r.map, r.mode, lean);
+        if (request_bytes(r) <= most) return;
+    }
+    const size_t region = most - bare, bounds = depth_bounds(r) + 256;
+    r.steps = StepsLayout{};
+    if (r.count.pass != MIG_COUNT_PAIRS && bounds < region) r.steps = steps_layout_in(d, pl.n, r.Lmax, region - bounds);
+    if (r.steps.cap == 0 && sample) {  // not one node: by (node, yaw) pairs, or ray by ray
+        r.count.pass = MIG_COUNT_PAIRS;
+        r.steps = steps_pairs_in(d, r.Lmax, region);
+    }
 }
 
 std::shared_ptr<Grid> current_grid(mig_server *s, mig_map *m) {
@@ -163,12 +196,16 @@ mig_status admit(mig_server *s, Request &r) {
     const size_t zero_end = cv.off;
     const size_t o_out = cv.take(12 * (size_t)n), o_sel = cv.take(4 * (size_t)n);
     const size_t o_arena = cv.take(4 * (size_t)std::max(1, pl.n_internal) * WH);
-    const size_t o_dpyr = cv.take(sizeof(uint2) * (size_t)std::max(1, pl.n_internal) * hz_entries(r.sensor.width, r.sensor.height));
     const size_t o_pcnt = pano ? cv.take(8 * (size_t)n * r.cam->pano_A) : 0;
-    size_t o_steps = 0;
+    size_t o_dpyr = 0, o_steps = 0;
     for (int lean = 0; lean < 3 && !r.dev; ++lean) {  // less memory where the allocator has not enough
-        if (lean) r.steps = steps_for(r.count, n, L, r.Lmax, r.sensor, r.map, r.mode, lean);
+        if (lean) {
+            const StepsLayout less = steps_for(r.count, n, L, r.Lmax, r.sensor, r.map, r.mode, lean);
+            if (less.bytes >= r.steps.bytes) continue;
+            r.steps = less;
+        }
         Carve c = cv;
+        o_dpyr = c.take(dpyr_bytes(r));
         o_steps = c.take(r.steps.bytes);
         r.dev_bytes = c.off;
         r.dev = (char *)ctx->alloc.alloc(r.dev_bytes, ctx->stream);
@@ -233,7 +270,7 @@ mig_status admit(mig_server *s, Request &r) {
     p.max_anc = std::max(1, pl.max_depth);
     if (pano) set_pano_params(p, r.cam, (int32_t *)(r.dev + o_pcnt));
     if (r.steps.cap) set_steps(p, r.dev + o_steps, r.steps);
-    p.dpyr = (uint2 *)(r.dev + o_dpyr);
+    p.dpyr = r.steps.queue_cap ? (uint2 *)(r.dev + o_dpyr) : nullptr;
     p.voxel_pass = r.count.pass;
     r.level = 0;
     return MIG_OK;
@@ -480,11 +517,7 @@ extern "C" mig_status mig_server_submit(mig_server *s, const mig_tree_desc *d, u
     }
     for (int lv = 0; lv <= r->plan.max_depth; ++lv)
         r->Lmax = std::max(r->Lmax, r->plan.level_off[lv + 1] - r->plan.level_off[lv]);
-    // the whole tree's step counts only where as many such requests as may be in flight fit the budget
-    for (int lean = 0; lean < 2; ++lean) {
-        r->steps = steps_for(r->count, r->plan.n, r->plan.max_depth + 1, r->Lmax, d->sensor, d->map, d->mode, lean);
-        if (!r->steps.tree || request_bytes(*r) <= s->budget / (size_t)s->max_inflight) break;
-    }
+    choose_region(s, *r);
     r->out_abs = d->abs_gain;
     r->out_marg = d->marg_gain;
     r->out_yaw = d->best_yaw;

@@ -1,0 +1,81 @@
+"""Device memory at its limits: a server's budget holds as many requests in flight as their depth buffers and
+the step counts of their largest levels allow, whatever else their counts could use; and an allocator that has
+refused a large workspace is not asked for it again by every later call."""
+import math
+import threading
+import time
+
+import numpy as np
+import pytest
+
+import synth
+from synth import Sensor
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():  # pragma: no cover
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+import paper_2609_40297_gb300 as mig  # noqa: E402
+
+
+def _problem(seed, sensor, n=24, depth=6):
+    return synth.random_small(seed, nx=60, ny=60, nz=30, v=0.1, p_occ=0.001, n_nodes=n, max_depth=depth, sensor=sensor)
+
+
+def _bytes(parent, s, counts, columns):
+    """Depth buffers, plan, counters (also per column) and, with counts, a uint16 per ray of the largest level."""
+    parent = np.asarray(parent)
+    depth = np.zeros(len(parent), int)
+    for i in range(len(parent)):
+        j = parent[i]
+        while j >= 0:
+            depth[i] += 1
+            j = parent[j]
+    n, levels, rays, K = len(parent), depth.max() + 1, s.width * s.height, s.yaw_bins
+    parts = [16 * n, 8 * n, 4 * max(1, depth.sum()), 4 * (levels + 1), 4 * levels, 4 * n, 8 * n * K, 4 * levels, 12 * n, 4 * n,
+             4 * max(1, len(set(parent[parent >= 0]))) * rays]
+    if counts:
+        parts += [2 * np.bincount(depth).max() * K * rays, 256]
+    if columns:
+        parts += [8 * n * K * math.ceil(s.width * 360 / (s.hfov_deg * K))]
+    return int(sum((p + 255) // 256 * 256 for p in parts))
+
+
+@pytest.mark.parametrize("mode", [mig.MODE_MARGINAL, mig.MODE_ABSOLUTE, mig.MODE_INTERVAL, mig.MODE_PANORAMIC])
+@pytest.mark.parametrize("image", [(40, 30, 8), (9, 6, 3), (96, 72, 2)])
+def test_budget_holds_its_requests(image, mode):
+    w, h, yaws = image
+    p = _problem(141, Sensor(90, 60, w, h, 2.0, yaws, 0.0))
+    busy = _problem(142, Sensor(90, 60, 320, 240, 2.0, 36, 0.0), 600, 12)
+    counts = mode in (mig.MODE_MARGINAL, mig.MODE_ABSOLUTE)
+    flight = 5
+    budget = flight * _bytes(p.tree.parent, p.sensor, counts, mode == mig.MODE_PANORAMIC)
+    ctx = mig.Context(0, stream=torch.cuda.Stream())
+    m = mig.Map(ctx, p.map.grid, p.map.voxel_size, p.map.origin)
+    try:
+        want = mig.tree_eval(m, p.tree.parent, p.tree.pos, p.sensor, mode=mode)
+        peaks = []
+        for k in (1, flight):
+            srv = mig.Server(ctx, arena_budget_bytes=budget, max_inflight=4096)
+            try:
+                # a long call holds the context until all requests wait, so that they are admitted together
+                holds = threading.Thread(target=mig.tree_eval_stats, args=(m, busy.tree.parent, busy.tree.pos, busy.sensor))
+                holds.start()
+                time.sleep(0.02)
+                subs = [srv.submit(m, p.tree.parent, p.tree.pos, p.sensor, mode=mode) for _ in range(k)]
+                assert holds.is_alive()
+                for t, _ in subs:
+                    assert srv.poll(t, timeout_us=30_000_000)
+                holds.join()
+                peaks.append(srv.memory()["peak"])
+                for _, got in subs:
+                    for key in ("abs", "marg", "yaw"):
+                        assert np.array_equal(got[key], want[key]), key
+            finally:
+                srv.close()
+        assert peaks[1] == flight * peaks[0] and peaks[1] <= budget
+    finally:
+        m.close()
+        ctx.close()
