@@ -52,7 +52,10 @@ mig_status ctx_workspace(mig_ctx *ctx, size_t bytes, void **out) {
         void *p = ctx->alloc.alloc(want, ctx->stream);
         if (!p) {
             p = ctx->alloc.alloc(bytes, ctx->stream);
-            if (!p) return fail(MIG_ENOMEM, "device workspace allocation of " + std::to_string(bytes) + " bytes failed");
+            if (!p) {
+                ctx->ws_refused.note(bytes);
+                return fail(MIG_ENOMEM, "device workspace allocation of " + std::to_string(bytes) + " bytes failed");
+            }
             ctx->ws.bytes = bytes;
         } else {
             ctx->ws.bytes = want;
@@ -62,6 +65,8 @@ mig_status ctx_workspace(mig_ctx *ctx, size_t bytes, void **out) {
     *out = ctx->ws.ptr;
     return MIG_OK;
 }
+
+bool ctx_workspace_refused(mig_ctx *ctx, size_t bytes) { return bytes > ctx->ws.bytes && ctx->ws_refused.skip(bytes); }
 
 mig_status ctx_pinned(mig_ctx *ctx, size_t bytes, void **out) {
     if (ctx->pinned_bytes < bytes) {
@@ -699,6 +704,7 @@ static mig_status eval_host(mig_map *m, int n, const int32_t *parent, const floa
         // for the method's own work counts (rays, DDA steps, owner tests) and as a cross-check
         rerun = stats && steps.cap > 0;
         o_cnt2 = c.take<int32_t>(rerun ? (size_t)n * K * 2 + L : 1);
+        if (lean < 2 && ctx_workspace_refused(ctx, c.off)) continue;
         st = ctx_workspace(ctx, c.off, (void **)&dev);
         if (st != MIG_ENOMEM) break;
     }
@@ -886,6 +892,7 @@ mig_status mig_tree_eval_device(mig_map *m, int n, const int32_t *parent, const 
         o_arena = cv.take<uint32_t>((size_t)n * WH);
         o_dpyr = cv.take<uint2>(steps.cap ? (size_t)n * hz_entries(cam->W, cam->H) : 0);
         o_steps = cv.take<char>(steps.bytes);
+        if (lean < 2 && ctx_workspace_refused(ctx, cv.off)) continue;
         st = ctx_workspace(ctx, cv.off, (void **)&dev);
         if (st != MIG_ENOMEM) break;
     }

@@ -655,6 +655,7 @@ mig_status batch_run_streams(mig_ctx *ctx, std::vector<BatchItem> &items) {
         }
         Carve c = cv;
         for (int i = 0; i < S; ++i) o_steps[i] = c.take(std::max<size_t>(stream_steps[i], 1));
+        if (lean < 2 && ctx_workspace_refused(ctx, c.off)) continue;
         st = ctx_workspace(ctx, c.off, (void **)&dev);
         if (st != MIG_ENOMEM) break;
     }

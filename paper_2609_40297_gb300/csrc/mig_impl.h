@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <cstring>
 #include <map>
@@ -37,6 +38,23 @@ struct DeviceAllocator {
     bool has_user = false;
     void *alloc(size_t bytes, cudaStream_t s);
     void free(void *p, size_t bytes, cudaStream_t s);
+};
+
+// What an allocator refused last: callers that can do with less do not ask for that much again for a while
+// (a failed attempt costs a freed workspace, two failed allocations and the captured graphs).
+struct Refused {
+    size_t least = SIZE_MAX;
+    int left = 0;  // requests still to be skipped
+    void note(size_t bytes) {
+        least = std::min(least, bytes);
+        left = 256;
+    }
+    bool skip(size_t bytes) {
+        if (bytes < least) return false;
+        if (left-- > 0) return true;
+        least = SIZE_MAX;
+        return false;
+    }
 };
 
 // Grow-only device buffer owned by a context.
@@ -132,6 +150,7 @@ struct mig_ctx {
     std::mutex count_mu;       // for readers that do not wait for the device (mig_server_submit)
     std::vector<std::unique_ptr<mig::Camera>> cameras;
     mig::DevBuf ws;          // per-call workspace (plan, counters, outputs, arena)
+    mig::Refused ws_refused;
     void *pinned = nullptr;  // pinned host staging
     size_t pinned_bytes = 0;
     int32_t *d_err = nullptr;  // device-side check word (device planning)
@@ -158,6 +177,8 @@ struct mig_map {
 namespace mig {
 // workspace / staging helpers (api.cu)
 mig_status ctx_workspace(mig_ctx *ctx, size_t bytes, void **out);
+// Should a caller that can do with less go on to that at once? (the workspace is smaller, and so much was refused)
+bool ctx_workspace_refused(mig_ctx *ctx, size_t bytes);
 mig_status ctx_pinned(mig_ctx *ctx, size_t bytes, void **out);
 mig_status ctx_camera(mig_ctx *ctx, const mig_sensor &s, const Camera **out);
 // The panoramic tables of a context camera, built and uploaded on first use (ctx->mu held).

@@ -89,6 +89,7 @@ struct Carve {
 struct mig_server {
     mig_ctx *ctx = nullptr;
     size_t budget = 0, in_use = 0;
+    Refused refused;  // by the allocator, for requests in flight (worker thread)
     // device bytes of superseded map grids that requests in flight still read (copy-on-write
     // snapshots), and the largest in_use + snapshot bytes seen; written by the worker only
     std::atomic<size_t> snap_bytes{0}, peak_bytes{0};
@@ -208,7 +209,9 @@ mig_status admit(mig_server *s, Request &r) {
         o_dpyr = c.take(dpyr_bytes(r));
         o_steps = c.take(r.steps.bytes);
         r.dev_bytes = c.off;
+        if (lean < 2 && s->refused.skip(r.dev_bytes)) continue;
         r.dev = (char *)ctx->alloc.alloc(r.dev_bytes, ctx->stream);
+        if (!r.dev) s->refused.note(r.dev_bytes);
     }
     if (!r.dev) return fail(MIG_ENOMEM, "server: request allocation failed");
     if (s->pinned_bytes < up) {

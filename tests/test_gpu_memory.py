@@ -79,3 +79,62 @@ def test_budget_holds_its_requests(image, mode):
     finally:
         m.close()
         ctx.close()
+
+
+@pytest.mark.parametrize("call", ["host", "device", "batch", "server"])
+def test_refused_memory_is_not_asked_for_by_every_call(monkeypatch, call):
+    """An allocator with a limit below the largest workspace: the first call finds the one that fits, the next
+    ones ask for no more than that (calls whose memory is kept: for nothing), with the same results."""
+    limit, asked = [1 << 62], []
+    real = mig._torch_allocator
+
+    def limited(device):
+        a = real(device)
+
+        def alloc(nbytes, stream, user):
+            asked.append(int(nbytes))
+            return None if nbytes > limit[0] else a.alloc(nbytes, stream, user)
+
+        b = mig.Allocator(mig.ALLOC_FN(alloc), a.free, None)
+        b.keep = (a, alloc)
+        return b
+
+    monkeypatch.setattr(mig, "_torch_allocator", limited)
+    p = _problem(143, Sensor(90, 60, 40, 30, 2.0, 8, 0.0))
+    c = mig.Context(0, stream=torch.cuda.Stream())
+    m = mig.Map(c, p.map.grid, p.map.voxel_size, p.map.origin)
+    srv = mig.Server(c, arena_budget_bytes=1 << 30, max_inflight=2) if call == "server" else None
+    par, pos = torch.from_numpy(p.tree.parent).cuda(), torch.from_numpy(p.tree.pos).cuda()
+    out = [torch.empty(p.tree.n, dtype=torch.int32, device="cuda") for _ in range(3)]
+
+    def run():
+        if call == "device":
+            mig.tree_eval_device(m, par, pos, p.sensor, 6, *out)
+            c.sync()
+            return [t.cpu().numpy() for t in out]
+        if call == "batch":
+            got = mig.tree_eval_batch(c, [(p.tree.parent, p.tree.pos, p.sensor)] * 2, [m, m])[1]
+        elif call == "server":
+            ticket, got = srv.submit(m, p.tree.parent, p.tree.pos, p.sensor)
+            assert srv.poll(ticket, timeout_us=30_000_000)
+        else:
+            got = mig.tree_eval(m, p.tree.parent, p.tree.pos, p.sensor)
+        return [got[k] for k in ("abs", "marg", "yaw")]
+
+    try:
+        mig.tree_eval(m, p.tree.parent[:1], p.tree.pos[:1], p.sensor)  # the camera's tables and a small workspace
+        asked.clear()
+        limit[0] = (1 << 20) if call == "batch" else (1 << 19)  # no room for any step counts beside the queue
+        first = run()
+        assert any(b > limit[0] for b in asked)
+        for i in range(20):
+            asked.clear()
+            assert all(np.array_equal(a, b) for a, b in zip(run(), first))
+            assert all(b <= limit[0] for b in asked), (i, asked)
+            assert call == "server" or not asked
+    finally:
+        limit[0] = 1 << 62
+        if srv is not None:
+            srv.close()
+        m.close()
+        c.close()
