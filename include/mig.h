@@ -369,7 +369,8 @@ mig_status mig_tree_eval_stats(mig_map *map, int n, const int32_t *parent, const
 const char *mig_last_error(void);
 
 /* Build of this library (no counterpart in the paper). MIG_BUILD_CHECKED: built with
- * MIG_DEBUG_BOUNDS=1, where every voxel load and depth-buffer write checks its index; an index
+ * MIG_DEBUG_BOUNDS=1, where every load of the map (codes, brick masks and distances), of step counts,
+ * their bounds, queued bricks and depth buffers, and every write of these checks its index; an index
  * outside its buffer skips the access and makes the host-array evaluation calls return MIG_ECUDA
  * ("bounds check") instead of touching memory outside the buffer. Slower; for testing. */
 #define MIG_BUILD_CHECKED 1

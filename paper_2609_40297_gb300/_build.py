@@ -16,7 +16,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libmig.so")
-# checked build (MIG_DEBUG_BOUNDS=1: every voxel load and depth-buffer write checks its index)
+# checked build (MIG_DEBUG_BOUNDS=1: loads of the map and loads and writes of what the counts keep check their index)
 BUILD_CHECKED = os.path.join(HERE, "_build_checked")
 LIB_CHECKED = os.path.join(HERE, "libmig_checked.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

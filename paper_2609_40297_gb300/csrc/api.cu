@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
 
 #include "interval.h"
@@ -746,6 +747,7 @@ static mig_status eval_host(mig_map *m, int n, const int32_t *parent, const floa
 #if defined(MIG_DEBUG_BOUNDS) && MIG_DEBUG_BOUNDS
     p.bounds_err = ctx->d_err + 16;  // checked build: out-of-buffer indices are recorded here
     MIG_CUDA_TRY(cudaMemsetAsync(p.bounds_err, 0, 4, ctx->stream));
+    if (const char *half = std::getenv("MIG_BOUNDS_HALF")) p.bounds_half = std::atoi(half);
 #endif
     if (steps.cap) set_steps(p, dev + o_steps, steps);
     p.dpyr = steps.cap ? (uint2 *)(dev + o_dpyr) : nullptr;

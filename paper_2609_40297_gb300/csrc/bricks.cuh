@@ -57,6 +57,20 @@ MIG_HD uint64_t ld_u64(const uint64_t *p) {
 #endif
 }
 
+// Mask and distance of brick i; a checked build's skipped access reads an occupied brick.
+MIG_HD uint64_t ld_mask(const uint64_t *m, size_t i MIG_CHECKED(, const LevelParams *p)) {
+#if MIG_DEBUG_BOUNDS && defined(__CUDA_ARCH__)
+    if (!at_ok(*p, m + i, m, brick_count(p->grid.nx, p->grid.ny, p->grid.nz), kBoundsBrick)) return ~0ull;
+#endif
+    return ld_u64(m + i);
+}
+MIG_HD int ld_dist(const uint8_t *d, size_t i MIG_CHECKED(, const LevelParams *p)) {
+#if MIG_DEBUG_BOUNDS && defined(__CUDA_ARCH__)
+    if (!at_ok(*p, d + i, d, brick_count(p->grid.nx, p->grid.ny, p->grid.nz), kBoundsBrick)) return 0;
+#endif
+    return ld_u8(d + i);
+}
+
 // ------------------------------------------------------------------------------------- cast
 // Crossings of an axis (face distances n0 + k 2^16, speed ad) that start before the time ts (Q16
 // voxel units along the ray), exactly.
@@ -104,7 +118,7 @@ struct ExactWalk {
     float t;
 };
 MIG_HD ExactWalk exact_walk(const uint64_t *om, int gnx, int gny, int gnz, int Px, int Py, int Pz, int dx, int dy, int dz, int64_t Tq,
-                     uint32_t ts, float tf) {
+                     uint32_t ts, float tf MIG_CHECKED(, const LevelParams *lp)) {
     int v0x, v0y, v0z, sx, sy, sz;
     uint32_t n0x, n0y, n0z, ax, ay, az;
     ray_axis(Px, dx, v0x, sx, n0x, ax);
@@ -124,7 +138,7 @@ MIG_HD ExactWalk exact_walk(const uint64_t *om, int gnx, int gny, int gnz, int P
     w.t = 0.0f;
     w.more = true;
     uint32_t nx = n0x + ((uint32_t)cx << 16), ny = n0y + ((uint32_t)cy << 16), nz = n0z + ((uint32_t)cz << 16);
-    uint64_t m = ld_u64(om + ((size_t)((w.vz >> 2) * nby + (w.vy >> 2)) * nbx + (w.vx >> 2)));
+    uint64_t m = ld_mask(om, (size_t)((w.vz >> 2) * nby + (w.vy >> 2)) * nbx + (w.vx >> 2) MIG_CHECKED(, lp));
     bool walk = true;
     while (walk) {
         ++w.steps;
@@ -146,7 +160,7 @@ MIG_HD ExactWalk exact_walk(const uint64_t *om, int gnx, int gny, int gnz, int P
             if (((uint64_t)w.en << 30) >= (uint64_t)Tq * w.ea || (unsigned)v >= (unsigned)(a == 0 ? gnx : (a == 1 ? gny : gnz))) {
                 walk = w.more = false;  // the crossing starts at or beyond the range, or leaves the grid
             } else if ((v & 3) == (s > 0 ? 0 : 3)) {  // entered another brick
-                m = ld_u64(om + ((size_t)((w.vz >> 2) * nby + (w.vy >> 2)) * nbx + (w.vx >> 2)));
+                m = ld_mask(om, (size_t)((w.vz >> 2) * nby + (w.vy >> 2)) * nbx + (w.vx >> 2) MIG_CHECKED(, lp));
                 // en / ea in voxels (Q16 over Q30)
                 w.t = (float)w.en * fast_divf(16384.0f, (float)w.ea);
                 walk = w.t < tf;
@@ -190,7 +204,7 @@ MIG_HD bool mask_box(uint64_t m, int lx, int hx, int ly, int hy, int lz, int hz)
 template <bool DEPTH, bool STATS>
 MIG_HD uint32_t cast_bricks(const uint64_t *om, const uint8_t *oct, int gnx, int gny, int gnz, int Px, int Py, int Pz,
                             int dx, int dy, int dz, int64_t Tq, float t0, uint32_t &ne, uint32_t &ade, uint32_t &fine,
-                            uint32_t &coarse) {
+                            uint32_t &coarse MIG_CHECKED(, const LevelParams *lp)) {
     const float q30 = 9.31322574615478515625e-10f, q16 = 1.52587890625e-5f, q18 = 3.814697265625e-6f;
     const int nbx = (gnx + 3) >> 2, nby = (gny + 3) >> 2, nbz = (gnz + 3) >> 2;
     const int b0x = Px >> 18, b0y = Py >> 18, b0z = Pz >> 18;
@@ -231,7 +245,7 @@ MIG_HD uint32_t cast_bricks(const uint64_t *om, const uint8_t *oct, int gnx, int
     float r = 1.0f;
     if (sure) {
         bi = oct_at();
-        d = ld_u8(oct + bi);
+        d = ld_dist(oct, bi MIG_CHECKED(, lp));
     }
     int rounds = 0;  // every round passes a brick face; beyond kCastRounds the exact walk runs to the end
     for (bool more = true; more;) {
@@ -250,7 +264,7 @@ MIG_HD uint32_t cast_bricks(const uint64_t *om, const uint8_t *oct, int gnx, int
                 const float e = fmaf(t, kTimeErr, 2.0f * eps);
                 auto at = [&](float v) { return float_bits(fminf(fmaxf(v, 0.0f), 3.0f) + kMagic) & 3; };
                 const float cx = fmaf(-4.0f, bx, 1.5f), cy = fmaf(-4.0f, by, 1.5f), cz = fmaf(-4.0f, bz, 1.5f);
-                dda = mask_box(ld_u64(om + bi), at(fmaf(4.0f, fminf(px, qx), cx - e)), at(fmaf(4.0f, fmaxf(px, qx), cx + e)),
+                dda = mask_box(ld_mask(om, bi MIG_CHECKED(, lp)), at(fmaf(4.0f, fminf(px, qx), cx - e)), at(fmaf(4.0f, fmaxf(px, qx), cx + e)),
                                at(fmaf(4.0f, fminf(py, qy), cy - e)), at(fmaf(4.0f, fmaxf(py, qy), cy + e)),
                                at(fmaf(4.0f, fminf(pz, qz), cz - e)), at(fmaf(4.0f, fmaxf(pz, qz), cz + e)));
             }
@@ -267,7 +281,7 @@ MIG_HD uint32_t cast_bricks(const uint64_t *om, const uint8_t *oct, int gnx, int
                 if constexpr (DEPTH) last = ox ? 0 : (oy ? 1 : 2);
                 if (sure) {
                     bi = oct_at();
-                    d = ld_u8(oct + bi);
+                    d = ld_dist(oct, bi MIG_CHECKED(, lp));
                 }
             }
         }
@@ -278,7 +292,7 @@ MIG_HD uint32_t cast_bricks(const uint64_t *om, const uint8_t *oct, int gnx, int
             // brick's voxels; the entry face itself is exact), next crossing times, and a packed state: bits
             // 0-5 the mask's bit (plus 64), above them a guard per axis whose third bit is set while the
             // coordinate is in 0..3
-            const uint64_t m = ld_u64(om + bi);
+            const uint64_t m = ld_mask(om, bi MIG_CHECKED(, lp));
             const float e = fmaf(t, kTimeErr, eps);
             const float lx = fminf(fmaxf(4.0f * (px - bx) + 1.5f, -0.5f), 3.499f), ly = fminf(fmaxf(4.0f * (py - by) + 1.5f, -0.5f), 3.499f),
                         lz = fminf(fmaxf(4.0f * (pz - bz) + 1.5f, -0.5f), 3.499f);  // minus 1/2
@@ -344,7 +358,7 @@ MIG_HD uint32_t cast_bricks(const uint64_t *om, const uint8_t *oct, int gnx, int
                 r = 1.0f;
                 if (sure) {
                     bi = oct_at();
-                    d = ld_u8(oct + bi);
+                    d = ld_dist(oct, bi MIG_CHECKED(, lp));
                 }
             } else if (mn > T + eps) {
                 more = false;  // the next crossing is beyond the range
@@ -356,7 +370,7 @@ MIG_HD uint32_t cast_bricks(const uint64_t *om, const uint8_t *oct, int gnx, int
             const float slack = fmaf(t, kTimeErr, eps);
             const ExactWalk w = exact_walk(om, gnx, gny, gnz, Px, Py, Pz, dx, dy, dz, Tq,
                                            (uint32_t)(int)(fmaxf(0.0f, fminf(t, t_end) - slack) * 65536.0f),
-                                           ++rounds < kCastRounds ? t + slack : 1e30f);
+                                           ++rounds < kCastRounds ? t + slack : 1e30f MIG_CHECKED(, lp));
             if constexpr (STATS) fine += w.steps;
             if constexpr (DEPTH) {
                 ne = w.en;
@@ -377,7 +391,7 @@ MIG_HD uint32_t cast_bricks(const uint64_t *om, const uint8_t *oct, int gnx, int
                 sure = t < t_sure;
                 if (sure) {
                     bi = oct_at();
-                    d = ld_u8(oct + bi);
+                    d = ld_dist(oct, bi MIG_CHECKED(, lp));
                 }
             }
         }
@@ -400,7 +414,7 @@ MIG_HD uint32_t cast_bricks(const uint64_t *om, const uint8_t *oct, int gnx, int
 // axes), s_end: the largest camera depth of a ray's range. The bounds are widened by 4e-6 of w (the
 // rounding of w and of the positions) and the result is kCastEps short.
 MIG_HD float beam_free(const uint8_t *dist, int gnx, int gny, int gnz, int Px, int Py, int Pz, const float wlo[3],
-                       const float whi[3], float s_end) {
+                       const float whi[3], float s_end MIG_CHECKED(, const LevelParams *lp)) {
     const int nb[3] = {(gnx + 3) >> 2, (gny + 3) >> 2, (gnz + 3) >> 2}, P[3] = {Px, Py, Pz};
     const float q18 = 3.814697265625e-6f;
     float p0[3], lo[3], hi[3];
@@ -414,7 +428,7 @@ MIG_HD float beam_free(const uint8_t *dist, int gnx, int gny, int gnz, int Px, i
     }
     float s = 0.0f;
     for (bool go = true; go;) {
-        const int d = ld_u8(dist + ((size_t)(b[2] * nb[1] + b[1]) * nb[0] + b[0]));
+        const int d = ld_dist(dist, (size_t)(b[2] * nb[1] + b[1]) * nb[0] + b[0] MIG_CHECKED(, lp));
         float s1 = 1e30f;
         bool in = d > 0;
         for (int a = 0; a < 3; ++a) {

@@ -39,7 +39,8 @@ constexpr int kOcc = 2;
 
 // Checked builds (MIG_DEBUG_BOUNDS=1): an index outside its buffer sets `bit` in *err (when err is
 // not NULL) and the access is skipped; other builds compile the check away.
-constexpr int kBoundsVoxel = 1, kBoundsArena = 2, kBoundsDepth = 4;
+constexpr int kBoundsVoxel = 1, kBoundsArena = 2, kBoundsDepth = 4;  // codes; depth buffers written, read
+constexpr int kBoundsBrick = 8, kBoundsSteps = 16, kBoundsTiles = 32, kBoundsQueue = 64;  // masks and distances; step counts; bounds
 __device__ __forceinline__ bool in_bounds(int32_t *err, bool ok, int bit) {
 #if MIG_DEBUG_BOUNDS
     if (!ok && err) atomicOr(err, bit);
@@ -61,6 +62,22 @@ __device__ __forceinline__ T ld_written(const T *p) {
     __builtin_assume(__isGlobal(p));
     return *p;
 }
+
+// Is `at` one of the n elements from base on? In other builds always.
+template <class T>
+__device__ __forceinline__ bool at_ok(const LevelParams &p, const T *at, const T *base, size_t n, int bit) {
+#if MIG_DEBUG_BOUNDS
+    return in_bounds(p.bounds_err, (size_t)(at - base) < (p.bounds_half & bit ? n / 2 : n), bit);
+#else
+    return true;
+#endif
+}
+// Arguments that only checked builds have.
+#if MIG_DEBUG_BOUNDS
+#define MIG_CHECKED(...) __VA_ARGS__
+#else
+#define MIG_CHECKED(...)
+#endif
 
 __device__ __forceinline__ uint32_t grid_cells(int nx, int ny, int nz) {
     return (uint32_t)nx * (uint32_t)ny * (uint32_t)nz;

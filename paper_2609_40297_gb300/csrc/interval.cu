@@ -93,7 +93,7 @@ __device__ bool iv_observed(const LevelParams &p, const IvAnc *anc, int na, cons
         const int32_t *m = p.yawtab + A.yaw * 12 + 2;
         if (!seg_setup(m, A.U0, A.V0, A.Z0, make_int3(E[0] - A.px, E[1] - A.py, E[2] - A.pz), zf, p.W, p.H, lam, g)) continue;
         float s;
-        if (seg_param(g, lam, s) && seg_lookup(g, p.W, p.H, A.D, s)) return true;
+        if (seg_param(g, lam, s) && seg_lookup(g, p.W, p.H, A.D, s MIG_CHECKED(, &p))) return true;
     }
     return false;
 }

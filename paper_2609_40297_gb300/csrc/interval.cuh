@@ -148,7 +148,7 @@ __device__ __forceinline__ int count_crossings(float a0, float r, float d, int b
 // it is in column i0 + si * (column crossings <= s) and row j0 + sj * (row crossings <= s), in the
 // portion from the latest crossing at or before s (s0 if none) to the next one (capped at s1).
 // True if that portion is observed; false if not, or if the walk leaves the buffer before s.
-__device__ __forceinline__ bool seg_lookup(const Seg &g, int W, int H, const uint32_t *D, float s) {
+__device__ __forceinline__ bool seg_lookup(const Seg &g, int W, int H, const uint32_t *D, float s MIG_CHECKED(, const LevelParams *p)) {
     const float du = fsub(g.ub, g.ua), dv = fsub(g.vb, g.va);
     const float ru = g.ru, rv = g.rv;
     const float fi = floorf(fadd(g.ua, fmul(g.s0, du))), fj = floorf(fadd(g.va, fmul(g.s0, dv)));
@@ -173,6 +173,10 @@ __device__ __forceinline__ bool seg_lookup(const Seg &g, int W, int H, const uin
     if (g.s1 < s_out) s_out = g.s1;
     const float sm = fmul(fadd(s_in, s_out), 0.5f);
     const float wm = fadd(g.wa, fmul(sm, fsub(g.wb, g.wa)));
+#if MIG_DEBUG_BOUNDS
+    const uint32_t *at = D + (size_t)j * W + i;
+    if (p->arena_slots && !at_ok(*p, at, (const uint32_t *)p->arena, (size_t)p->arena_slots * W * H, kBoundsDepth)) return false;
+#endif
     const float Dv = fmul(__uint2float_rn(ld_written(D + (size_t)j * W + i)), 1.52587890625e-05f);
     return fmul(wm, Dv) >= 1.0f;  // z <= D in inverse depth
 }

@@ -60,6 +60,7 @@ struct LevelParams {
     // not recorded) and the access is skipped; arena_slots = depth buffers in the arena (0: unchecked)
     int32_t *bounds_err;
     int arena_slots;
+    int bounds_half;  // checked builds: kinds of buffers that count as half as large (a test of the checks)
     // owned-voxel count (voxcount.cu): per-ray DDA step counts of a chunk of (node, yaw) pairs
     // [q0, q1) of the level, steps_cap pairs of W * H each; NULL = the ray-by-ray count kernel
     uint16_t *steps;

@@ -227,7 +227,7 @@ __device__ __forceinline__ bool iv_observed(const LevelParams &p, const NodeAnc 
         Seg g;
         float s;
         obs = seg_setup(p.yawtab + A.yaw * 12 + 2, A.U0, A.V0, A.Z0, make_int3(Ex - A.px, Ey - A.py, Ez - A.pz), zf, p.W, p.H, lam, g) &&
-              seg_param(g, lam, s) && seg_lookup(g, p.W, p.H, A.D, s);
+              seg_param(g, lam, s) && seg_lookup(g, p.W, p.H, A.D, s MIG_CHECKED(, &p));
     }
     return obs;
 }
@@ -316,7 +316,7 @@ __device__ __forceinline__ void count_brick(const LevelParams &p, const VoxConst
                 int m[2] = {0, 0};
 #pragma unroll
                 for (int h = 0; h < 2; ++h)
-                    if (c[h]) m[h] = ld_written(stp + pix[h]);
+                    if (c[h] && steps_ok(p, stp + pix[h])) m[h] = ld_written(stp + pix[h]);
                 c[0] = man[0] < m[0];
                 c[1] = man[1] < m[1];
             }
@@ -445,7 +445,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, 3) node_kernel(const LevelParams
             // ---- lane = brick
             const int bx = X + (lane & 3), by = Y + ((lane >> 2) & 3), bz = Z + (lane >> 4);
             uint64_t U = 0;
-            if (bx < bd.nbx && by < bd.nby && bz < bd.nbz) U = ld_u64(umask + ((size_t)(bz * bd.nby + by) * bd.nbx + bx));
+            if (bx < bd.nbx && by < bd.nby && bz < bd.nbz) U = ld_mask(umask, (size_t)(bz * bd.nby + by) * bd.nbx + bx MIG_CHECKED(, &p));
             const float cx = q16f(((4 * bx + 2) << 16) - nd.x), cy = q16f(((4 * by + 2) << 16) - nd.y),
                         cz = q16f(((4 * bz + 2) << 16) - nd.z);
             float far;
@@ -478,7 +478,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, 3) node_kernel(const LevelParams
                         const BoxView b = box_view<false>(s_y[k], gx, gy, gz, 7.5f, 7.5f, 3.5f, W, H);
                         may = b.in >= 0;
                         if (may && box_lookup(b)) {
-                            const uint32_t hm = hz_box(hz + (size_t)k * pyr.n, pyr, top, b);
+                            const uint32_t hm = hz_box(p, hz + (size_t)k * pyr.n, pyr, top, b);
                             may = mac_man0 < (int)((hm >> 16) ^ 0xFFFFu);  // else every ray stops before the block
                         }
                     }
@@ -498,7 +498,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, 3) node_kernel(const LevelParams
                         }
                         if (some && b.zlo >= 0.5f) {
                             if (box_lookup(b)) {
-                                const uint32_t hm = hz_box(hz + (size_t)(kb + j) * pyr.n, pyr, top, b);
+                                const uint32_t hm = hz_box(p, hz + (size_t)(kb + j) * pyr.n, pyr, top, b);
                                 some = man0 < (int)((hm >> 16) ^ 0xFFFFu);
                                 reach = man1 < (int)(hm & 0xFFFFu);
                             }
@@ -548,7 +548,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, 3) node_kernel(const LevelParams
                     at = __shfl_sync(0xffffffffu, at, 0) + __popc(recs & ((1u << lane) - 1u));
                     BrickRec r{U, O, left, all, part, rch, vis, (uint32_t)bx | ((uint32_t)by << 10) | ((uint32_t)bz << 20),
                                (uint32_t)ln | ((uint32_t)(kb >> 6) << kRecNodeBits)};
-                    if (rec && at < p.queue_cap) p.queue[at] = r;
+                    if (rec && at < p.queue_cap && queue_ok(p, at)) p.queue[at] = r;
 #pragma unroll 1
                     for (unsigned full = __ballot_sync(0xffffffffu, rec && at >= p.queue_cap); full; full &= full - 1) {
                         const int s = __ffs(full) - 1;
@@ -598,6 +598,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, 4) brick_kernel(const LevelParam
         const int end = min(i + slice, total);
 #pragma unroll 1
         for (; i < end; ++i) {
+            if (!queue_ok(p, i)) continue;
             const BrickRec r = p.queue[i];
             if (r.node != cur) {
                 if (cur != 0xFFFFFFFFu) flush_counts<STATS>(p, n, (int)(cur >> kRecNodeBits) * 64, lane, c_abs, c_mrg, st);

@@ -78,7 +78,7 @@ struct CameraRays {
         const float b0 = ((float)j0 + 0.5f - 0.5f * (float)H) * p.ify, b1 = ((float)j1 + 0.5f - 0.5f * (float)H) * p.ify;
         const float am = a0 * a1 <= 0.0f ? 0.0f : fminf(fabsf(a0), fabsf(a1)), bm = b0 * b1 <= 0.0f ? 0.0f : fminf(fabsf(b0), fabsf(b1));
         const float s_end = q16f((int)p.Tq) * rsqrtf(1.0f + am * am + bm * bm) * 1.00001f;
-        return beam_free(dist, p.grid.nx, p.grid.ny, p.grid.nz, nd.x, nd.y, nd.z, lo, hi, s_end);
+        return beam_free(dist, p.grid.nx, p.grid.ny, p.grid.nz, nd.x, nd.y, nd.z, lo, hi, s_end MIG_CHECKED(, &p));
     }
 };
 // The time before which a ray of camera depth cz (Q30, per unit length) of a beam free to depth s
@@ -90,6 +90,22 @@ __device__ __forceinline__ float beam_time(float s, int cz) {
 struct CastCnt {  // statistics
     uint32_t rays = 0, fine = 0, jump = 0;
 };
+
+// The rays of an image that a node's count casts, and the images' (tiles') number in the region.
+__device__ __forceinline__ int image_width(const LevelParams &p) { return p.mode == MIG_MODE_PANORAMIC ? p.pano_A : p.W; }
+__device__ __forceinline__ bool steps_ok(const LevelParams &p, const uint16_t *at) {
+    return at_ok(p, at, (const uint16_t *)p.steps, (size_t)p.steps_cap * image_width(p) * p.H, kBoundsSteps);
+}
+__device__ __forceinline__ bool hz_ok(const LevelParams &p, const uint32_t *at) {
+    return at_ok(p, at, (const uint32_t *)p.hz, (size_t)p.steps_cap * pyramid(image_width(p), p.H).n, kBoundsTiles);
+}
+__device__ __forceinline__ bool dpyr_ok(const LevelParams &p, const uint2 *at) {
+    return p.arena_slots == 0 || at_ok(p, at, (const uint2 *)p.dpyr, (size_t)p.arena_slots * pyramid(p.W, p.H).n, kBoundsTiles);
+}
+__device__ __forceinline__ bool depth_ok(const LevelParams &p, const uint32_t *at) {
+    return p.arena_slots == 0 || at_ok(p, at, (const uint32_t *)p.arena, (size_t)p.arena_slots * p.W * p.H, kBoundsDepth);
+}
+__device__ __forceinline__ bool queue_ok(const LevelParams &p, int i) { return at_ok(p, p.queue + i, (const BrickRec *)p.queue, p.queue_cap, kBoundsQueue); }
 
 // What a pass keeps per ray and per tile: the cast the step index (16 bits, bounds packed as min |
 // ~max << 16), the render the depth.
@@ -103,11 +119,13 @@ struct CastOut {
     __device__ __forceinline__ bool stored() const { return false; }
     __device__ __forceinline__ uint32_t load(const LevelParams &, size_t) const { return 0u; }
     __device__ __forceinline__ uint32_t put(const LevelParams &p, size_t i, int dzc, uint32_t m, uint32_t ne, uint32_t ade) const {
-        out[i] = (uint16_t)m;
-        if (DEPTH && depth) depth[i] = hit_depth(m != kNoHit, ne, ade, dzc, p.Tq);
+        if (steps_ok(p, out + i)) out[i] = (uint16_t)m;
+        if (DEPTH && depth && at_ok(p, depth + i, p.depths, (size_t)p.steps_cap * p.W * p.H, kBoundsSteps)) depth[i] = hit_depth(m != kNoHit, ne, ade, dzc, p.Tq);
         return m;
     }
-    __device__ __forceinline__ void tile(size_t i, uint32_t lo, uint32_t hi) const { hz[i] = lo | ((hi ^ 0xFFFFu) << 16); }
+    __device__ __forceinline__ void tile(const LevelParams &p, size_t i, uint32_t lo, uint32_t hi) const {
+        if (hz_ok(p, hz + i)) hz[i] = lo | ((hi ^ 0xFFFFu) << 16);
+    }
 };
 struct RenderOut {
     uint2 *pyr;  // NULL: not kept
@@ -117,7 +135,7 @@ struct RenderOut {
     static constexpr uint32_t kMin = 0xFFFFFFFFu;
     __device__ __forceinline__ bool stored() const { return src != nullptr; }
     __device__ __forceinline__ uint32_t load(const LevelParams &p, size_t i) const {
-        const uint32_t D = ld_written(src + i);
+        const uint32_t D = at_ok(p, src + i, (const uint32_t *)p.depths, (size_t)p.steps_cap * p.W * p.H, kBoundsSteps) ? ld_written(src + i) : 0u;
         arena_store(p.arena, p.arena_slots, slot, i, (size_t)p.W * p.H, D, p.bounds_err);
         return D;
     }
@@ -126,8 +144,8 @@ struct RenderOut {
         arena_store(p.arena, p.arena_slots, slot, i, (size_t)p.W * p.H, D, p.bounds_err);
         return D;
     }
-    __device__ __forceinline__ void tile(size_t i, uint32_t lo, uint32_t hi) const {
-        if (pyr) pyr[i] = make_uint2(lo, hi);
+    __device__ __forceinline__ void tile(const LevelParams &p, size_t i, uint32_t lo, uint32_t hi) const {
+        if (pyr && dpyr_ok(p, pyr + i)) pyr[i] = make_uint2(lo, hi);
     }
 };
 
@@ -137,10 +155,10 @@ struct RayHit {
 };
 template <bool STATS, bool DEPTH>
 __device__ __noinline__ RayHit cast_ray(const uint64_t *om, const uint8_t *oct, int gnx, int gny, int gnz, int Px, int Py, int Pz,
-                                       int dx, int dy, int dz, int Tq, float t0, CastCnt *st) {
+                                       int dx, int dy, int dz, int Tq, float t0, CastCnt *st MIG_CHECKED(, const LevelParams *lp)) {
     RayHit h{0, 0, 1};
     uint32_t fine = 0, jump = 0;
-    h.m = cast_bricks<DEPTH, STATS>(om, oct, gnx, gny, gnz, Px, Py, Pz, dx, dy, dz, Tq, t0, h.ne, h.ade, fine, jump);
+    h.m = cast_bricks<DEPTH, STATS>(om, oct, gnx, gny, gnz, Px, Py, Pz, dx, dy, dz, Tq, t0, h.ne, h.ade, fine, jump MIG_CHECKED(, lp));
     if constexpr (STATS) {
         st->fine += fine;
         st->jump += jump;
@@ -170,7 +188,7 @@ __device__ __forceinline__ void cast_part(const LevelParams &p, const uint64_t *
                 r.dir(b, dx, dy, dz);
                 const uint8_t *oct = p.grid.g + oct_offset(p.grid.nx, p.grid.ny, p.grid.nz, octant_of(dx, dy, dz));
                 hit = cast_ray<STATS, OUT::kDepth>(om, oct, p.grid.nx, p.grid.ny, p.grid.nz, r.nd.x, r.nd.y, r.nd.z, dx, dy, dz, (int)p.Tq,
-                                                   beam_time(beam, b.w), &st);
+                                                   beam_time(beam, b.w), &st MIG_CHECKED(, &p));
             }
         }
         v = o.put(p, at, dzc, hit.m, hit.ne, hit.ade);
@@ -200,14 +218,14 @@ __device__ __forceinline__ uint2 cast_quad(const LevelParams &p, const uint64_t 
         if (t & 1) {
             lo = __reduce_min_sync(0xffffffffu, lo);
             hi = __reduce_max_sync(0xffffffffu, hi);
-            if (lane == 0 && at.x < r.W && at.y - 4 < r.H) o.tile((size_t)(at.y >> 3) * y.w0 + (at.x >> 3), lo, hi);
+            if (lane == 0 && at.x < r.W && at.y - 4 < r.H) o.tile(p, (size_t)(at.y >> 3) * y.w0 + (at.x >> 3), lo, hi);
             lo16 = min(lo16, lo);
             hi16 = max(hi16, hi);
             lo = OUT::kMin;
             hi = 0u;
         }
     }
-    if (lane == 0 && x0 < r.W && y0 < r.H) o.tile(y.o1 + (size_t)(y0 >> 4) * y.w1 + (x0 >> 4), lo16, hi16);
+    if (lane == 0 && x0 < r.W && y0 < r.H) o.tile(p, y.o1 + (size_t)(y0 >> 4) * y.w1 + (x0 >> 4), lo16, hi16);
     return make_uint2(lo16, hi16);
 }
 
@@ -223,7 +241,7 @@ __device__ __forceinline__ void cast_large(const LevelParams &p, const uint64_t 
         const uint2 v = cast_quad<STATS>(p, om, dist, y, r, x0 + (q & 1) * 16, y0 + (q >> 1) * 16, s, 8 * q, o, lane, st);
         b = make_uint2(min(b.x, v.x), max(b.y, v.y));
     }
-    if (lane == 0) o.tile(y.o2 + (size_t)(y0 >> 5) * y.w2 + (x0 >> 5), b.x, b.y);
+    if (lane == 0) o.tile(p, y.o2 + (size_t)(y0 >> 5) * y.w2 + (x0 >> 5), b.x, b.y);
 }
 
 // One 32x32 tile at pixel (x0, y0) by a CTA of 8 warps: warp w casts half of quadrant w >> 1.
@@ -246,7 +264,7 @@ __device__ __forceinline__ void cast_mid(const LevelParams &p, const uint64_t *o
         if (t & 1) {
             lo = __reduce_min_sync(0xffffffffu, lo);
             hi = __reduce_max_sync(0xffffffffu, hi);
-            if (lane == 0 && at.x < r.W && at.y - 4 < r.H) o.tile((size_t)(at.y >> 3) * y.w0 + (at.x >> 3), lo, hi);
+            if (lane == 0 && at.x < r.W && at.y - 4 < r.H) o.tile(p, (size_t)(at.y >> 3) * y.w0 + (at.x >> 3), lo, hi);
             lo2 = min(lo2, lo);
             hi2 = max(hi2, hi);
             lo = OUT::kMin;
@@ -260,10 +278,10 @@ __device__ __forceinline__ void cast_mid(const LevelParams &p, const uint64_t *o
         lo = min(a.x, b.x);
         hi = max(a.y, b.y);
         const int i0 = x0 + (threadIdx.x & 1) * 16, j0 = y0 + (threadIdx.x >> 1) * 16;
-        if (i0 < r.W && j0 < r.H) o.tile(y.o1 + (size_t)(j0 >> 4) * y.w1 + (i0 >> 4), lo, hi);
+        if (i0 < r.W && j0 < r.H) o.tile(p, y.o1 + (size_t)(j0 >> 4) * y.w1 + (i0 >> 4), lo, hi);
         lo = __reduce_min_sync(0xfu, lo);
         hi = __reduce_max_sync(0xfu, hi);
-        if (threadIdx.x == 0) o.tile(y.o2 + (size_t)(y0 >> 5) * y.w2 + (x0 >> 5), lo, hi);
+        if (threadIdx.x == 0) o.tile(p, y.o2 + (size_t)(y0 >> 5) * y.w2 + (x0 >> 5), lo, hi);
     }
     __syncthreads();
 }
@@ -286,10 +304,10 @@ __device__ __forceinline__ void cast_small(const LevelParams &p, const uint64_t 
         lo = min(a.x, b.x);
         hi = max(a.y, b.y);
         const int i0 = x0 + (threadIdx.x & 1) * 8, j0 = y0 + (threadIdx.x >> 1) * 8;
-        if (i0 < r.W && j0 < r.H) o.tile((size_t)(j0 >> 3) * y.w0 + (i0 >> 3), lo, hi);
+        if (i0 < r.W && j0 < r.H) o.tile(p, (size_t)(j0 >> 3) * y.w0 + (i0 >> 3), lo, hi);
         lo = __reduce_min_sync(0xfu, lo);
         hi = __reduce_max_sync(0xfu, hi);
-        if (threadIdx.x == 0) o.tile(y.o1 + (size_t)(y0 >> 4) * y.w1 + (x0 >> 4), lo, hi);
+        if (threadIdx.x == 0) o.tile(p, y.o1 + (size_t)(y0 >> 4) * y.w1 + (x0 >> 4), lo, hi);
     }
     __syncthreads();
 }
@@ -337,7 +355,7 @@ __device__ __forceinline__ uint64_t or64(uint64_t v) {  // over the warp
 }
 
 // Bounds of the step counts under a pixel box: min in the low half, ~max in the high half.
-__device__ __forceinline__ uint32_t hz_box(const uint32_t *hz, const Pyramid &y, int top, const BoxView &b) {
+__device__ __forceinline__ uint32_t hz_box(const LevelParams &p, const uint32_t *hz, const Pyramid &y, int top, const BoxView &b) {
     int sh, off, w;
     pyramid_level(y, max(b.u1 - b.u0, b.v1 - b.v0), top, sh, off, w);
     const uint32_t *t = hz + off;
@@ -345,11 +363,11 @@ __device__ __forceinline__ uint32_t hz_box(const uint32_t *hz, const Pyramid &y,
 #pragma unroll 1
     for (int ty = b.v0 >> sh; ty <= (b.v1 >> sh); ++ty)
 #pragma unroll 1
-        for (int tx = b.u0 >> sh; tx <= (b.u1 >> sh); ++tx) r = __vminu2(r, ld_written(t + ty * w + tx));
+        for (int tx = b.u0 >> sh; tx <= (b.u1 >> sh); ++tx) r = __vminu2(r, hz_ok(p, t + ty * w + tx) ? ld_written(t + ty * w + tx) : 0u);
     return r;
 }
 // Bounds of the stored depths under a pixel box (the 32x32 level is not kept by every render).
-__device__ __forceinline__ uint2 depth_box(const uint2 *pyr, const Pyramid &y, const BoxView &b) {
+__device__ __forceinline__ uint2 depth_box(const LevelParams &p, const uint2 *pyr, const Pyramid &y, const BoxView &b) {
     int sh, off, w;
     pyramid_level(y, max(b.u1 - b.u0, b.v1 - b.v0), 4, sh, off, w);
     const uint2 *t = pyr + off;
@@ -358,7 +376,7 @@ __device__ __forceinline__ uint2 depth_box(const uint2 *pyr, const Pyramid &y, c
     for (int ty = b.v0 >> sh; ty <= (b.v1 >> sh); ++ty)
 #pragma unroll 1
         for (int tx = b.u0 >> sh; tx <= (b.u1 >> sh); ++tx) {
-            const uint2 v = ld_written(t + ty * w + tx);
+            const uint2 v = dpyr_ok(p, t + ty * w + tx) ? ld_written(t + ty * w + tx) : make_uint2(0u, 0xFFFFFFFFu);
             r.x = min(r.x, v.x);
             r.y = max(r.y, v.y);
         }
@@ -402,9 +420,13 @@ __device__ __noinline__ int pixel_exact(const int32_t *row, int rx, int ry, int 
     return pixel_index(row, rx, ry, rz, W, H, Z);
 }
 // The exact ancestor test (Sec. IV-B): inside the image and z <= D.
-__device__ __noinline__ bool observed_exact(const int32_t *row, int rx, int ry, int rz, int W, int H, const uint32_t *D) {
+__device__ __noinline__ bool observed_exact(const int32_t *row, int rx, int ry, int rz, int W, int H, const uint32_t *D
+                                              MIG_CHECKED(, const LevelParams *p)) {
     int64_t Z;
     const int pix = pixel_index(row, rx, ry, rz, W, H, Z);
+#if MIG_DEBUG_BOUNDS
+    if (pix >= 0 && !depth_ok(*p, D + pix)) return false;
+#endif
     return pix >= 0 && Z < (((int64_t)ld_written(D + pix) + 1) << 16);
 }
 // The exact visit test of a voxel by its owner ray.
@@ -495,7 +517,7 @@ __device__ __forceinline__ void block_ancestors(const LevelParams &p, const YawR
                 const BoxView b = box_view<false>(s_y[A.yaw], ox, oy, oz, 7.5f, 7.5f, 3.5f, W, H);
                 rel = b.in >= 0;
                 if (rel && box_lookup(b)) {
-                    const uint2 D = depth_box(A.pyr, pyr, b);
+                    const uint2 D = depth_box(p, A.pyr, pyr, b);
                     rel = b.zlo * (65536.0f * (1.0f - 1e-6f)) <= (float)D.y + 1.5f;
                 }
             }
@@ -514,7 +536,7 @@ __device__ __forceinline__ void block_ancestors(const LevelParams &p, const YawR
                     const BoxView b = box_view<true>(s_y[A.yaw], ox, oy, oz, 1.5f, 1.5f, 1.5f, W, H);
                     vox = b.in >= 0;
                     if (vox && box_lookup(b)) {
-                        const uint2 D = depth_box(A.pyr, pyr, b);
+                        const uint2 D = depth_box(p, A.pyr, pyr, b);
                         if (b.zlo * (65536.0f * (1.0f - 1e-6f)) > (float)D.y + 1.5f) {
                             vox = false;
                         } else if (b.in > 0 && b.zhi * (65536.0f * (1.0f + 1e-6f)) < (float)D.x) {
@@ -562,7 +584,7 @@ __device__ __forceinline__ uint64_t voxel_ancestors(const LevelParams &p, const 
         uint32_t D[2] = {0u, 0u};
 #pragma unroll
         for (int h = 0; h < 2; ++h)
-            if (in[h] > 0) D[h] = ld_written(A.D + pix[h]);
+            if (in[h] > 0 && depth_ok(p, A.D + pix[h])) D[h] = ld_written(A.D + pix[h]);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             if constexpr (STATS) st.reads += in[h] > 0;
@@ -571,7 +593,7 @@ __device__ __forceinline__ uint64_t voxel_ancestors(const LevelParams &p, const 
             obs[h] = in[h] > 0 && Zf[h] + e_z < lim * (1.0f - 2.4e-7f);
             if (in[h] < 0 || (in[h] > 0 && !obs[h] && Zf[h] - e_z < lim * (1.0f + 2.4e-7f)))
                 obs[h] = observed_exact(p.yawtab + A.yaw * 12, (x << 16) + 32768 - A.px, (y << 16) + 32768 - A.py,
-                                        (z0 << 16) + 32768 + (h << 17) - A.pz, W, H, A.D);
+                                        (z0 << 16) + 32768 + (h << 17) - A.pz, W, H, A.D MIG_CHECKED(, &p));
         }
         O |= (uint64_t)__ballot_sync(0xffffffffu, obs[0]) | ((uint64_t)__ballot_sync(0xffffffffu, obs[1]) << 32);
     }

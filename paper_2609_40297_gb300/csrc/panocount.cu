@@ -75,7 +75,7 @@ struct PanoRays {
         const float hi[3] = {fmaxf(ax, bx) * ic, fmaxf(ay, by) * ic, fmaxf(fmaxf(z0, z1), fmaxf(z0, z1) * ic)};
         const float zm = z0 * z1 <= 0.0f ? 0.0f : fminf(fabsf(z0), fabsf(z1));
         const float s_end = q16f((int)p.Tq) * rsqrtf(1.0f + zm * zm) * 1.00001f;
-        return beam_free(dist, p.grid.nx, p.grid.ny, p.grid.nz, nd.x, nd.y, nd.z, lo, hi, s_end);
+        return beam_free(dist, p.grid.nx, p.grid.ny, p.grid.nz, nd.x, nd.y, nd.z, lo, hi, s_end MIG_CHECKED(, &p));
     }
 };
 
@@ -182,21 +182,21 @@ __device__ __forceinline__ PanoBox pano_box(const PanoConst &c, float cx, float 
     return b;
 }
 // Bounds of the step counts under a box (hz_box), over the seam between the last and the first column.
-__device__ __forceinline__ uint32_t pano_hz(const uint32_t *hz, const Pyramid &y, int top, const PanoBox &b, int A) {
+__device__ __forceinline__ uint32_t pano_hz(const LevelParams &p, const uint32_t *hz, const Pyramid &y, int top, const PanoBox &b, int A) {
     BoxView v;
     v.v0 = b.r0;
     v.v1 = b.r1;
     v.u0 = max(b.c0, 0);
     v.u1 = min(b.c1, A - 1);
-    uint32_t r = hz_box(hz, y, top, v);
+    uint32_t r = hz_box(p, hz, y, top, v);
     if (b.c0 < 0) {
         v.u0 = b.c0 + A;
         v.u1 = A - 1;
-        r = __vminu2(r, hz_box(hz, y, top, v));
+        r = __vminu2(r, hz_box(p, hz, y, top, v));
     } else if (b.c1 >= A) {
         v.u0 = 0;
         v.u1 = b.c1 - A;
-        r = __vminu2(r, hz_box(hz, y, top, v));
+        r = __vminu2(r, hz_box(p, hz, y, top, v));
     }
     return r;
 }
@@ -272,7 +272,10 @@ __device__ __forceinline__ void count_pano_brick(const LevelParams &p, const Vox
                 else row = row_exact(m0, m1, rx, ry, rz0 + (h << 17), H);
                 in = row >= 0;
             }
-            if (in && r.rch) in = mxy + abs(z0 + 2 * h - (nd.z >> 16)) < (int)ld_written(steps + (size_t)row * A + col);
+            if (in && r.rch) {
+                const uint16_t *s = steps + (size_t)row * A + col;
+                in = steps_ok(p, s) && mxy + abs(z0 + 2 * h - (nd.z >> 16)) < (int)ld_written(s);
+            }
             if (in && r.vis && !(Z >= 0.5f && r2 < vc.l22 && Z < p.vis_zl2)) {
                 const int4 d = p.pano_dir[(size_t)col * H + row];
                 const float q30 = 9.31322574615478515625e-10f;
@@ -352,7 +355,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, 3) pano_node_kernel(const LevelP
                       Z = __shfl_sync(0xffffffffu, mZ, src) * 2;  // the block's first brick
             const int bx = X + (lane & 3), by = Y + ((lane >> 2) & 3), bz = Z + (lane >> 4);
             uint64_t U = 0;
-            if (bx < bd.nbx && by < bd.nby && bz < bd.nbz) U = ld_u64(umask + ((size_t)(bz * bd.nby + by) * bd.nbx + bx));
+            if (bx < bd.nbx && by < bd.nby && bz < bd.nbz) U = ld_mask(umask, (size_t)(bz * bd.nby + by) * bd.nbx + bx MIG_CHECKED(, &p));
             const float cx = q16f(((4 * bx + 2) << 16) - nd.x), cy = q16f(((4 * by + 2) << 16) - nd.y),
                         cz = q16f(((4 * bz + 2) << 16) - nd.z);
             float far;
@@ -372,7 +375,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, 3) pano_node_kernel(const LevelP
                     const int ax = 4 * bx - v0x, ay = 4 * by - v0y, az = 4 * bz - v0z;
                     const int man0 = max(max(ax, -ax - 3), 0) + max(max(ay, -ay - 3), 0) + max(max(az, -az - 3), 0);
                     const int man1 = max(abs(ax), abs(ax + 3)) + max(abs(ay), abs(ay + 3)) + max(abs(az), abs(az + 3));
-                    const uint32_t hm = pano_hz(hz, ppyr, top, b, A);
+                    const uint32_t hm = pano_hz(p, hz, ppyr, top, b, A);
                     want = man0 < (int)((hm >> 16) ^ 0xFFFFu);
                     reach = man1 < (int)(hm & 0xFFFFu);
                 }
@@ -388,7 +391,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, 3) pano_node_kernel(const LevelP
             at = __shfl_sync(0xffffffffu, at, 0) + __popc(recs & ((1u << lane) - 1u));
             BrickRec r{U, O, left, in && reach && sure, 0ull, !reach, !sure, (uint32_t)bx | ((uint32_t)by << 10) | ((uint32_t)bz << 20),
                        (uint32_t)ln};
-            if (want && at < p.queue_cap) p.queue[at] = r;
+            if (want && at < p.queue_cap && queue_ok(p, at)) p.queue[at] = r;
 #pragma unroll 1
             for (unsigned full = __ballot_sync(0xffffffffu, want && at >= p.queue_cap); full; full &= full - 1) {
                 const int s = __ffs(full) - 1;
@@ -431,6 +434,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, 4) pano_brick_kernel(const Level
         const int end = min(i + slice, total);
 #pragma unroll 1
         for (; i < end; ++i) {
+            if (!queue_ok(p, i)) continue;
             const BrickRec r = p.queue[i];
             if (r.node != cur) {
                 cur = r.node;

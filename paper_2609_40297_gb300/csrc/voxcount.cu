@@ -131,7 +131,8 @@ __global__ void __launch_bounds__(kVoxWarps * 32, 3) voxel_kernel(const LevelPar
                     if (pixel_in(U, Z, uf, p.W, pu) && pixel_in(V, Z, vf, p.H, pv)) {
                         pix = pv * p.W + pu;
                         const int man = abs(x - v0x) + abs(y - v0y) + abs(z - v0z);
-                        keep = man < (int)ld_written(steps + pix);
+                        keep = at_ok(p, steps + pix, (const uint16_t *)p.steps, (size_t)p.steps_cap * p.W * p.H, kBoundsSteps) &&
+                               man < (int)ld_written(steps + pix);
                     }
                 }
             }
