@@ -255,33 +255,36 @@ void launch_device_levels(mig_ctx *ctx, LevelParams p, int n, int levels, int2 *
     }
 }
 
-// Microseconds of the two ways to count a tree, fitted to 2800 timings (5 to 1500 nodes, ranges of R = 5 to 200
-// voxels, images of 8x4 to 320x240, 1 to 48 yaws; rooms, terrain and a map full of boxes, ranges within the
+// Microseconds of the two ways to count a tree, fitted to 4400 timings (5 to 1500 nodes, ranges of R = 5 to 200
+// voxels, images of 8x4 to 320x240, 1 to 250 yaws; rooms, terrain and a map full of boxes, ranges within the
 // grid and far beyond it):
 //   ray by ray - per level two launches and a chain of voxel loads as long as a ray's way, and each ray's walk;
 //                a ray's way ends at the range or about a third of the grid away;
-//   by voxels  - per round (a level or a chunk of one) three launches; the cast of each ray; and, over the part
+//   by voxels  - per round (a level or a chunk of one) three launches and the yaws that an undecided brick goes
+//                through one by one; the cast of each ray; and, over the part
 //                of the range ball between the image's elevations that lies in the grid, each node's voxels
 //                and each yaw's frustum of them.
 // Voxels that lie closer than the image's pixels are mostly on no ray at all, so that a coarse image over a
 // long range is walked sooner than enumerated: 1000 nodes, R = 150, 16 yaws of 56x42 count in 68 ms ray by
-// ray and 184 by voxels, of 128x96 in 251 and 201. The slower way by more than a quarter is chosen in 66 of
-// the 2800, 3 of them among images 36 pixels wide or more, 4 yaws, 20 nodes and ranges of 15 voxels or more.
+// ray and 184 by voxels, of 128x96 in 251 and 201. The slower way by more than a quarter is chosen in 119 of
+// the 4400; in 2 of the 345 with at least 20 nodes, images 36 pixels wide, 4 to 36 yaws and ranges of 15 voxels
+// up to half the grid.
 // margin: what the caller adds to the voxels' side.
 bool rays_cheaper(const mig_sensor &s, const mig_map *m, int n, int levels, int rounds, int mode, double margin) {
     struct {
-        double level, chain, walk, start, way, round, cast, cast_way, node, yaw;
-    } c = {18.0, 1.65, 3.9e-6, 1.7, 0.35, 28.0, 12e-6, 1e-6, 6e-6, 2.4e-6};
+        double level, chain, walk, start, way, round, serial, cast, cast_way, node, yaw;
+    } c = {21.0, 1.44, 4.2e-6, 0.9, 0.38, 28.0, 0.36, 2.8e-6, 1.12e-6, 7.2e-6, 2.14e-6};
     double rays = (double)s.yaw_bins * s.width * s.height * n;
-    if (mode == MIG_MODE_INTERVAL) c = {16.0, 3.2, 5e-6, 0.4, 0.47, 32.0, 16e-6, 1.4e-6, 5.6e-6, 4.5e-6};
+    if (mode == MIG_MODE_INTERVAL) c = {12.0, 3.46, 5.3e-6, 0.34, 0.45, 32.0, 0.25, 9.3e-6, 1.7e-6, 2.2e-6, 4.5e-6};
     if (mode == MIG_MODE_PANORAMIC) {
-        c = {20.0, 1.4, 7.5e-6, 1.2, 0.23, 35.0, 7e-6, 1.35e-6, 15.5e-6, 0.43e-6};
+        c = {20.0, 1.4, 7.5e-6, 1.2, 0.23, 35.0, 0.0, 7e-6, 1.35e-6, 15.5e-6, 0.43e-6};
         rays = (double)pano_columns(s) * s.height * n;
     }
     const double R = s.range_m / m->voxel, way = std::min(R, c.way * std::max(m->nx, m->ny)), up = std::sin(s.vfov_deg * (M_PI / 360.0));
     const double ball = R * R * R * up * std::min(1.0, m->nx / (2.0 * R)) * std::min(1.0, m->ny / (2.0 * R)) * std::min(1.0, m->nz / (2.0 * R * up));
+    const double views = s.yaw_bins * (s.hfov_deg / 90.0);
     return levels * (c.level + c.chain * way) + c.walk * rays * (way + c.start) <
-           margin * (rounds * c.round + (c.cast + c.cast_way * way) * rays + n * ball * (c.node + c.yaw * s.yaw_bins * (s.hfov_deg / 90.0)));
+           margin * (rounds * (c.round + c.serial * views) + (c.cast + c.cast_way * way) * rays + n * ball * (c.node + c.yaw * views));
 }
 
 SensorDims steps_dims(const mig_sensor &s, const mig_map *m, int mode) {
