@@ -570,11 +570,11 @@ mig_status mig_map_create(mig_ctx *ctx, int nx, int ny, int nz, float voxel_size
             return fail(MIG_ENOMEM, "map_create: staging allocation failed");
         }
         MIG_CUDA_TRY(cudaMemcpyAsync(tmp, host_voxels, nvox, cudaMemcpyHostToDevice, ctx->stream));
-        launch_map_write(m->d_grid, m->nx, m->ny, m->nz, tmp, 0, 0, 0, nx, ny, nz, ctx->stream);
+        launch_map_write(m->d_grid, m->nx, m->ny, m->nz, tmp, 0, 0, 0, nx, ny, nz, 0, ctx->stream);
         MIG_CUDA_TRY(cudaGetLastError());
         ctx->alloc.free(tmp, nvox, ctx->stream);
     } else {
-        launch_map_write(m->d_grid, nx, ny, nz, nullptr, 0, 0, 0, nx, ny, nz, ctx->stream);
+        launch_map_write(m->d_grid, nx, ny, nz, nullptr, 0, 0, 0, nx, ny, nz, 0, ctx->stream);
         MIG_CUDA_TRY(cudaGetLastError());
     }
     MIG_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
@@ -595,7 +595,7 @@ mig_status mig_map_update(mig_map *m, int x0, int y0, int z0, int dx, int dy, in
     uint8_t *tmp = (uint8_t *)ctx->alloc.alloc(nvox, ctx->stream);
     if (!tmp) return fail(MIG_ENOMEM, "map_update: staging allocation failed");
     MIG_CUDA_TRY(cudaMemcpyAsync(tmp, host_voxels, nvox, cudaMemcpyHostToDevice, ctx->stream));
-    launch_map_write(m->d_grid, m->nx, m->ny, m->nz, tmp, x0, y0, z0, dx, dy, dz, ctx->stream);
+    launch_map_write(m->d_grid, m->nx, m->ny, m->nz, tmp, x0, y0, z0, dx, dy, dz, (uint32_t)(m->version + 1), ctx->stream);
     MIG_CUDA_TRY(cudaGetLastError());
     ctx->alloc.free(tmp, nvox, ctx->stream);
     MIG_CUDA_TRY(cudaStreamSynchronize(ctx->stream));  // the host buffer may be reused on return

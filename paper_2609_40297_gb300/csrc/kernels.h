@@ -101,9 +101,10 @@ void launch_select(const LevelParams &p, int grid, cudaStream_t s);  // a level 
 void launch_select_render(const LevelParams &p, int nodes, int num_sms, cudaStream_t s);
 void set_visit_params(LevelParams &p, float hfov_deg, float vfov_deg);  // the vis_* fields, from p.W and p.H
 // Writes a box of voxel codes into a grid of nx * ny * nz (box NULL: they are in place) and refreshes the
-// occupancy bytes, masks and distances that depend on it (mapwrite.cu).
+// occupancy bytes, masks and distances that depend on it (mapwrite.cu). version: the map's after this write, or
+// 0 for its first.
 void launch_map_write(uint8_t *grid, int nx, int ny, int nz, const uint8_t *box, int x0, int y0, int z0, int dx, int dy, int dz,
-                      cudaStream_t s);
+                      uint32_t version, cudaStream_t s);
 // device bytes of an nx*ny*nz grid's voxel codes and occupancy bytes
 size_t map_codes_bytes(int nx, int ny, int nz);
 // device bytes of an nx*ny*nz grid with the masks and distances of its bricks

@@ -5,12 +5,13 @@
 //                      occupancy bytes of the 8x8x8 bricks they make up;
 //   dist_xy_kernel   - per brick, the distances to the occupied bricks of its own z layer; the occupancy bytes
 //                      of the 32x32x32 super-bricks;
-//   dist_z_kernel    - the octant distances and their minimum, from the layers ahead and behind.
+//   dist_z_kernel    - the octant distances and their minimum, from the layers ahead and behind; the clutter bit.
 // An update of a few voxels is a chain of launches and of dependent loads, so both are few: every kernel
 // issues its loads together, before any store, and a brick's row of neighbours is three words of bits. Codes,
 // two summaries, masks and three distance passes as seven launches took 75 us per mig_map_update of one voxel
-// of a 400x400x100 map (96 of 40x40x20 voxels, 75 of one voxel of 800x800x200); this takes 36 (52, 37), as
-// long as codes and summaries alone did (36, 52, 37).
+// of a 400x400x100 map (96 of 40x40x20 voxels, 75 of one voxel of 800x800x200); this takes 30 (43, 30) where no
+// brick is emptied or first occupied, which ends the second and third launch at once, and 37 (54, 40) else.
+// Codes and summaries alone took 36 (51, 35).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -32,10 +33,16 @@ __device__ __forceinline__ uint32_t *brick_bits(uint8_t *grid, int nx, int ny, i
     return reinterpret_cast<uint32_t *>(grid + bits_offset(nx, ny, nz)) + ((size_t)bz * n.nby + by) * bits_words(n.nbx);
 }
 
+// The version of the map whose write last emptied or occupied a brick: another one leaves distances and
+// super-bricks as they are.
+__device__ __forceinline__ uint32_t *changed_flag(uint8_t *grid, int nx, int ny, int nz) {
+    return reinterpret_cast<uint32_t *>(grid + changed_offset(nx, ny, nz));
+}
+
 // A CTA's four warps take the brick rows (2 Y + (warp & 1), 2 Z + (warp >> 1)), lane = x. box NULL: the codes
 // are in place.
 __global__ void __launch_bounds__(128) map_write_kernel(uint8_t *grid, int nx, int ny, int nz, const uint8_t *box, int x0, int y0,
-                                                        int z0, int dx, int dy, int dz) {
+                                                        int z0, int dx, int dy, int dz, uint32_t version) {
     __shared__ uint32_t s_occ[4];
     wait_previous();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -44,7 +51,8 @@ __global__ void __launch_bounds__(128) map_write_kernel(uint8_t *grid, int nx, i
     const BrickDims nb = brick_dims(nx, ny, nz);
     uint32_t occ = 0;
     if (by < nb.nby && bz < nb.nbz) {
-        uint8_t c[16];
+        uint8_t *bits = reinterpret_cast<uint8_t *>(brick_bits(grid, nx, ny, nz, by, bz)) + sx, c[16];
+        const uint32_t before = *bits;
         uint32_t in = 0;  // bit i: voxel i of the lane's column is in the box
         uint8_t *first = grid + ((size_t)(4 * bz) * ny + 4 * by) * nx + x;
 #pragma unroll
@@ -72,7 +80,10 @@ __global__ void __launch_bounds__(128) map_write_kernel(uint8_t *grid, int nx, i
             reinterpret_cast<uint64_t *>(grid + omask_offset(nx, ny, nz))[b] = o;
         }
         occ = __ballot_sync(0xffffffffu, o != 0) & 255u;
-        if (lane == 0) reinterpret_cast<uint8_t *>(brick_bits(grid, nx, ny, nz, by, bz))[sx] = (uint8_t)occ;
+        if (lane == 0 && occ != before) {
+            *bits = (uint8_t)occ;
+            *changed_flag(grid, nx, ny, nz) = version;
+        }
     }
     if (lane == 0) s_occ[warp] = occ;
     __syncthreads();
@@ -91,8 +102,10 @@ constexpr int kDistY = 4;
 // One-sided distances d = min over j >= 0 of max(j, the previous axis' distance j bricks ahead), capped at
 // kDistCap, as bytes: here the four combinations of directions along x (bit 0) and y (bit 1). The block
 // layers from box.wz on take the occupancy bytes of the super-bricks from (sx, sy, sz) on.
-__global__ void __launch_bounds__(32 * kDistY) dist_xy_kernel(uint8_t *grid, int nx, int ny, int nz, const BrickBox box, const BrickBox supers) {
+__global__ void __launch_bounds__(32 * kDistY) dist_xy_kernel(uint8_t *grid, int nx, int ny, int nz, const BrickBox box, const BrickBox supers,
+                                                              uint32_t version) {
     wait_previous();
+    if (version && *changed_flag(grid, nx, ny, nz) != version) return;
     const BrickDims n = brick_dims(nx, ny, nz);
     if ((int)blockIdx.z >= box.wz) {  // a byte of the bits for each of 8x8 brick rows, two per lane
         const int lane = threadIdx.x;
@@ -133,14 +146,28 @@ __global__ void __launch_bounds__(32 * kDistY) dist_xy_kernel(uint8_t *grid, int
 
 // ... and along z: the eight octants (octant_of) and their minimum. Lets no launch start early: what follows
 // reads the map through the read-only path.
-__global__ void __launch_bounds__(32 * kDistY) dist_z_kernel(uint8_t *grid, int nx, int ny, int nz, const BrickBox box) {
+__global__ void __launch_bounds__(32 * kDistY) dist_z_kernel(uint8_t *grid, int nx, int ny, int nz, const BrickBox box, uint32_t version) {
     cudaGridDependencySynchronize();
+    if (version && *changed_flag(grid, nx, ny, nz) != version) return;
     const BrickDims n = brick_dims(nx, ny, nz);
     const int ix = blockIdx.x * 32 + threadIdx.x, iy = blockIdx.y * kDistY + threadIdx.y;
     if (ix >= box.wx || iy >= box.wy) return;
     const int bx = box.ax + ix, by = box.ay + iy, bz = box.az + blockIdx.z, layer = n.nbx * n.nby;
     const size_t at = ((size_t)bz * n.nby + by) * n.nbx + bx;
     const uint32_t *xy = reinterpret_cast<const uint32_t *>(grid + dist_xy_offset(nx, ny, nz)) + at;
+    // occupied bricks among the 27 around it, loaded with the rest
+    const int words = bits_words(n.nbx), w = bx >> 5, sh = bx & 31;
+    const uint32_t *row = brick_bits(grid, nx, ny, nz, by, bz) + w;
+    int occ = 0;
+#pragma unroll
+    for (int r = 0; r < 9; ++r) {
+        const int dy = r % 3 - 1, dz = r / 3 - 1;
+        if ((unsigned)(by + dy) < (unsigned)n.nby && (unsigned)(bz + dz) < (unsigned)n.nbz) {
+            const uint32_t *q = row + (ptrdiff_t)(dz * n.nby + dy) * words;
+            const uint32_t before = sh == 0 && w > 0 ? q[-1] >> 31 : 0u, after = sh == 31 && w + 1 < words ? q[1] << 31 : 0u;
+            occ += __popc(sh == 0 ? (before | (*q << 1)) & 7u : ((*q >> (sh - 1)) & (sh == 31 ? 3u : 7u)) | (after >> 29));
+        }
+    }
     uint32_t lo = kDistCap * 0x01010101u, hi = lo;
 #pragma unroll
     for (int j = 0; j < kDistCap; ++j) {
@@ -156,7 +183,9 @@ __global__ void __launch_bounds__(32 * kDistY) dist_z_kernel(uint8_t *grid, int 
         dist[(o + 1) * plane] = (uint8_t)v;
         least = min(least, v);
     }
-    *dist = (uint8_t)least;
+    const int in = (min(bx + 1, n.nbx - 1) - max(bx - 1, 0) + 1) * (min(by + 1, n.nby - 1) - max(by - 1, 0) + 1) *
+                   (min(bz + 1, n.nbz - 1) - max(bz - 1, 0) + 1);
+    *dist = (uint8_t)(least | (least == 0 && 27 * occ >= 22 * in ? kClutter : 0));
 }
 
 }  // namespace
@@ -165,10 +194,10 @@ size_t map_codes_bytes(int nx, int ny, int nz) { return occ_summary_end(nx, ny, 
 size_t map_layout_bytes(int nx, int ny, int nz) { return brick_data_end(nx, ny, nz); }
 
 void launch_map_write(uint8_t *grid, int nx, int ny, int nz, const uint8_t *box, int x0, int y0, int z0, int dx, int dy, int dz,
-                      cudaStream_t s) {
+                      uint32_t version, cudaStream_t s) {
     const int x1 = x0 + dx - 1, y1 = y0 + dy - 1, z1 = z0 + dz - 1;
     const dim3 rows((unsigned)((x1 >> 5) - (x0 >> 5) + 1), (unsigned)((y1 >> 3) - (y0 >> 3) + 1), (unsigned)((z1 >> 3) - (z0 >> 3) + 1));
-    map_write_kernel<<<rows, 128, 0, s>>>(grid, nx, ny, nz, box, x0, y0, z0, dx, dy, dz);
+    map_write_kernel<<<rows, 128, 0, s>>>(grid, nx, ny, nz, box, x0, y0, z0, dx, dy, dz, version);
     // a brick's distances depend on the bricks up to kDistCap - 1 away along each axis
     const BrickDims n = brick_dims(nx, ny, nz);
     const int first[3] = {x0 >> 2, y0 >> 2, z0 >> 2}, last[3] = {x1 >> 2, y1 >> 2, z1 >> 2}, nb[3] = {n.nbx, n.nby, n.nbz};
@@ -183,8 +212,8 @@ void launch_map_write(uint8_t *grid, int nx, int ny, int nz, const uint8_t *box,
     dim3 g = blocks(xy);
     const unsigned per_layer = g.x * g.y * kDistY;
     g.z += ((unsigned)(supers.wx * supers.wy * supers.wz) + per_layer - 1) / per_layer;
-    launch_behind(dist_xy_kernel, g, dim3(32, kDistY), 0, s, grid, nx, ny, nz, xy, supers);
-    launch_behind(dist_z_kernel, blocks(all), dim3(32, kDistY), 0, s, grid, nx, ny, nz, all);
+    launch_behind(dist_xy_kernel, g, dim3(32, kDistY), 0, s, grid, nx, ny, nz, xy, supers, version);
+    launch_behind(dist_z_kernel, blocks(all), dim3(32, kDistY), 0, s, grid, nx, ny, nz, all, version);
 }
 
 }  // namespace mig

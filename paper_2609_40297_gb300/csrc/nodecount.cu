@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, kCastCtas) cast_kernel(const Lev
         const int q = q0 + ql;
         const int4 nd = p.node[p.level_nodes[l0 + q / p.K]];
         const int32_t *yk = p.yawtab + (q % p.K) * 12;
-        const CameraRays rays{p, nd, yk[0], yk[1], p.W, p.H};
+        const CameraRays rays{p, nd, in_clutter(p, dist, nd), yk[0], yk[1], p.W, p.H};
         const CastOut<DEPTH> o{p.steps + (size_t)ql * WH, p.hz + (size_t)ql * y.n,
                                DEPTH && nd.w >= 0 ? p.depths + (size_t)ql * WH : nullptr};
         const int x0 = tile % tx * T, y0 = tile / tx * T;
@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(kWarpsN * 32, kCastCtas) render_kernel(const L
         const int k = select_warp(p, n, tile == 0 && (lay == kCastLarge || warp == 0), lane);
         const int32_t *yk = p.yawtab + k * 12;
         if (nd.w < 0) continue;  // uniform over the warps of the item
-        const CameraRays rays{p, nd, yk[0], yk[1], p.W, p.H};
+        const CameraRays rays{p, nd, in_clutter(p, dist, nd), yk[0], yk[1], p.W, p.H};
         const RenderOut o{p.dpyr ? p.dpyr + (size_t)nd.w * y.n : nullptr, nd.w,
                           p.depths ? p.depths + ((size_t)(l0 + it / (tx * ty)) * p.K + k) * ((size_t)p.W * p.H) : nullptr};
         const int x0 = tile % tx * T, y0 = tile / tx * T;

@@ -48,17 +48,24 @@ __device__ __forceinline__ CastLayout cast_layout(long long images, int W, int H
     return tiles >= 3 * warps ? kCastLarge : (2 * tiles >= warps ? kCastMid : kCastSmall);
 }
 
+// Do nearly all bricks around a node hold occupied voxels (kClutter)?
+__device__ __forceinline__ bool in_clutter(const LevelParams &p, const uint8_t *dist, const int4 nd) {
+    const BrickDims n = brick_dims(p.grid.nx, p.grid.ny, p.grid.nz);
+    return ld_dist(dist, (size_t)((nd.z >> 18) * n.nby + (nd.y >> 18)) * n.nbx + (nd.x >> 18) MIG_CHECKED(, &p)) & kClutter;
+}
+
 // The rays of a yaw's image from node nd.
 struct CameraRays {
     const LevelParams &p;
     int4 nd;
+    bool clutter;  // nearly all bricks around the node hold occupied voxels
     int ck, sk, W, H;
     // pixel (i, j)'s direction (Q30, unit) and its camera depth per unit length
     __device__ __forceinline__ int4 ray(int i, int j) const { return p.body[j * W + i]; }
     __device__ __forceinline__ void dir(const int4 &b, int &dx, int &dy, int &dz) const { ray_dir(b, ck, sk, dx, dy, dz); }
     // the beam of the 8x4 part at pixel (i0, j0)
     __device__ __forceinline__ float beam(const uint8_t *dist, int i0, int j0) const {
-        if (i0 >= W || j0 >= H) return 0.0f;
+        if (i0 >= W || j0 >= H || clutter) return 0.0f;
         const int i1 = min(i0 + 7, W - 1), j1 = min(j0 + 3, H - 1);
         const float q30 = 9.31322574615478515625e-10f, c = (float)ck * q30, s = (float)sk * q30;
         float lo[3] = {1e30f, 1e30f, 1e30f}, hi[3] = {-1e30f, -1e30f, -1e30f};
@@ -155,15 +162,23 @@ struct RayHit {
 };
 template <bool STATS, bool DEPTH>
 __device__ __noinline__ RayHit cast_ray(const uint64_t *om, const uint8_t *oct, int gnx, int gny, int gnz, int Px, int Py, int Pz,
-                                       int dx, int dy, int dz, int Tq, float t0, CastCnt *st MIG_CHECKED(, const LevelParams *lp)) {
+                                       int dx, int dy, int dz, int Tq, float t0, int start, CastCnt *st MIG_CHECKED(, const LevelParams *lp)) {
     RayHit h{0, 0, 1};
     uint32_t fine = 0, jump = 0;
-    h.m = cast_bricks<DEPTH, STATS>(om, oct, gnx, gny, gnz, Px, Py, Pz, dx, dy, dz, Tq, t0, h.ne, h.ade, fine, jump MIG_CHECKED(, lp));
+    h.m = cast_bricks<DEPTH, STATS>(om, oct, gnx, gny, gnz, Px, Py, Pz, dx, dy, dz, Tq, t0, h.ne, h.ade, fine, jump, start MIG_CHECKED(, lp));
     if constexpr (STATS) {
         st->fine += fine;
         st->jump += jump;
     }
     return h;
+}
+
+template <bool STATS>
+__device__ __noinline__ NearWalk cast_near(const uint64_t *om, int gnx, int gny, int gnz, int Px, int Py, int Pz, int dx, int dy, int dz,
+                                           int Tq, CastCnt *st MIG_CHECKED(, const LevelParams *lp)) {
+    const NearWalk w = near_walk(om, gnx, gny, gnz, Px, Py, Pz, dx, dy, dz, Tq MIG_CHECKED(, lp));
+    if constexpr (STATS) st->fine += w.steps + 1;
+    return w;
 }
 
 // Casts the 8x4 part at pixel (i0, j0), lane l the pixel (l & 7, l >> 3); lo, hi gather its bounds.
@@ -186,9 +201,22 @@ __device__ __forceinline__ void cast_part(const LevelParams &p, const uint64_t *
             if (beam < 1e29f) {
                 int dx, dy, dz;
                 r.dir(b, dx, dy, dz);
-                const uint8_t *oct = p.grid.g + oct_offset(p.grid.nx, p.grid.ny, p.grid.nz, octant_of(dx, dy, dz));
-                hit = cast_ray<STATS, OUT::kDepth>(om, oct, p.grid.nx, p.grid.ny, p.grid.nz, r.nd.x, r.nd.y, r.nd.z, dx, dy, dz, (int)p.Tq,
-                                                   beam_time(beam, b.w), &st MIG_CHECKED(, &p));
+                float t0 = beam_time(beam, b.w);
+                int start = -1;
+                bool on = true;
+                if (r.clutter) {  // (the beam stops where it starts)
+                    const NearWalk w = cast_near<STATS>(om, p.grid.nx, p.grid.ny, p.grid.nz, r.nd.x, r.nd.y, r.nd.z, dx, dy, dz, (int)p.Tq, &st
+                                                        MIG_CHECKED(, &p));
+                    if (w.hit != kNoHit) hit = RayHit{w.hit, w.en, w.ea};
+                    on = w.brick >= 0;
+                    start = w.brick;
+                    t0 = w.t;
+                }
+                if (on) {
+                    const uint8_t *oct = p.grid.g + oct_offset(p.grid.nx, p.grid.ny, p.grid.nz, octant_of(dx, dy, dz));
+                    hit = cast_ray<STATS, OUT::kDepth>(om, oct, p.grid.nx, p.grid.ny, p.grid.nz, r.nd.x, r.nd.y, r.nd.z, dx, dy, dz, (int)p.Tq,
+                                                       t0, start, &st MIG_CHECKED(, &p));
+                }
             }
         }
         v = o.put(p, at, dzc, hit.m, hit.ne, hit.ade);

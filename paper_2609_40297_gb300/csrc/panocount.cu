@@ -46,6 +46,7 @@ __device__ __forceinline__ NodeRange node_range(const LevelParams &p, bool cast 
 struct PanoRays {
     const LevelParams &p;
     int4 nd;
+    bool clutter;  // as of CameraRays
     int W, H;
     // w: at least the horizontal part of the unit ray (Q30)
     __device__ __forceinline__ int4 ray(int i, int j) const {
@@ -62,7 +63,7 @@ struct PanoRays {
     // at unit depth its rays' horizontal parts lie on a line, and their heights between z / h and
     // z / (h cos) of the outermost columns. A unit ray's depth is at most h.
     __device__ __forceinline__ float beam(const uint8_t *dist, int i0, int j0) const {
-        if (i0 >= W || j0 >= H || W < 64) return 0.0f;  // 8 columns: at most 45 degrees
+        if (i0 >= W || j0 >= H || W < 64 || clutter) return 0.0f;  // 8 columns: at most 45 degrees
         const int i1 = min(i0 + 7, W - 1), j1 = min(j0 + 3, H - 1);
         const int4 a = p.pano_dir[(size_t)i0 * H + j0], b = p.pano_dir[(size_t)i1 * H + j0], d = p.pano_dir[(size_t)i0 * H + j1];
         const float ha = sqrtf((float)a.x * (float)a.x + (float)a.y * (float)a.y), ia = 1.0f / ha;
@@ -104,7 +105,8 @@ __global__ void __launch_bounds__(kWarpsN * 32, kCastCtas) pano_cast_kernel(cons
         if (dyn && lane == 0) more = atomicAdd(p.work, 1);
         const int tile = (int)(it % (tx * ty)), ln = (int)(it / (tx * ty));
         const int n = p.level_nodes[nr.l0 + nr.q0 + ln];
-        const PanoRays rays{p, p.node[n], A, H};
+        const int4 nd = p.node[n];
+        const PanoRays rays{p, nd, in_clutter(p, dist, nd), A, H};
         const CastOut<false> o{p.steps + (size_t)ln * AH, p.hz + (size_t)ln * y.n, nullptr};
         const int x0 = tile % tx * T, y0 = tile / tx * T;
         if (y0 == 0) {  // the first row of tiles clears its columns' counts

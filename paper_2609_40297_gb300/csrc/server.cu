@@ -319,7 +319,8 @@ mig_status apply_update(mig_server *s, Update &u) {
     uint8_t *tmp = (uint8_t *)ctx->alloc.alloc(nv, ctx->stream);
     if (!tmp) return fail(MIG_ENOMEM, "server: update staging allocation failed");
     MIG_CUDA_TRY(cudaMemcpyAsync(tmp, u.voxels.data(), nv, cudaMemcpyHostToDevice, ctx->stream));
-    launch_map_write(m->d_grid, m->nx, m->ny, m->nz, tmp, u.x0, u.y0, u.z0, u.dx, u.dy, u.dz, ctx->stream);
+    launch_map_write(m->d_grid, m->nx, m->ny, m->nz, tmp, u.x0, u.y0, u.z0, u.dx, u.dy, u.dz, (uint32_t)(m->version + 1),
+                     ctx->stream);
     MIG_CUDA_TRY(cudaGetLastError());
     ctx->alloc.free(tmp, nv, ctx->stream);
     MIG_CUDA_TRY(cudaStreamSynchronize(ctx->stream));  // the host voxels are freed with the update
