@@ -255,36 +255,42 @@ void launch_device_levels(mig_ctx *ctx, LevelParams p, int n, int levels, int2 *
     }
 }
 
-// Microseconds of the two ways to count a tree, fitted to 4400 timings (5 to 1500 nodes, ranges of R = 5 to 200
+// Microseconds of the two ways to count a tree, fitted to 4800 timings (5 to 1500 nodes, ranges of R = 5 to 200
 // voxels, images of 8x4 to 320x240, 1 to 250 yaws; rooms, terrain and a map full of boxes, ranges within the
 // grid and far beyond it):
-//   ray by ray - per level two launches and a chain of voxel loads as long as a ray's way, and each ray's walk;
-//                a ray's way ends at the range or about a third of the grid away;
+//   ray by ray - per level two launches and a chain of voxel loads as long as a ray's way, and each ray's walk; the
+//                way ends at the range or about 0.4 of the grid away, and long ways leave lanes idle (bend);
 //   by voxels  - per round (a level or a chunk of one) three launches and the yaws that an undecided brick goes
-//                through one by one; the cast of each ray; and, over the part
-//                of the range ball between the image's elevations that lies in the grid, each node's voxels
-//                and each yaw's frustum of them.
+//                through one by one; the cast of each ray; and, over the part of the range ball between the
+//                image's elevations that lies in the grid, each node's voxels and each yaw's frustum of them.
 // Voxels that lie closer than the image's pixels are mostly on no ray at all, so that a coarse image over a
 // long range is walked sooner than enumerated: 1000 nodes, R = 150, 16 yaws of 56x42 count in 68 ms ray by
-// ray and 184 by voxels, of 128x96 in 251 and 201. The slower way by more than a quarter is chosen in 119 of
-// the 4400; in 2 of the 345 with at least 20 nodes, images 36 pixels wide, 4 to 36 yaws and ranges of 15 voxels
+// ray and 184 by voxels, of 128x96 in 251 and 201. The slower way by more than a quarter is chosen in 129 of
+// the 4800; in 6 of the 745 with at least 20 nodes, images 36 pixels wide, 4 to 36 yaws and ranges of 15 voxels
 // up to half the grid.
-// margin: what the caller adds to the voxels' side.
-bool rays_cheaper(const mig_sensor &s, const mig_map *m, int n, int levels, int rounds, int mode, double margin) {
+// in_chunks: the allocation-free call, whose rounds are long ones (what they take varies with the chunks, so
+// that the voxels' side needs a quarter to spare, and more with more of them) and which loses most in clutter:
+// 50 nodes of 320x240x8 among 20 % of occupied voxels 0.98 ms ray by ray and 1.23 by voxels, 0.97 and 1.04 with
+// memory for whole levels.
+bool rays_cheaper(const mig_sensor &s, const mig_map *m, int n, int levels, int rounds, int mode, bool in_chunks) {
     struct {
-        double level, chain, walk, start, way, round, serial, cast, cast_way, node, yaw;
-    } c = {21.0, 1.44, 4.2e-6, 0.9, 0.38, 28.0, 0.36, 2.8e-6, 1.12e-6, 7.2e-6, 2.14e-6};
+        double level, chain, walk, start, way, bend, round, serial, cast, cast_way, node, yaw;
+    } c = {17.5, 1.77, 3.9e-6, 3.9, 0.41, 144.0, 25.0, 0.47, 2.9e-6, 1.17e-6, 5.0e-6, 3.0e-6};
     double rays = (double)s.yaw_bins * s.width * s.height * n;
-    if (mode == MIG_MODE_INTERVAL) c = {12.0, 3.46, 5.3e-6, 0.34, 0.45, 32.0, 0.25, 9.3e-6, 1.7e-6, 2.2e-6, 4.5e-6};
+    if (mode == MIG_MODE_INTERVAL) c = {12.0, 3.46, 5.3e-6, 0.34, 0.45, 1e9, 32.0, 0.25, 9.3e-6, 1.7e-6, 2.2e-6, 4.5e-6};
     if (mode == MIG_MODE_PANORAMIC) {
-        c = {20.0, 1.4, 7.5e-6, 1.2, 0.23, 35.0, 0.0, 7e-6, 1.35e-6, 15.5e-6, 0.43e-6};
+        c = {20.0, 1.4, 7.5e-6, 1.2, 0.23, 1e9, 35.0, 0.0, 7e-6, 1.35e-6, 15.5e-6, 0.43e-6};
         rays = (double)pano_columns(s) * s.height * n;
     }
     const double R = s.range_m / m->voxel, way = std::min(R, c.way * std::max(m->nx, m->ny)), up = std::sin(s.vfov_deg * (M_PI / 360.0));
     const double ball = R * R * R * up * std::min(1.0, m->nx / (2.0 * R)) * std::min(1.0, m->ny / (2.0 * R)) * std::min(1.0, m->nz / (2.0 * R * up));
     const double views = s.yaw_bins * (s.hfov_deg / 90.0);
-    return levels * (c.level + c.chain * way) + c.walk * rays * (way + c.start) <
-           margin * (rounds * (c.round + c.serial * views) + (c.cast + c.cast_way * way) * rays + n * ball * (c.node + c.yaw * views));
+    // clutter ends the rays of a walk early, and keeps a cast from jumping that far
+    const double path = in_chunks ? (double)m->free_path : 1e9, clear = std::min(way, path),
+                 margin = in_chunks ? 1.25 * (1.0 + 0.06 * ((double)rounds / levels - 1.0)) : 1.0;
+    return levels * (c.level + c.chain * clear) + c.walk * rays * (clear * (1.0 + clear / c.bend) + c.start) <
+           margin * (rounds * (c.round + c.serial * views) + (c.cast + c.cast_way * way + 2.5e-6 * std::min(1.0, R / path) * clear) * rays +
+                     n * ball * (c.node + c.yaw * views));
 }
 
 SensorDims steps_dims(const mig_sensor &s, const mig_map *m, int mode) {
@@ -301,7 +307,7 @@ StepsLayout steps_for(const CountChoice &c, int n, int levels, int Lmax, const m
     if (pano && (size_t)d.W * d.H * sizeof(uint16_t) > c.steps_budget) return StepsLayout{};
     const StepsLayout L = steps_layout(d, n, Lmax, c.steps_budget, lean == 0 ? kTreeSteps : 0, c.pass != MIG_COUNT_PAIRS, mode);
     if (whole && L.queue_cap == 0) return StepsLayout{};
-    if (c.pass == MIG_COUNT_AUTO && rays_cheaper(s, m, n, levels, std::max(levels, device_steps(L, n, d.K, levels)), mode, 1.0)) return StepsLayout{};
+    if (c.pass == MIG_COUNT_AUTO && rays_cheaper(s, m, n, levels, std::max(levels, device_steps(L, n, d.K, levels)), mode, false)) return StepsLayout{};
     return L;
 }
 
@@ -362,10 +368,39 @@ struct Carver {
     }
 };
 
-static mig_status check_codes(const uint8_t *v, size_t n) {
-    for (size_t i = 0; i < n; ++i)
-        if (v[i] > 2) return fail(MIG_EINVAL, "map: voxel code " + std::to_string(v[i]) + " at index " + std::to_string(i) + " (codes are 0, 1, 2)");
-    return MIG_OK;
+CodeScan scan_codes(const uint8_t *v, size_t n) {
+    CodeScan r;
+    for (size_t i0 = 0; i0 < n; i0 += 128) {  // sums of a block fit a byte, so that the loop runs on bytes
+        const size_t m = std::min<size_t>(128, n - i0);
+        const uint8_t *b = v + i0;
+        uint8_t most = 0, open = 0, entries = 0;
+        for (size_t i = 0; i < m; ++i) {
+            most = std::max(most, b[i]);
+            open = (uint8_t)(open + (b[i] != 2));
+        }
+        for (size_t i = 1; i < m; ++i) entries = (uint8_t)(entries + ((b[i] == 2) & (b[i - 1] != 2)));
+        if (most > 2) {
+            for (size_t i = 0; i < m; ++i)
+                if (b[i] > 2) {
+                    r.bad = i0 + i;
+                    return r;
+                }
+        }
+        r.open += open;
+        r.entries += entries;
+    }
+    return r;
+}
+
+static mig_status bad_code(const uint8_t *v, const CodeScan &s) {
+    return fail(MIG_EINVAL, "map: voxel code " + std::to_string(v[s.bad]) + " at index " + std::to_string(s.bad) + " (codes are 0, 1, 2)");
+}
+
+void map_written(mig_map *m, size_t voxels, const CodeScan &scan) {
+    const double keep = 1.0 - (double)voxels / ((double)m->nx * m->ny * m->nz);
+    m->open_voxels = keep * m->open_voxels + (double)scan.open;
+    m->entries = keep * m->entries + (double)scan.entries;
+    m->free_path = (float)std::min(1e9, std::max(1.0, m->open_voxels / std::max(m->entries, 1e-3)));
 }
 
 static LevelParams level_params(const mig_map *m, const Camera *cam, const mig_ctx *ctx) {
@@ -555,8 +590,9 @@ mig_status mig_map_create(mig_ctx *ctx, int nx, int ny, int nz, float voxel_size
     for (int a = 0; a < 3; ++a) m->origin[a] = origin_m ? origin_m[a] : 0.f;
     const size_t nvox = (size_t)nx * ny * nz;
     if (host_voxels) {
-        mig_status st = check_codes(host_voxels, nvox);
-        if (st != MIG_OK) return st;
+        const CodeScan scan = scan_codes(host_voxels, nvox);
+        if (scan.bad != SIZE_MAX) return bad_code(host_voxels, scan);
+        map_written(m.get(), nvox, scan);
     }
     std::lock_guard<std::mutex> lk(ctx->mu);
     MIG_CUDA_TRY(cudaSetDevice(ctx->device));
@@ -587,8 +623,8 @@ mig_status mig_map_update(mig_map *m, int x0, int y0, int z0, int dx, int dy, in
     if (dx < 1 || dy < 1 || dz < 1 || x0 < 0 || y0 < 0 || z0 < 0 || x0 + dx > m->nx || y0 + dy > m->ny || z0 + dz > m->nz)
         return fail(MIG_EINVAL, "map_update: box outside the grid or empty");
     const size_t nvox = (size_t)dx * dy * dz;
-    mig_status st = check_codes(host_voxels, nvox);
-    if (st != MIG_OK) return st;
+    const CodeScan scan = scan_codes(host_voxels, nvox);
+    if (scan.bad != SIZE_MAX) return bad_code(host_voxels, scan);
     mig_ctx *ctx = m->ctx;
     std::lock_guard<std::mutex> lk(ctx->mu);
     MIG_CUDA_TRY(cudaSetDevice(ctx->device));
@@ -600,6 +636,7 @@ mig_status mig_map_update(mig_map *m, int x0, int y0, int z0, int dx, int dy, in
     ctx->alloc.free(tmp, nvox, ctx->stream);
     MIG_CUDA_TRY(cudaStreamSynchronize(ctx->stream));  // the host buffer may be reused on return
     m->version++;
+    map_written(m, nvox, scan);
     return MIG_OK;
 }
 

@@ -5,6 +5,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstdint>
 #include <cstring>
 #include <map>
@@ -172,6 +173,10 @@ struct mig_map {
     uint8_t *d_grid = nullptr;       // voxel codes, summaries, brick data (bricks.cuh)
     size_t grid_bytes = 0;
     uint64_t version = 0;
+    // how far a ray goes along x between occupied voxels, about (voxels): what the two ways to count a tree cost
+    // depends on it. Written with the context's lock held, the shares of the voxels written last kept as a sum.
+    std::atomic<float> free_path{1e9f};
+    double open_voxels = 0.0, entries = 0.0;
 };
 
 namespace mig {
@@ -183,6 +188,13 @@ mig_status ctx_pinned(mig_ctx *ctx, size_t bytes, void **out);
 mig_status ctx_camera(mig_ctx *ctx, const mig_sensor &s, const Camera **out);
 // The panoramic tables of a context camera, built and uploaded on first use (ctx->mu held).
 mig_status ctx_pano(mig_ctx *ctx, const Camera *cam);
+// The codes of a box: are they codes (else the first bad index in *bad), and how many are not occupied, how many
+// of these are followed by an occupied one.
+struct CodeScan {
+    size_t bad = SIZE_MAX, open = 0, entries = 0;
+};
+CodeScan scan_codes(const uint8_t *v, size_t n);
+void map_written(mig_map *m, size_t voxels, const CodeScan &scan);  // (ctx->mu held)
 // The frustum band of the per-node voxel pass, from the camera.
 void set_band(LevelParams &p, const Camera *cam);
 // Panoramic level parameters from the camera's tables; pcnt = n * A * 2 int32 of workspace.
@@ -203,7 +215,7 @@ void launch_level_count_timed(mig_ctx *ctx, const LevelParams &p, int Ld, int co
 struct StepsLayout;
 struct SensorDims;
 SensorDims steps_dims(const mig_sensor &s, const mig_map *m, int mode);  // the images of one node
-bool rays_cheaper(const mig_sensor &s, const mig_map *m, int n, int levels, int rounds, int mode, double margin);
+bool rays_cheaper(const mig_sensor &s, const mig_map *m, int n, int levels, int rounds, int mode, bool in_chunks);
 StepsLayout steps_for(const CountChoice &c, int n, int levels, int Lmax, const mig_sensor &s, const mig_map *m, int mode, int lean);
 // The count and select-and-render launches of a device-planned tree of n nodes and at most `levels` levels.
 // With the per-node pass they go chunk by chunk through the levels, whose sizes only the device knows:

@@ -117,7 +117,7 @@ extern "C" mig_status mig_tree_eval_device_noalloc(mig_map *m, int n, const int3
     const size_t o_cursor = cv.take(sizeof(int2) * ((size_t)n + L + 1)), o_steps = cv.take(0);
     const SensorDims dims{W, H, K, range_q16(sensor->range_m, m->voxel)};
     const StepsLayout steps = o_steps < (size_t)MIG_NOALLOC_SCRATCH_BYTES
-                                  ? steps_layout_in(dims, n, n, (size_t)MIG_NOALLOC_SCRATCH_BYTES - o_steps)
+                                  ? steps_layout_in(dims, n, n, (size_t)MIG_NOALLOC_SCRATCH_BYTES - o_steps, true)
                                   : StepsLayout{};
     if (need > (size_t)MIG_NOALLOC_SCRATCH_BYTES)
         return fail(MIG_EINVAL, "tree_eval_device_noalloc: needs " + std::to_string(need) + " bytes of scratch, above the " +
@@ -232,9 +232,8 @@ extern "C" mig_status mig_tree_eval_device_noalloc(mig_map *m, int n, const int3
     elevation_band(*sensor, p.band_tlo, p.band_thi);
     p.voxel_pass = MIG_COUNT_AUTO;
     set_visit_params(p, sensor->hfov_deg, sensor->vfov_deg);
-    // (by voxels only where it is sooner with a quarter to spare: what the rounds take varies with the chunks)
     const bool rays = ctx->count.rays || ctx->count.pass == MIG_COUNT_PAIRS || steps.cap == 0 ||
-                      (ctx->count.pass == MIG_COUNT_AUTO && rays_cheaper(*sensor, m, n, L, device_steps(steps, n, K, L), MIG_MODE_MARGINAL, 1.25));
+                      (ctx->count.pass == MIG_COUNT_AUTO && rays_cheaper(*sensor, m, n, L, device_steps(steps, n, K, L), MIG_MODE_MARGINAL, true));
     if (!rays) {
         set_steps(p, dev + o_steps, steps);
         p.dpyr = (uint2 *)(dev + o_dpyr);

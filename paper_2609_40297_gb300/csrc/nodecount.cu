@@ -747,7 +747,7 @@ StepsLayout steps_layout(const SensorDims &d, int n, int max_nodes, size_t budge
     return L;
 }
 
-StepsLayout steps_layout_in(const SensorDims &d, int n, int max_nodes, size_t bytes) {
+StepsLayout steps_layout_in(const SensorDims &d, int n, int max_nodes, size_t bytes, bool with_depths) {
     // per node: its step counts, their bounds and 0.7 of the usual queue (a full queue only slows the
     // bricks beyond it), so that a fixed region holds more nodes at a time
     const size_t recs = (size_t)(0.7 * kQueueShare * (double)node_bricks(d.Tq)) + 1;
@@ -762,6 +762,11 @@ StepsLayout steps_layout_in(const SensorDims &d, int n, int max_nodes, size_t by
     // room for the whole tree: one cast
     if (nodes == n && (double)nodes * (double)node_items(d.Tq) * d.K < (double)(1ll << 30)) L.tree = n;
     place(L, d);
+    const size_t depths = (size_t)L.cap * d.W * d.H * sizeof(uint32_t);
+    if (L.tree && with_depths && depths <= kTreeDepths && L.bytes + depths <= bytes) {
+        L.depths = true;
+        place(L, d);
+    }
     return L;
 }
 

@@ -68,6 +68,7 @@ struct Update {
     mig_map *map;
     int x0, y0, z0, dx, dy, dz;
     std::vector<uint8_t> voxels;
+    CodeScan scan;
 };
 
 struct Entry {  // queue entry: a request or a map update
@@ -160,7 +161,7 @@ void choose_region(const mig_server *s, Request &r) {
     }
     const size_t region = most - bare, bounds = depth_bounds(r) + 256;
     r.steps = StepsLayout{};
-    if (r.count.pass != MIG_COUNT_PAIRS && bounds < region) r.steps = steps_layout_in(d, pl.n, r.Lmax, region - bounds);
+    if (r.count.pass != MIG_COUNT_PAIRS && bounds < region) r.steps = steps_layout_in(d, pl.n, r.Lmax, region - bounds, sample);
     if (r.steps.cap == 0 && sample) {  // not one node: by (node, yaw) pairs, or ray by ray
         r.count.pass = MIG_COUNT_PAIRS;
         r.steps = steps_pairs_in(d, r.Lmax, region);
@@ -325,6 +326,7 @@ mig_status apply_update(mig_server *s, Update &u) {
     ctx->alloc.free(tmp, nv, ctx->stream);
     MIG_CUDA_TRY(cudaStreamSynchronize(ctx->stream));  // the host voxels are freed with the update
     m->version++;
+    map_written(m, nv, u.scan);
     return MIG_OK;
 }
 
@@ -551,8 +553,8 @@ extern "C" mig_status mig_server_map_update(mig_server *s, mig_map *m, int x0, i
     u->dy = dy;
     u->dz = dz;
     u->voxels.assign(host_voxels, host_voxels + (size_t)dx * dy * dz);
-    for (uint8_t c : u->voxels)
-        if (c > 2) return fail(MIG_EINVAL, "server_map_update: voxel code above 2");
+    u->scan = scan_codes(u->voxels.data(), u->voxels.size());
+    if (u->scan.bad != SIZE_MAX) return fail(MIG_EINVAL, "server_map_update: voxel code above 2");
     std::lock_guard<std::mutex> lk(s->mu);
     Entry e;
     e.upd = std::move(u);

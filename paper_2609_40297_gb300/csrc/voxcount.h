@@ -32,8 +32,8 @@ struct StepsLayout {
 // tree_bytes: the most step counts for the whole tree (0: level by level)
 StepsLayout steps_layout(const SensorDims &d, int n, int max_nodes, size_t budget_bytes, size_t tree_bytes, bool node_pass, int mode);
 // The same for as many whole nodes as fit in a region of at most `bytes` bytes, and for single pairs (without a
-// queue) as many as fit (cap 0: not one does).
-StepsLayout steps_layout_in(const SensorDims &d, int n, int max_nodes, size_t bytes);
+// queue) as many as fit (cap 0: not one does). with_depths: also a whole tree's depth buffers, where they fit.
+StepsLayout steps_layout_in(const SensorDims &d, int n, int max_nodes, size_t bytes, bool with_depths);
 StepsLayout steps_pairs_in(const SensorDims &d, int max_nodes, size_t bytes);
 void set_steps(LevelParams &p, void *base, const StepsLayout &L);  // the region's fields
 // Step-count buffer budget per evaluation (device bytes).

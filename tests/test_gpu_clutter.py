@@ -57,3 +57,24 @@ def test_clutter(ctx, dims, share, image):
     finally:
         ctx.set_count_kernel(mig.COUNT_AUTO, 0)
         m.close()
+
+
+def test_bad_codes_are_refused(ctx):
+    """Codes above 2 are refused wherever they stand, by create and update, and leave the map as it was."""
+    grid = np.zeros((5, 7, 300), np.uint8)
+    for at in (0, 127, 128, 5 * 7 * 300 - 1):
+        bad = grid.copy()
+        bad.reshape(-1)[at] = 3
+        with pytest.raises(mig.MigError) as e:
+            mig.Map(ctx, bad, 0.1)
+        assert e.value.status == mig.MIG_EINVAL and f"index {at} " in str(e.value)
+    m = mig.Map(ctx, grid, 0.1)
+    try:
+        box = np.full((2, 2, 200), 2, np.uint8)
+        box.reshape(-1)[777] = 255
+        with pytest.raises(mig.MigError) as e:
+            m.update(0, 0, 0, box)
+        assert e.value.status == mig.MIG_EINVAL and "index 777 " in str(e.value)
+        assert np.array_equal(m.read(), grid)
+    finally:
+        m.close()
