@@ -273,11 +273,11 @@ mig_status mig_batch_trace_read(mig_ctx *ctx, mig_trace_rec *out, int cap, int *
 
 /* ---------------------------------------------------------------------------------------
  * Serving: continuous batching of replanning requests. Submitted trees wait in an admission
- * queue until their device bytes (depth-buffer arena nodes * W * H * 4, counters, and their share of the
- * budget, budget / max_inflight, or at most the step counts of their largest level where that is more) plus
- * the bytes already held (requests in flight and map snapshots) fit the budget, then
- * join the device work of the requests already running; each request's results are the same
- * as a lone mig_tree_eval on the map contents at submission time. The descriptor's host arrays
+ * queue until their device bytes plus the bytes already held (requests in flight and map snapshots) fit
+ * the budget. A request's bytes are its depth-buffer arena (nodes * W * H * 4), plan, counters and a region
+ * for its counts, which fills the request's share budget / max_inflight at most, and beyond that takes no
+ * more than the step counts of its largest level. Admitted requests join the device work of the requests
+ * already running; each request's results are the same as a lone mig_tree_eval on the map contents at submission time. The descriptor's host arrays
  * are copied at submit; outputs are written when the request completes. A worker thread
  * drives the device; submit and poll are thread-safe.
  * mig_server_poll: MIG_OK = done (outputs written), MIG_EBUSY = not yet (timeout_us = 0),
@@ -322,16 +322,17 @@ typedef struct mig_kernel_times {
  * each pixel ray once to its first occupied voxel, then tests every unknown voxel of the frustum
  * against the ray of the pixel that owns it (its centre's projection): MIG_COUNT_PAIRS enumerates each
  * (node, yaw) frustum, MIG_COUNT_NODES each node's voxels once for all yaws, whole 4x4x4 bricks at a
- * time (its ancestor test runs once per voxel), MIG_COUNT_AUTO (the default) takes the per-node pass.
- * In the marginal, single-parent and absolute modes either falls back to the pairs when the buffer
- * below does not hold all yaws of one node. The interval and panoramic modes have no pass per pair:
+ * time (its ancestor test runs once per voxel). MIG_COUNT_AUTO (the default) takes the per-node pass, or
+ * walks the rays where an estimate from sensor, range, tree and map finds that sooner (coarse images over
+ * long ranges, mostly). In the marginal, single-parent and absolute modes the per-node pass falls back to
+ * the pairs when the buffer below does not hold all yaws of one node. The interval and panoramic modes have no pass per pair:
  * there, and with MIG_COUNT_PAIRS, they count like MIG_COUNT_RAYS, which walks every ray through every
  * voxel it crosses and owner-tests the unknown ones. The owned-voxel kernels keep one uint16 step count
- * per (node, yaw, pixel) of a level (panoramic mode: per node, column and row) in a buffer of at most
- * steps_budget_bytes (0 = the default, 1 GiB); a level that does not fit is counted in chunks. The
- * per-node pass keeps a queue of undecided bricks beside it (at most 512 MiB). A server's requests keep
- * the kernel and budget that were set when they were submitted. Errors: MIG_EINVAL (ctx NULL, unknown
- * kernel). */
+ * per (node, yaw, pixel) of a level, or of a small tree (panoramic mode: per node, column and row), in a
+ * buffer of at most steps_budget_bytes (0 = the default, 1 GiB); a level that does not fit is counted in
+ * chunks. The per-node pass keeps a queue of undecided bricks beside it (at most 512 MiB). A server's
+ * requests keep the kernel and budget that were set when they were submitted. Errors: MIG_EINVAL (ctx
+ * NULL, unknown kernel). */
 #define MIG_COUNT_AUTO 0
 #define MIG_COUNT_RAYS 1
 #define MIG_COUNT_PAIRS 2

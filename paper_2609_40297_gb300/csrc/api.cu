@@ -1,5 +1,6 @@
 // C ABI of the marginal-gain library: contexts, maps, and tree evaluation in depth order
-// (Sec. IV-C) with one count / select / render launch triple per level on the context stream.
+// (Sec. IV-C): the cast of a small tree, then per level its count (by voxels, or ray by ray) and the yaw
+// selection with the depth-buffer render, on the context stream.
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -260,7 +260,7 @@ MIG_HD bool mask_box(uint64_t m, int lx, int hx, int ly, int hy, int lz, int hz)
 // Bound by instruction issue (about 65 % of the slots, 23 of 32 lanes active). Cast per replan at
 // paper scale / on the large workload: 12.3 / 493 ms with 64-bit compared crossings, 8.2 / 219 ms with
 // one distance for all directions, 8.0 / 208 ms without the box test of occupied bricks, 6.4 / 166 ms;
-// 5.3 ms at paper scale with all levels in one launch.
+// 5.3 ms at paper scale with all levels in one launch, 4.8 / 148 ms with tiles taken one at a time by warps.
 // The step index of a voxel is its Manhattan distance from the start voxel, so the walk need not
 // count steps. With DEPTH, ne / ade return the face distance and speed of the hit voxel's entry
 // (0 / 1 for the start voxel). fine, coarse: voxel steps and jumps taken (STATS).

@@ -649,7 +649,7 @@ void launch_select_render(const LevelParams &p, int nodes, int num_sms, cudaStre
 }
 
 int node_ctas_per_sm() {
-    // the most yaws and the deepest tree: 112 KB
+    // the most yaws and the deepest tree: 120 KiB
     const int smem = (int)node_dyn_smem(MIG_MAX_YAW_BINS, MIG_MAX_DEPTH);
     cudaFuncSetAttribute(node_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     cudaFuncSetAttribute(node_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -704,8 +704,9 @@ void launch_node_chunk(const LevelParams &c, int num_sms, int node_ctas, cudaStr
     }
 }
 
-// The share of them that a chunk's queue has room for (measured: up to 0.27 of a node's bricks are left
-// undecided as a whole; a fuller queue only sends its last bricks through the slower path inside node_kernel).
+// The share of them that a chunk's queue has room for (measured with up to 64 yaws: up to 0.27 of a node's bricks
+// are left undecided as a whole; every further 64 yaws queue a brick again). A fuller queue only sends its last
+// bricks through the slower path inside node_kernel.
 constexpr double kQueueShare = 0.3;
 constexpr double kQueueShareInterval = 0.7;  // there every counted brick that an ancestor looks at
 constexpr double kQueueSharePano = 0.5;      // every brick that a ray can reach
@@ -728,7 +729,7 @@ static void place(StepsLayout &L, const SensorDims &d) {
 StepsLayout steps_layout(const SensorDims &d, int n, int max_nodes, size_t budget_bytes, size_t tree_bytes, bool node_pass, int mode) {
     StepsLayout L{};
     const long long pairs = (long long)std::max(1, max_nodes) * d.K;
-    L.cap = (int)steps_pairs(pairs, d.W, d.H, budget_bytes);
+    L.cap = (int)std::min<size_t>(steps_pairs(pairs, d.W, d.H, budget_bytes), (size_t)1 << 30);
     const long long per_node = (long long)(queue_share(mode) * (double)node_bricks(d.Tq)) + 1;
     if (node_pass && L.cap >= d.K) {  // whole nodes, as many as the queue has room for
         const long long nodes = std::max<long long>(1, std::min<long long>(L.cap / d.K, kQueueMax / per_node));

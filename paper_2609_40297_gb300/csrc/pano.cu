@@ -11,8 +11,8 @@
 // selected yaw then run unchanged.
 //
 // The kernel here walks every ray voxel by voxel. It runs where panocount.cu's count by bricks has no
-// room for a node's step counts, and where the ray-by-ray or pairs count is asked for (3.2 times as slow
-// at 500 nodes of 640 columns).
+// room for a node's step counts, where the ray-by-ray or pairs count is asked for (3.2 times as slow at 500
+// nodes of 640 columns), and where it is the sooner way (rays_cheaper).
 //
 // Layout: one warp per work item (node, column); its lanes take the column's H rays, a new one
 // as soon as their ray ends. Owned samples go to a per-warp queue and are tested against the
