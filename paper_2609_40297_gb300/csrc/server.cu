@@ -203,7 +203,7 @@ mig_status admit(mig_server *s, Request &r) {
     for (int lean = 0; lean < 3 && !r.dev; ++lean) {  // less memory where the allocator has not enough
         if (lean) {
             const StepsLayout less = steps_for(r.count, n, L, r.Lmax, r.sensor, r.map, r.mode, lean);
-            if (less.bytes >= r.steps.bytes) continue;
+            if (lean < 2 && less.bytes >= r.steps.bytes) continue;  // (the least is always asked for)
             r.steps = less;
         }
         Carve c = cv;

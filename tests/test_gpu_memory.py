@@ -138,3 +138,45 @@ def test_refused_memory_is_not_asked_for_by_every_call(monkeypatch, call):
             srv.close()
         m.close()
         c.close()
+
+
+def test_request_is_retried_once_memory_is_there(monkeypatch):
+    """A request that needs the least it can and is refused fails; the next one like it is asked for again."""
+    limit = [1 << 62]
+    real = mig._torch_allocator
+
+    def limited(device):
+        a = real(device)
+
+        def alloc(nbytes, stream, user):
+            return None if nbytes > limit[0] else a.alloc(nbytes, stream, user)
+
+        b = mig.Allocator(mig.ALLOC_FN(alloc), a.free, None)
+        b.keep = (a, alloc)
+        return b
+
+    monkeypatch.setattr(mig, "_torch_allocator", limited)
+    p = _problem(144, Sensor(90, 60, 40, 30, 2.0, 8, 0.0))
+    c = mig.Context(0, stream=torch.cuda.Stream())
+    m = mig.Map(c, p.map.grid, p.map.voxel_size, p.map.origin)
+    srv = mig.Server(c, arena_budget_bytes=1 << 30, max_inflight=2)
+    try:
+        want = mig.tree_eval(m, p.tree.parent, p.tree.pos, p.sensor)
+        for kernel in (mig.COUNT_RAYS, mig.COUNT_AUTO):  # without a region for the counts, and with one
+            c.set_count_kernel(kernel, 0)
+            limit[0] = 1 << 14
+            t, _ = srv.submit(m, p.tree.parent, p.tree.pos, p.sensor)
+            with pytest.raises(mig.MigError) as e:
+                srv.poll(t, timeout_us=30_000_000)
+            assert e.value.status == mig.MIG_ENOMEM
+            limit[0] = 1 << 62
+            for _ in range(2):
+                t, got = srv.submit(m, p.tree.parent, p.tree.pos, p.sensor)
+                assert srv.poll(t, timeout_us=30_000_000)
+                for k in ("abs", "marg", "yaw"):
+                    assert np.array_equal(got[k], want[k]), k
+    finally:
+        limit[0] = 1 << 62
+        srv.close()
+        m.close()
+        c.close()
