@@ -771,11 +771,11 @@ StepsLayout steps_layout_in(const SensorDims &d, int n, int max_nodes, size_t by
     return L;
 }
 
-StepsLayout steps_pairs_in(const SensorDims &d, int max_nodes, size_t bytes) {
+StepsLayout steps_pairs_in(const SensorDims &d, size_t max_pairs, size_t bytes) {
     const size_t pair = (size_t)d.W * d.H * sizeof(uint16_t) + hz_entries(d.W, d.H) * sizeof(uint32_t), fixed = 4 * 256;
     StepsLayout L{};
     if (bytes < fixed + pair) return L;
-    L.cap = (int)std::min<long long>((long long)std::min<size_t>((bytes - fixed) / pair, INT_MAX), (long long)max_nodes * d.K);
+    L.cap = (int)std::min({(bytes - fixed) / pair, max_pairs, (size_t)1 << 30});
     place(L, d);
     return L;
 }

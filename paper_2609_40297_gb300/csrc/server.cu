@@ -150,9 +150,8 @@ void choose_region(const mig_server *s, Request &r) {
     const size_t share = s->budget / (size_t)s->max_inflight;
     const SensorDims d = steps_dims(r.sensor, r.map, r.mode);
     const bool sample = r.mode != MIG_MODE_INTERVAL && r.mode != MIG_MODE_PANORAMIC;
-    size_t counts = 0;
-    if (sample)
-        counts = (steps_pairs((long long)r.Lmax * d.K, d.W, d.H, r.count.steps_budget) * d.W * d.H * sizeof(uint16_t) + 511) & ~(size_t)255;
+    const size_t pairs = steps_pairs((long long)r.Lmax * d.K, d.W, d.H, r.count.steps_budget);  // the context's budget of step counts
+    const size_t counts = sample ? (pairs * d.W * d.H * sizeof(uint16_t) + 511) & ~(size_t)255 : 0;
     r.steps = StepsLayout{};
     const size_t bare = request_bytes(r), most = std::max(share, bare + counts);
     for (int lean = 0; lean < 2; ++lean) {
@@ -161,10 +160,11 @@ void choose_region(const mig_server *s, Request &r) {
     }
     const size_t region = most - bare, bounds = depth_bounds(r) + 256;
     r.steps = StepsLayout{};
-    if (r.count.pass != MIG_COUNT_PAIRS && bounds < region) r.steps = steps_layout_in(d, pl.n, r.Lmax, region - bounds, sample);
+    if (r.count.pass != MIG_COUNT_PAIRS && bounds < region && pairs >= (size_t)d.K)
+        r.steps = steps_layout_in(d, pl.n, (int)(pairs / d.K), region - bounds, sample);
     if (r.steps.cap == 0 && sample) {  // not one node: by (node, yaw) pairs, or ray by ray
         r.count.pass = MIG_COUNT_PAIRS;
-        r.steps = steps_pairs_in(d, r.Lmax, region);
+        r.steps = steps_pairs_in(d, pairs, region);
     }
 }
 

@@ -34,7 +34,7 @@ StepsLayout steps_layout(const SensorDims &d, int n, int max_nodes, size_t budge
 // The same for as many whole nodes as fit in a region of at most `bytes` bytes, and for single pairs (without a
 // queue) as many as fit (cap 0: not one does). with_depths: also a whole tree's depth buffers, where they fit.
 StepsLayout steps_layout_in(const SensorDims &d, int n, int max_nodes, size_t bytes, bool with_depths);
-StepsLayout steps_pairs_in(const SensorDims &d, int max_nodes, size_t bytes);
+StepsLayout steps_pairs_in(const SensorDims &d, size_t max_pairs, size_t bytes);
 void set_steps(LevelParams &p, void *base, const StepsLayout &L);  // the region's fields
 // Step-count buffer budget per evaluation (device bytes).
 constexpr size_t kStepsBudget = (size_t)1 << 30;

@@ -180,3 +180,30 @@ def test_request_is_retried_once_memory_is_there(monkeypatch):
         srv.close()
         m.close()
         c.close()
+
+
+def test_step_budget_holds_in_small_regions():
+    """A request between its level's step counts and the queue's least size takes whole nodes into what its share
+    leaves, but no more of them than the context's budget of step counts."""
+    p = _problem(145, Sensor(90, 60, 40, 30, 2.0, 8, 0.0))
+    bare = _bytes(p.tree.parent, p.sensor, False, False)
+    node = 2 * 8 * 40 * 30
+    peaks = {}
+    for nodes in (1, 3, 1000):
+        ctx = mig.Context(0, stream=torch.cuda.Stream())
+        m = mig.Map(ctx, p.map.grid, p.map.voxel_size, p.map.origin)
+        want = mig.tree_eval(m, p.tree.parent, p.tree.pos, p.sensor)
+        ctx.set_count_kernel(mig.COUNT_NODES, nodes * node + 100)
+        srv = mig.Server(ctx, arena_budget_bytes=bare + (2 << 20), max_inflight=1)
+        try:
+            t, got = srv.submit(m, p.tree.parent, p.tree.pos, p.sensor)
+            assert srv.poll(t, timeout_us=30_000_000)
+            peaks[nodes] = srv.memory()["peak"]
+            for k in ("abs", "marg", "yaw"):
+                assert np.array_equal(got[k], want[k]), k
+        finally:
+            srv.close()
+            m.close()
+            ctx.close()
+    assert bare + node < peaks[1] <= peaks[3] - 2 * node and peaks[3] <= peaks[1000] - node
+    assert peaks[1000] <= bare + (2 << 20)
