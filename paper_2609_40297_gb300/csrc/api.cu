@@ -388,8 +388,9 @@ CodeScan scan_codes(const uint8_t *v, size_t n) {
                 }
         }
         r.open += open;
-        r.entries += entries;
+        r.entries += entries;  // without those that begin a block: about one in 128
     }
+    r.entries += n > 0 && v[0] == 2;  // read before the loop, it keeps gcc from vectorizing it: 1.3 -> 12 ms for 16 MB
     return r;
 }
 
@@ -590,6 +591,7 @@ mig_status mig_map_create(mig_ctx *ctx, int nx, int ny, int nz, float voxel_size
     m->voxel = voxel_size_m;
     for (int a = 0; a < 3; ++a) m->origin[a] = origin_m ? origin_m[a] : 0.f;
     const size_t nvox = (size_t)nx * ny * nz;
+    m->open_voxels = (double)nvox;  // unknown without voxels
     if (host_voxels) {
         const CodeScan scan = scan_codes(host_voxels, nvox);
         if (scan.bad != SIZE_MAX) return bad_code(host_voxels, scan);

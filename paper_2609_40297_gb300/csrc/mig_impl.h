@@ -188,8 +188,8 @@ mig_status ctx_pinned(mig_ctx *ctx, size_t bytes, void **out);
 mig_status ctx_camera(mig_ctx *ctx, const mig_sensor &s, const Camera **out);
 // The panoramic tables of a context camera, built and uploaded on first use (ctx->mu held).
 mig_status ctx_pano(mig_ctx *ctx, const Camera *cam);
-// The codes of a box: are they codes (else the first bad index in *bad), and how many are not occupied, how many
-// of these are followed by an occupied one.
+// The codes of a box: are they codes (else the first bad index in bad), how many are not occupied, and about
+// how many runs of occupied ones begin.
 struct CodeScan {
     size_t bad = SIZE_MAX, open = 0, entries = 0;
 };

@@ -1,6 +1,7 @@
 """Which way a tree is counted by default, and both ways where only one is the default: short ranges with
 fine images, ranges far beyond the grid and coarse images (the pass that ran is in the statistics); the
 longest range (1024 voxels) ray by ray and by voxels; and a queue of undecided bricks that overflows."""
+import ctypes as C
 import math
 
 import numpy as np
@@ -49,6 +50,43 @@ def test_default_pass(ctx, dims, v, sensor, nodes, want):
     try:
         assert mig.tree_eval_stats(m, parent, pos, sensor)[1]["voxel_pass"] == want
     finally:
+        m.close()
+
+
+@pytest.mark.parametrize("writes", ["whole", "one box", "one voxel", "voxel by voxel"])
+def test_allocation_free_choice_of_a_map_written_in_parts(ctx, writes):
+    """A few occupied voxels in an empty map are no clutter, however they came there: the allocation-free call
+    counts fine images over 20 voxels of range by voxels."""
+    dims, v, n = (64, 64, 32), 0.1, 30
+    rng = np.random.default_rng(11)
+    parent, pos = _tree(rng, n, dims, v, 8)
+    sensor = Sensor(90, 60, 160, 120, 2.0, 8, 0.0)
+    grid = np.zeros(dims[::-1], np.uint8)
+    at = rng.integers(0, 32, (1 if writes == "one voxel" else 20, 3))
+    grid[at[:, 0], at[:, 1], at[:, 2]] = 2
+    m = mig.Map(ctx, grid if writes == "whole" else np.zeros_like(grid), v)
+    if writes != "whole":  # a map created without voxels, through the C call
+        m.close()
+        m.h = C.c_void_p()
+        mig.check(mig.lib().mig_map_create(ctx.h, *dims, v, (C.c_float * 3)(), None, C.byref(m.h)))
+    dev = torch.device("cuda:0")
+    try:
+        if writes == "one box":
+            m.update(0, 0, 0, np.ascontiguousarray(grid[:, :32, :32]))
+        elif writes != "whole":
+            for z, y, x in at:
+                m.update(int(x), int(y), int(z), np.full((1, 1, 1), 2, np.uint8))
+        assert np.array_equal(m.read(), grid)
+        par, p = torch.from_numpy(parent).to(dev), torch.from_numpy(pos).to(dev)
+        out = [torch.empty(n, dtype=torch.int32, device=dev) for _ in range(3)]
+        ctx.profile(True)
+        ctx.profile_read()
+        mig.tree_eval_device_noalloc(m, par, p, sensor, 4, *out)
+        ctx.sync()
+        t = ctx.profile_read()
+        assert t["cast_launches"] > 0 and t["count_launches"] == 0
+    finally:
+        ctx.profile(False)
         m.close()
 
 
